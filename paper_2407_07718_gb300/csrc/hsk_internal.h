@@ -57,6 +57,8 @@ struct SmParams {
     int rec_words;            // 2 (k <= 32) or 4 (k <= 64)
     uint32_t grid;
     uint64_t tile_begin, tile_end;     // warp tiles [begin, end) of 1024 windows (end 0 = all)
+    int desc_sub;             // 1: windows with different sub-partitions (8 hash bits above the
+                              // bucket's) are different supermers, and descriptors carry them
     uint64_t* desc;                    // supermer descriptors (DESC)
     uint64_t desc_cap;
     unsigned long long* desc_count;    // descriptors produced (may exceed desc_cap)
@@ -78,15 +80,16 @@ struct SmParams {
 size_t supermer_smem_bytes(int mode, uint32_t n_buckets);
 int supermer_max_ctas_per_sm(int mode, bool wide, int nreg, uint32_t n_buckets);
 void launch_supermer(int mode, const SmParams& p, cudaStream_t st);
-// records from descriptors: bucket_off[B+1] record offsets; cursor[b *
+// records from descriptors (and, with rec_sub, each record's sub-partition):
+// bucket_off[B+1] record offsets; cursor[b *
 // SCATTER_CURSOR_STRIDE] zeroed for every bucket b.  The cursors take every
 // descriptor's atomic: packed into 16 KB they fell into a few L2 slices, and
 // 128 bytes apart they spread over all of them (S3 took 6.2 ms packed, 5.35 ms
 // spread, on the long-read workload)
 constexpr uint32_t SCATTER_CURSOR_STRIDE = 32;
 void launch_scatter_desc(const uint64_t* desc, uint64_t n_desc, const uint64_t* packed, int k,
-                         const uint64_t* bucket_off, uint32_t* cursor, uint64_t* records, uint64_t n_records,
-                         int* err, int grid, cudaStream_t st);
+                         const uint64_t* bucket_off, uint32_t* cursor, uint64_t* records, uint8_t* rec_sub,
+                         uint64_t n_records, int* err, int grid, cudaStream_t st);
 
 // exclusive scan of n uint32 counts into uint64 offsets; offsets[n] = total.
 // Scratch: scan_status_words(n) uint64 words.
@@ -175,6 +178,26 @@ void launch_range_sort(const void* kin, const uint32_t* vin, void* kout, uint32_
 void launch_ov_gather(const uint64_t* sub_off, const uint32_t* ov_list, uint32_t n_ov, uint64_t* ov_pre,
                       int key_words, const void* keys, void* dst, uint64_t dst_cap, int* err, int grid,
                       cudaStream_t st);
+
+// ---- S4 + S5 by hashing (k_hash.cu) -------------------------------------------
+constexpr uint32_t HASH_MAX_SUB = 256;       // sub-partitions of a bucket at most
+constexpr uint64_t HASH_MAX_BASES = 1ull << 36;  // bases a descriptor with a sub-partition can address
+uint32_t hash_count_cap(int key_words);      // distinct k-mers the first tier's table holds
+void launch_split(const uint64_t* records, const uint8_t* rec_sub, const uint64_t* bucket_off, uint32_t first_bucket,
+                  uint32_t last_bucket, uint32_t nsub, int rec_words, uint64_t* out, uint64_t* part_off, int num_sms,
+                  cudaStream_t st);
+// Counts partitions (all of them, or the n_part listed in `only`): kept pairs
+// appended to (out_keys, out_counts) in no particular order, *out_n of them;
+// partitions that overfill the tier's table listed in ov_list, ov_stats =
+// {listed, their records}; dig_hist[256] += kept pairs per top digit.
+void launch_hash_count(const uint64_t* records, const uint64_t* part_off, const uint32_t* only, uint32_t n_part,
+                       int tier, int k, int nmax, uint32_t lo, uint32_t hi, void* out_keys, uint32_t* out_counts,
+                       uint64_t out_cap, uint64_t* out_n, uint32_t* ov_list, uint64_t* ov_stats, uint64_t* hist,
+                       uint32_t hist_len, uint32_t* max_count, uint64_t* n_distinct, uint64_t* dig_hist,
+                       uint32_t* claim, int* err, int num_sms, cudaStream_t st);
+void launch_list_gather(const uint64_t* records, const uint64_t* part_off, const uint32_t* list, uint32_t n_list,
+                        const uint64_t* dst_off, uint64_t* dst, uint64_t* kmers, int rec_words, int num_sms,
+                        cudaStream_t st);
 
 uint64_t rle_tiles(uint64_t n, int key_words);
 uint64_t rle_bits_words(uint64_t n);

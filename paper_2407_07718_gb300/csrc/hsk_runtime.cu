@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <atomic>
 #include <chrono>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -36,6 +37,9 @@
 #include "hsk_runtime.h"
 
 using namespace hsk;
+
+// Jobs of fewer k-mers than this take the sorting path.
+static constexpr uint64_t HASH_MIN_KMERS = 1ull << 16;
 
 // ---------------------------------------------------------------------------
 // context
@@ -425,9 +429,10 @@ static void fill_sm_params(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t 
 // With a set map the bases hold packed sets and B is the buckets of all sets.
 static_assert(HSK_MAX_BUCKETS == 8192, "the S2 walk's shared-memory limit is sized for 8192 buckets");
 int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Supermers& S, cudaStream_t st,
-                  InputPipe* pipe, const SetMap* sets) {
+                  InputPipe* pipe, const SetMap* sets, bool want_sub) {
     SmParams P;
     fill_sm_params(c, E, k, m, B, P);
+    P.desc_sub = want_sub;
     if (sets) {
         P.set_tile0 = sets->tile0;
         P.set_bucket = sets->bucket;
@@ -523,9 +528,12 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
     S.rec_words = P.rec_words;
     S.nmax = P.nmax;
     TRY(hsk_ensure(c, c->records, std::max<uint64_t>(S.n_records, 1) * P.rec_words * 8, false));
+    if (want_sub) TRY(hsk_ensure(c, c->rec_sub, std::max<uint64_t>(S.n_records, 1), false));
+    S.rec_sub = want_sub ? (const uint8_t*)c->rec_sub.p : nullptr;
     prof_mark(c, st, 1);
     launch_scatter_desc((const uint64_t*)c->cta_off.p, n_desc, E.packed, k, (const uint64_t*)c->bucket_rec.p,
-                        d_cursor, (uint64_t*)c->records.p, S.n_records, c->d_err, c->num_sms * 8, st);
+                        d_cursor, (uint64_t*)c->records.p, (uint8_t*)S.rec_sub, S.n_records, c->d_err,
+                        c->num_sms * 8, st);
     CK(cudaGetLastError());
     S.records = (const uint64_t*)c->records.p;
     return HSK_OK;
@@ -996,6 +1004,166 @@ static int local_chunk(hsk_ctx* c, const Supermers& S, const std::vector<uint32_
     return HSK_OK;
 }
 
+// Pairs of (keys, counts), n of them in any order, into the output buffers
+// partitioned by their top digit (hist: pairs per top digit, on the device):
+// stage S6's first partition.
+static int top_digit_pass(hsk_ctx* c, const void* keys, const uint32_t* counts, uint64_t n, int kw, int key_bits,
+                          const uint64_t* d_hist, cudaStream_t st) {
+    const uint64_t TILE = onesweep_tile_keys(kw);
+    const uint64_t tiles = (n + TILE - 1) / TILE;
+    TRY(hsk_ensure(c, c->s6_bounds, 2 * 257 * 8, false));
+    uint64_t* d_bounds = (uint64_t*)c->s6_bounds.p;
+    const uint64_t base[2] = {0, n};
+    CK(cudaMemcpyAsync(d_bounds + 257, base, sizeof(base), cudaMemcpyHostToDevice, st));
+    launch_digit_offsets_seg(d_hist, d_bounds + 257, d_bounds, 1, 1, st);
+    CK(cudaMemcpyAsync(d_bounds + 256, &base[1], 8, cudaMemcpyHostToDevice, st));
+    TRY(hsk_ensure_status(c, tiles * 256 + 1, st));
+    uint32_t ep, *ctr;
+    TRY(hsk_next_epoch(c, st, &ep));
+    TRY(hsk_next_counter(c, st, &ctr));
+    launch_onesweep_seg(keys, c->out_keys.p, counts, (uint32_t*)c->out_counts.p, d_bounds + 257, 1, (uint32_t)tiles,
+                        nullptr, kw, key_bits - 8, d_bounds, (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st);
+    CK(cudaGetLastError());
+    return HSK_OK;
+}
+
+// The hash path needs partitions whose distinct k-mers fit its table.  The
+// fine partitions hold n_windows / (256 B) k-mers at best, and no fewer than
+// one minimizer's: of the 4^m / 2 canonical m-mers about 2 in w + 1 are ever a
+// window's minimum, so a minimizer has about n_windows (w + 1) / 4^m k-mers.
+static bool hash_path_fits(hsk_ctx* c, uint64_t n_windows, uint32_t B, int k, int m) {
+    if (!c->cfg.local_sort || k < 12 || k > 63) return false;
+    const double cap = hash_count_cap(k <= 32 ? 1 : 2);
+    const double per_part = (double)n_windows / ((double)B * HASH_MAX_SUB);
+    const double per_min = (double)n_windows * (k - m + 2) / std::pow(4.0, m);
+    return n_windows >= HASH_MIN_KMERS && per_part <= cap && per_min <= cap;
+}
+
+// Bytes hsk_ensure would add for a buffer of `bytes`.
+static size_t buf_growth(const DevBuf& b, size_t bytes) {
+    return bytes > b.cap ? ((bytes + (2u << 20) - 1) & ~size_t((2u << 20) - 1)) - b.cap : 0;
+}
+
+// One chunk of buckets [b0, b1) through the hash path.  Kept pairs end in the
+// output buffers: partitioned by their top digit when they are the only ones.
+// *done = false (nothing counted) when the split records do not fit the
+// budget beside the pairs; the sorting path needs less.
+static int hash_chunk(hsk_ctx* c, const Supermers& S, uint32_t b0, uint32_t b1, uint64_t nk, bool single, int k,
+                      uint32_t lo, uint32_t hi, uint32_t H, Output& O, cudaStream_t st, bool* done) {
+    *done = false;
+    const int kw = k <= 32 ? 1 : 2;
+    const size_t kb = (size_t)kw * 8;
+    const uint32_t nb = b1 - b0;
+    const uint64_t rec0 = S.h_bucket_rec[b0], n_rec = S.h_bucket_rec[b1] - rec0;
+    // sub-partitions per bucket: about half the table's k-mers per partition
+    uint32_t nsub = 1;
+    while (nsub < HASH_MAX_SUB && nk > (uint64_t)nb * nsub * (hash_count_cap(kw) / 2)) nsub *= 2;
+    const uint32_t n_part = nb * nsub;
+    const uint64_t cap = nk / std::max<uint32_t>(lo, 1) + 1;  // a kept k-mer has at least lo copies
+    {
+        size_t need = buf_growth(c->keys, cap * kb) + buf_growth(c->alt, cap * 4) +
+                      buf_growth(c->hash_ctl, (size_t)n_part * 8 + 4096);
+        if (nsub > 1)
+            need += buf_growth(c->records2, n_rec * S.rec_words * 8) + buf_growth(c->part_off, ((size_t)n_part + 1) * 8);
+        if (c->allocated + need > c->budget) return HSK_OK;
+    }
+    *done = true;
+    TRY(hsk_ensure(c, c->keys, cap * kb, false));
+    TRY(hsk_ensure(c, c->alt, cap * 4, false));
+    // control words: out_n, distinct, {listed, records} x 2, kept pairs per top digit; then the two lists
+    const size_t ctl_words = 8 + 256;
+    TRY(hsk_ensure(c, c->hash_ctl, ctl_words * 8 + (size_t)n_part * 8, false));
+    uint64_t* ctl = (uint64_t*)c->hash_ctl.p;
+    uint32_t* list1 = (uint32_t*)(ctl + ctl_words);
+    uint32_t* list2 = list1 + n_part;
+    CK(cudaMemsetAsync(ctl, 0, ctl_words * 8, st));
+    const uint64_t* recs = S.records;
+    const uint64_t* part_off = (const uint64_t*)c->bucket_rec.p + b0;
+    if (nsub > 1) {
+        TRY(hsk_ensure(c, c->records2, n_rec * S.rec_words * 8, false));
+        TRY(hsk_ensure(c, c->part_off, ((uint64_t)n_part + 1) * 8, false));
+        launch_split(S.records, S.rec_sub, (const uint64_t*)c->bucket_rec.p, b0, b1, nsub, S.rec_words,
+                     (uint64_t*)c->records2.p, (uint64_t*)c->part_off.p, c->num_sms, st);
+        recs = (const uint64_t*)c->records2.p;
+        part_off = (const uint64_t*)c->part_off.p;
+    }
+    prof_mark(c, st, 3);
+    uint32_t* ctr;
+    TRY(hsk_next_counter(c, st, &ctr));
+    launch_hash_count(recs, part_off, nullptr, n_part, 0, k, S.nmax, lo, hi, c->keys.p, (uint32_t*)c->alt.p, cap, ctl,
+                      list1, ctl + 2, (uint64_t*)c->hist.p, H, c->d_max, ctl + 1, ctl + 8, ctr, c->d_err, c->num_sms,
+                      st);
+    CK(cudaGetLastError());
+    uint64_t w[6];
+    CK(cudaMemcpyAsync(w, ctl, sizeof(w), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    const uint32_t n1 = (uint32_t)w[2];
+    if (n1) {
+        TRY(hsk_next_counter(c, st, &ctr));
+        launch_hash_count(recs, part_off, list1, n1, 1, k, S.nmax, lo, hi, c->keys.p, (uint32_t*)c->alt.p, cap, ctl,
+                          list2, ctl + 4, (uint64_t*)c->hist.p, H, c->d_max, ctl + 1, ctl + 8, ctr, c->d_err,
+                          c->num_sms, st);
+        CK(cudaGetLastError());
+        CK(cudaMemcpyAsync(w, ctl, sizeof(w), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+    }
+    const uint32_t n2 = (uint32_t)w[4];
+    const uint64_t kept = w[0];
+    O.n_distinct += w[1];
+    // the split records are no longer read: give them back where the pairs need their room
+    const bool tight = c->allocated + 3 * (O.n_pairs + kept) * (kb + 4) > c->budget;
+    if (tight && n2 == 0) free_buf(c, c->records2);
+    TRY(hsk_grow_output(c, O, O.n_pairs + kept, kw, st));
+    prof_mark(c, st, 4);
+    const bool only = single && O.n_pairs == 0 && n2 == 0;
+    if (only && 2 * k >= 24 && kept > 1) {
+        TRY(top_digit_pass(c, c->keys.p, (const uint32_t*)c->alt.p, kept, kw, 2 * k, ctl + 8, st));
+        c->s6_digit_major = true;
+    } else if (kept) {
+        CK(cudaMemcpyAsync((char*)c->out_keys.p + O.n_pairs * kb, c->keys.p, kept * kb, cudaMemcpyDeviceToDevice, st));
+        CK(cudaMemcpyAsync((uint32_t*)c->out_counts.p + O.n_pairs, c->alt.p, kept * 4, cudaMemcpyDeviceToDevice, st));
+        c->s6_digit_major = false;
+    }
+    O.n_pairs += kept;
+    if (n2) {  // partitions no table holds: their records as groups of the sorting path
+        std::vector<uint32_t> list(n2);
+        std::vector<uint64_t> poff((size_t)n_part + 1);
+        CK(cudaMemcpyAsync(list.data(), list2, (size_t)n2 * 4, cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(poff.data(), part_off, ((size_t)n_part + 1) * 8, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        Supermers L;
+        L.B = n2;
+        L.rec_words = S.rec_words;
+        L.nmax = S.nmax;
+        L.h_bucket_rec.resize((size_t)n2 + 1);
+        L.h_bucket_kmers.resize(n2);
+        for (uint32_t j = 0; j < n2; ++j) {
+            L.h_bucket_rec[j] = L.n_records;
+            L.n_records += poff[(size_t)list[j] + 1] - poff[list[j]];
+        }
+        L.h_bucket_rec[n2] = L.n_records;
+        TRY(hsk_ensure(c, c->ov_records, L.n_records * S.rec_words * 8 + (size_t)n2 * 16, false));
+        uint64_t* d_off = (uint64_t*)c->ov_records.p + L.n_records * S.rec_words;
+        uint64_t* d_kmers = d_off + n2;
+        CK(cudaMemcpyAsync(d_off, L.h_bucket_rec.data(), (size_t)n2 * 8, cudaMemcpyHostToDevice, st));
+        CK(cudaMemsetAsync(d_kmers, 0, (size_t)n2 * 8, st));
+        launch_list_gather(recs, part_off, list2, n2, d_off, (uint64_t*)c->ov_records.p, d_kmers, S.rec_words,
+                           c->num_sms, st);
+        CK(cudaGetLastError());
+        CK(cudaMemcpyAsync(L.h_bucket_kmers.data(), d_kmers, (size_t)n2 * 8, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        L.records = (const uint64_t*)c->ov_records.p;
+        if (tight) free_buf(c, c->records2);
+        for (uint64_t v : L.h_bucket_kmers) L.n_kmers += v;
+        const uint64_t per_group = 256ull * local_cap(kw) / (c->tune.group_div ? c->tune.group_div : 3);
+        const uint32_t C_want = (uint32_t)std::min<uint64_t>(n2, std::max<uint64_t>(1, L.n_kmers / per_group));
+        TRY(local_chunk(c, L, hsk_group_buckets(L, 0, n2, C_want), L.n_kmers, k, lo, hi, H, O, st));
+        if (kept) c->s6_digit_major = false;
+    }
+    prof_mark(c, st, 5);
+    return HSK_OK;
+}
+
 int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, uint64_t n_reads,
                   uint64_t n_bases, int k, int m, uint32_t lo, uint32_t hi, cudaStream_t st,
                   DevResult& R, InputPipe* pipe) {
@@ -1025,11 +1193,13 @@ int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, ui
     prof_mark(c, st, 0);
     Supermers S;
     uint32_t B = hsk_pick_buckets(c, n_bases, k);
+    const bool want_sub = n_bases < HASH_MAX_BASES && hash_path_fits(c, n_bases, B, k, m);
     {
         NvtxRange r("S2-S3 supermers");
-        TRY(hsk_supermers(c, E, k, m, B, S, st, pipe));
+        TRY(hsk_supermers(c, E, k, m, B, S, st, pipe, nullptr, want_sub));
     }
     prof_mark(c, st, 2);
+    const bool hash = want_sub && hash_path_fits(c, S.n_kmers, B, k, m);
     R.n_windows = S.n_kmers;
     R.n_supermers = S.n_records;
     std::vector<std::pair<uint32_t, uint32_t>> chunks;
@@ -1043,6 +1213,13 @@ int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, ui
         uint64_t nk = 0;
         for (uint32_t b = ch.first; b < ch.second; ++b) nk += S.h_bucket_kmers[b];
         if (nk == 0) continue;
+        if (hash) {
+            NvtxRange r("S4-S5 on-chip hash count");
+            bool done = false;
+            TRY(hash_chunk(c, S, ch.first, ch.second, nk, chunks.size() == 1, k, lo, hi, H, O, st, &done));
+            unordered = true;
+            if (done) continue;
+        }
         if (c->cfg.local_sort) {
             // groups of about a third of the on-chip capacity per top digit
             const uint64_t per_group = 256ull * local_cap(kw) / (c->tune.group_div ? c->tune.group_div : 3);

@@ -157,9 +157,16 @@ __device__ __forceinline__ u64 keep_bases(u64 x, int nb) {
     return x & (~0ULL << (64 - 2 * nb));
 }
 
-// Descriptor of a supermer: start base (40 bits), k-mers (8 bits), bucket (16 bits).
-__device__ __forceinline__ u64 make_desc(u64 pos, uint32_t n, uint32_t b) {
-    return pos | ((u64)n << 40) | ((u64)b << 48);
+// Descriptor of a supermer, from its combined bucket b = bucket | sub << 13.
+// Plain: start base (40 bits), k-mers (8), bucket (16).  With sub-partitions:
+// start base (36), k-mers (7), bucket (13), sub-partition (8).
+__device__ __forceinline__ u64 make_desc(u64 pos, uint32_t n, uint32_t b, int sub) {
+    return sub ? pos | ((u64)n << 36) | ((u64)b << 43) : pos | ((u64)n << 40) | ((u64)b << 48);
+}
+__device__ __forceinline__ void split_desc(u64 d, int sub, u64& pos, uint32_t& n, uint32_t& bucket) {
+    pos = d & (sub ? (1ULL << 36) - 1 : (1ULL << 40) - 1);
+    n = sub ? (uint32_t)(d >> 36) & 0x7F : (uint32_t)(d >> 40) & 0xFF;
+    bucket = sub ? (uint32_t)(d >> 43) & 0x1FFF : (uint32_t)(d >> 48);
 }
 
 template <int MODE, bool WIDE, int NREG, bool LEX>
@@ -206,6 +213,7 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_supermer(const SmParams P) {
         const u64 p0 = t * SM_TW;
         // buckets of the tile's set (packed sets: the set holding tile t)
         uint32_t bbase = 0, bmask = B - 1u;
+        const uint32_t subs = P.desc_sub ? 0xFFu : 0u;  // sub-partition: the hash bits above the bucket's
         if (P.n_sets) {
             uint32_t lo = 0, hi = P.n_sets;  // set_tile0[lo] <= t < set_tile0[hi]
             while (hi - lo > 1) {
@@ -291,9 +299,9 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_supermer(const SmParams P) {
             if (nbuf + cnt > SM_DBUF) flush();
             if (end) {
                 const int n = plp - psm + 1;
-                atomicAdd(&s_cnt[pb], 1u);
-                atomicAdd(&s_km[pb], (uint32_t)n);
-                wdesc[nbuf + __popc(ends & ((1u << lane) - 1u))] = make_desc(p0 + psm, (uint32_t)n, pb);
+                atomicAdd(&s_cnt[pb & 0x1FFFu], 1u);
+                atomicAdd(&s_km[pb & 0x1FFFu], (uint32_t)n);
+                wdesc[nbuf + __popc(ends & ((1u << lane) - 1u))] = make_desc(p0 + psm, (uint32_t)n, pb, P.desc_sub);
             }
             nbuf += cnt;
             __syncwarp();
@@ -324,7 +332,7 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_supermer(const SmParams P) {
                 mh = min(tc, q < 32 ? a : b);
                 t_cur = t_new;
             }
-            const uint32_t b = bbase + (mh & bmask);
+            const uint32_t b = (bbase + (mh & bmask)) | (((mh >> __popc(bmask)) & subs) << 13);
 
             if (MODE == SM_DUMP) {
                 if (p < P.n_bases) {
@@ -450,7 +458,9 @@ template <bool WIDE>
 __global__ void __launch_bounds__(256) k_scatter_desc(const u64* __restrict__ desc, u64 n_desc,
                                                       const u64* __restrict__ packed, int k,
                                                       const u64* __restrict__ bucket_off, uint32_t* cursor,
-                                                      u64* __restrict__ records, u64 n_records, int* err) {
+                                                      u64* __restrict__ records, uint8_t* __restrict__ rec_sub,
+                                                      u64 n_records, int* err) {
+    const int sub = rec_sub != nullptr;
     constexpr int SD = 4;
     const u64 stride = (u64)gridDim.x * blockDim.x * SD;
     for (u64 i0 = (u64)blockIdx.x * blockDim.x * SD + threadIdx.x; i0 < n_desc; i0 += stride) {
@@ -464,20 +474,23 @@ __global__ void __launch_bounds__(256) k_scatter_desc(const u64* __restrict__ de
         for (int j = 0; j < SD; ++j) {
             slot[j] = ~0ULL;
             if (dd[j] != ~0ULL) {
-                const uint32_t b = (uint32_t)(dd[j] >> 48);
+                u64 pos;
+                uint32_t n, b;
+                split_desc(dd[j], sub, pos, n, b);
                 slot[j] = bucket_off[b] + atomicAdd(cursor + (size_t)b * SCATTER_CURSOR_STRIDE, 1u);
             }
         }
 #pragma unroll
         for (int j = 0; j < SD; ++j) {
             if (dd[j] == ~0ULL) continue;
-            const u64 d = dd[j];
-            const u64 pos = d & ((1ULL << 40) - 1);
-            const uint32_t n = (uint32_t)(d >> 40) & 0xFF, b = (uint32_t)(d >> 48);
+            u64 pos;
+            uint32_t n, b;
+            split_desc(dd[j], sub, pos, n, b);
             if (slot[j] >= n_records || slot[j] >= bucket_off[b + 1]) {
                 raise_error(err, HSK_DERR_BOUNDS);
                 continue;
             }
+            if (sub) rec_sub[slot[j]] = (uint8_t)(dd[j] >> 56);
             const int nb = (int)n + k - 1;  // bases in the record
             if (!WIDE) {
                 u64 a = keep_bases(extract_k64(packed, pos, 32), nb);
@@ -497,18 +510,18 @@ __global__ void __launch_bounds__(256) k_scatter_desc(const u64* __restrict__ de
 }
 
 void launch_scatter_desc(const uint64_t* desc, uint64_t n_desc, const uint64_t* packed, int k,
-                         const uint64_t* bucket_off, uint32_t* cursor, uint64_t* records, uint64_t n_records,
-                         int* err, int grid, cudaStream_t st) {
+                         const uint64_t* bucket_off, uint32_t* cursor, uint64_t* records, uint8_t* rec_sub,
+                         uint64_t n_records, int* err, int grid, cudaStream_t st) {
     if (n_desc == 0) return;
     count_launch();
     uint64_t need = (n_desc + 4 * 256 - 1) / (4 * 256);  // four descriptors a thread
     unsigned g = (unsigned)(need < (uint64_t)grid ? need : (uint64_t)grid);
     if (k <= 32)
         k_scatter_desc<false><<<g, 256, 0, st>>>((const u64*)desc, n_desc, (const u64*)packed, k,
-                                                 (const u64*)bucket_off, cursor, (u64*)records, n_records, err);
+                                                 (const u64*)bucket_off, cursor, (u64*)records, rec_sub, n_records, err);
     else
         k_scatter_desc<true><<<g, 256, 0, st>>>((const u64*)desc, n_desc, (const u64*)packed, k,
-                                                (const u64*)bucket_off, cursor, (u64*)records, n_records, err);
+                                                (const u64*)bucket_off, cursor, (u64*)records, rec_sub, n_records, err);
 }
 
 // ---------------------------------------------------------------------------
