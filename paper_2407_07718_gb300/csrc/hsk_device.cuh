@@ -55,6 +55,12 @@ __device__ __forceinline__ u64 reverse_pairs(u64 x) {
     return ((x >> 1) & 0x5555555555555555ULL) | ((x & 0x5555555555555555ULL) << 1);
 }
 
+// Reverse complement of the 16 bases of a 32-bit word.
+__device__ __forceinline__ uint32_t revcomp32(uint32_t x) {
+    x = __brev(~x);
+    return ((x >> 1) & 0x55555555u) | ((x << 1) & 0xAAAAAAAAu);
+}
+
 // Reverse complement of a right-aligned code of k <= 32 bases.
 __device__ __forceinline__ u64 revcomp64(u64 fwd, int k) {
     return reverse_pairs(~fwd) >> (64 - 2 * k);

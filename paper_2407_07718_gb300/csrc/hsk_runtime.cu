@@ -1032,7 +1032,7 @@ static int top_digit_pass(hsk_ctx* c, const void* keys, const uint32_t* counts, 
 // one minimizer's: of the 4^m / 2 canonical m-mers about 2 in w + 1 are ever a
 // window's minimum, so a minimizer has about n_windows (w + 1) / 4^m k-mers.
 static bool hash_path_fits(hsk_ctx* c, uint64_t n_windows, uint32_t B, int k, int m) {
-    if (!c->cfg.local_sort || k < 12 || k > 63) return false;
+    if (!c->cfg.local_sort || k < 12) return false;
     const double cap = hash_count_cap(k <= 32 ? 1 : 2);
     const double per_part = (double)n_windows / ((double)B * HASH_MAX_SUB);
     const double per_min = (double)n_windows * (k - m + 2) / std::pow(4.0, m);

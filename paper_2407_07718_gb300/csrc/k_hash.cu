@@ -12,21 +12,22 @@
 //   k_split       -- records of a bucket -> its fine partitions (one CTA per
 //                    bucket: count, scan, scatter; no global atomics).
 //   k_hash_count  -- per batch of whole partitions: equal records are merged
-//                    first (reads of the same locus repeat whole supermers, and
-//                    the record of the other strand is the reverse complement),
-//                    then the k-mers of each distinct record are added to the
-//                    table with the record's multiplicity.  When the table is
-//                    full it is emptied: statistics, filter, kept pairs.
-//                    Tier 1 is the same kernel with a table of one CTA per SM,
-//                    for the partitions that overfill tier 0's; what overfills
-//                    that is listed for the sorting path (k_local.cu).
+//                    first (reads of the same locus repeat whole supermers;
+//                    the records come in one orientation for both strands),
+//                    then the k-mers of each distinct record are hashed with
+//                    the record's multiplicity, equal ones merged, and the
+//                    counts go to the statistics, the filter and the output.
+//                    Tier 1 is the same kernel with one CTA per SM and a
+//                    larger batch, for partitions that overfill tier 0's;
+//                    what overfills that is listed for the sorting path
+//                    (k_local.cu).
 //   k_list_gather -- records of listed partitions -> one array for that path.
 //
 // What it replaces and measured (one GB300): writing every key to its (group,
 // top digit) sub-segment and sorting the sub-segments on chip (k_local.cu)
 // took 39 ms on 1.5 G windows of 30x long reads (k = 31) and 45 ms on 1.27 G
 // of 20x short reads (k = 55); the split takes 2.1 and 1.3 ms, the counting
-// 10.2 and 26.8 ms.
+// 4.9 and 13.0 ms.
 #include "hsk_device.cuh"
 
 namespace hsk {
@@ -111,82 +112,116 @@ void launch_split(const uint64_t* records, const uint8_t* rec_sub, const uint64_
 // ---------------------------------------------------------------------------
 // count the k-mers of partitions in a shared-memory table
 // ---------------------------------------------------------------------------
-// SLOTS table slots (a multiple of NT), RB records per batch, DS slots of the
-// record table (a power of two, at least 2 * RB).
+// A batch holds RB records and ENT k-mers of distinct records at most; 2^LS
+// hash slots (of k-mers, and before them of records).
+//
+// Equal k-mers find each other without a probe sequence: every k-mer of the
+// batch has an entry of its own (key, count) and writes its entry's number to
+// the slot of its hash.  After a barrier the number in the slot is the
+// winner: a k-mer that is not the winner but equal to it adds its count to
+// the winner's; one that differs goes to the next round, with another hash.
+// All copies of a k-mer take the same slots, so they either merge or go on
+// together.  Nothing waits or loops in the first round, which settles most
+// k-mers.  What bounds the kernel is instructions and the barriers between
+// its phases (about half the issue slots used); an open-addressing table with
+// compare-and-swap took three times the instructions, as the lanes of a warp
+// wait for its longest probe sequence: 10.2 and 26.8 ms on the two workloads
+// above (four tags read at once 10.2 and 27.7), against 4.9 and 13.0.
+//
+// Sizes, by trial.  64-bit keys, on the long reads and on 8x short reads of a
+// 20 Mbp genome: 384 threads x 3 CTAs and 3072 entries 5.1 and 0.74 ms, 512 x
+// 2 and 4096 5.8 and 0.92, 256 x 4 and 2304 5.5 and 0.77.  128-bit keys, on
+// the short reads: 512 x 2 and 3840 entries 12.9 ms, 3584 13.3, 1024 x 1 and
+// 7680 14.1.
 template <bool WIDE, int TIER>
 struct HashCfg;
 template <>
 struct HashCfg<false, 0> {
-    static constexpr int NT = 512, CTAS = 2, SLOTS = 6656, RB = 1024, DS = 2048;
+    static constexpr int NT = 384, CTAS = 3, ENT = 3072, LS = 13, RB = 768;
 };
 template <>
 struct HashCfg<false, 1> {
-    static constexpr int NT = 1024, CTAS = 1, SLOTS = 15360, RB = 1024, DS = 2048;
+    static constexpr int NT = 1024, CTAS = 1, ENT = 8192, LS = 14, RB = 4096;
 };
 template <>
 struct HashCfg<true, 0> {
-    static constexpr int NT = 512, CTAS = 2, SLOTS = 4096, RB = 512, DS = 1024;
+    static constexpr int NT = 512, CTAS = 2, ENT = 3840, LS = 13, RB = 384;
 };
 template <>
 struct HashCfg<true, 1> {
-    static constexpr int NT = 512, CTAS = 1, SLOTS = 9216, RB = 512, DS = 1024;
+    static constexpr int NT = 512, CTAS = 1, ENT = 6144, LS = 14, RB = 1536;
 };
 constexpr int HC_HS = 128;      // count-histogram bins kept in shared memory
-constexpr int HC_SEG = 8;       // k-mers of a record one lane adds at a time
+constexpr int HC_SEG = 16;      // k-mers of a record one lane takes at a time (at most 16)
 constexpr int HC_CHUNK = 32;    // most partitions claimed at a time
-constexpr int HC_PROBES = 512;  // a longer probe sequence means that the table is full
-constexpr u64 HC_EMPTY = ~0ULL; // never a stored key word (see insert)
-constexpr uint32_t HC_NONE = 0xFFFFFFFFu;
 
-template <bool WIDE, int TIER>
-constexpr uint32_t hash_cap() { return HashCfg<WIDE, TIER>::SLOTS / 32 * 27; }  // distinct k-mers held at most
-
-uint32_t hash_count_cap(int key_words) { return key_words == 1 ? hash_cap<false, 0>() : hash_cap<true, 0>(); }
+uint32_t hash_count_cap(int key_words) { return key_words == 1 ? HashCfg<false, 0>::ENT : HashCfg<true, 0>::ENT; }
 
 template <bool WIDE, int TIER>
 constexpr size_t hash_smem() {
     using C = HashCfg<WIDE, TIER>;
-    return (size_t)C::SLOTS * ((WIDE ? 16 : 8) + 4) + (size_t)C::RB * (WIDE ? 32 : 16) + (size_t)C::DS * 4 +
-           (size_t)C::RB * 4;
+    return (size_t)C::ENT * ((WIDE ? 16 : 8) + 4) + (size_t)C::RB * ((WIDE ? 32 : 16) + 4 + 2) + ((size_t)2 << C::LS);
 }
 
-// Bases of a record (left aligned, nb of them, the rest 0) reversed and
-// complemented, left aligned again.
+// A record's segment of HC_SEG k-mers, in 32-bit words: the bases from the
+// first k-mer on, and their reverse complements shifted so that the first
+// k-mer's is left aligned in r[1..], the bases that later k-mers shift in
+// being in r[0].
 template <bool WIDE>
-__device__ __forceinline__ void record_revcomp(const u64 (&W)[4], uint32_t nb, u64 (&R)[4]) {
-    if constexpr (!WIDE) {
-        const u64 x0 = reverse_pairs(~W[1]), x1 = reverse_pairs(~W[0]);  // right aligned
-        const uint32_t s = 128 - 2 * nb;
-        if (s >= 64) {
-            R[0] = x1 << (s - 64);  // nb <= 32 here; s = 128 (no bases) does not occur
-            R[1] = 0;
-        } else {
-            R[0] = s ? (x0 << s) | (x1 >> (64 - s)) : x0;
-            R[1] = x1 << s;
-        }
-        R[2] = R[3] = 0;
-    } else {
-        u64 x[5];
+struct SegWords {
+    static constexpr int N = WIDE ? 4 : 2;   // words of a key
+    uint32_t f[N + 1], r[N + 1];
+    // words w (2 * RW of them, the record's), segment s, k-mer length k
+    __device__ __forceinline__ void load(uint32_t (&w)[WIDE ? 8 : 4], int s, int k) {
+        constexpr int NW = WIDE ? 8 : 4;
+        const int b0 = HC_SEG * s;  // first base; s is the same in the whole warp
+        for (int q = b0 >> 4; q > 0; --q) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) x[i] = reverse_pairs(~W[3 - i]);
-        x[4] = 0;
-        uint32_t s = 256 - 2 * nb;  // < 256
-        if (s >= 128) {
-            x[0] = x[2];
-            x[1] = x[3];
-            x[2] = x[3] = 0;
-            s -= 128;
+            for (int i = 0; i < NW; ++i) w[i] = i + 1 < NW ? w[i + 1] : 0u;
         }
-        if (s >= 64) {
-            x[0] = x[1];
-            x[1] = x[2];
-            x[2] = x[3];
-            x[3] = 0;
-            s -= 64;
+        if (b0 & 15) {
+#pragma unroll
+            for (int i = 0; i < NW; ++i) w[i] = __funnelshift_l(i + 1 < NW ? w[i + 1] : 0u, w[i], 2 * (b0 & 15));
+        }
+        // the first 16 (N + 1) bases reversed and complemented; the first k-mer
+        // starts at base 16 (N + 1) - k of them (16 or more: k <= 16 N)
+        uint32_t x[N + 4];
+#pragma unroll
+        for (int i = 0; i <= N; ++i) {
+            f[i] = w[i];
+            x[i] = revcomp32(w[N - i]);
+        }
+        x[N + 1] = x[N + 2] = x[N + 3] = 0;
+        const int o = 2 * (16 * (N + 1) - k);
+        if (o >= 64) {
+#pragma unroll
+            for (int i = 0; i < N + 3; ++i) x[i] = x[i + 1];
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) R[i] = funnel64(x[i], x[i + 1], s);
+        for (int i = 0; i <= N; ++i) r[i] = __funnelshift_l(x[i + 1], x[i], o & 31);
     }
+    // the next k-mer
+    __device__ __forceinline__ void step() {
+#pragma unroll
+        for (int i = 0; i < N; ++i) f[i] = __funnelshift_l(f[i + 1], f[i], 2);
+        f[N] <<= 2;
+#pragma unroll
+        for (int i = N; i > 0; --i) r[i] = __funnelshift_r(r[i], r[i - 1], 2);
+        r[0] >>= 2;
+    }
+};
+
+// Slot (of 2^LS) of a key in round `round`.
+template <int LS>
+__device__ __forceinline__ uint32_t key_slot(u64 key, uint32_t round) {
+    const uint32_t x = (uint32_t)key * 0x9E3779B1u + (uint32_t)(key >> 32) * 0x85EBCA77u;
+    return ((x ^ (x >> 15)) * (0x2C1B3C6Du + 2 * round)) >> (32 - LS);
+}
+template <int LS>
+__device__ __forceinline__ uint32_t key_slot(const key128& key, uint32_t round) {
+    const uint32_t x = (uint32_t)key.lo * 0x9E3779B1u + (uint32_t)(key.lo >> 32) * 0x85EBCA77u +
+                       (uint32_t)key.hi * 0xC2B2AE3Du + (uint32_t)(key.hi >> 32) * 0x27D4EB2Fu;
+    return ((x ^ (x >> 15)) * (0x2C1B3C6Du + 2 * round)) >> (32 - LS);
 }
 
 struct HashArgs {
@@ -216,44 +251,221 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
     k_hash_count(const __grid_constant__ HashArgs P) {
     using Cfg = HashCfg<WIDE, TIER>;
     using K = typename std::conditional<WIDE, key128, u64>::type;
-    constexpr int NT = Cfg::NT, NW = NT / 32, SLOTS = Cfg::SLOTS, RB = Cfg::RB, DS = Cfg::DS;
+    constexpr int NT = Cfg::NT, NW = NT / 32, ENT = Cfg::ENT, LS = Cfg::LS, RB = Cfg::RB;
     constexpr int RW = WIDE ? 4 : 2;
-    constexpr int RPT = (RB + NT - 1) / NT;  // records a thread stages per batch
-    constexpr uint32_t CAP = hash_cap<WIDE, TIER>();
-    static_assert(SLOTS % NT == 0 && DS >= 2 * RB && RB <= 1024, "table sizes");
+    constexpr int RPT = (RB + NT - 1) / NT;  // records a thread takes per batch
+    static_assert(ENT <= 65536 && RB <= 65536 && (ENT + 3) / 4 <= RB * RW, "16-bit numbers; the lists fit the records' room");
     extern __shared__ __align__(16) unsigned char smem_hc[];
-    u64* tk = reinterpret_cast<u64*>(smem_hc);                       // [SLOTS] keys (WIDE: their high words)
-    u64* tk2 = tk + SLOTS;                                           // WIDE: [SLOTS] low words
-    u64* s_rec = tk + (size_t)SLOTS * (WIDE ? 2 : 1);                // [RB * RW]
-    uint32_t* tc = reinterpret_cast<uint32_t*>(s_rec + (size_t)RB * RW);  // [SLOTS] counts
-    uint32_t* s_ds = tc + SLOTS;                                     // [DS] record table: index | copies << 16
-    uint32_t* s_ord = s_ds + DS;                                     // [RB] distinct records, longest first
-    __shared__ uint32_t s_bin[128], s_base[128];                     // distinct records by k-mers; first place of each
+    K* ek = reinterpret_cast<K*>(smem_hc);                           // [ENT] keys, left aligned
+    u64* s_rec = reinterpret_cast<u64*>(ek + ENT);                   // [RB * RW] records
+    uint16_t* s_list = reinterpret_cast<uint16_t*>(s_rec);           // [ENT] then: entries left for the next round
+    uint32_t* ec = reinterpret_cast<uint32_t*>(s_rec + (size_t)RB * RW);  // [ENT] counts
+    uint32_t* s_w = ec + ENT;                                        // [RB] copies of a record
+    uint16_t* s_slot = reinterpret_cast<uint16_t*>(s_w + RB);        // [2^LS]
+    uint16_t* s_ord = s_slot + (1 << LS);                            // [RB] distinct records, longest first
+    // distinct records by their number of k-mers; records of more than t k-mers
+    // (the first place of t in the order); entry of the first record's k-mer t
+    __shared__ uint32_t s_bin[128], s_base[128], s_ent[128];
     __shared__ uint32_t s_hist[HC_HS], s_dig[256], s_wk[NW];
     __shared__ u64 s_off[HC_CHUNK + 1], s_obase;
-    __shared__ uint32_t s_claim, s_U, s_D, s_fail;
+    __shared__ uint32_t s_claim, s_U, s_nl[2];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t hs = P.hist_len < (uint32_t)HC_HS ? P.hist_len : (uint32_t)HC_HS;
     const int k = P.k;
+    const u64 mask = ~0ULL << (WIDE ? 128 - 2 * k : 64 - 2 * k);  // a left-aligned key's (low) word
 
-    for (int i = tid; i < SLOTS; i += NT) {
-        tk[i] = HC_EMPTY;
-        if (WIDE) tk2[i] = HC_EMPTY;
-        tc[i] = 0;
-    }
-    for (int i = tid; i < DS; i += NT) s_ds[i] = HC_NONE;
     for (int i = tid; i < HC_HS; i += NT) s_hist[i] = 0;
     for (int i = tid; i < 256; i += NT) s_dig[i] = 0;
     if (tid < 128) s_bin[tid] = 0;
-    if (tid == 0) s_U = s_D = s_fail = 0;
+    if (tid < 2) s_nl[tid] = 0;
     u64 my_distinct = 0;
     uint32_t my_max = 0, my_ones = 0;
 
-    // Empties the table: every slot is one distinct k-mer with its count.
-    auto flush = [&]() {
+    // Records [r0, r0 + nr) into shared memory, equal ones merged (most of
+    // them: a record that meets another one in its slot stays distinct).
+    // Returns the k-mers of the distinct ones; when they fit, s_ord lists
+    // those records, longest first.
+    auto stage = [&](u64 r0, uint32_t nr) -> uint32_t {
+        uint32_t rn[RPT], rr[RPT];  // k-mers | slot << 16 of this thread's records; place among equal lengths
+#pragma unroll
+        for (int j = 0; j < RPT; ++j) {
+            const uint32_t i = (uint32_t)j * NT + tid;
+            rn[j] = 0;
+            if (i >= nr) continue;
+            const uint4* src = reinterpret_cast<const uint4*>(P.rec + (r0 + i) * RW);
+            uint4* dst = reinterpret_cast<uint4*>(s_rec + (size_t)i * RW);
+            const uint4 a = src[0];
+            dst[0] = a;
+            uint32_t x = a.x * 0x9E3779B1u + a.y * 0x85EBCA77u + a.z * 0xC2B2AE3Du + a.w * 0x27D4EB2Fu;
+            uint32_t n = a.z & 0x7Fu;
+            if (WIDE) {
+                const uint4 b = src[1];
+                dst[1] = b;
+                x += b.x * 0x165667B1u + b.y * 0xD3A2646Du + b.z * 0xFD7046C5u + b.w * 0xB55A4F09u;
+                n = b.z & 0x7Fu;
+            }
+            const uint32_t h = ((x ^ (x >> 15)) * 0x2C1B3C6Du) >> (32 - LS);
+            *(volatile uint16_t*)&s_slot[h] = (uint16_t)i;
+            s_w[i] = 1;
+            rn[j] = n | (h << 16);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < RPT; ++j) {
+            const uint32_t i = (uint32_t)j * NT + tid, n = rn[j] & 0xFFFFu;
+            if (i >= nr) continue;
+            const uint32_t win = s_slot[rn[j] >> 16];
+            if (win != i) {
+                const uint4* a = reinterpret_cast<const uint4*>(s_rec + (size_t)i * RW);
+                const uint4* b = reinterpret_cast<const uint4*>(s_rec + (size_t)win * RW);
+                const uint4 u = a[0], v = b[0];
+                bool eq = u.x == v.x && u.y == v.y && u.z == v.z && u.w == v.w;
+                if (WIDE && eq) {
+                    const uint4 u1 = a[1], v1 = b[1];
+                    eq = u1.x == v1.x && u1.y == v1.y && u1.z == v1.z && u1.w == v1.w;
+                }
+                if (eq) {
+                    atomicAdd(&s_w[win], 1u);
+                    rn[j] = 0;
+                    continue;
+                }
+            }
+            rr[j] = atomicAdd(&s_bin[n], 1u);
+        }
+        __syncthreads();
+        if (warp == 0) {
+            // s_base[t] = records of more than t k-mers, s_ent[t] = its sum over the t before
+            uint32_t c[4], sum = 0;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                c[t] = s_bin[127 - 4 * lane - t];
+                sum += c[t];
+            }
+            uint32_t e = warp_incl_sum<uint32_t>(sum) - sum;
+            sum = 0;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                s_base[127 - 4 * lane - t] = e;
+                sum += e;
+                e += c[t];
+                c[t] = e - c[t];
+            }
+            const uint32_t inc = warp_incl_sum<uint32_t>(sum);
+            const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
+            uint32_t g = total - inc;
+#pragma unroll
+            for (int t = 3; t >= 0; --t) {
+                s_ent[127 - 4 * lane - t] = g;
+                g += c[t];
+            }
+            if (lane == 0) s_U = total;
+        }
+        __syncthreads();
+        const uint32_t U = s_U;
+        if (tid < 128) s_bin[tid] = 0;
+        if (U <= (uint32_t)ENT) {
+#pragma unroll
+            for (int j = 0; j < RPT; ++j)
+                if (rn[j] & 0xFFFFu) s_ord[s_base[rn[j] & 0xFFFFu] + rr[j]] = (uint16_t)((uint32_t)j * NT + tid);
+        }
+        __syncthreads();
+        return U;
+    };
+
+    // The k-mers of the staged distinct records: key, count and slot of each.
+    // A warp takes 32 records' k-mers [HC_SEG s, HC_SEG s + HC_SEG); the order
+    // by length keeps its lanes equally busy, and k-mer t of the q-th record
+    // is entry D + s_ent[t] + q, so the lanes write side by side.
+    auto expand = [&](uint32_t D) {
+        uint32_t t = warp;
+        for (int s = 0; HC_SEG * s < P.rec_n; ++s) {
+            const uint32_t ge = s_base[HC_SEG * s], tiles = (ge + 31) / 32;
+            for (; t < tiles; t += NW) {
+                const uint32_t q = t * 32 + lane;
+                if (q < ge) {
+                    const uint32_t i = s_ord[q], w = s_w[i];
+                    uint32_t W[2 * RW];
+                    const uint4* d = reinterpret_cast<const uint4*>(s_rec + (size_t)i * RW);
+#pragma unroll
+                    for (int y = 0; y < RW / 2; ++y) {  // words of 64 bits, low half first
+                        const uint4 v = d[y];
+                        W[4 * y] = v.y;
+                        W[4 * y + 1] = v.x;
+                        W[4 * y + 2] = v.w;
+                        W[4 * y + 3] = v.z;
+                    }
+                    const int nk = min((int)(W[2 * RW - 1] & 0x7Fu) - HC_SEG * s, HC_SEG);
+                    SegWords<WIDE> S;
+                    S.load(W, s, k);
+                    for (int j = 0; j < nk; ++j) {
+                        K key;
+                        if constexpr (WIDE) {
+                            const u64 fh = ((u64)S.f[0] << 32) | S.f[1], fl = ((u64)S.f[2] << 32) | S.f[3];
+                            const u64 rh = ((u64)S.r[1] << 32) | S.r[2], rl = ((u64)S.r[3] << 32) | S.r[4];
+                            const bool fwd = fh < rh || (fh == rh && fl < rl);
+                            key.hi = fwd ? fh : rh;
+                            key.lo = (fwd ? fl : rl) & mask;
+                        } else {
+                            const u64 f = ((u64)S.f[0] << 32) | S.f[1], r = ((u64)S.r[1] << 32) | S.r[2];
+                            key = (f < r ? f : r) & mask;
+                        }
+                        S.step();
+                        const uint32_t own = D + s_ent[HC_SEG * s + j] + q;
+                        ek[own] = key;
+                        ec[own] = w;
+                        *(volatile uint16_t*)&s_slot[key_slot<LS>(key, 0)] = (uint16_t)own;
+                    }
+                }
+            }
+            t -= tiles;
+        }
+    };
+
+    // Entry i after its slot was written: merged into the winner, or listed
+    // for the next round.
+    auto settle = [&](uint32_t i, uint32_t round, uint32_t* nl) {
+        const K key = ek[i];
+        const uint32_t win = s_slot[key_slot<LS>(key, round)];
+        if (win != i) {
+            if (key_eq(ek[win], key)) {
+                atomicAdd(&ec[win], ec[i]);
+                ec[i] = 0;
+            } else {
+                s_list[atomicAdd(nl, 1u)] = (uint16_t)i;
+            }
+        }
+    };
+    // Merges equal k-mers of U entries.
+    auto merge = [&](uint32_t U) {
+        for (uint32_t i = tid; i < U; i += NT) settle(i, 0, &s_nl[0]);
+        __syncthreads();
+        for (uint32_t round = 1;; ++round) {  // at least one key a slot is settled every round
+            const uint32_t nl = s_nl[(round - 1) & 1];
+            if (nl == 0) break;
+            // this thread's entries, in registers: the list is written again
+            constexpr int LPT = (ENT + NT - 1) / NT;
+            uint32_t e[LPT];
+#pragma unroll
+            for (int j = 0; j < LPT; ++j) {
+                const uint32_t q = (uint32_t)j * NT + tid;
+                e[j] = q < nl ? s_list[q] : 0xFFFFFFFFu;
+                if (q < nl) *(volatile uint16_t*)&s_slot[key_slot<LS>(ek[e[j]], round)] = (uint16_t)e[j];
+            }
+            if (tid == 0) s_nl[round & 1] = 0;
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < LPT; ++j)
+                if (e[j] != 0xFFFFFFFFu) settle(e[j], round, &s_nl[round & 1]);
+            __syncthreads();
+        }
+        if (tid < 2) s_nl[tid] = 0;  // read next after later barriers
+    };
+
+    // Statistics, filter and kept pairs of the U merged entries (count 0: merged into another).
+    auto emit = [&](uint32_t U) {
         uint32_t kept = 0;
-        for (int i = tid; i < SLOTS; i += NT) {
-            const uint32_t cnt = tc[i];
+        for (uint32_t i = tid; i < U; i += NT) {
+            const uint32_t cnt = ec[i];
             if (!cnt) continue;
             ++my_distinct;
             if (cnt == 1) {
@@ -278,27 +490,27 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
                 u64 at = total ? atomicAdd(P.out_n, (unsigned long long)total) : 0ULL;
                 if (at + total > P.out_cap) {
                     raise_error(P.err, HSK_DERR_BOUNDS);
-                    at = HC_EMPTY;
+                    at = ~0ULL;
                 }
-                s_obase = at;
-                s_D = 0;
+                s_obase = total ? at : ~0ULL;
             }
         }
         __syncthreads();
-        const bool ok = s_obase != HC_EMPTY;
+        if (s_obase == ~0ULL) return;  // nothing kept
         u64 at = s_obase + s_wk[warp];
-        for (int i = tid; i < SLOTS; i += NT) {
-            const uint32_t cnt = tc[i];
-            const bool keep = ok && cnt && cnt >= P.lo && cnt <= P.hi;
+        for (uint32_t i0 = 0; i0 < U; i0 += NT) {
+            const uint32_t i = i0 + tid;
+            const uint32_t cnt = i < U ? ec[i] : 0u;
+            const bool keep = cnt && cnt >= P.lo && cnt <= P.hi;
             const uint32_t km = __ballot_sync(0xffffffffu, keep);
             if (keep) {
-                K key;
+                K key = ek[i];
                 if constexpr (WIDE) {
-                    const u64 h = tk[i], l = tk2[i];
-                    key.hi = h >> 2;
-                    key.lo = (h << 62) | l;
+                    const int sh = 128 - 2 * k;  // 0 .. 62
+                    key.lo = sh ? (key.lo >> sh) | (key.hi << (64 - sh)) : key.lo;
+                    key.hi >>= sh;
                 } else {
-                    key = tk[i];
+                    key >>= 64 - 2 * k;
                 }
                 atomicAdd(&s_dig[key_digit(key, P.dshift, 0xFF)], 1u);
                 const u64 o = at + (uint32_t)__popc(km & ((1u << lane) - 1u));
@@ -306,214 +518,78 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
                 P.out_counts[o] = cnt;
             }
             at += (uint32_t)__popc(km);
-            tk[i] = HC_EMPTY;
-            if (WIDE) tk2[i] = HC_EMPTY;
-            tc[i] = 0;
         }
-        __syncthreads();
-    };
-    // Empties the table without counting anything (a partition that overfilled it).
-    auto discard = [&]() {
-        for (int i = tid; i < SLOTS; i += NT) {
-            tk[i] = HC_EMPTY;
-            if (WIDE) tk2[i] = HC_EMPTY;
-            tc[i] = 0;
-        }
-        if (tid == 0) s_D = s_fail = 0;
-        __syncthreads();
     };
 
-    // Records [r0, r0 + nr) into shared memory, each in the smaller of its two
-    // orientations, equal ones merged.  Returns the k-mers of the distinct
-    // ones (s_U); s_ord lists them, longest first, with their copies.
-    auto stage = [&](u64 r0, uint32_t nr) -> uint32_t {
-        uint32_t rn[RPT], rr[RPT], rh[RPT];
-        uint32_t u = 0;
-#pragma unroll
-        for (int j = 0; j < RPT; ++j) {
-            const uint32_t i = (uint32_t)j * NT + tid;
-            rn[j] = 0;
-            if (i >= nr) continue;
-            u64 W[4] = {0, 0, 0, 0}, R[4];
-            const ulonglong2* q = reinterpret_cast<const ulonglong2*>(P.rec + (r0 + i) * RW);
-            const ulonglong2 a = q[0];
-            W[0] = a.x;
-            W[1] = a.y;
-            if (WIDE) {
-                const ulonglong2 b = q[1];
-                W[2] = b.x;
-                W[3] = b.y;
+    // Moves the entries in use to the front; returns their number.
+    auto close_up = [&](uint32_t D) -> uint32_t {
+        uint32_t at = 0;
+        for (uint32_t i0 = 0; i0 < D; i0 += NT) {  // in order: no entry is overwritten before it is read
+            const uint32_t i = i0 + tid;
+            const uint32_t cnt = i < D ? ec[i] : 0u;
+            K key{};
+            if (cnt) key = ek[i];
+            const uint32_t m = __ballot_sync(0xffffffffu, cnt != 0);
+            if (lane == 0) s_wk[warp] = (uint32_t)__popc(m);
+            __syncthreads();
+            uint32_t pos = at;
+            for (int w = 0; w < NW; ++w) {
+                if (w < warp) pos += s_wk[w];
+                at += s_wk[w];
             }
-            const uint32_t n = (uint32_t)(W[RW - 1] & 0x7F);
-            W[RW - 1] &= ~0xFFULL;
-            record_revcomp<WIDE>(W, n + k - 1, R);
-            bool less = R[0] < W[0];
-            if (!WIDE) {
-                less = less || (R[0] == W[0] && R[1] < W[1]);
-            } else if (R[0] == W[0]) {
-                less = R[1] < W[1] || (R[1] == W[1] && (R[2] < W[2] || (R[2] == W[2] && R[3] < W[3])));
+            if (cnt) {
+                pos += (uint32_t)__popc(m & ((1u << lane) - 1u));
+                ek[pos] = key;
+                ec[pos] = cnt;
             }
-            if (less) {
-#pragma unroll
-                for (int t = 0; t < RW; ++t) W[t] = R[t];
-            }
-            W[RW - 1] |= n;
-            ulonglong2* d = reinterpret_cast<ulonglong2*>(s_rec + (size_t)i * RW);
-            d[0] = make_ulonglong2(W[0], W[1]);
-            if (WIDE) d[1] = make_ulonglong2(W[2], W[3]);
-            __threadfence_block();
-            uint32_t x = (uint32_t)W[0] * 0x9E3779B1u + (uint32_t)(W[0] >> 32) * 0x85EBCA77u +
-                         (uint32_t)W[1] * 0xC2B2AE3Du + (uint32_t)(W[1] >> 32) * 0x27D4EB2Fu;
-            if (WIDE)
-                x += (uint32_t)W[2] * 0x165667B1u + (uint32_t)(W[2] >> 32) * 0xD3A2646Du +
-                     (uint32_t)W[3] * 0xFD7046C5u + (uint32_t)(W[3] >> 32) * 0xB55A4F09u;
-            uint32_t h = (x ^ (x >> 15)) & (DS - 1);
-            for (;;) {  // at most RB of the DS slots are taken: this ends
-                uint32_t prev = *(volatile uint32_t*)&s_ds[h];
-                if (prev == HC_NONE) prev = atomicCAS(&s_ds[h], HC_NONE, i | (1u << 16));
-                if (prev == HC_NONE) {
-                    rn[j] = n;
-                    rh[j] = h;
-                    u += n;
-                    break;
-                }
-                const volatile u64* o = s_rec + (size_t)(prev & 0xFFFFu) * RW;
-                bool eq = o[0] == W[0] && o[1] == W[1];
-                if (WIDE) eq = eq && o[2] == W[2] && o[3] == W[3];
-                if (eq) {
-                    atomicAdd(&s_ds[h], 1u << 16);
-                    break;
-                }
-                h = (h + 1) & (DS - 1);
-            }
-            if (rn[j]) rr[j] = atomicAdd(&s_bin[n], 1u);
+            __syncthreads();
         }
-        u = __reduce_add_sync(0xffffffffu, u);
-        if (lane == 0 && u) atomicAdd(&s_U, u);
-        __syncthreads();
-        if (warp == 0) {  // first place of each length, longest first
-            uint32_t c[4], sum = 0;
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                c[t] = s_bin[127 - 4 * lane - t];
-                sum += c[t];
-            }
-            uint32_t e = warp_incl_sum<uint32_t>(sum) - sum;
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                s_base[127 - 4 * lane - t] = e;
-                e += c[t];
-            }
-        }
-        const uint32_t U = s_U;
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < RPT; ++j)
-            if (rn[j]) s_ord[s_base[rn[j]] + rr[j]] = ((uint32_t)j * NT + tid) | (s_ds[rh[j]] & 0xFFFF0000u);
-        if (tid < 128) s_bin[tid] = 0;
-        if (tid == 0) s_U = 0;
-        __syncthreads();
-        for (int i = tid; i < DS; i += NT) s_ds[i] = HC_NONE;
-        return U;
+        return at;
     };
-
-    // The k-mers of the staged distinct records into the table.  A warp takes
-    // 32 records' k-mers [8 s, 8 s + 8); the order by length keeps its lanes
-    // equally busy.  s_base[8 s] is the number of records of more than 8 s
-    // k-mers.
-    auto insert_all = [&]() {
-        uint32_t fresh = 0;
-        bool fail = false;
-        auto insert = [&](const K& key, uint32_t w) {
-            u64 a;
-            [[maybe_unused]] u64 b = 0;
-            uint32_t x;
-            if constexpr (WIDE) {
-                // 2 k - 62 and 62 bits: the all-ones word is no low word, and no
-                // high word of a canonical code of k <= 63 bases (at k = 63 it
-                // would start with 32 T, and so end with 32 A)
-                a = (key.hi << 2) | (key.lo >> 62);
-                b = key.lo & (~0ULL >> 2);
-                x = (uint32_t)b * 0x9E3779B1u + (uint32_t)(b >> 32) * 0x85EBCA77u + (uint32_t)a * 0xC2B2AE3Du +
-                    (uint32_t)(a >> 32) * 0x27D4EB2Fu;
-            } else {
-                a = key;  // never all ones: the reverse complement of all T is smaller
-                x = (uint32_t)a * 0x9E3779B1u + (uint32_t)(a >> 32) * 0x85EBCA77u;
-            }
-            uint32_t h = __umulhi(x, (uint32_t)SLOTS);
-            for (int probe = 0; probe < HC_PROBES; ++probe) {
-                u64 prev = *(volatile u64*)&tk[h];
-                if (prev == HC_EMPTY) {
-                    prev = atomicCAS(reinterpret_cast<unsigned long long*>(&tk[h]), HC_EMPTY, a);
-                    if (!WIDE && prev == HC_EMPTY) ++fresh;
-                }
-                bool hit = prev == HC_EMPTY || prev == a;
-                if constexpr (WIDE) {
-                    // a slot whose high word is set gets its low word from one of
-                    // the keys with that high word; the others go on
-                    if (hit) {
-                        u64 p2 = *(volatile u64*)&tk2[h];
-                        if (p2 == HC_EMPTY) {
-                            p2 = atomicCAS(reinterpret_cast<unsigned long long*>(&tk2[h]), HC_EMPTY, b);
-                            if (p2 == HC_EMPTY) ++fresh;
-                        }
-                        hit = p2 == HC_EMPTY || p2 == b;
-                    }
-                }
-                if (hit) {
-                    atomicAdd(&tc[h], w);
-                    return;
-                }
-                if (++h == (uint32_t)SLOTS) h = 0;
-            }
-            fail = true;
-        };
-        uint32_t t = warp;
-        for (int s = 0; HC_SEG * s < P.rec_n; ++s) {
-            const uint32_t ge = s_base[HC_SEG * s], tiles = (ge + 31) / 32;
-            for (; t < tiles; t += NW) {
-                if (*(volatile uint32_t*)&s_fail) break;
-                const uint32_t q = t * 32 + lane;
-                if (q < ge) {
-                    const uint32_t e = s_ord[q], i = e & 0xFFFFu, w = e >> 16;
-                    u64 W[4] = {0, 0, 0, 0};
-                    const ulonglong2* d = reinterpret_cast<const ulonglong2*>(s_rec + (size_t)i * RW);
-                    const ulonglong2 a = d[0];
-                    W[0] = a.x;
-                    W[1] = a.y;
-                    if (WIDE) {
-                        const ulonglong2 b = d[1];
-                        W[2] = b.x;
-                        W[3] = b.y;
-                    }
-                    const uint32_t n = (uint32_t)(W[RW - 1] & 0x7F), j0 = HC_SEG * s;
-                    uint32_t sh = 2 * j0;  // drop the first j0 bases
-                    while (sh >= 64) {
-                        W[0] = W[1];
-                        W[1] = W[2];
-                        W[2] = W[3];
-                        W[3] = 0;
-                        sh -= 64;
-                    }
-                    if (sh) {
-#pragma unroll
-                        for (int y = 0; y < RW; ++y) W[y] = funnel64(W[y], y < 3 ? W[y + 1] : 0ULL, sh);
-                    }
-                    const uint32_t nk = n - j0 < (uint32_t)HC_SEG ? n - j0 : (uint32_t)HC_SEG;
-                    record_kmers<WIDE>(W, nk, k, [&](uint32_t, const K& key) { insert(key, w); });
-                }
-            }
-            t -= tiles;  // t >= tiles unless the loop stopped on a failure
-        }
-        fresh = __reduce_add_sync(0xffffffffu, fresh);
-        if (lane == 0 && fresh) atomicAdd(&s_D, fresh);
-        if (fail) s_fail = 1;
-        __syncthreads();
+    // records of a part: what fills half the room at U k-mers in n records
+    auto next_part = [&](uint32_t n, uint32_t U, uint32_t room) -> uint32_t {
+        const uint32_t t = (uint32_t)((u64)n * room / (2 * (u64)U));
+        return t < 16 ? 16 : t >= n ? (n > 32 ? n / 2 : 16) : t;
     };
-
-    uint32_t target = RB, D = 0;
-    __syncthreads();
+    // One partition of more than a batch, in parts: the distinct k-mers of the
+    // parts so far keep their entries (closed up when room runs out), and every
+    // part's are merged with them.  False when even those do not fit.
+    auto count_in_parts = [&](u64 r0, u64 nr, uint32_t U) -> bool {
+        uint32_t D = 0, take = (uint32_t)(nr < (u64)RB ? nr : (u64)RB);
+        if (U != 0xFFFFFFFFu) take = next_part(take, U, ENT);
+        for (u64 r = r0; r < r0 + nr;) {
+            const uint32_t n = r0 + nr - r < (u64)take ? (uint32_t)(r0 + nr - r) : take;
+            U = stage(r, n);
+            if (D + U > (uint32_t)ENT) {
+                const uint32_t before = D;
+                D = close_up(D);
+                if (D + U > (uint32_t)ENT) {  // a smaller part, unless the entries are nearly all distinct k-mers
+                    if (D > (uint32_t)ENT / 4 * 3 || (before == D && n <= 16)) return false;
+                    take = next_part(n, U, (uint32_t)ENT - D);
+                    continue;
+                }
+            }
+            expand(D);
+            for (uint32_t i = tid; i < D; i += NT) *(volatile uint16_t*)&s_slot[key_slot<LS>(ek[i], 0)] = (uint16_t)i;
+            __syncthreads();
+            merge(D + U);
+            __syncthreads();
+            D += U;
+            r += n;
+        }
+        emit(D);
+        __syncthreads();
+        return true;
+    };
+    // records of the next batch: as many as fill 15/16 of the entries at the
+    // last batch's k-mers per record
+    auto next_target = [&](uint32_t nr, uint32_t U) -> uint32_t {
+        const uint32_t t = nr * (uint32_t)(ENT / 16 * 15) / (U ? U : 1u);  // nr <= 4096, ENT <= 8192: no overflow
+        return t > (uint32_t)RB ? (uint32_t)RB : t;
+    };
+    uint32_t target = RB;
     for (;;) {
+        __syncthreads();
         if (tid == 0) s_claim = atomicAdd(P.claim, 1u);
         __syncthreads();
         const u64 c0 = (u64)s_claim * P.chunk;
@@ -524,6 +600,7 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
         if (tid <= (int)np) s_off[tid] = P.part_off[first + tid];
         __syncthreads();
         for (uint32_t p = 0; p < np;) {
+            // the batch: as many whole partitions as `target` records hold
             const u64 r0 = s_off[p];
             uint32_t q = p + 1;
             while (q < np && s_off[q + 1] - r0 <= (u64)target) ++q;
@@ -532,58 +609,33 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
                 p = q;
                 continue;
             }
-            bool over = false;  // more k-mers than the table surely holds: it may overfill
-            uint32_t U = 0;
-            if (nr <= (u64)RB) {
-                U = stage(r0, (uint32_t)nr);
-                if (D + U > CAP && D > 0) {
-                    flush();
-                    D = 0;
+            uint32_t U = nr <= (u64)RB ? stage(r0, (uint32_t)nr) : 0xFFFFFFFFu;
+            if (U > (uint32_t)ENT) {
+                if (q > p + 1) {  // take fewer partitions
+                    target = next_target((uint32_t)nr, U);
+                    if (target >= (uint32_t)nr) target = (uint32_t)nr - 1;
+                    continue;
                 }
-                if (U > CAP) {
-                    if (q > p + 1) {  // take fewer partitions
-                        target = target / 2 > 32 ? target / 2 : 32;
-                        __syncthreads();
-                        continue;
+                // partition p alone is more than a batch
+                if (TIER == 0 || !count_in_parts(r0, nr, U)) {
+                    if (tid == 0) {
+                        P.ov_list[atomicAdd(reinterpret_cast<unsigned int*>(P.ov_stats), 1u)] = (uint32_t)(first + p);
+                        atomicAdd(P.ov_stats + 1, (unsigned long long)nr);
                     }
-                    over = true;
+                    __syncthreads();
                 }
-                insert_all();
-            } else {  // one partition of more records than fit a batch
-                over = true;
-                if (D > 0) {
-                    flush();
-                    D = 0;
-                }
-                for (u64 r = r0; r < r0 + nr; r += RB) {
-                    const u64 left = r0 + nr - r;
-                    stage(r, (uint32_t)(left < (u64)RB ? left : (u64)RB));
-                    insert_all();
-                    if (s_fail) break;
-                }
+                ++p;
+                continue;
             }
-            D = s_D;
-            if (over && s_fail) {
-                __syncthreads();
-                discard();
-                D = 0;
-                if (tid == 0) {
-                    P.ov_list[atomicAdd(reinterpret_cast<unsigned int*>(P.ov_stats), 1u)] = (uint32_t)(first + p);
-                    atomicAdd(P.ov_stats + 1, (unsigned long long)nr);
-                }
-            } else if (s_fail) {  // cannot happen: D + U <= CAP < SLOTS
-                if (tid == 0) raise_error(P.err, HSK_DERR_BOUNDS);
-                __syncthreads();
-                discard();
-                D = 0;
-            } else if (U < CAP / 3 && target < (uint32_t)RB) {
-                target = target * 2 < (uint32_t)RB ? target * 2 : (uint32_t)RB;
-            }
+            expand(0);
+            __syncthreads();
+            merge(U);
+            emit(U);
+            __syncthreads();
+            target = next_target((uint32_t)nr, U);
             p = q;
         }
-        __syncthreads();
     }
-    if (D > 0) flush();
     if (my_ones) atomicAdd(&s_hist[1], my_ones);
     __syncthreads();
     for (uint32_t i = tid; i < hs; i += NT)

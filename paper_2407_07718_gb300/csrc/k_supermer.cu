@@ -446,6 +446,41 @@ int supermer_max_ctas_per_sm(int mode, bool wide, int nreg, uint32_t n_buckets) 
     return n > 0 ? n : 1;
 }
 
+// A record's nb bases (left aligned, the rest 0) or their reverse complement,
+// whichever is smaller: the supermers of one locus on both strands then have
+// one record.  (The k-mers are the same: they are canonical.)
+template <int RW>
+__device__ __forceinline__ void one_strand(u64 (&r)[RW], int nb) {
+    constexpr int NW = 2 * RW;
+    uint32_t x[NW + 1];  // the whole words reversed and complemented, then shifted left
+#pragma unroll
+    for (int i = 0; i < RW; ++i) {
+        x[2 * i] = revcomp32((uint32_t)r[RW - 1 - i]);
+        x[2 * i + 1] = revcomp32((uint32_t)(r[RW - 1 - i] >> 32));
+    }
+    x[NW] = 0;
+    const uint32_t s = 64 * RW - 2 * nb;  // bits of the shift, < 64 RW
+#pragma unroll
+    for (int d = NW / 2; d > 0; d /= 2)
+        if ((s >> 5) & d) {
+#pragma unroll
+            for (int i = 0; i < NW; ++i) x[i] = i + d < NW ? x[i + d < NW ? i + d : 0] : 0u;
+        }
+    u64 c[RW];
+    bool less = false, same = true;
+#pragma unroll
+    for (int i = 0; i < RW; ++i) {
+        c[i] = ((u64)__funnelshift_l(x[2 * i + 1], x[2 * i], s & 31) << 32) |
+               __funnelshift_l(x[2 * i + 2], x[2 * i + 1], s & 31);
+        less = less || (same && c[i] < r[i]);
+        same = same && c[i] == r[i];
+    }
+    if (less) {
+#pragma unroll
+        for (int i = 0; i < RW; ++i) r[i] = c[i];
+    }
+}
+
 // ---------------------------------------------------------------------------
 // records from descriptors
 // ---------------------------------------------------------------------------
@@ -492,19 +527,15 @@ __global__ void __launch_bounds__(256) k_scatter_desc(const u64* __restrict__ de
             }
             if (sub) rec_sub[slot[j]] = (uint8_t)(dd[j] >> 56);
             const int nb = (int)n + k - 1;  // bases in the record
-            if (!WIDE) {
-                u64 a = keep_bases(extract_k64(packed, pos, 32), nb);
-                u64 c = keep_bases(extract_k64(packed, pos + 32, 32), nb - 32) | (u64)n;
-                reinterpret_cast<ulonglong2*>(records)[slot[j]] = make_ulonglong2(a, c);
-            } else {
-                u64 r[4];
+            constexpr int RW = WIDE ? 4 : 2;
+            u64 r[RW];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) r[q] = keep_bases(extract_k64(packed, pos + 32 * q, 32), nb - 32 * q);
-                r[3] |= (u64)n;
-                ulonglong2* dst = reinterpret_cast<ulonglong2*>(records) + 2 * slot[j];
-                dst[0] = make_ulonglong2(r[0], r[1]);
-                dst[1] = make_ulonglong2(r[2], r[3]);
-            }
+            for (int q = 0; q < RW; ++q) r[q] = keep_bases(extract_k64(packed, pos + 32 * q, 32), nb - 32 * q);
+            if (sub) one_strand<RW>(r, nb);
+            r[RW - 1] |= (u64)n;
+            ulonglong2* dst = reinterpret_cast<ulonglong2*>(records) + (RW / 2) * slot[j];
+#pragma unroll
+            for (int q = 0; q < RW / 2; ++q) dst[q] = make_ulonglong2(r[2 * q], r[2 * q + 1]);
         }
     }
 }
