@@ -28,9 +28,7 @@ void launch_encode_range(const char* reads, uint64_t n_bases, uint64_t b0, uint6
                          uint64_t* invalid, uint64_t n_packed_words, cudaStream_t st);
 constexpr uint64_t SM_TILE_BASES = 1024;   // windows per S2 warp tile
 constexpr uint64_t SM_TILE_REACH = 1280;   // bases past a tile's start that its walk reads
-// warps per CTA of the walk; one bucket-counter table per CTA in shared
-// memory, so more warps share it (16: short-read S2 17.9 -> 16.1 ms against 8)
-constexpr int SM_CTA_WARPS = 16;
+constexpr int SM_CTA_WARPS = 8;            // warps per CTA of the walk
 void launch_mark_starts(const uint64_t* offsets, uint64_t n_reads, uint64_t n_bases,
                         uint64_t* start_mask, int* err, cudaStream_t st);
 
@@ -53,7 +51,6 @@ struct SmParams {
     int lexical;              // 1: m-mers ordered by their code (lexical), 0: by hash
     uint32_t n_buckets;       // a power of two (one set), or the buckets of all packed sets
     int nmax;                 // k-mers per supermer record at most
-    uint32_t nmax_magic;      // ceil(2^32 / nmax): q = umulhi(x, magic) = x / nmax for x < 2^24
     int rec_words;            // 2 (k <= 32) or 4 (k <= 64)
     uint32_t grid;
     uint64_t tile_begin, tile_end;     // warp tiles [begin, end) of 1024 windows (end 0 = all)
@@ -78,7 +75,7 @@ struct SmParams {
 };
 
 size_t supermer_smem_bytes(int mode, uint32_t n_buckets);
-int supermer_max_ctas_per_sm(int mode, bool wide, int nreg, uint32_t n_buckets);
+int supermer_max_ctas_per_sm(int mode, int m, bool lexical, uint32_t n_buckets);
 void launch_supermer(int mode, const SmParams& p, cudaStream_t st);
 // records from descriptors (and, with rec_sub, each record's sub-partition):
 // bucket_off[B+1] record offsets; cursor[b *

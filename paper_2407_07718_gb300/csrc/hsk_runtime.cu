@@ -421,7 +421,6 @@ static void fill_sm_params(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t 
     P.rec_words = k <= 32 ? 2 : 4;
     P.nmax = (P.rec_words * 32 - 4) - k + 1;  // bases per record minus (k - 1)
     if (P.nmax > 255) P.nmax = 255;
-    P.nmax_magic = (uint32_t)(((1ull << 32) + P.nmax - 1) / P.nmax);
     P.err = c->d_err;
 }
 
@@ -439,9 +438,7 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
         P.set_bmask = sets->bmask;
         P.n_sets = sets->n;
     }
-    const bool wide = k > 32;
-    const int nreg = P.w <= 33 ? 2 : 3;
-    const int occ = supermer_max_ctas_per_sm(SM_DESC, wide, nreg, B);
+    const int occ = supermer_max_ctas_per_sm(SM_DESC, m, P.lexical, B);
     const uint64_t warp_tiles = (E.n_bases + 1023) / 1024;
     uint64_t g = std::min<uint64_t>((uint64_t)c->num_sms * occ, (warp_tiles + SM_CTA_WARPS - 1) / SM_CTA_WARPS);
     P.grid = (uint32_t)std::max<uint64_t>(g, 1);

@@ -11,33 +11,36 @@
 // reverse complement the same minimizer score.
 //
 // GPU design (replaces the paper's per-read monotone deque): a warp walks a
-// tile of 1024 consecutive window starts in 32 steps, lane l handling window
-// 32*s + l.  The packed bases and masks of the tile are staged in shared
-// memory with 128-bit loads.  Each lane computes one new m-mer score per step;
-// the window minimum over w = k-m+1 scores comes from minima over 32-lane
-// blocks kept in registers: for w <= 33 the minima of runs of D = 2^L <= w
-// scores (doubling with shuffles, each block's computed once and carried to
-// the next step), for w > 33 suffix and prefix minima of the blocks (van
-// Herk / Gil-Werman with 32-lane blocks).  Supermer
-// cuts (bucket change, invalid window, cap of nmax k-mers, tile end) come
-// from ballots of run starts (the latest start at or before a lane is the
-// highest set bit below it).  The walk runs once (DESC): every
-// supermer becomes an 8-byte descriptor (start base, k-mer count, bucket),
-// buffered per warp in shared memory and appended to a global list with one
-// atomic per buffer; per-bucket record and k-mer counts are kept in shared
+// tile of 1024 consecutive window starts, lane l the 32 windows that start in
+// its 64-bit word of packed bases.  The tile's bases and masks are staged in
+// shared memory with 128-bit loads.  A lane computes its 32 m-mer scores from
+// two words by constant shifts, then the minima of runs of D scores (D the
+// largest power of two <= w) by doubling in registers; a window's minimum is
+// that of two overlapping runs.  Supermer cuts (bucket change, invalid window,
+// cap of nmax k-mers, tile end) are bit masks of the lane's windows: a
+// supermer starts where a bit is set, and ends at the next set bit of the
+// cuts, in this lane or a later one.  Every supermer becomes an 8-byte
+// descriptor (start base, k-mer count, bucket), appended to a global list with
+// one atomic per tile; per-bucket record and k-mer counts are kept in shared
 // memory.  A second, light kernel scatters records into their buckets from
 // the descriptors.  DUMP mode writes per-window keys and scores for the stage
 // test.
+//
+// The kernel is bound by instruction issue.  With 32 windows a lane it takes
+// 3.9 ms on 1.5 G windows of long reads (k = 31, w = 15) and 5.3 ms on 1.27 G
+// of short reads (k = 55, w = 35); one window a lane and step, with the window
+// minima and the cuts found by shuffles and ballots across lanes, took 8.7
+// warp instructions per window and 14.4 and 17.0 ms.
 #include "hsk_device.cuh"
 
 namespace hsk {
 
 constexpr int SM_WARPS = SM_CTA_WARPS;
-constexpr int SM_STEPS = 32;
-constexpr int SM_TW = 32 * SM_STEPS;      // windows per warp tile
+constexpr int SM_CTAS = 3;                // CTAs per SM (registers, shared memory)
+constexpr int SM_TW = 32 * 32;            // windows per warp tile, 32 per lane
 constexpr int SM_PW = SM_TW / 32 + 6;     // packed words staged per warp (even)
 constexpr int SM_MW = SM_TW / 64 + 4;     // mask words staged per warp (even)
-constexpr int SM_DBUF = 128;              // descriptors buffered per warp
+constexpr int SM_ROWS = 33 * 33;          // words of run minima per warp (33 padded rows of 32)
 constexpr int SM_VW = SM_TW / 64;         // valid-window words per warp
 static_assert(SM_TW == (int)SM_TILE_BASES, "tile size");
 static_assert(SM_PW * 32 <= (int)SM_TILE_REACH && SM_MW * 64 <= (int)SM_TILE_REACH,
@@ -50,8 +53,8 @@ static_assert(SM_PW * 32 <= (int)SM_TILE_REACH && SM_MW * 64 <= (int)SM_TILE_REA
 // one thread cannot lower it under another's launch.
 constexpr uint32_t SM_MAX_BUCKETS = 8192;
 size_t supermer_smem_bytes(int mode, uint32_t n_buckets) {
-    size_t s = (size_t)SM_WARPS * (SM_PW + 2 * SM_MW + SM_VW) * sizeof(u64);
-    if (mode == SM_DESC) s += (size_t)SM_WARPS * SM_DBUF * sizeof(u64) + (size_t)n_buckets * 2 * sizeof(uint32_t);
+    size_t s = (size_t)SM_WARPS * ((SM_PW + 2 * SM_MW + SM_VW) * sizeof(u64) + SM_ROWS * sizeof(uint32_t));
+    if (mode == SM_DESC) s += (size_t)n_buckets * 2 * sizeof(uint32_t);
     return s;
 }
 
@@ -79,60 +82,6 @@ __device__ __forceinline__ uint32_t mmer_score(const u64* pk, int q, int m, uint
     u64 c = f < r ? f : r;
     if constexpr (LEX) return m > 16 ? (uint32_t)(c >> (2 * m - 32)) : (uint32_t)c;
     else return fmix32((uint32_t)c ^ (uint32_t)(c >> 32) ^ seed);
-}
-
-// Minimum of v over lanes [lane, 31] (suffix) and over [0, lane] (prefix).
-__device__ __forceinline__ uint32_t lane_suffix_min(uint32_t v, int lane) {
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t o = __shfl_down_sync(0xffffffffu, v, d);
-        if (lane + d < 32) v = min(v, o);
-    }
-    return v;
-}
-__device__ __forceinline__ uint32_t lane_prefix_min(uint32_t v, int lane) {
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t o = __shfl_up_sync(0xffffffffu, v, d);
-        if (lane >= d) v = min(v, o);
-    }
-    return v;
-}
-
-// min(v[lane .. lane + 2^L - 1]) within the block (lanes past 31 ignored).
-__device__ __forceinline__ uint32_t lane_range_min_trunc(uint32_t v, int L, int lane) {
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        if (j < L) {
-            const uint32_t o = __shfl_down_sync(0xffffffffu, v, 1 << j);
-            if (lane + (1 << j) < 32) v = min(v, o);
-        }
-    }
-    return v;
-}
-// min(v[0 .. lane]) for lanes below n (n <= 32; other lanes: partial).
-__device__ __forceinline__ uint32_t lane_prefix_min_upto(uint32_t v, int n, int lane) {
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        if ((1 << j) < n) {
-            const uint32_t o = __shfl_up_sync(0xffffffffu, v, 1 << j);
-            if (lane >= (1 << j)) v = min(v, o);
-        }
-    }
-    return v;
-}
-
-// Window minimum for 33 <= w <= 65 (three score registers): a window that
-// starts at lane l of block 0 always runs past the block's end, so it is the
-// suffix of block 0 from l, then either a prefix of block 1 or all of block
-// 1 and a prefix of block 2 (van Herk / Gil-Werman with 32-lane blocks).
-// sm0 = suffix minima of block 0, pm1 / pm2 = prefix minima of blocks 1 / 2.
-__device__ __forceinline__ uint32_t window_min_wide(uint32_t sm0, uint32_t pm1, uint32_t pm2, int w, int lane) {
-    const int e = lane + w - 1;  // last position of the window, 32 <= e <= 95
-    const uint32_t a = __shfl_sync(0xffffffffu, pm1, (e - 32) & 31);
-    const uint32_t b = __shfl_sync(0xffffffffu, pm2, (e - 64) & 31);
-    const uint32_t full1 = __shfl_sync(0xffffffffu, pm1, 31);
-    return min(sm0, e < 64 ? a : min(full1, b));
 }
 
 // Bit t (most significant first) = OR of bits [t, t + L) of the 128-bit
@@ -169,16 +118,114 @@ __device__ __forceinline__ void split_desc(u64 d, int sub, u64& pos, uint32_t& n
     bucket = sub ? (uint32_t)(d >> 43) & 0x1FFF : (uint32_t)(d >> 48);
 }
 
-template <int MODE, bool WIDE, int NREG, bool LEX>
-__global__ void __launch_bounds__(SM_WARPS * 32) k_supermer(const SmParams P) {
+// Window minima of a tile.  Lane l holds the scores of positions 32 l .. 32 l
+// + 31 in a[0..31] and in h0, h1 those of positions 1024 + l and 1056 + l (h1
+// only read when w > 33).  With D = 2^L <= w < 2 D the minimum of a window is
+// that of two overlapping runs of D scores; the run minima come from doubling
+// in registers, and the entries past the lane's own 32 from the next lane
+// (its first d at level d), exchanged through rows of 33 words (lane l's word
+// j at l * 33 + j: no bank conflicts; row 32 holds the positions past the
+// tile).  Leaves the run minima in the rows too, and returns the distance of
+// the two runs; the window minimum of position j is then
+// min(row[j], row[j + off]) (row_at).
+__device__ __forceinline__ int run_minima(uint32_t (&a)[32], uint32_t h0, uint32_t h1, int w, uint32_t* rows, int lane) {
+    uint32_t* own = rows + lane * 33;
+    const uint32_t* nxt = own + 33;
+    int D = 1;
+#pragma unroll
+    for (int d = 1; d <= 16; d *= 2) {
+        if (2 * d <= w) {
+#pragma unroll
+            for (int j = 0; j < d; ++j) own[j] = a[j];
+            if (lane < d) rows[32 * 33 + lane] = h0;
+            __syncwarp();
+            uint32_t n[16];
+#pragma unroll
+            for (int j = 0; j < d; ++j) n[j] = nxt[j];
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 32; ++j) a[j] = min(a[j], j + d < 32 ? a[j + d < 32 ? j + d : 0] : n[j + d < 32 ? 0 : j + d - 32]);
+            const uint32_t o0 = __shfl_sync(0xffffffffu, h0, (lane + d) & 31);
+            const uint32_t o1 = __shfl_sync(0xffffffffu, h1, (lane + d) & 31);
+            h0 = min(h0, lane + d < 32 ? o0 : o1);
+            if (lane + d < 32) h1 = min(h1, o1);
+            D = 2 * d;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 32; ++j) own[j] = a[j];
+    rows[32 * 33 + lane] = h0;
+    __syncwarp();
+    if (w >= 64) {
+        uint32_t n[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) n[j] = nxt[j];
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) own[j] = a[j] = min(a[j], n[j]);
+        rows[32 * 33 + lane] = min(h0, h1);
+        __syncwarp();
+        D = 64;
+    }
+    return w - D;
+}
+// word of position 32 * lane + j (j < 63) in the rows
+__device__ __forceinline__ uint32_t row_at(const uint32_t* rows, int lane, int j) {
+    return rows[lane * 33 + j + (j >= 32 ? 1 : 0)];
+}
+
+// Scores of the 32 m-mers starting in word W0 of the packed bases (W1 the next
+// word).  The forward codes are funnels of W0:W1 by constant shifts; the
+// reverse complements are funnels of the reversed and complemented words,
+// shifted once so that those shifts are constant too.  Codes stay left
+// aligned with the following bases below them: two codes that differ compare
+// by their own bits, and equal ones are the same m-mer.
+template <bool SHORT, bool LEX>
+__device__ __forceinline__ void mmer_scores32(u64 W0, u64 W1, int m, uint32_t seed, uint32_t (&a)[32]) {
+    u64 R0 = reverse_pairs(~W1), R1 = reverse_pairs(~W0);
+    const uint32_t s = 2 * (33 - m);  // 2 .. 64
+    if (s == 64) {
+        R0 = R1;
+        R1 = 0;
+    } else {
+        R0 = (R0 << s) | (R1 >> (64 - s));
+        R1 <<= s;
+    }
+    const uint32_t F[5] = {(uint32_t)(W0 >> 32), (uint32_t)W0, (uint32_t)(W1 >> 32), (uint32_t)W1, 0u};
+    const uint32_t C[5] = {(uint32_t)(R0 >> 32), (uint32_t)R0, (uint32_t)(R1 >> 32), (uint32_t)R1, 0u};
+    const uint32_t sh = SHORT ? 32 - 2 * m : 64 - 2 * m;  // < 32
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        const int fi = j / 16, fs = 2 * (j % 16), ci = (31 - j) / 16, cs = 2 * ((31 - j) % 16);
+        const uint32_t fh = __funnelshift_l(F[fi + 1], F[fi], fs), ch = __funnelshift_l(C[ci + 1], C[ci], cs);
+        if constexpr (SHORT) {
+            const uint32_t c = min(fh, ch) >> sh;
+            a[j] = LEX ? c : fmix32(c ^ seed);
+        } else {
+            if constexpr (LEX) {
+                a[j] = min(fh, ch);
+            } else {
+                const uint32_t fl = __funnelshift_l(F[fi + 2], F[fi + 1], fs);
+                const uint32_t cl = __funnelshift_l(C[ci + 2], C[ci + 1], cs);
+                const u64 f = ((u64)fh << 32) | fl, r = ((u64)ch << 32) | cl;
+                const u64 c = f < r ? f : r;
+                const uint32_t h = (uint32_t)(c >> 32), l = (uint32_t)c;
+                a[j] = fmix32(__funnelshift_r(l, h, sh) ^ (h >> sh) ^ seed);
+            }
+        }
+    }
+}
+
+template <int MODE, bool SHORT, bool LEX>
+__global__ void __launch_bounds__(SM_WARPS * 32, SM_CTAS) k_supermer(const __grid_constant__ SmParams P) {
     extern __shared__ __align__(16) unsigned char smem[];
     u64* s_pk = reinterpret_cast<u64*>(smem);
     u64* s_iv = s_pk + SM_WARPS * SM_PW;
     u64* s_rs = s_iv + SM_WARPS * SM_MW;
     u64* s_val = s_rs + SM_WARPS * SM_MW;
-    u64* s_desc = s_val + SM_WARPS * SM_VW;                                      // DESC
-    uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_desc + SM_WARPS * SM_DBUF);  // DESC
-    uint32_t* s_km = s_cnt + P.n_buckets;                                        // DESC
+    uint32_t* s_rows = reinterpret_cast<uint32_t*>(s_val + SM_WARPS * SM_VW);
+    uint32_t* s_cnt = s_rows + SM_WARPS * SM_ROWS;  // DESC
+    uint32_t* s_km = s_cnt + P.n_buckets;           // DESC
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t B = P.n_buckets;
@@ -193,27 +240,13 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_supermer(const SmParams P) {
     u64* wiv = s_iv + warp * SM_MW;
     u64* wrs = s_rs + warp * SM_MW;
     u64* wval = s_val + warp * SM_VW;
-    u64* wdesc = s_desc + warp * SM_DBUF;
-    int nbuf = 0;  // descriptors buffered by this warp (warp-uniform)
+    uint32_t* rows = s_rows + warp * SM_ROWS;
     const u64 n_tiles = P.tile_end ? P.tile_end : (P.n_bases + SM_TW - 1) / SM_TW;
-
-    // append the buffered descriptors to the global list (one atomic per flush)
-    auto flush = [&]() {
-        if (nbuf == 0) return;
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(P.desc_count, (unsigned long long)nbuf);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        for (int i = lane; i < nbuf; i += 32)
-            if (base + i < P.desc_cap) P.desc[base + i] = wdesc[i];
-        __syncwarp();
-        nbuf = 0;
-    };
 
     for (u64 t = P.tile_begin + (u64)blockIdx.x * SM_WARPS + warp; t < n_tiles; t += (u64)gridDim.x * SM_WARPS) {
         const u64 p0 = t * SM_TW;
         // buckets of the tile's set (packed sets: the set holding tile t)
         uint32_t bbase = 0, bmask = B - 1u;
-        const uint32_t subs = P.desc_sub ? 0xFFu : 0u;  // sub-partition: the hash bits above the bucket's
         if (P.n_sets) {
             uint32_t lo = 0, hi = P.n_sets;  // set_tile0[lo] <= t < set_tile0[hi]
             while (hi - lo > 1) {
@@ -265,139 +298,107 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_supermer(const SmParams P) {
             }
             __syncwarp();
         }
+        // valid windows of this lane, window j at bit j
+        const u64 v64 = wval[lane >> 1];
+        uint32_t V = __brev(lane & 1 ? (uint32_t)v64 : (uint32_t)(v64 >> 32));
+        {
+            const u64 p = p0 + 32 * lane + k;  // end of window 0
+            const u64 left = P.n_bases + 1 > p ? P.n_bases + 1 - p : 0;  // windows that end inside the data
+            if (left < 32) V &= (1u << left) - 1u;
+        }
 
-        // rolling m-mer scores: X[r] = score at local base 32*(s + r) + lane
-        uint32_t X[NREG];
+        uint32_t a[32];
+        mmer_scores32<SHORT, LEX>(wpk[lane], wpk[lane + 1], m, P.seed32, a);
+        const uint32_t h0 = mmer_score<LEX>(wpk, SM_TW + lane, m, P.seed32);
+        const uint32_t h1 = w > 33 ? mmer_score<LEX>(wpk, SM_TW + 32 + lane, m, P.seed32) : 0xFFFFFFFFu;
+        const int off = run_minima(a, h0, h1, w, rows, lane);
+
+        if (MODE == SM_DUMP) {
+            for (int j = 0; j < 32; ++j) {
+                const u64 p = p0 + 32 * lane + j;
+                if (p >= P.n_bases) break;
+                const bool valid = (V >> j) & 1u;
+                P.dump_valid[p] = valid;
+                if (!valid) continue;
+                if (k <= 32) {
+                    P.dump_key[2 * p] = canonical64(extract_k64(wpk, 32 * lane + j, k), k);
+                    P.dump_key[2 * p + 1] = 0;
+                } else {
+                    const key128 c = canonical128(extract_k128(wpk, 32 * lane + j, k), k);
+                    P.dump_key[2 * p] = c.lo;
+                    P.dump_key[2 * p + 1] = c.hi;
+                }
+                P.dump_minhash[p] = min(row_at(rows, lane, j), row_at(rows, lane, j + off));
+            }
+        } else {
+            // id of a window: its bucket and, with sub-partitions, the hash bits
+            // above; D has bit j set where window j's id differs from window j - 1's
+            const int bb = __popc(bmask);
+            const uint32_t idmask = P.desc_sub ? (bmask << 8) | 0xFFu : bmask;
+            uint32_t D = 0, prev = 0;
 #pragma unroll
-        for (int r = 0; r < NREG; ++r) X[r] = mmer_score<LEX>(wpk, 32 * r + lane, m, P.seed32);
-        // wide windows (three registers): prefix minima of block 1, carried
-        // from one step to the next as block 2's
-        uint32_t pm_next = 0;
-        if constexpr (NREG == 3) pm_next = lane_prefix_min(X[1], lane);
-        // narrow windows (two registers, w <= 33): with D = 2^L <= w < 2D, a
-        // window is two overlapping runs of D scores.  t_cur = min over runs
-        // of D starting at each lane of block 0, counted within the block
-        // only; computed for each block when it enters as block 1, carried.
-        int nL = 0;
-        while ((2 << nL) <= w) ++nL;
-        const int nD = 1 << nL;
-        uint32_t t_cur = 0;
-        if constexpr (NREG == 2) t_cur = lane_range_min_trunc(X[0], nL, lane);
-
-        int c_valid = 0, c_runstart = -1;   // carry from lane 31 of the previous step
-        uint32_t c_b = 0;
-        int pv = 0, plp = 0, psm = 0;       // previous step, for delayed emission
-        uint32_t pb = 0, pvmask = 0, psmask = 0;
-
-        // emit the supermers that end in the previous step (end = valid and the
-        // next window is invalid or starts a new supermer)
-        auto emit_prev = [&](int nv, int ns) {
-            const bool end = pv && (!nv || ns);
-            const uint32_t ends = __ballot_sync(0xffffffffu, end);
-            if (!ends) return;
-            const int cnt = __popc(ends);
-            if (nbuf + cnt > SM_DBUF) flush();
-            if (end) {
-                const int n = plp - psm + 1;
-                atomicAdd(&s_cnt[pb & 0x1FFFu], 1u);
-                atomicAdd(&s_km[pb & 0x1FFFu], (uint32_t)n);
-                wdesc[nbuf + __popc(ends & ((1u << lane) - 1u))] = make_desc(p0 + psm, (uint32_t)n, pb, P.desc_sub);
+            for (int j = 0; j < 32; ++j) {
+                const uint32_t id = min(a[j], row_at(rows, lane, j + off)) & idmask;
+                if (j > 0) D |= id != prev ? 1u << j : 0u;
+                else a[0] = id;
+                prev = id;
             }
-            nbuf += cnt;
-            __syncwarp();
-        };
-
-        for (int s = 0; s < SM_STEPS; ++s) {
-            const int lp = 32 * s + lane;
-            const u64 p = p0 + lp;
-            int valid = (p + k <= P.n_bases) && ((wval[lp >> 6] >> (63 - (lp & 63))) & 1);
-            uint32_t mh;
-            if constexpr (NREG == 3) {
-                const uint32_t pm2 = lane_prefix_min(X[2], lane);
-                mh = window_min_wide(lane_suffix_min(X[0], lane), pm_next, pm2, w, lane);
-                pm_next = pm2;
-            } else {
-                // block 1's runs within block 1, and its prefix minima that
-                // complete block 0's runs reaching into it (lanes past 32 - D)
-                const uint32_t t_new = lane_range_min_trunc(X[1], nL, lane);
-                const uint32_t pm1 = lane_prefix_min_upto(X[1], nD - 1, lane);
-                const int i1 = lane + nD - 33;  // last lane of block 1 in this lane's run
-                const uint32_t pv = __shfl_sync(0xffffffffu, pm1, i1 & 31);
-                const uint32_t tc = i1 >= 0 ? min(t_cur, pv) : t_cur;
-                // the second run starts at q = lane + w - D (in block 1 when q >= 32,
-                // where its run lies inside block 1 because w <= 33)
-                const int q = lane + w - nD;
-                const uint32_t a = __shfl_sync(0xffffffffu, tc, q & 31);
-                const uint32_t b = __shfl_sync(0xffffffffu, t_new, (q - 32) & 31);
-                mh = min(tc, q < 32 ? a : b);
-                t_cur = t_new;
-            }
-            const uint32_t b = (bbase + (mh & bmask)) | (((mh >> __popc(bmask)) & subs) << 13);
-
-            if (MODE == SM_DUMP) {
-                if (p < P.n_bases) {
-                    P.dump_valid[p] = (uint8_t)valid;
-                    if (valid) {
-                        if (!WIDE) {
-                            P.dump_key[2 * p] = canonical64(extract_k64(wpk, lp, k), k);
-                            P.dump_key[2 * p + 1] = 0;
-                        } else {
-                            key128 c = canonical128(extract_k128(wpk, lp, k), k);
-                            P.dump_key[2 * p] = c.lo;
-                            P.dump_key[2 * p + 1] = c.hi;
-                        }
-                        P.dump_minhash[p] = mh;
+            const uint32_t before = __shfl_up_sync(0xffffffffu, prev, 1);
+            const uint32_t vb = __shfl_up_sync(0xffffffffu, V, 1);
+            D |= a[0] != before ? 1u : 0u;
+            const uint32_t Vp = (V << 1) | (lane ? vb >> 31 : 0u);  // window before is valid (and in the tile)
+            const uint32_t start = V & (D | ~Vp);
+            const uint32_t ev = start | ~V;  // a run that is open here ends
+            // the first such place after this lane's windows, in the tile
+            const uint32_t has = __ballot_sync(0xffffffffu, ev != 0);
+            const uint32_t later = lane < 31 ? has >> (lane + 1) << (lane + 1) : 0u;
+            const int nl = later ? __ffs(later) - 1 : lane;
+            const int fe = __shfl_sync(0xffffffffu, __ffs(ev) - 1, nl);
+            const int open_end = later ? 32 * nl + fe : SM_TW;
+            const uint32_t mine = (uint32_t)__popc(start);
+            const uint32_t incl = warp_incl_sum<uint32_t>(mine);
+            const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+            if (total) {
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(P.desc_count, (unsigned long long)total);
+                base = __shfl_sync(0xffffffffu, base, 0);
+                u64 o = base + incl - mine;
+                int extra = 0;  // pieces past the first of runs of more than nmax k-mers
+                auto desc_at = [&](u64 at, int pos, int n, uint32_t id) {
+                    const uint32_t b = bbase + (id & bmask);
+                    atomicAdd(&s_cnt[b], 1u);
+                    atomicAdd(&s_km[b], (uint32_t)n);
+                    if (at < P.desc_cap)
+                        P.desc[at] = make_desc(p0 + pos, (uint32_t)n, b | (id >> bb) << 13, P.desc_sub);
+                };
+                for (uint32_t S = start; S; S &= S - 1) {
+                    const int j = __ffs(S) - 1;
+                    const uint32_t rest = ev & ~((2u << j) - 1u);
+                    const int len = (rest ? 32 * lane + __ffs(rest) - 1 : open_end) - (32 * lane + j);
+                    const uint32_t id = min(row_at(rows, lane, j), row_at(rows, lane, j + off)) & idmask;
+                    if (len > nmax) extra += (len - 1) / nmax;
+                    desc_at(o++, 32 * lane + j, min(len, nmax), id);
+                }
+                if (__any_sync(0xffffffffu, extra)) {
+                    const uint32_t xi = warp_incl_sum<uint32_t>((uint32_t)extra);
+                    const uint32_t xt = __shfl_sync(0xffffffffu, xi, 31);
+                    if (lane == 0) base = atomicAdd(P.desc_count, (unsigned long long)xt);
+                    base = __shfl_sync(0xffffffffu, base, 0);
+                    o = base + xi - (uint32_t)extra;
+                    for (uint32_t S = extra ? start : 0u; S; S &= S - 1) {
+                        const int j = __ffs(S) - 1;
+                        const uint32_t rest = ev & ~((2u << j) - 1u);
+                        const int end = rest ? 32 * lane + __ffs(rest) - 1 : open_end;
+                        const uint32_t id = min(row_at(rows, lane, j), row_at(rows, lane, j + off)) & idmask;
+                        for (int q = 32 * lane + j + nmax; q < end; q += nmax) desc_at(o++, q, min(end - q, nmax), id);
                     }
                 }
-            } else {
-                // flags of neighbouring lanes come from ballots; only the
-                // bucket of the lane before needs a shuffle
-                const uint32_t vmask = __ballot_sync(0xffffffffu, valid);
-                uint32_t prev_b = __shfl_up_sync(0xffffffffu, b, 1);
-                int prev_valid = lane ? (int)((vmask >> (lane - 1)) & 1u) : c_valid;
-                if (lane == 0) prev_b = c_b;
-                const int start0 = valid && !(prev_valid && prev_b == b);
-                // the latest run start at or before this window
-                const uint32_t smask0 = __ballot_sync(0xffffffffu, start0);
-                const uint32_t le = smask0 & (0xFFFFFFFFu >> (31 - lane));
-                const int rs = le ? 32 * s + (31 - __clz(le)) : c_runstart;
-                const int pos_in_run = lp - rs;
-                // pos_in_run / nmax by a multiply: exact for pos_in_run < 2^24
-                const int q = (int)__umulhi((uint32_t)pos_in_run, P.nmax_magic);
-                const int start = valid && (start0 || pos_in_run == q * nmax);
-                const int smstart = rs + q * nmax;
-                const uint32_t smask = __ballot_sync(0xffffffffu, start);
-                if (s > 0) {
-                    // the window after this lane's window of the previous step
-                    const int nv = lane < 31 ? (int)((pvmask >> (lane + 1)) & 1u) : (int)(vmask & 1u);
-                    const int ns = lane < 31 ? (int)((psmask >> (lane + 1)) & 1u) : (int)(smask & 1u);
-                    emit_prev(nv, ns);
-                }
-                c_valid = (int)(vmask >> 31);
-                c_b = __shfl_sync(0xffffffffu, b, 31);
-                if (smask0) c_runstart = 32 * s + (31 - __clz(smask0));
-                pv = valid;
-                pvmask = vmask;
-                psmask = smask;
-                pb = b;
-                plp = lp;
-                psm = smstart;
             }
-            // roll the scores forward by one step
-#pragma unroll
-            for (int r = 0; r + 1 < NREG; ++r) X[r] = X[r + 1];
-            X[NREG - 1] = mmer_score<LEX>(wpk, 32 * (s + NREG) + lane, m, P.seed32);
-        }
-        if (MODE != SM_DUMP) {  // the tile edge ends every open supermer
-            const int nv = lane < 31 ? (int)((pvmask >> (lane + 1)) & 1u) : 0;
-            const int ns = lane < 31 ? (int)((psmask >> (lane + 1)) & 1u) : 0;
-            emit_prev(nv, ns);
         }
         __syncwarp();
     }
 
     if (MODE == SM_DESC) {
-        flush();
         __syncthreads();
         for (uint32_t b = threadIdx.x; b < B; b += blockDim.x) {
             if (s_cnt[b]) atomicAdd(P.bucket_rec + b, s_cnt[b]);
@@ -407,42 +408,29 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_supermer(const SmParams P) {
     }
 }
 
+using SmKernel = void (*)(SmParams);
 template <int MODE>
-static void launch_mode(const SmParams& p, cudaStream_t st) {
-    size_t sm = supermer_smem_bytes(MODE, p.n_buckets);
-    const size_t sm_cap = supermer_smem_bytes(MODE, SM_MAX_BUCKETS);
-    bool wide = p.k > 32;
-    int nreg = (p.w <= 33) ? 2 : 3;
-    unsigned grid = p.grid;
-    count_launch();
-#define HSK_SM_LAUNCH(W, NR)                                                                 \
-    do {                                                                                     \
-        auto fn = p.lexical ? k_supermer<MODE, W, NR, true> : k_supermer<MODE, W, NR, false>; \
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_cap);  \
-        fn<<<grid, SM_WARPS * 32, sm, st>>>(p);                                              \
-    } while (0)
-    if (!wide && nreg == 2) HSK_SM_LAUNCH(false, 2);
-    else if (!wide) HSK_SM_LAUNCH(false, 3);
-    else if (nreg == 2) HSK_SM_LAUNCH(true, 2);
-    else HSK_SM_LAUNCH(true, 3);
-#undef HSK_SM_LAUNCH
+static SmKernel walk_kernel(int m, bool lexical) {
+    if (m <= 16) return lexical ? (SmKernel)k_supermer<MODE, true, true> : (SmKernel)k_supermer<MODE, true, false>;
+    return lexical ? (SmKernel)k_supermer<MODE, false, true> : (SmKernel)k_supermer<MODE, false, false>;
+}
+static SmKernel walk_kernel(int mode, int m, bool lexical) {
+    SmKernel fn = mode == SM_DESC ? walk_kernel<SM_DESC>(m, lexical) : walk_kernel<SM_DUMP>(m, lexical);
+    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)supermer_smem_bytes(mode, SM_MAX_BUCKETS));
+    return fn;
 }
 
 void launch_supermer(int mode, const SmParams& p, cudaStream_t st) {
     if (p.n_bases == 0) return;
-    if (mode == SM_DESC) launch_mode<SM_DESC>(p, st);
-    else launch_mode<SM_DUMP>(p, st);
+    count_launch();
+    walk_kernel(mode, p.m, p.lexical)<<<p.grid, SM_WARPS * 32, supermer_smem_bytes(mode, p.n_buckets), st>>>(p);
 }
 
-int supermer_max_ctas_per_sm(int mode, bool wide, int nreg, uint32_t n_buckets) {
-    size_t sm = supermer_smem_bytes(mode, n_buckets);
+int supermer_max_ctas_per_sm(int mode, int m, bool lexical, uint32_t n_buckets) {
     int n = 0;
-    const void* fn = wide ? (nreg == 2 ? (const void*)k_supermer<SM_DESC, true, 2, false>
-                                       : (const void*)k_supermer<SM_DESC, true, 3, false>)
-                          : (nreg == 2 ? (const void*)k_supermer<SM_DESC, false, 2, false>
-                                       : (const void*)k_supermer<SM_DESC, false, 3, false>);
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)supermer_smem_bytes(mode, SM_MAX_BUCKETS));
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, SM_WARPS * 32, sm) != cudaSuccess) n = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel(mode, m, lexical), SM_WARPS * 32,
+                                                      supermer_smem_bytes(mode, n_buckets)) != cudaSuccess)
+        n = 1;
     return n > 0 ? n : 1;
 }
 
