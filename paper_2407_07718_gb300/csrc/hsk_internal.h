@@ -164,14 +164,17 @@ void launch_compact(const uint64_t* sub_off, const uint32_t* kc, const uint64_t*
                     uint32_t n_groups, int key_words, const void* keys, const uint32_t* kcount, void* out_keys,
                     uint32_t* out_counts, uint64_t out_cap, int* err, int grid, cudaStream_t st);
 void launch_transpose_kc(const uint32_t* kc, uint32_t n_groups, uint32_t* kc_t, int grid, cudaStream_t st);
-// S6 on chip: sub-range r holds pairs [bounds[r], bounds[r+1]) of (kin, vin)
-// that share their key bits from shift up; each is sorted by its key and
-// written to the same range of (kout, vout).  A sub-range over
-// range_sort_cap() sets *too_big and is skipped.
+// S6 on chip: range r holds pairs [bounds[r], bounds[r+1]) of (kin, vin) that
+// share their top fixed_bits key bits; every range is sorted by key and
+// written to its place in (kout, vout).  `group` ranges (1 to 64, a power of
+// two; they share all but log2(group) of those bits) are claimed at a time.
+// Ranges over range_sort_cap() pairs are listed in big[1 ...], big[0] (zeroed)
+// counting them; tier 1 sorts listed ranges of up to 8192 pairs (`only` =
+// big + 1 of the first launch, n_ranges of them, group 1).
 uint32_t range_sort_cap(int key_words);
 void launch_range_sort(const void* kin, const uint32_t* vin, void* kout, uint32_t* vout, const uint64_t* bounds,
-                       uint32_t n_ranges, int key_words, int shift, int* too_big, uint32_t* claim, int num_sms,
-                       cudaStream_t st);
+                       const uint32_t* only, uint32_t n_ranges, uint32_t group, int tier, int key_words, int key_bits,
+                       int fixed_bits, uint32_t* big, uint32_t* claim, int num_sms, cudaStream_t st);
 void launch_ov_gather(const uint64_t* sub_off, const uint32_t* ov_list, uint32_t n_ov, uint64_t* ov_pre,
                       int key_words, const void* keys, void* dst, uint64_t dst_cap, int* err, int grid,
                       cudaStream_t st);

@@ -199,7 +199,6 @@ extern "C" int hsk_create(hsk_ctx** out, const hsk_config* cfg_in) {
         c->d_ndesc = (uint64_t*)(s + 32);
         c->d_nlocal = (uint64_t*)(s + 40);
         c->d_ovstats = (uint64_t*)(s + 48);
-        c->d_flag = (int*)(s + 112);
         c->counters = (uint32_t*)(s + 256);
         *out = c;
         return HSK_OK;
@@ -700,24 +699,44 @@ int hsk_order_pairs(hsk_ctx* c, void* keys, uint32_t* counts, uint64_t n, int ke
 }
 
 // Stage S6 for kept pairs laid out by their top digit (c->s6_bounds holds
-// the 257 digit starts): one segmented LSD pass on the second digit groups
-// every top-digit range into 256 sub-ranges, then each of the 65,536
-// sub-ranges is sorted on chip (k_range_sort).  *done = false leaves the
-// pairs for the general path (keys of fewer than 24 bits, or a sub-range over
-// the on-chip capacity; the pairs are then back in place, unsorted).
+// the 257 digit starts): when every top-digit range fits the on-chip sort
+// (k_range_sort), they are sorted at once; else one segmented pass on the
+// second digit groups every range into 256 sub-ranges first.  *done = false
+// leaves the pairs for the general path (keys of fewer than 24 bits, or a
+// sub-range over the on-chip capacity; the pairs are then back in place,
+// unsorted).
 static int order_pairs_msd(hsk_ctx* c, uint64_t n, int kw, int key_bits, cudaStream_t st, bool* done) {
     *done = false;
-    const int shift1 = key_bits - 16, shift2 = key_bits - 24;
-    if (shift2 < 0 || n < 2) return HSK_OK;
+    if (key_bits < 24 || n < 2) return HSK_OK;
     const size_t kb = (size_t)kw * 8;
     const uint64_t* d_bounds = (const uint64_t*)c->s6_bounds.p;
-    std::vector<uint64_t> hb(257);
-    CK(cudaMemcpyAsync(hb.data(), d_bounds, 257 * 8, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
+    std::vector<uint64_t>& hb = c->s6_h;
+    if (hb.size() != 257) {
+        hb.resize(257);
+        CK(cudaMemcpyAsync(hb.data(), d_bounds, 257 * 8, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+    }
     if (hb[256] != n) {
         hsk_set_error(c, "S6: %llu pairs laid out by digit, %llu expected", (unsigned long long)hb[256],
                       (unsigned long long)n);
         return HSK_ECUDA;
+    }
+    uint64_t largest = 0;
+    for (int d = 0; d < 256; ++d) largest = std::max(largest, hb[d + 1] - hb[d]);
+    TRY(hsk_ensure(c, c->pair_alt_keys, n * kb, false));
+    TRY(hsk_ensure(c, c->pair_alt_counts, n * 4, false));
+    TRY(hsk_ensure(c, c->pass_hist, 2 * (65536 + 16) * 4, false));  // digit counts; later two lists of ranges
+    uint32_t ep, *ctr;
+    if (largest <= range_sort_cap(kw)) {
+        TRY(hsk_next_counter(c, st, &ctr));
+        launch_range_sort(c->out_keys.p, (const uint32_t*)c->out_counts.p, c->pair_alt_keys.p,
+                          (uint32_t*)c->pair_alt_counts.p, d_bounds, nullptr, 256, 1, 0, kw, key_bits, 8,
+                          (uint32_t*)c->pass_hist.p, ctr, c->num_sms, st);
+        CK(cudaGetLastError());
+        std::swap(c->out_keys, c->pair_alt_keys);
+        std::swap(c->out_counts, c->pair_alt_counts);
+        *done = true;
+        return HSK_OK;
     }
     const uint64_t TILE = onesweep_tile_keys(kw);
     std::vector<uint32_t> ts(257);
@@ -729,34 +748,46 @@ static int order_pairs_msd(hsk_ctx* c, uint64_t n, int kw, int key_bits, cudaStr
     ts[256] = (uint32_t)tiles;
     TRY(hsk_ensure(c, c->seg, 257 * 4, false));
     CK(cudaMemcpyAsync(c->seg.p, ts.data(), 257 * 4, cudaMemcpyHostToDevice, st));
-    TRY(hsk_ensure(c, c->pass_hist, 256 * 256 * 8, false));
     TRY(hsk_ensure(c, c->digit_off, (256 * 256 + 1) * 8, false));
-    TRY(hsk_ensure(c, c->pair_alt_keys, n * kb, false));
-    TRY(hsk_ensure(c, c->pair_alt_counts, n * 4, false));
     TRY(hsk_ensure_status(c, tiles * 256 + 1, st));
     uint64_t* doff = (uint64_t*)c->digit_off.p;
     CK(cudaMemsetAsync(c->pass_hist.p, 0, 256 * 256 * 8, st));
-    launch_digit_hist_seg(c->out_keys.p, kw, d_bounds, 256, n, (uint64_t*)c->pass_hist.p, 1, st, shift1);
+    launch_digit_hist_seg(c->out_keys.p, kw, d_bounds, 256, n, (uint64_t*)c->pass_hist.p, 1, st, key_bits - 16);
     launch_digit_offsets_seg((const uint64_t*)c->pass_hist.p, d_bounds, doff, 1, 256, st);
     CK(cudaMemcpyAsync(doff + 256 * 256, &hb[256], 8, cudaMemcpyHostToDevice, st));
-    uint32_t ep, *ctr;
     TRY(hsk_next_epoch(c, st, &ep));
     TRY(hsk_next_counter(c, st, &ctr));
     launch_onesweep_seg(c->out_keys.p, c->pair_alt_keys.p, (const uint32_t*)c->out_counts.p,
                         (uint32_t*)c->pair_alt_counts.p, d_bounds, 256, (uint32_t)tiles, (const uint32_t*)c->seg.p, kw,
-                        shift1, doff, (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st);
-    CK(cudaMemsetAsync(c->d_flag, 0, sizeof(int), st));
+                        key_bits - 16, doff, (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st);
+    // sub-ranges are sorted a group at a time: about a third of the capacity
+    uint32_t group = 1;
+    while (group < 64 && n / 65536 * group * 2 <= range_sort_cap(kw) / 3) group *= 2;
+    uint32_t* big = (uint32_t*)c->pass_hist.p;  // free again
+    CK(cudaMemsetAsync(big, 0, 4, st));
     TRY(hsk_next_counter(c, st, &ctr));
     launch_range_sort(c->pair_alt_keys.p, (const uint32_t*)c->pair_alt_counts.p, c->out_keys.p,
-                      (uint32_t*)c->out_counts.p, doff, 256 * 256, kw, shift2, c->d_flag, ctr, c->num_sms, st);
+                      (uint32_t*)c->out_counts.p, doff, nullptr, 256 * 256, group, 0, kw, key_bits, 16, big, ctr,
+                      c->num_sms, st);
     CK(cudaGetLastError());
-    int too_big = 0;
-    CK(cudaMemcpyAsync(&too_big, c->d_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    if (too_big) {  // a sub-range over the on-chip capacity: the general path sorts all pairs
-        CK(cudaMemcpyAsync(c->out_keys.p, c->pair_alt_keys.p, n * kb, cudaMemcpyDeviceToDevice, st));
-        CK(cudaMemcpyAsync(c->out_counts.p, c->pair_alt_counts.p, n * 4, cudaMemcpyDeviceToDevice, st));
-        return HSK_OK;
+    for (int tier = 1;; ++tier) {
+        uint32_t n_big = 0;
+        CK(cudaMemcpyAsync(&n_big, big, 4, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        if (!n_big) break;
+        if (tier == 2) {  // a sub-range over every on-chip capacity: the general path sorts all pairs
+            CK(cudaMemcpyAsync(c->out_keys.p, c->pair_alt_keys.p, n * kb, cudaMemcpyDeviceToDevice, st));
+            CK(cudaMemcpyAsync(c->out_counts.p, c->pair_alt_counts.p, n * 4, cudaMemcpyDeviceToDevice, st));
+            return HSK_OK;
+        }
+        uint32_t* list = big + 1;
+        big += 65536 + 8;  // the next list
+        CK(cudaMemsetAsync(big, 0, 4, st));
+        TRY(hsk_next_counter(c, st, &ctr));
+        launch_range_sort(c->pair_alt_keys.p, (const uint32_t*)c->pair_alt_counts.p, c->out_keys.p,
+                          (uint32_t*)c->out_counts.p, doff, list, n_big, 1, 1, kw, key_bits, 16, big, ctr,
+                          c->num_sms, st);
+        CK(cudaGetLastError());
     }
     *done = true;
     return HSK_OK;
@@ -984,6 +1015,7 @@ static int local_chunk(hsk_ctx* c, const Supermers& S, const std::vector<uint32_
         launch_gather_u64(kc_off, d_at, 257, (uint64_t*)c->s6_bounds.p, st);
         CK(cudaGetLastError());
         c->s6_digit_major = O.n_pairs == 0;
+        c->s6_h.clear();
     }
     O.n_pairs += kept;
     if (n_ov) {  // the sub-segments that did not fit: global radix passes, then S5
@@ -1002,18 +1034,20 @@ static int local_chunk(hsk_ctx* c, const Supermers& S, const std::vector<uint32_
 }
 
 // Pairs of (keys, counts), n of them in any order, into the output buffers
-// partitioned by their top digit (hist: pairs per top digit, on the device):
-// stage S6's first partition.
+// partitioned by their top digit (hist: pairs per top digit): stage S6's
+// first partition.
 static int top_digit_pass(hsk_ctx* c, const void* keys, const uint32_t* counts, uint64_t n, int kw, int key_bits,
-                          const uint64_t* d_hist, cudaStream_t st) {
+                          const uint64_t* hist, cudaStream_t st) {
     const uint64_t TILE = onesweep_tile_keys(kw);
     const uint64_t tiles = (n + TILE - 1) / TILE;
     TRY(hsk_ensure(c, c->s6_bounds, 2 * 257 * 8, false));
     uint64_t* d_bounds = (uint64_t*)c->s6_bounds.p;
-    const uint64_t base[2] = {0, n};
-    CK(cudaMemcpyAsync(d_bounds + 257, base, sizeof(base), cudaMemcpyHostToDevice, st));
-    launch_digit_offsets_seg(d_hist, d_bounds + 257, d_bounds, 1, 1, st);
-    CK(cudaMemcpyAsync(d_bounds + 256, &base[1], 8, cudaMemcpyHostToDevice, st));
+    std::vector<uint64_t>& hb = c->s6_h;
+    hb.assign(259, 0);
+    for (int d = 0; d < 256; ++d) hb[d + 1] = hb[d] + hist[d];
+    hb[258] = n;  // hb[257], hb[258]: the one segment of the pass
+    CK(cudaMemcpyAsync(d_bounds, hb.data(), 259 * 8, cudaMemcpyHostToDevice, st));
+    hb.resize(257);
     TRY(hsk_ensure_status(c, tiles * 256 + 1, st));
     uint32_t ep, *ctr;
     TRY(hsk_next_epoch(c, st, &ep));
@@ -1091,7 +1125,7 @@ static int hash_chunk(hsk_ctx* c, const Supermers& S, uint32_t b0, uint32_t b1, 
                       list1, ctl + 2, (uint64_t*)c->hist.p, H, c->d_max, ctl + 1, ctl + 8, ctr, c->d_err, c->num_sms,
                       st);
     CK(cudaGetLastError());
-    uint64_t w[6];
+    uint64_t w[8 + 256];
     CK(cudaMemcpyAsync(w, ctl, sizeof(w), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     const uint32_t n1 = (uint32_t)w[2];
@@ -1114,7 +1148,7 @@ static int hash_chunk(hsk_ctx* c, const Supermers& S, uint32_t b0, uint32_t b1, 
     prof_mark(c, st, 4);
     const bool only = single && O.n_pairs == 0 && n2 == 0;
     if (only && 2 * k >= 24 && kept > 1) {
-        TRY(top_digit_pass(c, c->keys.p, (const uint32_t*)c->alt.p, kept, kw, 2 * k, ctl + 8, st));
+        TRY(top_digit_pass(c, c->keys.p, (const uint32_t*)c->alt.p, kept, kw, 2 * k, w + 8, st));
         c->s6_digit_major = true;
     } else if (kept) {
         CK(cudaMemcpyAsync((char*)c->out_keys.p + O.n_pairs * kb, c->keys.p, kept * kb, cudaMemcpyDeviceToDevice, st));

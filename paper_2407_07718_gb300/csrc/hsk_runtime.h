@@ -273,7 +273,6 @@ struct hsk_ctx {
     uint64_t* d_ndesc = nullptr;
     uint64_t* d_nlocal = nullptr;   // distinct k-mers counted on chip
     uint64_t* d_ovstats = nullptr;  // per on-chip step: [2i] low half = sub-segments it listed, [2i+1] their keys
-    int* d_flag = nullptr;          // S6: a sub-range was over the on-chip capacity
     uint32_t* counters = nullptr;
     uint32_t ctr_used = 0;
     uint32_t epoch = 0;
@@ -292,6 +291,7 @@ struct hsk_ctx {
     DevBuf s6_bounds;                                              // S6: where each top digit's kept pairs start
     DevBuf rec_sub, records2, part_off, hash_ctl, ov_records;      // hash path: sub-partitions, split records
     bool s6_digit_major = false;                                   // the output holds only digit-major pairs
+    std::vector<uint64_t> s6_h;                                    // S6: host copy of s6_bounds, when known
 
     // tuned parameters (0 = built-in default); see hsk_tune.cu
     struct Tune {

@@ -756,117 +756,173 @@ void launch_onesweep_seg(const void* kin, void* kout, const uint32_t* vin, uint3
 }
 
 // ---------------------------------------------------------------------------
-// S6 on chip: sort sub-ranges that already share their top digits
+// S6 on chip: sort ranges of pairs that already share their top bits
 // ---------------------------------------------------------------------------
-// After the kept pairs are laid out by their top digit and one segmented pass
-// has grouped each top-digit range by the second digit, every sub-range
-// holds pairs whose keys agree above bit `shift + 8`.  One CTA takes a
-// sub-range: it counts the keys' digit at `shift` (256 bins), places the
-// pairs bin by bin in shared memory, and writes each key to its sorted place:
-// the start of its bin plus the number of smaller keys in the bin (the keys
-// are distinct, so the places are too).
+// The kept pairs are laid out by their top digit, and for many pairs by the
+// second one too.  A CTA claims `group` consecutive ranges (1, or a power of
+// two of them that share their bits above the group) and sorts as many of them
+// together as fit its shared memory: pairs are counted into 4096 bins by the
+// next 12 bits, placed bin by bin, and every key goes to the start of its bin
+// plus the number of smaller keys in the bin (the keys are distinct, so the
+// places are too).  A pair's arrival number in its bin comes from the counting
+// atomic, so the placing needs none.
+//
+// Bound by latency between barriers for small ranges and by HBM for large
+// ones; 4096 bins leave about one key a bin, and one claim for many small
+// ranges replaces one claim each: 65,536 ranges of a few pairs took 0.43 ms
+// whatever the number of pairs (256 bins, one range a claim; now 0.01 ms for
+// 20,000 pairs), and 104 M 128-bit pairs 3.6 ms (now 1.6).
 constexpr int RS_NT = 512;
-template <typename K>
+constexpr int RS_BITS = 12;
+constexpr int RS_BINS = 1 << RS_BITS;
+constexpr int RS_GROUP = 64;  // most ranges a claim
+template <typename K, int TIER>
 struct RangeCfg;
 template <>
-struct RangeCfg<u64> {
-    static constexpr int CAP = 8192;  // 96 KB: two CTAs per SM
+struct RangeCfg<u64, 0> {
+    static constexpr int CAP = 6144, CTAS = 2;  // 72 + 16 KB
 };
 template <>
-struct RangeCfg<key128> {
-    static constexpr int CAP = 8192;  // 160 KB
+struct RangeCfg<key128, 0> {
+    static constexpr int CAP = 4096, CTAS = 2;  // 80 + 16 KB
 };
-uint32_t range_sort_cap(int key_words) { return key_words == 1 ? RangeCfg<u64>::CAP : RangeCfg<key128>::CAP; }
+template <>
+struct RangeCfg<u64, 1> {
+    static constexpr int CAP = 8192, CTAS = 1;
+};
+template <>
+struct RangeCfg<key128, 1> {
+    static constexpr int CAP = 8192, CTAS = 1;
+};
+uint32_t range_sort_cap(int key_words) { return key_words == 1 ? RangeCfg<u64, 0>::CAP : RangeCfg<key128, 0>::CAP; }
 
-template <typename K>
-__global__ void __launch_bounds__(RS_NT) k_range_sort(const K* __restrict__ kin, const uint32_t* __restrict__ vin,
-                                                      K* __restrict__ kout, uint32_t* __restrict__ vout,
-                                                      const u64* __restrict__ bounds, uint32_t n_ranges, int shift,
-                                                      int* too_big, uint32_t* claim) {
-    constexpr int CAP = RangeCfg<K>::CAP;
+template <typename K, int TIER>
+__global__ void __launch_bounds__(RS_NT, RangeCfg<K, TIER>::CTAS)
+    k_range_sort(const K* __restrict__ kin, const uint32_t* __restrict__ vin, K* __restrict__ kout,
+                 uint32_t* __restrict__ vout, const u64* __restrict__ bounds, const uint32_t* __restrict__ only,
+                 uint32_t n_claims, uint32_t group, int group_shift, int range_shift, uint32_t mask, uint32_t* big,
+                 uint32_t* claim) {
+    constexpr int CAP = RangeCfg<K, TIER>::CAP;
+    constexpr int PT = CAP / RS_NT, BPT = RS_BINS / RS_NT;
+    static_assert(CAP % RS_NT == 0, "pairs per thread");
     extern __shared__ __align__(16) unsigned char smem_rs[];
     K* sk = reinterpret_cast<K*>(smem_rs);
     uint32_t* sv = reinterpret_cast<uint32_t*>(sk + CAP);
-    __shared__ uint32_t s_cnt[RADIX], s_start[RADIX], s_fill[RADIX];
-    __shared__ uint32_t s_scr[RS_NT / 32 + 1];
+    uint32_t* s_bin = sv + CAP;  // [RS_BINS] counts, then starts
+    __shared__ uint32_t s_scr[RS_NT / 32];
+    __shared__ u64 s_b[RS_GROUP + 1];
     __shared__ uint32_t s_next;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (;;) {
         __syncthreads();
         if (tid == 0) s_next = atomicAdd(claim, 1u);
-        if (tid < RADIX) s_cnt[tid] = 0;
         __syncthreads();
-        const uint32_t r = s_next;
-        if (r >= n_ranges) break;
-        const u64 b = bounds[r], e = bounds[r + 1];
-        if (e <= b) continue;
-        const uint32_t n = (uint32_t)(e - b);
-        if (e - b > (u64)CAP) {
-            if (tid == 0) atomicExch(too_big, 1);
-            continue;
-        }
-        if (n == 1) {
-            if (tid == 0) {
-                kout[b] = kin[b];
-                vout[b] = vin[b];
+        if (s_next >= n_claims) break;
+        const uint32_t r0 = only ? only[s_next] : s_next * group;
+        if (tid <= (int)group) s_b[tid] = bounds[r0 + tid];
+        __syncthreads();
+        for (uint32_t i = 0; i < group;) {
+            uint32_t j = i + 1;
+            while (j < group && s_b[j + 1] - s_b[i] <= (u64)CAP) ++j;
+            const u64 b = s_b[i], len = s_b[j] - b;
+            const int shift = j == i + 1 ? range_shift : group_shift;
+            const uint32_t first = i;
+            i = j;
+            if (len == 0) continue;
+            if (len > (u64)CAP) {  // one range over the capacity: big[0] of them, listed
+                if (tid == 0) big[1 + atomicAdd(big, 1u)] = r0 + first;
+                continue;
             }
-            continue;
-        }
-        for (uint32_t i = tid; i < n; i += RS_NT) atomicAdd(&s_cnt[key_digit(kin[b + i], shift, 0xFF)], 1u);
-        __syncthreads();
-        uint32_t tot;
-        const uint32_t c = tid < RADIX ? s_cnt[tid] : 0u;
-        const uint32_t ex = block_excl_sum<RS_NT, uint32_t>(c, s_scr, tot);
-        if (tid < RADIX) {
-            s_start[tid] = ex;
-            s_fill[tid] = ex;
-        }
-        __syncthreads();
-        for (uint32_t i = tid; i < n; i += RS_NT) {
-            const K key = kin[b + i];
-            const uint32_t at = atomicAdd(&s_fill[key_digit(key, shift, 0xFF)], 1u);
-            sk[at] = key;
-            sv[at] = vin[b + i];
-        }
-        __syncthreads();
-        for (uint32_t i = tid; i < n; i += RS_NT) {
-            const K key = sk[i];
-            const uint32_t d = key_digit(key, shift, 0xFF);
-            const uint32_t bs = s_start[d], be = bs + s_cnt[d];
-            uint32_t rank = 0;
-            for (uint32_t j = bs; j < be; ++j) rank += key_lt(sk[j], key) ? 1u : 0u;
-            kout[b + bs + rank] = key;
-            vout[b + bs + rank] = sv[i];
+            const uint32_t n = (uint32_t)len;
+#pragma unroll
+            for (int t = 0; t < BPT; ++t) s_bin[t * RS_NT + tid] = 0;
+            __syncthreads();
+            K key[PT];
+            uint32_t at[PT];
+#pragma unroll
+            for (int t = 0; t < PT; ++t) {
+                const uint32_t q = (uint32_t)t * RS_NT + tid;
+                if (q < n) key[t] = kin[b + q];
+            }
+#pragma unroll
+            for (int t = 0; t < PT; ++t) {
+                const uint32_t q = (uint32_t)t * RS_NT + tid;
+                if (q < n) at[t] = atomicAdd(&s_bin[key_digit(key[t], shift, mask)], 1u);
+            }
+            __syncthreads();
+            uint32_t c[BPT], sum = 0;
+#pragma unroll
+            for (int t = 0; t < BPT; ++t) {
+                c[t] = s_bin[tid * BPT + t];
+                sum += c[t];
+            }
+            const uint32_t inc = warp_incl_sum<uint32_t>(sum);
+            if (lane == 31) s_scr[warp] = inc;
+            __syncthreads();
+            uint32_t run = inc - sum;
+            for (int w = 0; w < warp; ++w) run += s_scr[w];
+#pragma unroll
+            for (int t = 0; t < BPT; ++t) {
+                s_bin[tid * BPT + t] = run;
+                run += c[t];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int t = 0; t < PT; ++t) {
+                const uint32_t q = (uint32_t)t * RS_NT + tid;
+                if (q < n) {
+                    const uint32_t o = s_bin[key_digit(key[t], shift, mask)] + at[t];
+                    sk[o] = key[t];
+                    sv[o] = vin[b + q];
+                }
+            }
+            __syncthreads();
+            for (uint32_t q = tid; q < n; q += RS_NT) {
+                const K x = sk[q];
+                const uint32_t d = key_digit(x, shift, mask);
+                const uint32_t bs = s_bin[d], be = d + 1 < (uint32_t)RS_BINS ? s_bin[d + 1] : n;
+                uint32_t rank = 0;
+                if (be - bs > 1)
+                    for (uint32_t y = bs; y < be; ++y) rank += key_lt(sk[y], x) ? 1u : 0u;
+                kout[b + bs + rank] = x;
+                vout[b + bs + rank] = sv[q];
+            }
+            __syncthreads();
         }
     }
 }
 
 void launch_range_sort(const void* kin, const uint32_t* vin, void* kout, uint32_t* vout, const uint64_t* bounds,
-                       uint32_t n_ranges, int key_words, int shift, int* too_big, uint32_t* claim, int num_sms,
-                       cudaStream_t st) {
+                       const uint32_t* only, uint32_t n_ranges, uint32_t group, int tier, int key_words, int key_bits,
+                       int fixed_bits, uint32_t* big, uint32_t* claim, int num_sms, cudaStream_t st) {
     if (n_ranges == 0) return;
     count_launch();
+    // a group fixes log2(group) fewer of the keys' top bits than a range; the
+    // bins take the 12 bits below (all that are left, when fewer)
+    int gb = 0;
+    while ((1u << gb) < group) ++gb;
+    const int left = key_bits - fixed_bits, bits = left < RS_BITS ? left : RS_BITS;
+    const int range_shift = left - bits, group_shift = left + gb - RS_BITS > 0 ? left + gb - RS_BITS : 0;
+    const uint32_t mask = (1u << RS_BITS) - 1;
+    auto go = [&](auto kern, auto* kp, int cap, int ctas) {
+        const size_t dyn = (size_t)cap * (8 * key_words + 4) + RS_BINS * 4;
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+        const uint32_t claims = n_ranges / group;
+        const uint32_t want = (uint32_t)num_sms * ctas;
+        // with few bits left a range's mask covers them all: higher bits are fixed, so masking 12 is the same
+        kern<<<claims < want ? claims : want, RS_NT, dyn, st>>>((decltype(kp))kin, vin, kp, vout, (const u64*)bounds,
+                                                                only, claims, group, group_shift, range_shift, mask,
+                                                                big, claim);
+    };
+#define RS_GO(K, T) go(k_range_sort<K, T>, (K*)kout, RangeCfg<K, T>::CAP, RangeCfg<K, T>::CTAS)
     if (key_words == 1) {
-        const size_t dyn = (size_t)RangeCfg<u64>::CAP * 12;
-        cudaFuncSetAttribute(k_range_sort<u64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-        int occ = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_range_sort<u64>, RS_NT, dyn);
-        if (occ < 1) occ = 1;
-        const uint64_t want = (uint64_t)num_sms * occ;
-        const unsigned g = (unsigned)(n_ranges < want ? n_ranges : want);
-        k_range_sort<u64><<<g, RS_NT, dyn, st>>>((const u64*)kin, vin, (u64*)kout, vout, (const u64*)bounds,
-                                                 n_ranges, shift, too_big, claim);
+        if (tier) RS_GO(u64, 1);
+        else RS_GO(u64, 0);
     } else {
-        const size_t dyn = (size_t)RangeCfg<key128>::CAP * 20;
-        cudaFuncSetAttribute(k_range_sort<key128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-        int occ = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_range_sort<key128>, RS_NT, dyn);
-        if (occ < 1) occ = 1;
-        const uint64_t want = (uint64_t)num_sms * occ;
-        const unsigned g = (unsigned)(n_ranges < want ? n_ranges : want);
-        k_range_sort<key128><<<g, RS_NT, dyn, st>>>((const key128*)kin, vin, (key128*)kout, vout,
-                                                    (const u64*)bounds, n_ranges, shift, too_big, claim);
+        if (tier) RS_GO(key128, 1);
+        else RS_GO(key128, 0);
     }
+#undef RS_GO
 }
 
 // ---------------------------------------------------------------------------
