@@ -54,8 +54,12 @@ struct SmParams {
     int rec_words;            // 2 (k <= 32) or 4 (k <= 64)
     uint32_t grid;
     uint64_t tile_begin, tile_end;     // warp tiles [begin, end) of 1024 windows (end 0 = all)
-    int desc_sub;             // 1: windows with different sub-partitions (8 hash bits above the
-                              // bucket's) are different supermers, and descriptors carry them
+    // Fine partitions (part_rec != nullptr): the sub_bits (at most 8) hash bits
+    // above the bucket's split every bucket into 2^sub_bits of them; windows of
+    // different partitions are different supermers, descriptors carry the
+    // sub-partition, and records are counted per partition, bucket-major.
+    uint32_t* part_rec;                // [n_buckets << sub_bits] records per partition (atomic adds)
+    int sub_bits;
     uint64_t* desc;                    // supermer descriptors (DESC)
     uint64_t desc_cap;
     unsigned long long* desc_count;    // descriptors produced (may exceed desc_cap)
@@ -77,22 +81,25 @@ struct SmParams {
 size_t supermer_smem_bytes(int mode, uint32_t n_buckets);
 int supermer_max_ctas_per_sm(int mode, int m, bool lexical, uint32_t n_buckets);
 void launch_supermer(int mode, const SmParams& p, cudaStream_t st);
-// records from descriptors (and, with rec_sub, each record's sub-partition):
-// bucket_off[B+1] record offsets; cursor[b *
+// records from descriptors, in bucket order, or with part_cursor in order of
+// fine partitions (their first records; advanced) and in one orientation for
+// both strands: bucket_off[B+1] record offsets; cursor[b *
 // SCATTER_CURSOR_STRIDE] zeroed for every bucket b.  The cursors take every
 // descriptor's atomic: packed into 16 KB they fell into a few L2 slices, and
 // 128 bytes apart they spread over all of them (S3 took 6.2 ms packed, 5.35 ms
 // spread, on the long-read workload)
 constexpr uint32_t SCATTER_CURSOR_STRIDE = 32;
 void launch_scatter_desc(const uint64_t* desc, uint64_t n_desc, const uint64_t* packed, int k,
-                         const uint64_t* bucket_off, uint32_t* cursor, uint64_t* records, uint8_t* rec_sub,
-                         uint64_t n_records, int* err, int grid, cudaStream_t st);
+                         const uint64_t* bucket_off, uint32_t* cursor, uint64_t* part_cursor, int sub_bits,
+                         uint64_t* records, uint64_t n_records, int* err, int grid, cudaStream_t st);
 
 // exclusive scan of n uint32 counts into uint64 offsets; offsets[n] = total.
-// Scratch: scan_status_words(n) uint64 words.
+// Scratch: scan_status_words(n) uint64 words.  copy: the offsets once more;
+// bnd: every 2^bnd_bits-th of them, then the total.
 uint64_t scan_status_words(uint64_t n);
 void launch_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, uint64_t* status,
-                     uint32_t* tile_ctr, uint32_t epoch, int* err, cudaStream_t st);
+                     uint32_t* tile_ctr, uint32_t epoch, int* err, cudaStream_t st, uint64_t* copy = nullptr,
+                     uint64_t* bnd = nullptr, int bnd_bits = 0);
 
 // ---- S4 sort ---------------------------------------------------------------
 // Segment c: records [rec_base[c], rec_base[c+1]) expand to keys
@@ -180,12 +187,9 @@ void launch_ov_gather(const uint64_t* sub_off, const uint32_t* ov_list, uint32_t
                       cudaStream_t st);
 
 // ---- S4 + S5 by hashing (k_hash.cu) -------------------------------------------
-constexpr uint32_t HASH_MAX_SUB = 256;       // sub-partitions of a bucket at most
+constexpr int HASH_MAX_SUB_BITS = 8;             // fine partitions of a bucket: 2^8 at most
 constexpr uint64_t HASH_MAX_BASES = 1ull << 36;  // bases a descriptor with a sub-partition can address
 uint32_t hash_count_cap(int key_words);      // distinct k-mers the first tier's table holds
-void launch_split(const uint64_t* records, const uint8_t* rec_sub, const uint64_t* bucket_off, uint32_t first_bucket,
-                  uint32_t last_bucket, uint32_t nsub, int rec_words, uint64_t* out, uint64_t* part_off, int num_sms,
-                  cudaStream_t st);
 // Counts partitions (all of them, or the n_part listed in `only`): kept pairs
 // appended to (out_keys, out_counts) in no particular order, *out_n of them;
 // partitions that overfill the tier's table listed in ov_list, ov_stats =

@@ -423,45 +423,58 @@ static void fill_sm_params(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t 
     P.err = c->d_err;
 }
 
-// Count supermers per (bucket, CTA), scan to record offsets, scatter records.
-// With a set map the bases hold packed sets and B is the buckets of all sets.
+// S2 and S3: count supermers per bucket, scan to record offsets, scatter
+// records.  With a set map the bases hold packed sets and B is the buckets of
+// all sets.  sub_bits >= 0: every bucket is cut into 2^sub_bits fine
+// partitions, and the records come in their order (c->part_off: their first
+// records).
 static_assert(HSK_MAX_BUCKETS == 8192, "the S2 walk's shared-memory limit is sized for 8192 buckets");
 int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Supermers& S, cudaStream_t st,
-                  InputPipe* pipe, const SetMap* sets, bool want_sub) {
+                  InputPipe* pipe, const SetMap* sets, int sub_bits) {
     SmParams P;
     fill_sm_params(c, E, k, m, B, P);
-    P.desc_sub = want_sub;
     if (sets) {
         P.set_tile0 = sets->tile0;
         P.set_bucket = sets->bucket;
         P.set_bmask = sets->bmask;
         P.n_sets = sets->n;
     }
+    const bool fine = sub_bits >= 0;
+    const uint64_t F = fine ? (uint64_t)B << sub_bits : 0;
     const int occ = supermer_max_ctas_per_sm(SM_DESC, m, P.lexical, B);
     const uint64_t warp_tiles = (E.n_bases + 1023) / 1024;
     uint64_t g = std::min<uint64_t>((uint64_t)c->num_sms * occ, (warp_tiles + SM_CTA_WARPS - 1) / SM_CTA_WARPS);
     P.grid = (uint32_t)std::max<uint64_t>(g, 1);
     TRY(hsk_ensure(c, c->bucket_kmers, (uint64_t)B * 8, false));
     TRY(hsk_ensure(c, c->bucket_rec, ((uint64_t)B + 1) * 8, false));
-    // records per bucket, then the bucket cursors of the scatter (spread out)
-    const size_t cnt_bytes = (size_t)B * 4 * (1 + SCATTER_CURSOR_STRIDE);
+    // records per bucket, then the bucket cursors of the scatter (spread out);
+    // or the partitions' cursors, then records per partition
+    const size_t cnt_bytes = fine ? F * 12 : (size_t)B * 4 * (1 + SCATTER_CURSOR_STRIDE);
     TRY(hsk_ensure(c, c->cta_cnt, cnt_bytes, false));
-    uint32_t* d_rec_cnt = (uint32_t*)c->cta_cnt.p;
-    uint32_t* d_cursor = d_rec_cnt + B;
+    if (fine) TRY(hsk_ensure(c, c->part_off, (F + 1) * 8, false));
+    uint64_t* d_part_cursor = fine ? (uint64_t*)c->cta_cnt.p : nullptr;
+    uint32_t* d_rec_cnt = fine ? (uint32_t*)(d_part_cursor + F) : (uint32_t*)c->cta_cnt.p;
+    uint32_t* d_cursor = fine ? nullptr : d_rec_cnt + B;
     // descriptors: about 2/(w+1) supermers per window (random minimizers), plus
     // cuts at invalid bases, tile ends and the record cap; re-run if short
     uint64_t cap = std::min<uint64_t>(E.n_bases + 1, (uint64_t)((double)E.n_bases *
                                        (3.0 / (P.w + 1) + 1.0 / P.nmax + 1.0 / 256)) + (1u << 16));
     uint64_t n_desc = 0;
+    S.B = B;
+    S.h_bucket_kmers.resize(B);
+    S.h_bucket_rec.resize((size_t)B + 1);
     for (int attempt = 0; attempt < 2; ++attempt) {
         TRY(hsk_ensure(c, c->cta_off, cap * 8, false));
         CK(cudaMemsetAsync(c->bucket_kmers.p, 0, (size_t)B * 8, st));
-        CK(cudaMemsetAsync(d_rec_cnt, 0, cnt_bytes, st));
+        if (fine) CK(cudaMemsetAsync(d_rec_cnt, 0, F * 4, st));
+        else CK(cudaMemsetAsync(d_rec_cnt, 0, cnt_bytes, st));
         CK(cudaMemsetAsync(c->d_ndesc, 0, 8, st));
         P.desc = (uint64_t*)c->cta_off.p;
         P.desc_cap = cap;
         P.desc_count = (unsigned long long*)c->d_ndesc;
         P.bucket_rec = d_rec_cnt;
+        P.part_rec = fine ? d_rec_cnt : nullptr;
+        P.sub_bits = fine ? sub_bits : 0;
         P.bucket_kmers = (uint64_t*)c->bucket_kmers.p;
         if (pipe && attempt == 0) {
             // chunk i's bytes arrive on the copy stream: encode them, then walk
@@ -494,25 +507,25 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
             launch_supermer(SM_DESC, P, st);
         }
         CK(cudaGetLastError());
+        // record offsets of the buckets (and fine partitions)
+        TRY(hsk_ensure_status(c, scan_status_words(fine ? F : B), st));
+        uint32_t ep, *ctr;
+        TRY(hsk_next_epoch(c, st, &ep));
+        TRY(hsk_next_counter(c, st, &ctr));
+        if (fine)
+            launch_scan_u32(d_rec_cnt, F, (uint64_t*)c->part_off.p, (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st,
+                            d_part_cursor, (uint64_t*)c->bucket_rec.p, sub_bits);
+        else
+            launch_scan_u32(d_rec_cnt, B, (uint64_t*)c->bucket_rec.p, (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st);
+        CK(cudaGetLastError());
+        // bucket statistics to the host (needed to size records and plan chunks)
         CK(cudaMemcpyAsync(&n_desc, c->d_ndesc, 8, cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
+        CK(cudaMemcpyAsync(S.h_bucket_kmers.data(), c->bucket_kmers.p, (size_t)B * 8, cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(S.h_bucket_rec.data(), c->bucket_rec.p, ((size_t)B + 1) * 8, cudaMemcpyDeviceToHost, st));
+        TRY(hsk_read_device_error(c, st));
         if (n_desc <= cap) break;
         cap = n_desc;  // the walk counted every supermer: one more run fits them all
     }
-    // record offsets of the buckets
-    TRY(hsk_ensure_status(c, scan_status_words(B), st));
-    uint32_t ep, *ctr;
-    TRY(hsk_next_epoch(c, st, &ep));
-    TRY(hsk_next_counter(c, st, &ctr));
-    launch_scan_u32(d_rec_cnt, B, (uint64_t*)c->bucket_rec.p, (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st);
-    CK(cudaGetLastError());
-    // bucket statistics to the host (needed to size records and plan chunks)
-    S.B = B;
-    S.h_bucket_kmers.resize(B);
-    S.h_bucket_rec.resize((size_t)B + 1);
-    CK(cudaMemcpyAsync(S.h_bucket_kmers.data(), c->bucket_kmers.p, (size_t)B * 8, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(S.h_bucket_rec.data(), c->bucket_rec.p, ((size_t)B + 1) * 8, cudaMemcpyDeviceToHost, st));
-    TRY(hsk_read_device_error(c, st));
     S.n_records = S.h_bucket_rec[B];
     if (S.n_records != n_desc) {
         hsk_set_error(c, "supermer count mismatch: %llu descriptors, %llu records",
@@ -523,12 +536,11 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
     for (uint64_t v : S.h_bucket_kmers) S.n_kmers += v;
     S.rec_words = P.rec_words;
     S.nmax = P.nmax;
+    S.sub_bits = sub_bits;
     TRY(hsk_ensure(c, c->records, std::max<uint64_t>(S.n_records, 1) * P.rec_words * 8, false));
-    if (want_sub) TRY(hsk_ensure(c, c->rec_sub, std::max<uint64_t>(S.n_records, 1), false));
-    S.rec_sub = want_sub ? (const uint8_t*)c->rec_sub.p : nullptr;
     prof_mark(c, st, 1);
     launch_scatter_desc((const uint64_t*)c->cta_off.p, n_desc, E.packed, k, (const uint64_t*)c->bucket_rec.p,
-                        d_cursor, (uint64_t*)c->records.p, (uint8_t*)S.rec_sub, S.n_records, c->d_err,
+                        d_cursor, d_part_cursor, fine ? sub_bits : 0, (uint64_t*)c->records.p, S.n_records, c->d_err,
                         c->num_sms * 8, st);
     CK(cudaGetLastError());
     S.records = (const uint64_t*)c->records.p;
@@ -1065,40 +1077,19 @@ static int top_digit_pass(hsk_ctx* c, const void* keys, const uint32_t* counts, 
 static bool hash_path_fits(hsk_ctx* c, uint64_t n_windows, uint32_t B, int k, int m) {
     if (!c->cfg.local_sort || k < 12) return false;
     const double cap = hash_count_cap(k <= 32 ? 1 : 2);
-    const double per_part = (double)n_windows / ((double)B * HASH_MAX_SUB);
+    const double per_part = (double)n_windows / ((double)B * (1 << HASH_MAX_SUB_BITS));
     const double per_min = (double)n_windows * (k - m + 2) / std::pow(4.0, m);
     return n_windows >= HASH_MIN_KMERS && per_part <= cap && per_min <= cap;
 }
 
-// Bytes hsk_ensure would add for a buffer of `bytes`.
-static size_t buf_growth(const DevBuf& b, size_t bytes) {
-    return bytes > b.cap ? ((bytes + (2u << 20) - 1) & ~size_t((2u << 20) - 1)) - b.cap : 0;
-}
-
 // One chunk of buckets [b0, b1) through the hash path.  Kept pairs end in the
 // output buffers: partitioned by their top digit when they are the only ones.
-// *done = false (nothing counted) when the split records do not fit the
-// budget beside the pairs; the sorting path needs less.
 static int hash_chunk(hsk_ctx* c, const Supermers& S, uint32_t b0, uint32_t b1, uint64_t nk, bool single, int k,
-                      uint32_t lo, uint32_t hi, uint32_t H, Output& O, cudaStream_t st, bool* done) {
-    *done = false;
+                      uint32_t lo, uint32_t hi, uint32_t H, Output& O, cudaStream_t st) {
     const int kw = k <= 32 ? 1 : 2;
     const size_t kb = (size_t)kw * 8;
-    const uint32_t nb = b1 - b0;
-    const uint64_t rec0 = S.h_bucket_rec[b0], n_rec = S.h_bucket_rec[b1] - rec0;
-    // sub-partitions per bucket: about half the table's k-mers per partition
-    uint32_t nsub = 1;
-    while (nsub < HASH_MAX_SUB && nk > (uint64_t)nb * nsub * (hash_count_cap(kw) / 2)) nsub *= 2;
-    const uint32_t n_part = nb * nsub;
+    const uint32_t n_part = (b1 - b0) << S.sub_bits;
     const uint64_t cap = nk / std::max<uint32_t>(lo, 1) + 1;  // a kept k-mer has at least lo copies
-    {
-        size_t need = buf_growth(c->keys, cap * kb) + buf_growth(c->alt, cap * 4) +
-                      buf_growth(c->hash_ctl, (size_t)n_part * 8 + 4096);
-        if (nsub > 1)
-            need += buf_growth(c->records2, n_rec * S.rec_words * 8) + buf_growth(c->part_off, ((size_t)n_part + 1) * 8);
-        if (c->allocated + need > c->budget) return HSK_OK;
-    }
-    *done = true;
     TRY(hsk_ensure(c, c->keys, cap * kb, false));
     TRY(hsk_ensure(c, c->alt, cap * 4, false));
     // control words: out_n, distinct, {listed, records} x 2, kept pairs per top digit; then the two lists
@@ -1109,15 +1100,7 @@ static int hash_chunk(hsk_ctx* c, const Supermers& S, uint32_t b0, uint32_t b1, 
     uint32_t* list2 = list1 + n_part;
     CK(cudaMemsetAsync(ctl, 0, ctl_words * 8, st));
     const uint64_t* recs = S.records;
-    const uint64_t* part_off = (const uint64_t*)c->bucket_rec.p + b0;
-    if (nsub > 1) {
-        TRY(hsk_ensure(c, c->records2, n_rec * S.rec_words * 8, false));
-        TRY(hsk_ensure(c, c->part_off, ((uint64_t)n_part + 1) * 8, false));
-        launch_split(S.records, S.rec_sub, (const uint64_t*)c->bucket_rec.p, b0, b1, nsub, S.rec_words,
-                     (uint64_t*)c->records2.p, (uint64_t*)c->part_off.p, c->num_sms, st);
-        recs = (const uint64_t*)c->records2.p;
-        part_off = (const uint64_t*)c->part_off.p;
-    }
+    const uint64_t* part_off = (const uint64_t*)c->part_off.p + ((uint64_t)b0 << S.sub_bits);
     prof_mark(c, st, 3);
     uint32_t* ctr;
     TRY(hsk_next_counter(c, st, &ctr));
@@ -1141,9 +1124,6 @@ static int hash_chunk(hsk_ctx* c, const Supermers& S, uint32_t b0, uint32_t b1, 
     const uint32_t n2 = (uint32_t)w[4];
     const uint64_t kept = w[0];
     O.n_distinct += w[1];
-    // the split records are no longer read: give them back where the pairs need their room
-    const bool tight = c->allocated + 3 * (O.n_pairs + kept) * (kb + 4) > c->budget;
-    if (tight && n2 == 0) free_buf(c, c->records2);
     TRY(hsk_grow_output(c, O, O.n_pairs + kept, kw, st));
     prof_mark(c, st, 4);
     const bool only = single && O.n_pairs == 0 && n2 == 0;
@@ -1184,7 +1164,6 @@ static int hash_chunk(hsk_ctx* c, const Supermers& S, uint32_t b0, uint32_t b1, 
         CK(cudaMemcpyAsync(L.h_bucket_kmers.data(), d_kmers, (size_t)n2 * 8, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
         L.records = (const uint64_t*)c->ov_records.p;
-        if (tight) free_buf(c, c->records2);
         for (uint64_t v : L.h_bucket_kmers) L.n_kmers += v;
         const uint64_t per_group = 256ull * local_cap(kw) / (c->tune.group_div ? c->tune.group_div : 3);
         const uint32_t C_want = (uint32_t)std::min<uint64_t>(n2, std::max<uint64_t>(1, L.n_kmers / per_group));
@@ -1224,13 +1203,20 @@ int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, ui
     prof_mark(c, st, 0);
     Supermers S;
     uint32_t B = hsk_pick_buckets(c, n_bases, k);
-    const bool want_sub = n_bases < HASH_MAX_BASES && hash_path_fits(c, n_bases, B, k, m);
+    int sub_bits = -1;
+    if (n_bases < HASH_MAX_BASES && hash_path_fits(c, n_bases, B, k, m)) {
+        // fine partitions of half a batch's k-mers at most
+        for (sub_bits = 0; sub_bits < HASH_MAX_SUB_BITS;) {
+            if (n_bases <= ((uint64_t)B << sub_bits) * (hash_count_cap(kw) / 2)) break;
+            ++sub_bits;
+        }
+    }
     {
         NvtxRange r("S2-S3 supermers");
-        TRY(hsk_supermers(c, E, k, m, B, S, st, pipe, nullptr, want_sub));
+        TRY(hsk_supermers(c, E, k, m, B, S, st, pipe, nullptr, sub_bits));
     }
     prof_mark(c, st, 2);
-    const bool hash = want_sub && hash_path_fits(c, S.n_kmers, B, k, m);
+    const bool hash = sub_bits >= 0 && hash_path_fits(c, S.n_kmers, B, k, m);
     R.n_windows = S.n_kmers;
     R.n_supermers = S.n_records;
     std::vector<std::pair<uint32_t, uint32_t>> chunks;
@@ -1246,10 +1232,9 @@ int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, ui
         if (nk == 0) continue;
         if (hash) {
             NvtxRange r("S4-S5 on-chip hash count");
-            bool done = false;
-            TRY(hash_chunk(c, S, ch.first, ch.second, nk, chunks.size() == 1, k, lo, hi, H, O, st, &done));
+            TRY(hash_chunk(c, S, ch.first, ch.second, nk, chunks.size() == 1, k, lo, hi, H, O, st));
             unordered = true;
-            if (done) continue;
+            continue;
         }
         if (c->cfg.local_sort) {
             // groups of about a third of the on-chip capacity per top digit

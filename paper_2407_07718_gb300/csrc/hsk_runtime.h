@@ -46,7 +46,7 @@ struct Supermers {
     uint64_t n_records = 0, n_kmers = 0;
     int rec_words = 2, nmax = 0;
     const uint64_t* records = nullptr;
-    const uint8_t* rec_sub = nullptr;      // each record's sub-partition (hash path), or none
+    int sub_bits = -1;                     // records in order of 2^sub_bits fine partitions per bucket; -1: none
 };
 
 struct Output {
@@ -289,7 +289,7 @@ struct hsk_ctx {
     DevBuf pack_tab, pack_stat;                                    // packed sets: set tables, per-set statistics
     DevBuf ext_tab, ext_occ;                                       // extension information: key table, occurrence arrays
     DevBuf s6_bounds;                                              // S6: where each top digit's kept pairs start
-    DevBuf rec_sub, records2, part_off, hash_ctl, ov_records;      // hash path: sub-partitions, split records
+    DevBuf part_off, hash_ctl, ov_records;                         // hash path: partitions, control words and lists
     bool s6_digit_major = false;                                   // the output holds only digit-major pairs
     std::vector<uint64_t> s6_h;                                    // S6: host copy of s6_bounds, when known
 
@@ -335,7 +335,7 @@ struct hsk_ctx {
                 &bucket_rec, &records, &keys, &alt, &pass_hist, &digit_off, &lb_status, &seg, &heads, &rle_tiles,
                 &out_keys, &out_counts, &hist, &pair_alt_keys, &pair_alt_counts, &loc_tab, &batch_a,
                 &batch_b, &batch_c, &batch_d, &pack_tab, &pack_stat, &ext_tab, &ext_occ, &s6_bounds,
-                &rec_sub, &records2, &part_off, &hash_ctl, &ov_records};
+                &part_off, &hash_ctl, &ov_records};
     }
 };
 
@@ -406,7 +406,7 @@ int hsk_grow_output(hsk_ctx* c, const Output& O, uint64_t need, int key_words, c
 std::vector<uint32_t> hsk_group_buckets(const Supermers& S, uint32_t b0, uint32_t b1, uint32_t C_want);
 int hsk_plan_chunks(hsk_ctx* c, const Supermers& S, int key_words, std::vector<std::pair<uint32_t, uint32_t>>& chunks);
 int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Supermers& S, cudaStream_t st,
-                  InputPipe* pipe, const SetMap* sets = nullptr, bool want_sub = false);
+                  InputPipe* pipe, const SetMap* sets = nullptr, int sub_bits = -1);
 uint32_t hsk_pick_buckets(hsk_ctx* c, uint64_t n_bases, int k);
 int hsk_plain_sort(hsk_ctx* c, void* keys, uint32_t* vals, uint64_t n, int key_words, int key_bits, DevBuf& alt_keys,
                    DevBuf* alt_vals, cudaStream_t st);

@@ -1,7 +1,7 @@
-// k_hash.cu -- stage S4 + S5 by hashing on chip: the supermer records of a
-// bucket are split further by the minimizer's hash into fine partitions, and
-// one CTA counts the k-mers of a few partitions at a time in a shared-memory
-// table, straight from the records.
+// k_hash.cu -- stage S4 + S5 by hashing on chip: the supermer records come
+// scattered into fine partitions (the minimizer's bucket and more bits of its
+// hash), and one CTA counts the k-mers of a few partitions at a time in shared
+// memory, straight from the records.
 //
 // A k-mer value never lands in two partitions (all its occurrences share the
 // canonical minimizer and so its hash), so partitions are the paper's tasks
@@ -9,8 +9,6 @@
 // The k-mers themselves are never written to memory: a record of 16 (k <= 32)
 // or 32 bytes stands for all k-mers of its supermer.
 //
-//   k_split       -- records of a bucket -> its fine partitions (one CTA per
-//                    bucket: count, scan, scatter; no global atomics).
 //   k_hash_count  -- per batch of whole partitions: equal records are merged
 //                    first (reads of the same locus repeat whole supermers;
 //                    the records come in one orientation for both strands),
@@ -26,88 +24,10 @@
 // What it replaces and measured (one GB300): writing every key to its (group,
 // top digit) sub-segment and sorting the sub-segments on chip (k_local.cu)
 // took 39 ms on 1.5 G windows of 30x long reads (k = 31) and 45 ms on 1.27 G
-// of 20x short reads (k = 55); the split takes 2.1 and 1.3 ms, the counting
-// 4.9 and 13.0 ms.
+// of 20x short reads (k = 55); this takes 4.9 and 13.0 ms.
 #include "hsk_device.cuh"
 
 namespace hsk {
-
-// ---------------------------------------------------------------------------
-// fine partitions
-// ---------------------------------------------------------------------------
-constexpr int SPLIT_NT = 512;
-
-// Bucket b (first_bucket <= b < last_bucket) holds records
-// [bucket_off[b], bucket_off[b+1]) with their sub-partition in rec_sub; they
-// go to partitions b * nsub + (sub & (nsub - 1)), in order of partition, at
-// out (record bucket_off[first_bucket] first).  part_off receives each
-// partition's first record, relative to out.
-template <int RW>
-__global__ void __launch_bounds__(SPLIT_NT) k_split(const u64* __restrict__ rec, const uint8_t* __restrict__ rec_sub,
-                                                    const u64* __restrict__ bucket_off, uint32_t first_bucket,
-                                                    uint32_t last_bucket, uint32_t nsub, u64* __restrict__ out,
-                                                    u64* __restrict__ part_off) {
-    __shared__ uint32_t s_cnt[256];
-    __shared__ uint32_t s_scr[SPLIT_NT / 32 + 1];
-    const int tid = threadIdx.x;
-    const u64 rec0 = bucket_off[first_bucket];
-    for (uint32_t b = first_bucket + blockIdx.x; b < last_bucket; b += gridDim.x) {
-        const u64 r0 = bucket_off[b];
-        const uint32_t n = (uint32_t)(bucket_off[b + 1] - r0);
-        const uint8_t* sub = rec_sub + r0;
-        if (tid < 256) s_cnt[tid] = 0;
-        __syncthreads();
-        for (uint32_t i = tid; i < n; i += SPLIT_NT) atomicAdd(&s_cnt[sub[i] & (nsub - 1)], 1u);
-        __syncthreads();
-        const uint32_t c = tid < 256 ? s_cnt[tid] : 0u;
-        uint32_t total;
-        const uint32_t e = block_excl_sum<SPLIT_NT, uint32_t>(c, s_scr, total);
-        if (tid < 256) s_cnt[tid] = e;
-        if (tid < (int)nsub) part_off[(u64)(b - first_bucket) * nsub + tid] = r0 - rec0 + e;
-        if (b + 1 == last_bucket && tid == 0) part_off[(u64)(last_bucket - first_bucket) * nsub] = r0 - rec0 + n;
-        __syncthreads();
-        constexpr int UR = RW == 2 ? 4 : 2;  // records a thread holds at a time
-        const ulonglong2* src = reinterpret_cast<const ulonglong2*>(rec + r0 * RW);
-        ulonglong2* dst = reinterpret_cast<ulonglong2*>(out + (r0 - rec0) * RW);
-        for (uint32_t i0 = tid; i0 < n; i0 += SPLIT_NT * UR) {
-            ulonglong2 v[UR][RW / 2];
-            uint32_t d[UR];
-#pragma unroll
-            for (int j = 0; j < UR; ++j) {
-                const uint32_t i = i0 + j * SPLIT_NT;
-                if (i < n) {
-                    d[j] = sub[i] & (nsub - 1);
-#pragma unroll
-                    for (int q = 0; q < RW / 2; ++q) v[j][q] = src[(size_t)i * (RW / 2) + q];
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < UR; ++j) {
-                if (i0 + j * SPLIT_NT < n) {
-                    const uint32_t at = atomicAdd(&s_cnt[d[j]], 1u);
-#pragma unroll
-                    for (int q = 0; q < RW / 2; ++q) dst[(size_t)at * (RW / 2) + q] = v[j][q];
-                }
-            }
-        }
-        __syncthreads();
-    }
-}
-
-void launch_split(const uint64_t* records, const uint8_t* rec_sub, const uint64_t* bucket_off, uint32_t first_bucket,
-                  uint32_t last_bucket, uint32_t nsub, int rec_words, uint64_t* out, uint64_t* part_off, int num_sms,
-                  cudaStream_t st) {
-    if (last_bucket <= first_bucket) return;
-    count_launch();
-    const uint32_t nb = last_bucket - first_bucket;
-    const unsigned g = nb < (uint32_t)num_sms * 4 ? nb : (unsigned)num_sms * 4;
-    if (rec_words == 2)
-        k_split<2><<<g, SPLIT_NT, 0, st>>>((const u64*)records, rec_sub, (const u64*)bucket_off, first_bucket,
-                                           last_bucket, nsub, (u64*)out, (u64*)part_off);
-    else
-        k_split<4><<<g, SPLIT_NT, 0, st>>>((const u64*)records, rec_sub, (const u64*)bucket_off, first_bucket,
-                                           last_bucket, nsub, (u64*)out, (u64*)part_off);
-}
 
 // ---------------------------------------------------------------------------
 // count the k-mers of partitions in a shared-memory table

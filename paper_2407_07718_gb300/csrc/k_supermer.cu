@@ -107,15 +107,10 @@ __device__ __forceinline__ u64 keep_bases(u64 x, int nb) {
 }
 
 // Descriptor of a supermer, from its combined bucket b = bucket | sub << 13.
-// Plain: start base (40 bits), k-mers (8), bucket (16).  With sub-partitions:
+// Plain: start base (40 bits), k-mers (8), bucket (16).  With fine partitions:
 // start base (36), k-mers (7), bucket (13), sub-partition (8).
-__device__ __forceinline__ u64 make_desc(u64 pos, uint32_t n, uint32_t b, int sub) {
-    return sub ? pos | ((u64)n << 36) | ((u64)b << 43) : pos | ((u64)n << 40) | ((u64)b << 48);
-}
-__device__ __forceinline__ void split_desc(u64 d, int sub, u64& pos, uint32_t& n, uint32_t& bucket) {
-    pos = d & (sub ? (1ULL << 36) - 1 : (1ULL << 40) - 1);
-    n = sub ? (uint32_t)(d >> 36) & 0x7F : (uint32_t)(d >> 40) & 0xFF;
-    bucket = sub ? (uint32_t)(d >> 43) & 0x1FFF : (uint32_t)(d >> 48);
+__device__ __forceinline__ u64 make_desc(u64 pos, uint32_t n, uint32_t b, bool fine) {
+    return fine ? pos | ((u64)n << 36) | ((u64)b << 43) : pos | ((u64)n << 40) | ((u64)b << 48);
 }
 
 // Window minima of a tile.  Lane l holds the scores of positions 32 l .. 32 l
@@ -331,10 +326,10 @@ __global__ void __launch_bounds__(SM_WARPS * 32, SM_CTAS) k_supermer(const __gri
                 P.dump_minhash[p] = min(row_at(rows, lane, j), row_at(rows, lane, j + off));
             }
         } else {
-            // id of a window: its bucket and, with sub-partitions, the hash bits
-            // above; D has bit j set where window j's id differs from window j - 1's
+            // id of a window: its bucket and, with fine partitions, the hash bits
+            // above it; D has bit j set where window j's id differs from window j - 1's
             const int bb = __popc(bmask);
-            const uint32_t idmask = P.desc_sub ? (bmask << 8) | 0xFFu : bmask;
+            const uint32_t idmask = (((bmask + 1u) << P.sub_bits) - 1u);
             uint32_t D = 0, prev = 0;
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
@@ -366,10 +361,11 @@ __global__ void __launch_bounds__(SM_WARPS * 32, SM_CTAS) k_supermer(const __gri
                 int extra = 0;  // pieces past the first of runs of more than nmax k-mers
                 auto desc_at = [&](u64 at, int pos, int n, uint32_t id) {
                     const uint32_t b = bbase + (id & bmask);
-                    atomicAdd(&s_cnt[b], 1u);
+                    if (P.part_rec) atomicAdd(P.part_rec + ((b << P.sub_bits) | (id >> bb)), 1u);
+                    else atomicAdd(&s_cnt[b], 1u);
                     atomicAdd(&s_km[b], (uint32_t)n);
                     if (at < P.desc_cap)
-                        P.desc[at] = make_desc(p0 + pos, (uint32_t)n, b | (id >> bb) << 13, P.desc_sub);
+                        P.desc[at] = make_desc(p0 + pos, (uint32_t)n, b | (id >> bb) << 13, P.part_rec != nullptr);
                 };
                 for (uint32_t S = start; S; S &= S - 1) {
                     const int j = __ffs(S) - 1;
@@ -477,14 +473,24 @@ __device__ __forceinline__ void one_strand(u64 (&r)[RW], int nb) {
 // one tile, so these reads hit L1/L2).  The kernel waits on memory: each
 // thread takes SD descriptors at a time and issues their loads and cursor
 // atomics together (SD = 4: long-read S3 5.35 -> 4.40 ms; 8 was slower).
-template <bool WIDE>
+//
+// FINE: straight into the fine partitions, whose cursors start at their first
+// record.  The records of a partition arrive one by one, but the partitions'
+// open sectors (1 M x 32 bytes) stay in L2, so they leave it whole.  What
+// bounds it is L2 requests: one atomic and one write per record.  Scattering
+// into the buckets (4.4 and 3.8 ms; 5.9 and 4.4 with the sub-partition beside
+// each record) and from there into the partitions (2.1 and 1.3 ms) took 8.0
+// and 5.7 ms on the long- and short-read workloads; this takes 5.0 to 5.8 and
+// 3.9 (and 0.1 of the walk, which counts records per partition).  Two passes,
+// each over half of the partitions, took 4.7 and 4.3.
+template <bool WIDE, bool FINE>
 __global__ void __launch_bounds__(256) k_scatter_desc(const u64* __restrict__ desc, u64 n_desc,
                                                       const u64* __restrict__ packed, int k,
                                                       const u64* __restrict__ bucket_off, uint32_t* cursor,
-                                                      u64* __restrict__ records, uint8_t* __restrict__ rec_sub,
-                                                      u64 n_records, int* err) {
-    const int sub = rec_sub != nullptr;
+                                                      unsigned long long* part_cursor, int sub_bits,
+                                                      u64* __restrict__ records, u64 n_records, int* err) {
     constexpr int SD = 4;
+    constexpr int RW = WIDE ? 4 : 2;
     const u64 stride = (u64)gridDim.x * blockDim.x * SD;
     for (u64 i0 = (u64)blockIdx.x * blockDim.x * SD + threadIdx.x; i0 < n_desc; i0 += stride) {
         u64 dd[SD], slot[SD];
@@ -497,29 +503,30 @@ __global__ void __launch_bounds__(256) k_scatter_desc(const u64* __restrict__ de
         for (int j = 0; j < SD; ++j) {
             slot[j] = ~0ULL;
             if (dd[j] != ~0ULL) {
-                u64 pos;
-                uint32_t n, b;
-                split_desc(dd[j], sub, pos, n, b);
-                slot[j] = bucket_off[b] + atomicAdd(cursor + (size_t)b * SCATTER_CURSOR_STRIDE, 1u);
+                if constexpr (FINE) {
+                    const uint32_t b = (uint32_t)(dd[j] >> 43) & 0x1FFFu, sub = (uint32_t)(dd[j] >> 56);
+                    slot[j] = atomicAdd(part_cursor + ((b << sub_bits) | sub), 1ULL);
+                } else {
+                    const uint32_t b = (uint32_t)(dd[j] >> 48);
+                    slot[j] = bucket_off[b] + atomicAdd(cursor + (size_t)b * SCATTER_CURSOR_STRIDE, 1u);
+                }
             }
         }
 #pragma unroll
         for (int j = 0; j < SD; ++j) {
             if (dd[j] == ~0ULL) continue;
-            u64 pos;
-            uint32_t n, b;
-            split_desc(dd[j], sub, pos, n, b);
-            if (slot[j] >= n_records || slot[j] >= bucket_off[b + 1]) {
+            const u64 d = dd[j];
+            const u64 pos = d & (FINE ? (1ULL << 36) - 1 : (1ULL << 40) - 1);
+            const uint32_t n = FINE ? (uint32_t)(d >> 36) & 0x7F : (uint32_t)(d >> 40) & 0xFF;
+            if (slot[j] >= n_records || (!FINE && slot[j] >= bucket_off[(uint32_t)(d >> 48) + 1])) {
                 raise_error(err, HSK_DERR_BOUNDS);
                 continue;
             }
-            if (sub) rec_sub[slot[j]] = (uint8_t)(dd[j] >> 56);
             const int nb = (int)n + k - 1;  // bases in the record
-            constexpr int RW = WIDE ? 4 : 2;
             u64 r[RW];
 #pragma unroll
             for (int q = 0; q < RW; ++q) r[q] = keep_bases(extract_k64(packed, pos + 32 * q, 32), nb - 32 * q);
-            if (sub) one_strand<RW>(r, nb);
+            if (FINE) one_strand<RW>(r, nb);
             r[RW - 1] |= (u64)n;
             ulonglong2* dst = reinterpret_cast<ulonglong2*>(records) + (RW / 2) * slot[j];
 #pragma unroll
@@ -529,18 +536,23 @@ __global__ void __launch_bounds__(256) k_scatter_desc(const u64* __restrict__ de
 }
 
 void launch_scatter_desc(const uint64_t* desc, uint64_t n_desc, const uint64_t* packed, int k,
-                         const uint64_t* bucket_off, uint32_t* cursor, uint64_t* records, uint8_t* rec_sub,
-                         uint64_t n_records, int* err, int grid, cudaStream_t st) {
+                         const uint64_t* bucket_off, uint32_t* cursor, uint64_t* part_cursor, int sub_bits,
+                         uint64_t* records, uint64_t n_records, int* err, int grid, cudaStream_t st) {
     if (n_desc == 0) return;
     count_launch();
     uint64_t need = (n_desc + 4 * 256 - 1) / (4 * 256);  // four descriptors a thread
     unsigned g = (unsigned)(need < (uint64_t)grid ? need : (uint64_t)grid);
-    if (k <= 32)
-        k_scatter_desc<false><<<g, 256, 0, st>>>((const u64*)desc, n_desc, (const u64*)packed, k,
-                                                 (const u64*)bucket_off, cursor, (u64*)records, rec_sub, n_records, err);
-    else
-        k_scatter_desc<true><<<g, 256, 0, st>>>((const u64*)desc, n_desc, (const u64*)packed, k,
-                                                (const u64*)bucket_off, cursor, (u64*)records, rec_sub, n_records, err);
+    auto go = [&](auto kern) {
+        kern<<<g, 256, 0, st>>>((const u64*)desc, n_desc, (const u64*)packed, k, (const u64*)bucket_off, cursor,
+                                (unsigned long long*)part_cursor, sub_bits, (u64*)records, n_records, err);
+    };
+    if (part_cursor) {
+        if (k <= 32) go(k_scatter_desc<false, true>);
+        else go(k_scatter_desc<true, true>);
+    } else {
+        if (k <= 32) go(k_scatter_desc<false, false>);
+        else go(k_scatter_desc<true, false>);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -551,8 +563,11 @@ constexpr int SCAN_TILE = 256 * SCAN_ITEMS;
 
 uint64_t scan_status_words(uint64_t n) { return ((n + SCAN_TILE - 1) / SCAN_TILE + 1) * LB_PAD; }
 
+// Also, when asked: a second copy of the offsets (cursors), and every
+// 2^bnd_bits-th offset and the total (bnd).
 __global__ void __launch_bounds__(256) k_scan_u32(const uint32_t* __restrict__ in, uint64_t n,
-                                                  u64* __restrict__ out, u64* status,
+                                                  u64* __restrict__ out, u64* __restrict__ copy,
+                                                  u64* __restrict__ bnd, int bnd_bits, u64* status,
                                                   uint32_t* tile_ctr, uint32_t epoch, int* err) {
     __shared__ uint32_t s_tile;
     __shared__ u64 s_scr[9];
@@ -585,21 +600,31 @@ __global__ void __launch_bounds__(256) k_scan_u32(const uint32_t* __restrict__ i
     u64 run = s_prefix + excl;
 #pragma unroll
     for (int i = 0; i < SCAN_ITEMS; ++i) {
-        if (base + i < n) out[base + i] = run;
+        const u64 at = base + i;
+        if (at < n) {
+            out[at] = run;
+            if (copy) copy[at] = run;
+            if (bnd && (at & ((1ULL << bnd_bits) - 1)) == 0) bnd[at >> bnd_bits] = run;
+        }
         run += v[i];
     }
-    if (base < n && base + SCAN_ITEMS >= n) out[n] = run;  // total
+    if (base < n && base + SCAN_ITEMS >= n) {  // total
+        out[n] = run;
+        if (bnd) bnd[(n + (1ULL << bnd_bits) - 1) >> bnd_bits] = run;
+    }
 }
 
 void launch_scan_u32(const uint32_t* in, uint64_t n, uint64_t* out, uint64_t* status,
-                     uint32_t* tile_ctr, uint32_t epoch, int* err, cudaStream_t st) {
+                     uint32_t* tile_ctr, uint32_t epoch, int* err, cudaStream_t st, uint64_t* copy, uint64_t* bnd,
+                     int bnd_bits) {
     if (n == 0) {
         cudaMemsetAsync(out, 0, sizeof(uint64_t), st);
         return;
     }
     uint64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
     count_launch();
-    k_scan_u32<<<(unsigned)tiles, 256, 0, st>>>(in, n, (u64*)out, (u64*)status, tile_ctr, epoch, err);
+    k_scan_u32<<<(unsigned)tiles, 256, 0, st>>>(in, n, (u64*)out, (u64*)copy, (u64*)bnd, bnd_bits, (u64*)status,
+                                                tile_ctr, epoch, err);
 }
 
 }  // namespace hsk
