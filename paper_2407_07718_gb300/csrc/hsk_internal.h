@@ -191,14 +191,22 @@ constexpr int HASH_MAX_SUB_BITS = 8;             // fine partitions of a bucket:
 constexpr uint64_t HASH_MAX_BASES = 1ull << 36;  // bases a descriptor with a sub-partition can address
 uint32_t hash_count_cap(int key_words);      // distinct k-mers the first tier's table holds
 // Counts partitions (all of them, or the n_part listed in `only`): kept pairs
-// appended to (out_keys, out_counts) in no particular order, *out_n of them;
-// partitions that overfill the tier's table listed in ov_list, ov_stats =
-// {listed, their records}; dig_hist[256] += kept pairs per top digit.
+// to places out_base[0] .. out_base[1] of (out_keys, out_counts) in no
+// particular order, out_n[0] of them; partitions that overfill the tier's
+// batch listed in ov_list, ov_stats = {listed, their records}; dig_hist[256]
+// += kept pairs per top digit.  bucket_set (packed passes): the set of every
+// bucket of 2^sub_bits partitions, with out_base, out_n, dig_hist and the
+// statistics per set.
 void launch_hash_count(const uint64_t* records, const uint64_t* part_off, const uint32_t* only, uint32_t n_part,
                        int tier, int k, int nmax, uint32_t lo, uint32_t hi, void* out_keys, uint32_t* out_counts,
-                       uint64_t out_cap, uint64_t* out_n, uint32_t* ov_list, uint64_t* ov_stats, uint64_t* hist,
-                       uint32_t hist_len, uint32_t* max_count, uint64_t* n_distinct, uint64_t* dig_hist,
-                       uint32_t* claim, int* err, int num_sms, cudaStream_t st);
+                       const uint32_t* bucket_set, int sub_bits, const uint64_t* out_base, uint64_t* out_n,
+                       uint32_t* ov_list, uint64_t* ov_stats, uint64_t* hist, uint32_t hist_len, uint32_t* max_count,
+                       uint64_t* n_distinct, uint64_t* dig_hist, uint32_t* claim, int* err, int num_sms,
+                       cudaStream_t st);
+// sets' pairs from src_off[s] on -> dst_off[s] .. dst_off[s + 1] (n in all)
+void launch_close_sets(const void* src_keys, const uint32_t* src_counts, const uint64_t* src_off,
+                       const uint64_t* dst_off, uint32_t n_sets, uint64_t n, int key_words, void* dst_keys,
+                       uint32_t* dst_counts, int num_sms, cudaStream_t st);
 void launch_list_gather(const uint64_t* records, const uint64_t* part_off, const uint32_t* list, uint32_t n_list,
                         const uint64_t* dst_off, uint64_t* dst, uint64_t* kmers, int rec_words, int num_sms,
                         cudaStream_t st);

@@ -91,6 +91,9 @@ static void empty_result(hsk_ctx* c, HostResult& HR, int kw) {
     HR.R.hist = HR.hist.data();
 }
 
+// Packs of fewer bases than this are counted by sorting.
+constexpr uint64_t PACK_HASH_MIN_BASES = 1ull << 22;
+
 // Device arrays the pass keeps for the sets (one allocation): see the offsets
 // computed in pack_pass.
 struct PackTables {
@@ -197,7 +200,24 @@ static int pack_pass(hsk_ctx* c, std::vector<PackSet*>& sets, const std::vector<
     map.bmask = T.bmask;
     map.n = S;
     Supermers SMR;
-    TRY(hsk_supermers(c, E, k, m, B_total, SMR, st, nullptr, &map));
+    // large packs are counted by hashing, every bucket cut into fine partitions
+    // of half a batch's k-mers at most; small ones, and packs whose buckets are
+    // too large for that (or whose largest set's minimizers are), by sorting
+    int sub_bits = -1;
+    if (NB >= PACK_HASH_MIN_BASES && NB < HASH_MAX_BASES) {
+        sub_bits = 0;
+        uint64_t largest = 0;
+        for (uint32_t j = 0; j < S; ++j) {
+            while (sub_bits <= HASH_MAX_SUB_BITS &&
+                   nb[j] > ((uint64_t)(bmask[j] + 1) << sub_bits) * (hash_count_cap(kw) / 2))
+                ++sub_bits;
+            largest = std::max(largest, nb[j]);
+        }
+        if (sub_bits > HASH_MAX_SUB_BITS ||
+            !hsk_hash_path_fits(c, std::max<uint64_t>(largest, HASH_MIN_KMERS), HSK_MAX_BUCKETS, k, m))
+            sub_bits = -1;
+    }
+    TRY(hsk_supermers(c, E, k, m, B_total, SMR, st, nullptr, &map, sub_bits));
 
     // ---- bucket groups, set by set (a group never spans two sets)
     std::vector<uint64_t> set_kmers(S, 0), set_recs(S, 0);
@@ -231,6 +251,7 @@ static int pack_pass(hsk_ctx* c, std::vector<PackSet*>& sets, const std::vector<
     CK(cudaMemsetAsync(c->hist.p, 0, (size_t)S * H * 8, st));
     CK(cudaMemsetAsync(c->pack_stat.p, 0, (size_t)S * 12, st));
 
+    bool ordered = false;
     if (C > 0) {
         // the pack must fit the budget as one sort chunk
         std::vector<std::pair<uint32_t, uint32_t>> chunks;
@@ -239,6 +260,50 @@ static int pack_pass(hsk_ctx* c, std::vector<PackSet*>& sets, const std::vector<
             hsk_set_error(c, "a pack of %llu k-mers does not fit one sort chunk", (unsigned long long)nk);
             return HSK_ENOMEM;
         }
+    }
+    if (C > 0 && sub_bits >= 0) {
+        // S4/S5 by hashing: set j's kept pairs (each of at least lo k-mers) from place base_j on
+        std::vector<uint64_t> at(S + 1, 0);
+        std::vector<uint32_t> bset(B_total, 0);
+        for (uint32_t j = 0; j < S; ++j) {
+            at[j + 1] = at[j] + set_kmers[j] / std::max<uint32_t>(lo, 1) + 1;
+            for (uint32_t b = bkt[j]; b < bkt[j + 1]; ++b) bset[b] = j;
+        }
+        TRY(hsk_ensure(c, c->keys, at[S] * kb, false));
+        TRY(hsk_ensure(c, c->alt, at[S] * 4, false));
+        TRY(hsk_ensure(c, c->batch_d, (size_t)B_total * 4, false));
+        CK(cudaMemcpyAsync(c->batch_d.p, bset.data(), (size_t)B_total * 4, cudaMemcpyHostToDevice, st));
+        HashRun R;
+        TRY(hsk_hash_tiers(c, SMR.records, (const uint64_t*)c->part_off.p, B_total << sub_bits, SMR, k, lo, hi, H, S,
+                           at.data(), (const uint32_t*)c->batch_d.p, d_max, R, st));
+        if (R.n_left) {  // sets with a partition that no tier holds: counted again alone
+            std::vector<uint32_t> left(R.n_left);
+            CK(cudaMemcpyAsync(left.data(), R.list, (size_t)R.n_left * 4, cudaMemcpyDeviceToHost, st));
+            CK(cudaStreamSynchronize(st));
+            for (uint32_t p : left) redo[bset[p >> sub_bits]] = 1;
+        }
+        for (uint32_t j = 0; j < S; ++j) {
+            pair_off[j + 1] = pair_off[j] + R.out_n()[j];
+            distinct[j] = R.distinct()[j];
+        }
+        const uint64_t kept = pair_off[S];
+        Output O;
+        TRY(hsk_grow_output(c, O, std::max<uint64_t>(kept, 1), kw, st));
+        if (kept) {
+            // the sets' pairs one after the other, then S6
+            TRY(hsk_ensure(c, c->pair_alt_keys, kept * kb, false));
+            TRY(hsk_ensure(c, c->pair_alt_counts, kept * 4, false));
+            TRY(hsk_ensure(c, c->batch_c, (2 * (size_t)S + 2) * 8, false));
+            uint64_t* d_src = (uint64_t*)c->batch_c.p;
+            CK(cudaMemcpyAsync(d_src, at.data(), (S + 1) * 8, cudaMemcpyHostToDevice, st));
+            CK(cudaMemcpyAsync(d_src + S + 1, pair_off.data(), (S + 1) * 8, cudaMemcpyHostToDevice, st));
+            launch_close_sets(c->keys.p, (const uint32_t*)c->alt.p, d_src, d_src + S + 1, S, kept, kw,
+                              c->pair_alt_keys.p, (uint32_t*)c->pair_alt_counts.p, c->num_sms, st);
+            TRY(hsk_top_digit_pass(c, c->pair_alt_keys.p, (const uint32_t*)c->pair_alt_counts.p, S, pair_off.data(),
+                                   R.digits(), kw, 2 * k, st));
+            TRY(hsk_order_partitioned(c, kept, S, kw, 2 * k, st, &ordered));
+        }
+    } else if (C > 0) {
         const uint64_t NS = (uint64_t)C * 256;
         const int key_bits = 2 * k;
         const int shift0 = key_bits > 8 ? key_bits - 8 : 0;
@@ -343,7 +408,7 @@ static int pack_pass(hsk_ctx* c, std::vector<PackSet*>& sets, const std::vector<
     const uint64_t kept = pair_off[S];
     void* fin_keys = c->out_keys.p;
     uint32_t* fin_counts = (uint32_t*)c->out_counts.p;
-    if (kept > 1) {
+    if (kept > 1 && !ordered) {
         const int key_bits = 2 * k;
         const int P = (key_bits + 7) / 8;
         const int cshift = 8 * P;
@@ -398,7 +463,7 @@ static int pack_pass(hsk_ctx* c, std::vector<PackSet*>& sets, const std::vector<
     CK(cudaEventRecord(c->ev1, st));
     // device statistics of the sets
     if (C > 0) {
-        CK(cudaMemcpyAsync(distinct.data(), d_distinct, (size_t)S * 8, cudaMemcpyDeviceToHost, st));
+        if (sub_bits < 0) CK(cudaMemcpyAsync(distinct.data(), d_distinct, (size_t)S * 8, cudaMemcpyDeviceToHost, st));
         CK(cudaMemcpyAsync(maxc.data(), d_max, (size_t)S * 4, cudaMemcpyDeviceToHost, st));
     }
     TRY(hsk_read_device_error(c, st));

@@ -38,9 +38,6 @@
 
 using namespace hsk;
 
-// Jobs of fewer k-mers than this take the sorting path.
-static constexpr uint64_t HASH_MIN_KMERS = 1ull << 16;
-
 // ---------------------------------------------------------------------------
 // context
 // ---------------------------------------------------------------------------
@@ -710,76 +707,126 @@ int hsk_order_pairs(hsk_ctx* c, void* keys, uint32_t* counts, uint64_t n, int ke
     return hsk_plain_sort(c, keys, counts, n, key_words, key_bits, c->pair_alt_keys, &c->pair_alt_counts, st);
 }
 
-// Stage S6 for kept pairs laid out by their top digit (c->s6_bounds holds
-// the 257 digit starts): when every top-digit range fits the on-chip sort
-// (k_range_sort), they are sorted at once; else one segmented pass on the
-// second digit groups every range into 256 sub-ranges first.  *done = false
-// leaves the pairs for the general path (keys of fewer than 24 bits, or a
-// sub-range over the on-chip capacity; the pairs are then back in place,
-// unsorted).
-static int order_pairs_msd(hsk_ctx* c, uint64_t n, int kw, int key_bits, cudaStream_t st, bool* done) {
+// Stage S6's first partition: pairs of S sets (set s's at [seg[s], seg[s + 1])
+// of (keys, counts), in any order) into the output buffers, every set's pairs
+// partitioned by their top digit (hist: S x 256 pairs per set and digit).
+int hsk_top_digit_pass(hsk_ctx* c, const void* keys, const uint32_t* counts, uint32_t S, const uint64_t* seg,
+                       const uint64_t* hist, int kw, int key_bits, cudaStream_t st) {
+    const uint64_t TILE = onesweep_tile_keys(kw);
+    std::vector<uint64_t>& hb = c->s6_h;
+    hb.resize((size_t)S * 256 + 1);
+    std::vector<uint64_t> up(S + 1 + (S + 2) / 2);  // segments, then their first tiles
+    uint32_t* ts = reinterpret_cast<uint32_t*>(up.data() + S + 1);
+    uint64_t tiles = 0;
+    for (uint32_t i = 0; i < S; ++i) {
+        up[i] = seg[i];
+        ts[i] = (uint32_t)tiles;
+        tiles += (seg[i + 1] - seg[i] + TILE - 1) / TILE;
+        uint64_t at = seg[i];
+        for (int d = 0; d < 256; ++d) {
+            hb[(size_t)i * 256 + d] = at;
+            at += hist[(size_t)i * 256 + d];
+        }
+    }
+    up[S] = seg[S];
+    ts[S] = (uint32_t)tiles;
+    hb[(size_t)S * 256] = seg[S];
+    if (tiles >= 0xFFFFFFFFull) {
+        hsk_set_error(c, "%llu sort tiles", (unsigned long long)tiles);
+        return HSK_EOVERFLOW;
+    }
+    TRY(hsk_ensure(c, c->s6_bounds, hb.size() * 8, false));
+    TRY(hsk_ensure(c, c->seg, up.size() * 8, false));
+    CK(cudaMemcpyAsync(c->s6_bounds.p, hb.data(), hb.size() * 8, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(c->seg.p, up.data(), up.size() * 8, cudaMemcpyHostToDevice, st));
+    TRY(hsk_ensure_status(c, tiles * 256 + 1, st));
+    uint32_t ep, *ctr;
+    TRY(hsk_next_epoch(c, st, &ep));
+    TRY(hsk_next_counter(c, st, &ctr));
+    const uint64_t* d_seg = (const uint64_t*)c->seg.p;
+    launch_onesweep_seg(keys, c->out_keys.p, counts, (uint32_t*)c->out_counts.p, d_seg, S, (uint32_t)tiles,
+                        (const uint32_t*)(d_seg + S + 1), kw, key_bits - 8, (const uint64_t*)c->s6_bounds.p,
+                        (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st);
+    CK(cudaGetLastError());
+    return HSK_OK;
+}
+
+// Stage S6 for n kept pairs of S sets laid out by set and top digit
+// (c->s6_bounds holds the S x 256 range starts and n, c->s6_h the same or
+// nothing): when every range fits the on-chip sort (k_range_sort), they are
+// sorted at once; else one segmented pass on the second digit groups every
+// range into 256 sub-ranges first.  *done = false leaves the pairs for the
+// general path (keys of fewer than 24 bits, a sub-range over the on-chip
+// capacity, or more sets than the second digit's tables are kept for; the
+// pairs are then back in place, unsorted).
+int hsk_order_partitioned(hsk_ctx* c, uint64_t n, uint32_t S, int kw, int key_bits, cudaStream_t st, bool* done) {
     *done = false;
     if (key_bits < 24 || n < 2) return HSK_OK;
     const size_t kb = (size_t)kw * 8;
+    const uint32_t R = S * 256;
     const uint64_t* d_bounds = (const uint64_t*)c->s6_bounds.p;
     std::vector<uint64_t>& hb = c->s6_h;
-    if (hb.size() != 257) {
-        hb.resize(257);
-        CK(cudaMemcpyAsync(hb.data(), d_bounds, 257 * 8, cudaMemcpyDeviceToHost, st));
+    if (hb.size() != (size_t)R + 1) {
+        hb.resize((size_t)R + 1);
+        CK(cudaMemcpyAsync(hb.data(), d_bounds, hb.size() * 8, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
     }
-    if (hb[256] != n) {
-        hsk_set_error(c, "S6: %llu pairs laid out by digit, %llu expected", (unsigned long long)hb[256],
+    if (hb[R] != n) {
+        hsk_set_error(c, "S6: %llu pairs laid out by digit, %llu expected", (unsigned long long)hb[R],
                       (unsigned long long)n);
         return HSK_ECUDA;
     }
-    uint64_t largest = 0;
-    for (int d = 0; d < 256; ++d) largest = std::max(largest, hb[d + 1] - hb[d]);
+    uint64_t largest = 0, largest_set = 0;
+    for (uint32_t d = 0; d < R; ++d) largest = std::max(largest, hb[d + 1] - hb[d]);
+    for (uint32_t i = 0; i < S; ++i) largest_set = std::max(largest_set, hb[(size_t)i * 256 + 256] - hb[(size_t)i * 256]);
+    const bool one_pass = largest <= range_sort_cap(kw);
+    if (!one_pass && S > 256) return HSK_OK;  // 0.5 MB of tables per set
     TRY(hsk_ensure(c, c->pair_alt_keys, n * kb, false));
     TRY(hsk_ensure(c, c->pair_alt_counts, n * 4, false));
-    TRY(hsk_ensure(c, c->pass_hist, 2 * (65536 + 16) * 4, false));  // digit counts; later two lists of ranges
     uint32_t ep, *ctr;
-    if (largest <= range_sort_cap(kw)) {
+    if (one_pass) {
         TRY(hsk_next_counter(c, st, &ctr));
         launch_range_sort(c->out_keys.p, (const uint32_t*)c->out_counts.p, c->pair_alt_keys.p,
-                          (uint32_t*)c->pair_alt_counts.p, d_bounds, nullptr, 256, 1, 0, kw, key_bits, 8,
-                          (uint32_t*)c->pass_hist.p, ctr, c->num_sms, st);
+                          (uint32_t*)c->pair_alt_counts.p, d_bounds, nullptr, R, 1, 0, kw, key_bits, 8, nullptr, ctr,
+                          c->num_sms, st);
         CK(cudaGetLastError());
         std::swap(c->out_keys, c->pair_alt_keys);
         std::swap(c->out_counts, c->pair_alt_counts);
         *done = true;
         return HSK_OK;
     }
+    const uint64_t R2 = (uint64_t)R * 256;
+    TRY(hsk_ensure(c, c->pass_hist, R2 * 8 + 256, false));  // digit counts; later two lists of ranges
     const uint64_t TILE = onesweep_tile_keys(kw);
-    std::vector<uint32_t> ts(257);
+    std::vector<uint32_t> ts((size_t)R + 1);
     uint64_t tiles = 0;
-    for (int d = 0; d < 256; ++d) {
+    for (uint32_t d = 0; d < R; ++d) {
         ts[d] = (uint32_t)tiles;
         tiles += (hb[d + 1] - hb[d] + TILE - 1) / TILE;
     }
-    ts[256] = (uint32_t)tiles;
-    TRY(hsk_ensure(c, c->seg, 257 * 4, false));
-    CK(cudaMemcpyAsync(c->seg.p, ts.data(), 257 * 4, cudaMemcpyHostToDevice, st));
-    TRY(hsk_ensure(c, c->digit_off, (256 * 256 + 1) * 8, false));
+    ts[R] = (uint32_t)tiles;
+    TRY(hsk_ensure(c, c->seg, ts.size() * 4, false));
+    CK(cudaMemcpyAsync(c->seg.p, ts.data(), ts.size() * 4, cudaMemcpyHostToDevice, st));
+    TRY(hsk_ensure(c, c->digit_off, (R2 + 1) * 8, false));
     TRY(hsk_ensure_status(c, tiles * 256 + 1, st));
     uint64_t* doff = (uint64_t*)c->digit_off.p;
-    CK(cudaMemsetAsync(c->pass_hist.p, 0, 256 * 256 * 8, st));
-    launch_digit_hist_seg(c->out_keys.p, kw, d_bounds, 256, n, (uint64_t*)c->pass_hist.p, 1, st, key_bits - 16);
-    launch_digit_offsets_seg((const uint64_t*)c->pass_hist.p, d_bounds, doff, 1, 256, st);
-    CK(cudaMemcpyAsync(doff + 256 * 256, &hb[256], 8, cudaMemcpyHostToDevice, st));
+    CK(cudaMemsetAsync(c->pass_hist.p, 0, R2 * 8, st));
+    launch_digit_hist_seg(c->out_keys.p, kw, d_bounds, R, n, (uint64_t*)c->pass_hist.p, 1, st, key_bits - 16);
+    launch_digit_offsets_seg((const uint64_t*)c->pass_hist.p, d_bounds, doff, 1, R, st);
+    CK(cudaMemcpyAsync(doff + R2, &hb[R], 8, cudaMemcpyHostToDevice, st));
     TRY(hsk_next_epoch(c, st, &ep));
     TRY(hsk_next_counter(c, st, &ctr));
     launch_onesweep_seg(c->out_keys.p, c->pair_alt_keys.p, (const uint32_t*)c->out_counts.p,
-                        (uint32_t*)c->pair_alt_counts.p, d_bounds, 256, (uint32_t)tiles, (const uint32_t*)c->seg.p, kw,
+                        (uint32_t*)c->pair_alt_counts.p, d_bounds, R, (uint32_t)tiles, (const uint32_t*)c->seg.p, kw,
                         key_bits - 16, doff, (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st);
     // sub-ranges are sorted a group at a time: about a third of the capacity
     uint32_t group = 1;
-    while (group < 64 && n / 65536 * group * 2 <= range_sort_cap(kw) / 3) group *= 2;
+    while (group < 64 && largest_set / 65536 * group * 2 <= range_sort_cap(kw) / 3) group *= 2;
     uint32_t* big = (uint32_t*)c->pass_hist.p;  // free again
     CK(cudaMemsetAsync(big, 0, 4, st));
     TRY(hsk_next_counter(c, st, &ctr));
     launch_range_sort(c->pair_alt_keys.p, (const uint32_t*)c->pair_alt_counts.p, c->out_keys.p,
-                      (uint32_t*)c->out_counts.p, doff, nullptr, 256 * 256, group, 0, kw, key_bits, 16, big, ctr,
+                      (uint32_t*)c->out_counts.p, doff, nullptr, (uint32_t)R2, group, 0, kw, key_bits, 16, big, ctr,
                       c->num_sms, st);
     CK(cudaGetLastError());
     for (int tier = 1;; ++tier) {
@@ -793,7 +840,7 @@ static int order_pairs_msd(hsk_ctx* c, uint64_t n, int kw, int key_bits, cudaStr
             return HSK_OK;
         }
         uint32_t* list = big + 1;
-        big += 65536 + 8;  // the next list
+        big += R2 + 8;  // the next list
         CK(cudaMemsetAsync(big, 0, 4, st));
         TRY(hsk_next_counter(c, st, &ctr));
         launch_range_sort(c->pair_alt_keys.p, (const uint32_t*)c->pair_alt_counts.p, c->out_keys.p,
@@ -1045,41 +1092,52 @@ static int local_chunk(hsk_ctx* c, const Supermers& S, const std::vector<uint32_
     return HSK_OK;
 }
 
-// Pairs of (keys, counts), n of them in any order, into the output buffers
-// partitioned by their top digit (hist: pairs per top digit): stage S6's
-// first partition.
-static int top_digit_pass(hsk_ctx* c, const void* keys, const uint32_t* counts, uint64_t n, int kw, int key_bits,
-                          const uint64_t* hist, cudaStream_t st) {
-    const uint64_t TILE = onesweep_tile_keys(kw);
-    const uint64_t tiles = (n + TILE - 1) / TILE;
-    TRY(hsk_ensure(c, c->s6_bounds, 2 * 257 * 8, false));
-    uint64_t* d_bounds = (uint64_t*)c->s6_bounds.p;
-    std::vector<uint64_t>& hb = c->s6_h;
-    hb.assign(259, 0);
-    for (int d = 0; d < 256; ++d) hb[d + 1] = hb[d] + hist[d];
-    hb[258] = n;  // hb[257], hb[258]: the one segment of the pass
-    CK(cudaMemcpyAsync(d_bounds, hb.data(), 259 * 8, cudaMemcpyHostToDevice, st));
-    hb.resize(257);
-    TRY(hsk_ensure_status(c, tiles * 256 + 1, st));
-    uint32_t ep, *ctr;
-    TRY(hsk_next_epoch(c, st, &ep));
-    TRY(hsk_next_counter(c, st, &ctr));
-    launch_onesweep_seg(keys, c->out_keys.p, counts, (uint32_t*)c->out_counts.p, d_bounds + 257, 1, (uint32_t)tiles,
-                        nullptr, kw, key_bits - 8, d_bounds, (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st);
-    CK(cudaGetLastError());
-    return HSK_OK;
-}
-
 // The hash path needs partitions whose distinct k-mers fit its table.  The
 // fine partitions hold n_windows / (256 B) k-mers at best, and no fewer than
 // one minimizer's: of the 4^m / 2 canonical m-mers about 2 in w + 1 are ever a
 // window's minimum, so a minimizer has about n_windows (w + 1) / 4^m k-mers.
-static bool hash_path_fits(hsk_ctx* c, uint64_t n_windows, uint32_t B, int k, int m) {
+bool hsk_hash_path_fits(hsk_ctx* c, uint64_t n_windows, uint32_t B, int k, int m) {
     if (!c->cfg.local_sort || k < 12) return false;
     const double cap = hash_count_cap(k <= 32 ? 1 : 2);
     const double per_part = (double)n_windows / ((double)B * (1 << HASH_MAX_SUB_BITS));
     const double per_min = (double)n_windows * (k - m + 2) / std::pow(4.0, m);
     return n_windows >= HASH_MIN_KMERS && per_part <= cap && per_min <= cap;
+}
+
+// The hash count of n_part partitions of S sets (bucket_set: the set of every
+// bucket; nullptr with one set): kept pairs of set s to places out_base[s] ..
+// out_base[s + 1] of (c->keys, c->alt); histograms to c->hist, largest counts
+// to d_max[s].  R receives the rest.
+int hsk_hash_tiers(hsk_ctx* c, const uint64_t* recs, const uint64_t* part_off, uint32_t n_part, const Supermers& SM,
+                   int k, uint32_t lo, uint32_t hi, uint32_t H, uint32_t S, const uint64_t* out_base,
+                   const uint32_t* bucket_set, uint32_t* d_max, HashRun& R, cudaStream_t st) {
+    // {listed, their records} of the two tiers | kept pairs, distinct k-mers
+    // and kept pairs per top digit of every set || out_base || two lists
+    const size_t words = 4 + 258 * (size_t)S;
+    TRY(hsk_ensure(c, c->hash_ctl, (words + S + 1) * 8 + (size_t)n_part * 8, false));
+    uint64_t* ctl = (uint64_t*)c->hash_ctl.p;
+    uint64_t* d_base = ctl + words;
+    uint32_t* list1 = (uint32_t*)(d_base + S + 1);
+    R.list = list1 + n_part;
+    R.S = S;
+    R.h.resize(words);
+    CK(cudaMemsetAsync(ctl, 0, words * 8, st));
+    CK(cudaMemcpyAsync(d_base, out_base, ((size_t)S + 1) * 8, cudaMemcpyHostToDevice, st));
+    for (int tier = 0; tier < 2; ++tier) {
+        const uint32_t n = tier ? (uint32_t)R.h[0] : n_part;
+        if (n == 0) break;
+        uint32_t* ctr;
+        TRY(hsk_next_counter(c, st, &ctr));
+        launch_hash_count(recs, part_off, tier ? list1 : nullptr, n, tier, k, SM.nmax, lo, hi, c->keys.p,
+                          (uint32_t*)c->alt.p, bucket_set, SM.sub_bits, d_base, ctl + 4, tier ? R.list : list1,
+                          ctl + 2 * tier, (uint64_t*)c->hist.p, H, d_max, ctl + 4 + S, ctl + 4 + 2 * (size_t)S, ctr,
+                          c->d_err, c->num_sms, st);
+        CK(cudaGetLastError());
+        CK(cudaMemcpyAsync(R.h.data(), ctl, words * 8, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+    }
+    R.n_left = (uint32_t)R.h[2];
+    return HSK_OK;
 }
 
 // One chunk of buckets [b0, b1) through the hash path.  Kept pairs end in the
@@ -1092,43 +1150,21 @@ static int hash_chunk(hsk_ctx* c, const Supermers& S, uint32_t b0, uint32_t b1, 
     const uint64_t cap = nk / std::max<uint32_t>(lo, 1) + 1;  // a kept k-mer has at least lo copies
     TRY(hsk_ensure(c, c->keys, cap * kb, false));
     TRY(hsk_ensure(c, c->alt, cap * 4, false));
-    // control words: out_n, distinct, {listed, records} x 2, kept pairs per top digit; then the two lists
-    const size_t ctl_words = 8 + 256;
-    TRY(hsk_ensure(c, c->hash_ctl, ctl_words * 8 + (size_t)n_part * 8, false));
-    uint64_t* ctl = (uint64_t*)c->hash_ctl.p;
-    uint32_t* list1 = (uint32_t*)(ctl + ctl_words);
-    uint32_t* list2 = list1 + n_part;
-    CK(cudaMemsetAsync(ctl, 0, ctl_words * 8, st));
     const uint64_t* recs = S.records;
     const uint64_t* part_off = (const uint64_t*)c->part_off.p + ((uint64_t)b0 << S.sub_bits);
     prof_mark(c, st, 3);
-    uint32_t* ctr;
-    TRY(hsk_next_counter(c, st, &ctr));
-    launch_hash_count(recs, part_off, nullptr, n_part, 0, k, S.nmax, lo, hi, c->keys.p, (uint32_t*)c->alt.p, cap, ctl,
-                      list1, ctl + 2, (uint64_t*)c->hist.p, H, c->d_max, ctl + 1, ctl + 8, ctr, c->d_err, c->num_sms,
-                      st);
-    CK(cudaGetLastError());
-    uint64_t w[8 + 256];
-    CK(cudaMemcpyAsync(w, ctl, sizeof(w), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    const uint32_t n1 = (uint32_t)w[2];
-    if (n1) {
-        TRY(hsk_next_counter(c, st, &ctr));
-        launch_hash_count(recs, part_off, list1, n1, 1, k, S.nmax, lo, hi, c->keys.p, (uint32_t*)c->alt.p, cap, ctl,
-                          list2, ctl + 4, (uint64_t*)c->hist.p, H, c->d_max, ctl + 1, ctl + 8, ctr, c->d_err,
-                          c->num_sms, st);
-        CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(w, ctl, sizeof(w), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-    }
-    const uint32_t n2 = (uint32_t)w[4];
-    const uint64_t kept = w[0];
-    O.n_distinct += w[1];
+    HashRun R;
+    const uint64_t base[2] = {0, cap};
+    TRY(hsk_hash_tiers(c, recs, part_off, n_part, S, k, lo, hi, H, 1, base, nullptr, c->d_max, R, st));
+    const uint32_t n2 = R.n_left;
+    const uint64_t kept = R.out_n()[0];
+    O.n_distinct += R.distinct()[0];
     TRY(hsk_grow_output(c, O, O.n_pairs + kept, kw, st));
     prof_mark(c, st, 4);
     const bool only = single && O.n_pairs == 0 && n2 == 0;
     if (only && 2 * k >= 24 && kept > 1) {
-        TRY(top_digit_pass(c, c->keys.p, (const uint32_t*)c->alt.p, kept, kw, 2 * k, w + 8, st));
+        const uint64_t seg[2] = {0, kept};
+        TRY(hsk_top_digit_pass(c, c->keys.p, (const uint32_t*)c->alt.p, 1, seg, R.digits(), kw, 2 * k, st));
         c->s6_digit_major = true;
     } else if (kept) {
         CK(cudaMemcpyAsync((char*)c->out_keys.p + O.n_pairs * kb, c->keys.p, kept * kb, cudaMemcpyDeviceToDevice, st));
@@ -1139,7 +1175,7 @@ static int hash_chunk(hsk_ctx* c, const Supermers& S, uint32_t b0, uint32_t b1, 
     if (n2) {  // partitions no table holds: their records as groups of the sorting path
         std::vector<uint32_t> list(n2);
         std::vector<uint64_t> poff((size_t)n_part + 1);
-        CK(cudaMemcpyAsync(list.data(), list2, (size_t)n2 * 4, cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(list.data(), R.list, (size_t)n2 * 4, cudaMemcpyDeviceToHost, st));
         CK(cudaMemcpyAsync(poff.data(), part_off, ((size_t)n_part + 1) * 8, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
         Supermers L;
@@ -1158,7 +1194,7 @@ static int hash_chunk(hsk_ctx* c, const Supermers& S, uint32_t b0, uint32_t b1, 
         uint64_t* d_kmers = d_off + n2;
         CK(cudaMemcpyAsync(d_off, L.h_bucket_rec.data(), (size_t)n2 * 8, cudaMemcpyHostToDevice, st));
         CK(cudaMemsetAsync(d_kmers, 0, (size_t)n2 * 8, st));
-        launch_list_gather(recs, part_off, list2, n2, d_off, (uint64_t*)c->ov_records.p, d_kmers, S.rec_words,
+        launch_list_gather(recs, part_off, R.list, n2, d_off, (uint64_t*)c->ov_records.p, d_kmers, S.rec_words,
                            c->num_sms, st);
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(L.h_bucket_kmers.data(), d_kmers, (size_t)n2 * 8, cudaMemcpyDeviceToHost, st));
@@ -1204,7 +1240,7 @@ int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, ui
     Supermers S;
     uint32_t B = hsk_pick_buckets(c, n_bases, k);
     int sub_bits = -1;
-    if (n_bases < HASH_MAX_BASES && hash_path_fits(c, n_bases, B, k, m)) {
+    if (n_bases < HASH_MAX_BASES && hsk_hash_path_fits(c, n_bases, B, k, m)) {
         // fine partitions of half a batch's k-mers at most
         for (sub_bits = 0; sub_bits < HASH_MAX_SUB_BITS;) {
             if (n_bases <= ((uint64_t)B << sub_bits) * (hash_count_cap(kw) / 2)) break;
@@ -1216,7 +1252,7 @@ int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, ui
         TRY(hsk_supermers(c, E, k, m, B, S, st, pipe, nullptr, sub_bits));
     }
     prof_mark(c, st, 2);
-    const bool hash = sub_bits >= 0 && hash_path_fits(c, S.n_kmers, B, k, m);
+    const bool hash = sub_bits >= 0 && hsk_hash_path_fits(c, S.n_kmers, B, k, m);
     R.n_windows = S.n_kmers;
     R.n_supermers = S.n_records;
     std::vector<std::pair<uint32_t, uint32_t>> chunks;
@@ -1297,7 +1333,7 @@ int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, ui
         NvtxRange r("S6 order");
         bool done = false;
         if (chunks.size() == 1 && c->cfg.local_sort && c->s6_digit_major)
-            TRY(order_pairs_msd(c, O.n_pairs, kw, 2 * k, st, &done));
+            TRY(hsk_order_partitioned(c, O.n_pairs, 1, kw, 2 * k, st, &done));
         if (!done) TRY(hsk_order_pairs(c, c->out_keys.p, (uint32_t*)c->out_counts.p, O.n_pairs, kw, 2 * k, st, hi));
     }
     prof_mark(c, st, 6);

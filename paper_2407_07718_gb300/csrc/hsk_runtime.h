@@ -49,6 +49,21 @@ struct Supermers {
     int sub_bits = -1;                     // records in order of 2^sub_bits fine partitions per bucket; -1: none
 };
 
+// What a hash count leaves on the host (and its list of uncounted partitions
+// on the device).
+struct HashRun {
+    uint32_t S = 1;              // sets
+    std::vector<uint64_t> h;     // control words
+    uint32_t n_left = 0;         // partitions that no tier holds
+    uint32_t* list = nullptr;
+    const uint64_t* out_n() const { return h.data() + 4; }             // kept pairs per set
+    const uint64_t* distinct() const { return h.data() + 4 + S; }
+    const uint64_t* digits() const { return h.data() + 4 + 2 * (size_t)S; }  // S x 256 kept pairs per top digit
+};
+
+// Jobs of fewer k-mers than this take the sorting path.
+constexpr uint64_t HASH_MIN_KMERS = 1ull << 16;
+
 struct Output {
     uint64_t n_pairs = 0;
     uint64_t n_distinct = 0;
@@ -408,6 +423,13 @@ int hsk_plan_chunks(hsk_ctx* c, const Supermers& S, int key_words, std::vector<s
 int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Supermers& S, cudaStream_t st,
                   InputPipe* pipe, const SetMap* sets = nullptr, int sub_bits = -1);
 uint32_t hsk_pick_buckets(hsk_ctx* c, uint64_t n_bases, int k);
+bool hsk_hash_path_fits(hsk_ctx* c, uint64_t n_windows, uint32_t B, int k, int m);
+int hsk_hash_tiers(hsk_ctx* c, const uint64_t* recs, const uint64_t* part_off, uint32_t n_part, const Supermers& SM,
+                   int k, uint32_t lo, uint32_t hi, uint32_t H, uint32_t S, const uint64_t* out_base,
+                   const uint32_t* bucket_set, uint32_t* d_max, HashRun& R, cudaStream_t st);
+int hsk_top_digit_pass(hsk_ctx* c, const void* keys, const uint32_t* counts, uint32_t S, const uint64_t* seg,
+                       const uint64_t* hist, int kw, int key_bits, cudaStream_t st);
+int hsk_order_partitioned(hsk_ctx* c, uint64_t n, uint32_t S, int kw, int key_bits, cudaStream_t st, bool* done);
 int hsk_plain_sort(hsk_ctx* c, void* keys, uint32_t* vals, uint64_t n, int key_words, int key_bits, DevBuf& alt_keys,
                    DevBuf* alt_vals, cudaStream_t st);
 int hsk_local_overflow(hsk_ctx* c, const uint64_t* sub_off, uint32_t n_ov1, uint32_t* ov_list, uint32_t* ov_list_m,

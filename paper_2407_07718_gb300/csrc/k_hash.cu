@@ -153,7 +153,14 @@ struct HashArgs {
     uint32_t lo, hi;
     void* out_keys;
     uint32_t* out_counts;
-    u64 out_cap;
+    // Sets (packed passes): bucket b belongs to set bucket_set[b] (nullptr: one
+    // set); partition p to bucket p >> sub_bits.  Set s's kept pairs go to
+    // places out_base[s] .. out_base[s + 1], out_n[s] of them, and its
+    // statistics to hist + s * hist_len, max_count[s], n_distinct[s] and
+    // dig_hist + s * 256.
+    const uint32_t* bucket_set;
+    int sub_bits;
+    const u64* out_base;
     unsigned long long* out_n;  // kept pairs
     uint32_t* ov_list;
     unsigned long long* ov_stats;  // {partitions listed, their records}
@@ -200,6 +207,9 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
     if (tid < 2) s_nl[tid] = 0;
     u64 my_distinct = 0;
     uint32_t my_max = 0, my_ones = 0;
+    uint32_t set = 0;  // the set whose statistics are held here
+    u64 out0 = P.out_base[0], out1 = P.out_base[1];
+    u64* hist = P.hist;
 
     // Records [r0, r0 + nr) into shared memory, equal ones merged (most of
     // them: a record that meets another one in its slot stays distinct).
@@ -393,7 +403,7 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
             } else {
                 const uint32_t b = cnt < P.hist_len - 1 ? cnt : P.hist_len - 1;
                 if (b < hs) atomicAdd(&s_hist[b], 1u);
-                else atomicAdd(reinterpret_cast<unsigned long long*>(P.hist + b), 1ULL);
+                else atomicAdd(reinterpret_cast<unsigned long long*>(hist + b), 1ULL);
             }
             my_max = cnt > my_max ? cnt : my_max;
             kept += (cnt >= P.lo && cnt <= P.hi) ? 1u : 0u;
@@ -407,8 +417,8 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
             if (lane < NW) s_wk[lane] = inc - v;
             const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
             if (lane == 0) {
-                u64 at = total ? atomicAdd(P.out_n, (unsigned long long)total) : 0ULL;
-                if (at + total > P.out_cap) {
+                u64 at = out0 + (total ? atomicAdd(P.out_n + set, (unsigned long long)total) : 0ULL);
+                if (at + total > out1) {
                     raise_error(P.err, HSK_DERR_BOUNDS);
                     at = ~0ULL;
                 }
@@ -441,6 +451,26 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
         }
     };
 
+    // The held statistics to their set; leaves them cleared.
+    auto flush_stats = [&]() {
+        if (my_ones) atomicAdd(&s_hist[1], my_ones);  // hist_len >= 2: count 1 has its own bin
+        __syncthreads();
+        for (uint32_t i = tid; i < hs; i += NT) {
+            if (s_hist[i]) atomicAdd(reinterpret_cast<unsigned long long*>(hist + i), (unsigned long long)s_hist[i]);
+            s_hist[i] = 0;
+        }
+        for (int i = tid; i < 256; i += NT) {
+            if (s_dig[i]) atomicAdd(P.dig_hist + (u64)set * 256 + i, (unsigned long long)s_dig[i]);
+            s_dig[i] = 0;
+        }
+        const u64 d = warp_incl_sum<u64>(my_distinct);
+        const uint32_t mx = __reduce_max_sync(0xffffffffu, my_max);
+        if (lane == 31 && d) atomicAdd(P.n_distinct + set, (unsigned long long)d);
+        if (lane == 0 && mx) atomicMax(P.max_count + set, mx);
+        my_distinct = 0;
+        my_max = my_ones = 0;
+        __syncthreads();
+    };
     // Moves the entries in use to the front; returns their number.
     auto close_up = [&](uint32_t D) -> uint32_t {
         uint32_t at = 0;
@@ -518,6 +548,16 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
         u64 first = c0;
         if (P.only) first = P.only[c0];  // listed partitions are claimed one at a time
         if (tid <= (int)np) s_off[tid] = P.part_off[first + tid];
+        if (P.bucket_set) {  // a claim lies within one bucket
+            const uint32_t now = P.bucket_set[first >> P.sub_bits];
+            if (now != set) {
+                flush_stats();
+                set = now;
+                out0 = P.out_base[set];
+                out1 = P.out_base[set + 1];
+                hist = P.hist + (u64)set * P.hist_len;
+            }
+        }
         __syncthreads();
         for (uint32_t p = 0; p < np;) {
             // the batch: as many whole partitions as `target` records hold
@@ -556,23 +596,15 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
             p = q;
         }
     }
-    if (my_ones) atomicAdd(&s_hist[1], my_ones);
-    __syncthreads();
-    for (uint32_t i = tid; i < hs; i += NT)
-        if (s_hist[i]) atomicAdd(reinterpret_cast<unsigned long long*>(P.hist + i), (unsigned long long)s_hist[i]);
-    for (int i = tid; i < 256; i += NT)
-        if (s_dig[i]) atomicAdd(P.dig_hist + i, (unsigned long long)s_dig[i]);
-    const u64 d = warp_incl_sum<u64>(my_distinct);
-    const uint32_t mx = __reduce_max_sync(0xffffffffu, my_max);
-    if (lane == 31 && d) atomicAdd(P.n_distinct, (unsigned long long)d);
-    if (lane == 0 && mx) atomicMax(P.max_count, mx);
+    flush_stats();
 }
 
 void launch_hash_count(const uint64_t* records, const uint64_t* part_off, const uint32_t* only, uint32_t n_part,
                        int tier, int k, int nmax, uint32_t lo, uint32_t hi, void* out_keys, uint32_t* out_counts,
-                       uint64_t out_cap, uint64_t* out_n, uint32_t* ov_list, uint64_t* ov_stats, uint64_t* hist,
-                       uint32_t hist_len, uint32_t* max_count, uint64_t* n_distinct, uint64_t* dig_hist,
-                       uint32_t* claim, int* err, int num_sms, cudaStream_t st) {
+                       const uint32_t* bucket_set, int sub_bits, const uint64_t* out_base, uint64_t* out_n,
+                       uint32_t* ov_list, uint64_t* ov_stats, uint64_t* hist, uint32_t hist_len, uint32_t* max_count,
+                       uint64_t* n_distinct, uint64_t* dig_hist, uint32_t* claim, int* err, int num_sms,
+                       cudaStream_t st) {
     if (n_part == 0) return;
     count_launch();
     HashArgs P;
@@ -587,7 +619,9 @@ void launch_hash_count(const uint64_t* records, const uint64_t* part_off, const 
     P.hi = hi;
     P.out_keys = out_keys;
     P.out_counts = out_counts;
-    P.out_cap = out_cap;
+    P.bucket_set = bucket_set;
+    P.sub_bits = sub_bits;
+    P.out_base = (const u64*)out_base;
     P.out_n = (unsigned long long*)out_n;
     P.ov_list = ov_list;
     P.ov_stats = (unsigned long long*)ov_stats;
@@ -603,7 +637,14 @@ void launch_hash_count(const uint64_t* records, const uint64_t* part_off, const 
         const uint64_t slots = (uint64_t)num_sms * ctas;
         // enough claims that the CTAs end together, few enough that a claim spans several batches
         uint64_t ch = only ? 1 : n_part / (slots * 8);
-        P.chunk = (uint32_t)(ch < 1 ? 1 : ch > HC_CHUNK ? HC_CHUNK : ch);
+        if (ch < 1) ch = 1;
+        if (ch > HC_CHUNK) ch = HC_CHUNK;
+        if (bucket_set) {  // a power of two, at most a bucket's partitions
+            uint64_t c2 = 1;
+            while (c2 * 2 <= ch && c2 * 2 <= (1ull << sub_bits)) c2 *= 2;
+            ch = c2;
+        }
+        P.chunk = (uint32_t)ch;
         const uint64_t want = (n_part + P.chunk - 1) / P.chunk;
         kern<<<(unsigned)(want < slots ? want : slots), nt, dyn, st>>>(P);
     };
@@ -616,6 +657,45 @@ void launch_hash_count(const uint64_t* records, const uint64_t* part_off, const 
         else HC_GO(true, 0);
     }
 #undef HC_GO
+}
+
+// ---------------------------------------------------------------------------
+// the sets' kept pairs -> one after the other
+// ---------------------------------------------------------------------------
+// dst pairs [dst_off[s], dst_off[s + 1]) = src pairs from src_off[s] on.
+template <typename K>
+__global__ void __launch_bounds__(256) k_close_sets(const K* __restrict__ ks, const uint32_t* __restrict__ cs,
+                                                    const u64* __restrict__ src_off, const u64* __restrict__ dst_off,
+                                                    uint32_t n_sets, K* __restrict__ kd, uint32_t* __restrict__ cd) {
+    const u64 n = dst_off[n_sets];
+    for (u64 b = (u64)blockIdx.x * 2048; b < n; b += (u64)gridDim.x * 2048) {
+        for (u64 i = b + threadIdx.x; i < b + 2048 && i < n; i += 256) {
+            uint32_t lo = 0, hi = n_sets;  // dst_off[lo] <= i < dst_off[hi]
+            while (hi - lo > 1) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (dst_off[mid] <= i) lo = mid;
+                else hi = mid;
+            }
+            const u64 q = src_off[lo] + (i - dst_off[lo]);
+            kd[i] = ks[q];
+            cd[i] = cs[q];
+        }
+    }
+}
+
+void launch_close_sets(const void* src_keys, const uint32_t* src_counts, const uint64_t* src_off,
+                       const uint64_t* dst_off, uint32_t n_sets, uint64_t n, int key_words, void* dst_keys,
+                       uint32_t* dst_counts, int num_sms, cudaStream_t st) {
+    if (n == 0) return;
+    count_launch();
+    const uint64_t want = (n + 2047) / 2048;
+    const unsigned g = (unsigned)(want < (uint64_t)num_sms * 8 ? want : (uint64_t)num_sms * 8);
+    if (key_words == 1)
+        k_close_sets<u64><<<g, 256, 0, st>>>((const u64*)src_keys, src_counts, (const u64*)src_off,
+                                             (const u64*)dst_off, n_sets, (u64*)dst_keys, dst_counts);
+    else
+        k_close_sets<key128><<<g, 256, 0, st>>>((const key128*)src_keys, src_counts, (const u64*)src_off,
+                                                (const u64*)dst_off, n_sets, (key128*)dst_keys, dst_counts);
 }
 
 // ---------------------------------------------------------------------------

@@ -100,3 +100,28 @@ def test_chunks_and_small_histogram(hsk):
         got = ctx.count(rs.reads, rs.offsets, 31, 17, 1, 5)
     assert got.n_chunks > 3
     assert_same_result(got, want, "chunks")
+
+
+@pytest.mark.parametrize("k,m", [(31, 17), (21, 11), (55, 21), (64, 32)])
+def test_large_packs_are_counted_by_hashing(hsk, k, m):
+    """Packed passes of several million bases: sets of very different sizes
+    (among them empty ones and one of a single repeated read) and filters that
+    keep everything or little; each result is the oracle's for the set alone."""
+    rng = np.random.default_rng(k)
+    jobs = []
+    for i in range(20):
+        g = int(np.exp(rng.uniform(np.log(3_000), np.log(400_000))))
+        rs = datagen.batched_set(datagen.derive_seed(k, i), g, float(rng.uniform(5, 30)))
+        jobs.append((rs.reads, rs.offsets))
+    jobs.insert(3, (np.zeros(0, np.uint8), np.zeros(1, np.uint64)))
+    jobs.insert(7, _join(["ACGT" * 30] * 3000))
+    jobs.insert(9, _join(["N" * 5000, "A" * 20000]))
+    for lo, hi in ((1, 1 << 30), (2, 1000)):
+        wants = [oracle.count(r, o, k, lo, hi) for r, o in jobs]
+        with hsk.Context() as ctx:
+            ctx.tune_set(slots=1)
+            for _ in range(2):
+                got = ctx.count_batch([(r, o, k, m, lo, hi) for r, o in jobs])
+                for i, (a, b) in enumerate(zip(got, wants)):
+                    assert_same_result(a, b, f"k={k} lo={lo} set {i}")
+            assert ctx.pack_stats()["failed_passes"] == 0
