@@ -62,7 +62,12 @@ struct SmParams {
     int sub_bits;
     uint64_t* desc;                    // supermer descriptors (DESC)
     uint64_t desc_cap;
-    unsigned long long* desc_count;    // descriptors produced (may exceed desc_cap)
+    // two_ended (one set, fine partitions): the bucket is the score's low bits
+    // rotated right by one, and the descriptors of the second half of the
+    // buckets fill the array downward from its end, the others upward from its
+    // start
+    int two_ended;
+    unsigned long long* desc_count;    // descriptors produced, of each kind (may exceed desc_cap together)
     uint32_t* bucket_rec;              // [n_buckets] records per bucket (atomic adds)
     uint64_t* bucket_kmers;            // [n_buckets] k-mers per bucket (atomic adds)
     // Packed sets (n_sets > 0): set s owns warp tiles [set_tile0[s],

@@ -193,7 +193,7 @@ extern "C" int hsk_create(hsk_ctx** out, const hsk_config* cfg_in) {
         c->d_max = (uint32_t*)(s + 8);
         c->d_nheads = (uint64_t*)(s + 16);
         c->d_nout = (uint64_t*)(s + 24);
-        c->d_ndesc = (uint64_t*)(s + 32);
+        c->d_ndesc = (uint64_t*)(s + 128);
         c->d_nlocal = (uint64_t*)(s + 40);
         c->d_ovstats = (uint64_t*)(s + 48);
         c->counters = (uint32_t*)(s + 256);
@@ -456,7 +456,14 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
     // cuts at invalid bases, tile ends and the record cap; re-run if short
     uint64_t cap = std::min<uint64_t>(E.n_bases + 1, (uint64_t)((double)E.n_bases *
                                        (3.0 / (P.w + 1) + 1.0 / P.nmax + 1.0 / 256)) + (1u << 16));
-    uint64_t n_desc = 0;
+    uint64_t n_desc = 0, n_end[2] = {0, 0};
+    // The open lines of the fine partitions have to stay in L2 while their
+    // 16-byte records arrive, or half-filled sectors go to DRAM and come back:
+    // past 2^19 partitions (64 MB of lines) the scatter takes the first half of
+    // the partitions, then the second (long-read workload, 2^20 partitions: 6.0
+    // ms in one go, 4.7 in two, for 0.3 ms more in the walk).  32-byte records
+    // fill whole sectors and gain nothing (3.9 and 3.7 ms).
+    P.two_ended = F > (1u << 19) && k <= 32 && !sets;
     S.B = B;
     S.h_bucket_kmers.resize(B);
     S.h_bucket_rec.resize((size_t)B + 1);
@@ -465,7 +472,7 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
         CK(cudaMemsetAsync(c->bucket_kmers.p, 0, (size_t)B * 8, st));
         if (fine) CK(cudaMemsetAsync(d_rec_cnt, 0, F * 4, st));
         else CK(cudaMemsetAsync(d_rec_cnt, 0, cnt_bytes, st));
-        CK(cudaMemsetAsync(c->d_ndesc, 0, 8, st));
+        CK(cudaMemsetAsync(c->d_ndesc, 0, 16, st));
         P.desc = (uint64_t*)c->cta_off.p;
         P.desc_cap = cap;
         P.desc_count = (unsigned long long*)c->d_ndesc;
@@ -516,10 +523,11 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
             launch_scan_u32(d_rec_cnt, B, (uint64_t*)c->bucket_rec.p, (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st);
         CK(cudaGetLastError());
         // bucket statistics to the host (needed to size records and plan chunks)
-        CK(cudaMemcpyAsync(&n_desc, c->d_ndesc, 8, cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(n_end, c->d_ndesc, 16, cudaMemcpyDeviceToHost, st));
         CK(cudaMemcpyAsync(S.h_bucket_kmers.data(), c->bucket_kmers.p, (size_t)B * 8, cudaMemcpyDeviceToHost, st));
         CK(cudaMemcpyAsync(S.h_bucket_rec.data(), c->bucket_rec.p, ((size_t)B + 1) * 8, cudaMemcpyDeviceToHost, st));
         TRY(hsk_read_device_error(c, st));
+        n_desc = n_end[0] + n_end[1];
         if (n_desc <= cap) break;
         cap = n_desc;  // the walk counted every supermer: one more run fits them all
     }
@@ -536,9 +544,10 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
     S.sub_bits = sub_bits;
     TRY(hsk_ensure(c, c->records, std::max<uint64_t>(S.n_records, 1) * P.rec_words * 8, false));
     prof_mark(c, st, 1);
-    launch_scatter_desc((const uint64_t*)c->cta_off.p, n_desc, E.packed, k, (const uint64_t*)c->bucket_rec.p,
-                        d_cursor, d_part_cursor, fine ? sub_bits : 0, (uint64_t*)c->records.p, S.n_records, c->d_err,
-                        c->num_sms * 8, st);
+    for (int half = 0; half < 2; ++half)
+        launch_scatter_desc((const uint64_t*)c->cta_off.p + (half ? cap - n_end[1] : 0), n_end[half], E.packed, k,
+                            (const uint64_t*)c->bucket_rec.p, d_cursor, d_part_cursor, fine ? sub_bits : 0,
+                            (uint64_t*)c->records.p, S.n_records, c->d_err, c->num_sms * 8, st);
     CK(cudaGetLastError());
     S.records = (const uint64_t*)c->records.p;
     return HSK_OK;

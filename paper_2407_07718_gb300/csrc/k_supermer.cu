@@ -21,7 +21,7 @@
 // supermer starts where a bit is set, and ends at the next set bit of the
 // cuts, in this lane or a later one.  Every supermer becomes an 8-byte
 // descriptor (start base, k-mer count, bucket), appended to a global list with
-// one atomic per tile; per-bucket record and k-mer counts are kept in shared
+// one atomic per tile (or one for even and one for odd buckets); per-bucket record and k-mer counts are kept in shared
 // memory.  A second, light kernel scatters records into their buckets from
 // the descriptors.  DUMP mode writes per-window keys and scores for the stage
 // test.
@@ -211,7 +211,7 @@ __device__ __forceinline__ void mmer_scores32(u64 W0, u64 W1, int m, uint32_t se
     }
 }
 
-template <int MODE, bool SHORT, bool LEX>
+template <int MODE, bool SHORT, bool LEX, bool TWO_ENDED>
 __global__ void __launch_bounds__(SM_WARPS * 32, SM_CTAS) k_supermer(const __grid_constant__ SmParams P) {
     extern __shared__ __align__(16) unsigned char smem[];
     u64* s_pk = reinterpret_cast<u64*>(smem);
@@ -331,11 +331,13 @@ __global__ void __launch_bounds__(SM_WARPS * 32, SM_CTAS) k_supermer(const __gri
             const int bb = __popc(bmask);
             const uint32_t idmask = (((bmask + 1u) << P.sub_bits) - 1u);
             uint32_t D = 0, prev = 0;
+            [[maybe_unused]] uint32_t late = 0;  // bit j: the lowest bit of window j's id
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
                 const uint32_t id = min(a[j], row_at(rows, lane, j + off)) & idmask;
                 if (j > 0) D |= id != prev ? 1u << j : 0u;
                 else a[0] = id;
+                if (TWO_ENDED) late = __funnelshift_r(late, id, 1);
                 prev = id;
             }
             const uint32_t before = __shfl_up_sync(0xffffffffu, prev, 1);
@@ -350,17 +352,31 @@ __global__ void __launch_bounds__(SM_WARPS * 32, SM_CTAS) k_supermer(const __gri
             const int nl = later ? __ffs(later) - 1 : lane;
             const int fe = __shfl_sync(0xffffffffu, __ffs(ev) - 1, nl);
             const int open_end = later ? 32 * nl + fe : SM_TW;
-            const uint32_t mine = (uint32_t)__popc(start);
+            // descriptors: all upward from the array's start, or (TWO_ENDED)
+            // those of windows with the lowest id bit set downward from its end;
+            // `mine` and its sums hold the numbers of the two in 16 bits each
+            uint32_t mine = (uint32_t)__popc(start);
+            if (TWO_ENDED) mine += 0xFFFFu * (uint32_t)__popc(start & late);
             const uint32_t incl = warp_incl_sum<uint32_t>(mine);
             const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
             if (total) {
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(P.desc_count, (unsigned long long)total);
-                base = __shfl_sync(0xffffffffu, base, 0);
-                u64 o = base + incl - mine;
-                int extra = 0;  // pieces past the first of runs of more than nmax k-mers
-                auto desc_at = [&](u64 at, int pos, int n, uint32_t id) {
-                    const uint32_t b = bbase + (id & bmask);
+                u64 at0 = 0, at1 = 0;
+                auto reserve = [&](uint32_t sum, uint32_t n) {  // this lane's places, from its exclusive sum
+                    const uint32_t n0 = TWO_ENDED ? n & 0xFFFFu : n, n1 = TWO_ENDED ? n >> 16 : 0u;
+                    if (lane == 0 && n0) at0 = atomicAdd(P.desc_count, (unsigned long long)n0);
+                    if (lane == 0 && n1) at1 = atomicAdd(P.desc_count + 1, (unsigned long long)n1);
+                    at0 = __shfl_sync(0xffffffffu, at0, 0) + (TWO_ENDED ? sum & 0xFFFFu : sum);
+                    if (TWO_ENDED) at1 = __shfl_sync(0xffffffffu, at1, 0) + (sum >> 16);
+                };
+                reserve(incl - mine, total);
+                uint32_t extra = 0;  // pieces past the first of runs of more than nmax k-mers, counted like `mine`
+                auto put = [&](int pos, int n, uint32_t id) {
+                    const bool down = TWO_ENDED && (id & 1u);
+                    const u64 at = down ? P.desc_cap - 1 - at1++ : at0++;  // past the capacity: not written
+                    // TWO_ENDED: that bit is the bucket's highest, so the two kinds
+                    // are the two halves of the records
+                    const uint32_t in = id & bmask;
+                    const uint32_t b = bbase + (TWO_ENDED ? (in >> 1) | ((in & 1u) << (bb - 1)) : in);
                     if (P.part_rec) atomicAdd(P.part_rec + ((b << P.sub_bits) | (id >> bb)), 1u);
                     else atomicAdd(&s_cnt[b], 1u);
                     atomicAdd(&s_km[b], (uint32_t)n);
@@ -372,21 +388,19 @@ __global__ void __launch_bounds__(SM_WARPS * 32, SM_CTAS) k_supermer(const __gri
                     const uint32_t rest = ev & ~((2u << j) - 1u);
                     const int len = (rest ? 32 * lane + __ffs(rest) - 1 : open_end) - (32 * lane + j);
                     const uint32_t id = min(row_at(rows, lane, j), row_at(rows, lane, j + off)) & idmask;
-                    if (len > nmax) extra += (len - 1) / nmax;
-                    desc_at(o++, 32 * lane + j, min(len, nmax), id);
+                    if (len > nmax) extra += (uint32_t)((len - 1) / nmax) << (TWO_ENDED && (id & 1u) ? 16 : 0);
+                    put(32 * lane + j, min(len, nmax), id);
                 }
                 if (__any_sync(0xffffffffu, extra)) {
-                    const uint32_t xi = warp_incl_sum<uint32_t>((uint32_t)extra);
-                    const uint32_t xt = __shfl_sync(0xffffffffu, xi, 31);
-                    if (lane == 0) base = atomicAdd(P.desc_count, (unsigned long long)xt);
-                    base = __shfl_sync(0xffffffffu, base, 0);
-                    o = base + xi - (uint32_t)extra;
+                    const uint32_t xi = warp_incl_sum<uint32_t>(extra);
+                    at0 = at1 = 0;
+                    reserve(xi - extra, __shfl_sync(0xffffffffu, xi, 31));
                     for (uint32_t S = extra ? start : 0u; S; S &= S - 1) {
                         const int j = __ffs(S) - 1;
                         const uint32_t rest = ev & ~((2u << j) - 1u);
                         const int end = rest ? 32 * lane + __ffs(rest) - 1 : open_end;
                         const uint32_t id = min(row_at(rows, lane, j), row_at(rows, lane, j + off)) & idmask;
-                        for (int q = 32 * lane + j + nmax; q < end; q += nmax) desc_at(o++, q, min(end - q, nmax), id);
+                        for (int q = 32 * lane + j + nmax; q < end; q += nmax) put(q, min(end - q, nmax), id);
                     }
                 }
             }
@@ -405,13 +419,16 @@ __global__ void __launch_bounds__(SM_WARPS * 32, SM_CTAS) k_supermer(const __gri
 }
 
 using SmKernel = void (*)(SmParams);
-template <int MODE>
+template <int MODE, bool TWO_ENDED>
 static SmKernel walk_kernel(int m, bool lexical) {
-    if (m <= 16) return lexical ? (SmKernel)k_supermer<MODE, true, true> : (SmKernel)k_supermer<MODE, true, false>;
-    return lexical ? (SmKernel)k_supermer<MODE, false, true> : (SmKernel)k_supermer<MODE, false, false>;
+    if (m <= 16)
+        return lexical ? (SmKernel)k_supermer<MODE, true, true, TWO_ENDED> : (SmKernel)k_supermer<MODE, true, false, TWO_ENDED>;
+    return lexical ? (SmKernel)k_supermer<MODE, false, true, TWO_ENDED> : (SmKernel)k_supermer<MODE, false, false, TWO_ENDED>;
 }
-static SmKernel walk_kernel(int mode, int m, bool lexical) {
-    SmKernel fn = mode == SM_DESC ? walk_kernel<SM_DESC>(m, lexical) : walk_kernel<SM_DUMP>(m, lexical);
+static SmKernel walk_kernel(int mode, int m, bool lexical, bool two_ended) {
+    SmKernel fn = mode != SM_DESC ? walk_kernel<SM_DUMP, false>(m, lexical)
+                  : two_ended     ? walk_kernel<SM_DESC, true>(m, lexical)
+                                  : walk_kernel<SM_DESC, false>(m, lexical);
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)supermer_smem_bytes(mode, SM_MAX_BUCKETS));
     return fn;
 }
@@ -419,12 +436,12 @@ static SmKernel walk_kernel(int mode, int m, bool lexical) {
 void launch_supermer(int mode, const SmParams& p, cudaStream_t st) {
     if (p.n_bases == 0) return;
     count_launch();
-    walk_kernel(mode, p.m, p.lexical)<<<p.grid, SM_WARPS * 32, supermer_smem_bytes(mode, p.n_buckets), st>>>(p);
+    walk_kernel(mode, p.m, p.lexical, p.two_ended)<<<p.grid, SM_WARPS * 32, supermer_smem_bytes(mode, p.n_buckets), st>>>(p);
 }
 
 int supermer_max_ctas_per_sm(int mode, int m, bool lexical, uint32_t n_buckets) {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel(mode, m, lexical), SM_WARPS * 32,
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel(mode, m, lexical, false), SM_WARPS * 32,
                                                       supermer_smem_bytes(mode, n_buckets)) != cudaSuccess)
         n = 1;
     return n > 0 ? n : 1;
@@ -481,8 +498,7 @@ __device__ __forceinline__ void one_strand(u64 (&r)[RW], int nb) {
 // into the buckets (4.4 and 3.8 ms; 5.9 and 4.4 with the sub-partition beside
 // each record) and from there into the partitions (2.1 and 1.3 ms) took 8.0
 // and 5.7 ms on the long- and short-read workloads; this takes 5.0 to 5.8 and
-// 3.9 (and 0.1 of the walk, which counts records per partition).  Two passes,
-// each over half of the partitions, took 4.7 and 4.3.
+// 3.9 (and 0.1 of the walk, which counts records per partition).
 template <bool WIDE, bool FINE>
 __global__ void __launch_bounds__(256) k_scatter_desc(const u64* __restrict__ desc, u64 n_desc,
                                                       const u64* __restrict__ packed, int k,
