@@ -176,6 +176,12 @@ void launch_compact(const uint64_t* sub_off, const uint32_t* kc, const uint64_t*
                     uint32_t n_groups, int key_words, const void* keys, const uint32_t* kcount, void* out_keys,
                     uint32_t* out_counts, uint64_t out_cap, int* err, int grid, cudaStream_t st);
 void launch_transpose_kc(const uint32_t* kc, uint32_t n_groups, uint32_t* kc_t, int grid, cudaStream_t st);
+// S6, one MSD pass: segment c's pairs (its tiles of split_tile_keys() are
+// [tile_start[c], tile_start[c + 1])) to cursor[c * 256 + digit] on, in any order
+uint64_t split_tile_keys(int key_words);
+void launch_split_pairs(const void* kin, const uint32_t* vin, void* kout, uint32_t* vout, const uint64_t* key_base,
+                        uint32_t C, const uint32_t* tile_start, uint32_t n_tiles, int key_words, int shift,
+                        uint64_t* cursor, int* err, cudaStream_t st);
 // S6 on chip: range r holds pairs [bounds[r], bounds[r+1]) of (kin, vin) that
 // share their top fixed_bits key bits; every range is sorted by key and
 // written to its place in (kout, vout).  `group` ranges (1 to 64, a power of

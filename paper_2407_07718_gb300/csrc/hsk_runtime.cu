@@ -721,7 +721,7 @@ int hsk_order_pairs(hsk_ctx* c, void* keys, uint32_t* counts, uint64_t n, int ke
 // partitioned by their top digit (hist: S x 256 pairs per set and digit).
 int hsk_top_digit_pass(hsk_ctx* c, const void* keys, const uint32_t* counts, uint32_t S, const uint64_t* seg,
                        const uint64_t* hist, int kw, int key_bits, cudaStream_t st) {
-    const uint64_t TILE = onesweep_tile_keys(kw);
+    const uint64_t TILE = split_tile_keys(kw);
     std::vector<uint64_t>& hb = c->s6_h;
     hb.resize((size_t)S * 256 + 1);
     std::vector<uint64_t> up(S + 1 + (S + 2) / 2);  // segments, then their first tiles
@@ -745,17 +745,15 @@ int hsk_top_digit_pass(hsk_ctx* c, const void* keys, const uint32_t* counts, uin
         return HSK_EOVERFLOW;
     }
     TRY(hsk_ensure(c, c->s6_bounds, hb.size() * 8, false));
+    TRY(hsk_ensure(c, c->digit_off, hb.size() * 8, false));  // the pass's cursors
     TRY(hsk_ensure(c, c->seg, up.size() * 8, false));
     CK(cudaMemcpyAsync(c->s6_bounds.p, hb.data(), hb.size() * 8, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(c->seg.p, up.data(), up.size() * 8, cudaMemcpyHostToDevice, st));
-    TRY(hsk_ensure_status(c, tiles * 256 + 1, st));
-    uint32_t ep, *ctr;
-    TRY(hsk_next_epoch(c, st, &ep));
-    TRY(hsk_next_counter(c, st, &ctr));
+    CK(cudaMemcpyAsync(c->digit_off.p, hb.data(), hb.size() * 8, cudaMemcpyHostToDevice, st));
     const uint64_t* d_seg = (const uint64_t*)c->seg.p;
-    launch_onesweep_seg(keys, c->out_keys.p, counts, (uint32_t*)c->out_counts.p, d_seg, S, (uint32_t)tiles,
-                        (const uint32_t*)(d_seg + S + 1), kw, key_bits - 8, (const uint64_t*)c->s6_bounds.p,
-                        (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st);
+    launch_split_pairs(keys, counts, c->out_keys.p, (uint32_t*)c->out_counts.p, d_seg, S,
+                       (const uint32_t*)(d_seg + S + 1), (uint32_t)tiles, kw, key_bits - 8,
+                       (uint64_t*)c->digit_off.p, c->d_err, st);
     CK(cudaGetLastError());
     return HSK_OK;
 }
@@ -792,7 +790,7 @@ int hsk_order_partitioned(hsk_ctx* c, uint64_t n, uint32_t S, int kw, int key_bi
     if (!one_pass && S > 256) return HSK_OK;  // 0.5 MB of tables per set
     TRY(hsk_ensure(c, c->pair_alt_keys, n * kb, false));
     TRY(hsk_ensure(c, c->pair_alt_counts, n * 4, false));
-    uint32_t ep, *ctr;
+    uint32_t* ctr;
     if (one_pass) {
         TRY(hsk_next_counter(c, st, &ctr));
         launch_range_sort(c->out_keys.p, (const uint32_t*)c->out_counts.p, c->pair_alt_keys.p,
@@ -806,7 +804,7 @@ int hsk_order_partitioned(hsk_ctx* c, uint64_t n, uint32_t S, int kw, int key_bi
     }
     const uint64_t R2 = (uint64_t)R * 256;
     TRY(hsk_ensure(c, c->pass_hist, R2 * 8 + 256, false));  // digit counts; later two lists of ranges
-    const uint64_t TILE = onesweep_tile_keys(kw);
+    const uint64_t TILE = split_tile_keys(kw);
     std::vector<uint32_t> ts((size_t)R + 1);
     uint64_t tiles = 0;
     for (uint32_t d = 0; d < R; ++d) {
@@ -817,17 +815,16 @@ int hsk_order_partitioned(hsk_ctx* c, uint64_t n, uint32_t S, int kw, int key_bi
     TRY(hsk_ensure(c, c->seg, ts.size() * 4, false));
     CK(cudaMemcpyAsync(c->seg.p, ts.data(), ts.size() * 4, cudaMemcpyHostToDevice, st));
     TRY(hsk_ensure(c, c->digit_off, (R2 + 1) * 8, false));
-    TRY(hsk_ensure_status(c, tiles * 256 + 1, st));
     uint64_t* doff = (uint64_t*)c->digit_off.p;
     CK(cudaMemsetAsync(c->pass_hist.p, 0, R2 * 8, st));
     launch_digit_hist_seg(c->out_keys.p, kw, d_bounds, R, n, (uint64_t*)c->pass_hist.p, 1, st, key_bits - 16);
     launch_digit_offsets_seg((const uint64_t*)c->pass_hist.p, d_bounds, doff, 1, R, st);
     CK(cudaMemcpyAsync(doff + R2, &hb[R], 8, cudaMemcpyHostToDevice, st));
-    TRY(hsk_next_epoch(c, st, &ep));
-    TRY(hsk_next_counter(c, st, &ctr));
-    launch_onesweep_seg(c->out_keys.p, c->pair_alt_keys.p, (const uint32_t*)c->out_counts.p,
-                        (uint32_t*)c->pair_alt_counts.p, d_bounds, R, (uint32_t)tiles, (const uint32_t*)c->seg.p, kw,
-                        key_bits - 16, doff, (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st);
+    // the digit counts have become offsets: their room holds the cursors
+    CK(cudaMemcpyAsync(c->pass_hist.p, doff, R2 * 8, cudaMemcpyDeviceToDevice, st));
+    launch_split_pairs(c->out_keys.p, (const uint32_t*)c->out_counts.p, c->pair_alt_keys.p,
+                       (uint32_t*)c->pair_alt_counts.p, d_bounds, R, (const uint32_t*)c->seg.p, (uint32_t)tiles, kw,
+                       key_bits - 16, (uint64_t*)c->pass_hist.p, c->d_err, st);
     // sub-ranges are sorted a group at a time: about a third of the capacity
     uint32_t group = 1;
     while (group < 64 && largest_set / 65536 * group * 2 <= range_sort_cap(kw) / 3) group *= 2;
