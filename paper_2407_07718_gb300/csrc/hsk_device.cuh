@@ -400,4 +400,81 @@ __device__ __forceinline__ void record_kmers(const u64 (&W)[4], uint32_t n, int 
     }
 }
 
+// Bit t (most significant first) = OR of bits [t, t + L) of the 128-bit
+// value a:b, for t = 0..63 and 1 <= L <= 64: OR over windows of doubling
+// width, then two overlapping windows of that width.
+__device__ __forceinline__ u64 window_or64(u64 a, u64 b, int L) {
+    u64 hi = a, lo = b;
+    int width = 1;
+    while (2 * width <= L) {
+        hi |= (hi << width) | (lo >> (64 - width));
+        lo |= lo << width;
+        width *= 2;
+    }
+    const int d = L - width;  // 0 <= d < width
+    return d ? hi | (hi << d) | (lo >> (64 - d)) : hi;
+}
+
+// The canonical codes of up to 16 consecutive k-mers, rolled in 32-bit words
+// by constant shifts: the bases from the current k-mer on (f), and the
+// reversed and complemented ones shifted so that the current k-mer's code is
+// left aligned in r[1..], the bases that later k-mers shift in being in r[0].
+template <bool WIDE>
+struct KmerRoll {
+    static constexpr int N = WIDE ? 4 : 2;  // words of a key
+    using K = typename std::conditional<WIDE, key128, u64>::type;
+    uint32_t f[N + 1], r[N + 1];
+    // w: N + 1 words of bases (16 a word), the first k-mer at the top of w[0]; k <= 16 N
+    __device__ __forceinline__ void start(const uint32_t* w, int k) {
+        // all of them reversed and complemented; the first k-mer starts at base
+        // 16 (N + 1) - k (16 or more)
+        uint32_t x[N + 4];
+#pragma unroll
+        for (int i = 0; i <= N; ++i) {
+            f[i] = w[i];
+            x[i] = revcomp32(w[N - i]);
+        }
+        x[N + 1] = x[N + 2] = x[N + 3] = 0;
+        const int o = 2 * (16 * (N + 1) - k);
+        if (o >= 64) {
+#pragma unroll
+            for (int i = 0; i < N + 3; ++i) x[i] = x[i + 1];
+        }
+#pragma unroll
+        for (int i = 0; i <= N; ++i) r[i] = __funnelshift_l(x[i + 1], x[i], o & 31);
+    }
+    // the next k-mer
+    __device__ __forceinline__ void step() {
+#pragma unroll
+        for (int i = 0; i < N; ++i) f[i] = __funnelshift_l(f[i + 1], f[i], 2);
+        f[N] <<= 2;
+#pragma unroll
+        for (int i = N; i > 0; --i) r[i] = __funnelshift_r(r[i], r[i - 1], 2);
+        r[0] >>= 2;
+    }
+    // the smaller code, left aligned; mask: the bits of its low word that are code
+    __device__ __forceinline__ K left(u64 mask) const {
+        if constexpr (WIDE) {
+            const u64 fh = ((u64)f[0] << 32) | f[1], fl = ((u64)f[2] << 32) | f[3];
+            const u64 rh = ((u64)r[1] << 32) | r[2], rl = ((u64)r[3] << 32) | r[4];
+            const bool fwd = fh < rh || (fh == rh && fl < rl);
+            K key;
+            key.hi = fwd ? fh : rh;
+            key.lo = (fwd ? fl : rl) & mask;
+            return key;
+        } else {
+            const u64 a = ((u64)f[0] << 32) | f[1], b = ((u64)r[1] << 32) | r[2];
+            return (a < b ? a : b) & mask;
+        }
+    }
+};
+// Left-aligned code of k bases -> right aligned.
+__device__ __forceinline__ u64 right_aligned(u64 key, int k) { return key >> (64 - 2 * k); }
+__device__ __forceinline__ key128 right_aligned(key128 key, int k) {
+    const int sh = 128 - 2 * k;  // 0 .. 62
+    key.lo = sh ? (key.lo >> sh) | (key.hi << (64 - sh)) : key.lo;
+    key.hi >>= sh;
+    return key;
+}
+
 }  // namespace hsk

@@ -43,11 +43,12 @@ extern "C" int hsk_count_ext(hsk_ctx* c, const char* reads, const uint64_t* offs
             // the kept keys (sorted, on the device since the count) into a table of indices
             uint32_t slots = 1024;
             while (slots < 2 * np) slots <<= 1;
-            // composites: (index << 40) | start, 64-bit while the index fits 24 bits
-            int ib = 0;
-            while ((1ull << ib) < np) ++ib;
-            const bool wide = ib > 24;
-            const int comp_bits = 40 + std::max(ib, 1);
+            // composites: index above the start's bits, in 64 bits while they fit
+            int ib = 1, pb = 1;
+            while ((1ull << ib) <= np) ++ib;
+            while ((1ull << pb) < n_bases) ++pb;
+            const bool wide = ib + pb > 64;
+            const int comp_bits = ib + pb;
             const size_t cb = wide ? 16 : 8;
             // occurrence offsets = exclusive scan of the kept counts
             TRY(hsk_ensure(c, c->ext_tab, (size_t)slots * 4 + (np + 1) * 8 + 64, false));
@@ -55,7 +56,7 @@ extern "C" int hsk_count_ext(hsk_ctx* c, const char* reads, const uint64_t* offs
             uint64_t* occ_off = (uint64_t*)((char*)c->ext_tab.p + (size_t)slots * 4);
             CK(cudaMemsetAsync(table, 0, (size_t)slots * 4, st));
             CK(cudaMemsetAsync(c->small, 0, 64, st));
-            launch_ext_insert(c->out_keys.p, kw, np, table, slots - 1, c->d_err, st);
+            launch_ext_insert(c->out_keys.p, kw, np, table, slots - 1, ib, c->d_err, st);
             TRY(hsk_ensure_status(c, scan_status_words(np), st));
             uint32_t ep, *ctr;
             TRY(hsk_next_epoch(c, st, &ep));
@@ -69,7 +70,7 @@ extern "C" int hsk_count_ext(hsk_ctx* c, const char* reads, const uint64_t* offs
             TRY(hsk_ensure(c, c->batch_a, std::max<uint64_t>(n_occ, 1) * cb, false));
             TRY(hsk_ensure(c, c->ext_occ, std::max<uint64_t>(n_occ, 1) * 8, false));
             launch_ext_scan((const uint64_t*)c->pk.p, (const uint64_t*)c->iv.p, (const uint64_t*)c->rs.p, n_bases, k,
-                            c->out_keys.p, table, slots - 1, wide, c->batch_a.p, n_occ, c->d_nout, c->d_err,
+                            c->out_keys.p, table, slots - 1, ib, pb, wide, c->batch_a.p, n_occ, c->d_nout, c->d_err,
                             c->num_sms * 8, st);
             CK(cudaGetLastError());
             uint64_t emitted = 0;
@@ -83,7 +84,7 @@ extern "C" int hsk_count_ext(hsk_ctx* c, const char* reads, const uint64_t* offs
             TRY(hsk_plain_sort(c, c->batch_a.p, nullptr, n_occ, wide ? 2 : 1, comp_bits, c->batch_b, nullptr, st));
             uint32_t* occ_read = (uint32_t*)c->ext_occ.p;
             uint32_t* occ_pos = occ_read + n_occ;
-            launch_ext_decode_pos(c->batch_a.p, wide, n_occ, (const uint64_t*)c->in_offsets.p, n_reads, occ_read,
+            launch_ext_decode_pos(c->batch_a.p, wide, pb, n_occ, (const uint64_t*)c->in_offsets.p, n_reads, occ_read,
                                   occ_pos, c->num_sms * 8, st);
             CK(cudaGetLastError());
             c->ext_read.resize(n_occ);

@@ -2,15 +2,14 @@
 // read and position of every occurrence of every k-mer the filter kept.
 //
 // After a count, the kept k-mers are sorted and distinct.  They are entered
-// into a table of indices (open addressing over 32-bit slots holding index+1;
-// a probe compares the query with the kept key at that index, so one 32-bit
-// compare-and-swap claims a slot whatever the key width).  A scan over every
-// window then looks its canonical key up and, when the key is kept, emits the
-// composite (k-mer index, global window start).  Sorting the composites (the
-// LSD radix sort of k_sort.cu) puts each k-mer's occurrences together in
-// position order, which is (read, position) order; a last pass turns the
-// global start into (read, position in read) with a binary search over the
-// read offsets.
+// into a table of indices (open addressing over 32-bit slots holding index + 1
+// and, above it, more hash bits, so one 32-bit compare-and-swap claims a slot
+// whatever the key width).  A scan over every window then looks its canonical
+// key up and, when the key is kept, emits the composite (k-mer index, global
+// window start).  Sorting the composites (the LSD radix sort of k_sort.cu)
+// puts each k-mer's occurrences together in position order, which is (read,
+// position) order; a last pass turns the global start into (read, position in
+// read) with a binary search over the read offsets.
 //
 // The payload codec (k_ext_encode / k_ext_decode) is the paper's encoding of
 // extension information on its way to a destination: each item is
@@ -23,25 +22,44 @@
 
 namespace hsk {
 
-constexpr uint32_t EXT_EMPTY = 0;
-
-__device__ __forceinline__ uint32_t ext_hash(u64 k) { return (uint32_t)((k * 0x9E3779B97F4A7C15ULL) >> 32); }
-__device__ __forceinline__ uint32_t ext_hash(const key128& k) {
-    return (uint32_t)(((k.lo ^ (k.hi * 0xC2B2AE3D27D4EB4FULL)) * 0x9E3779B97F4A7C15ULL) >> 32);
+// A slot of the table: the low idx_bits hold a kept k-mer's index + 1 (0: the
+// slot is empty), the bits above some more hash bits of the k-mer, so that a
+// probe reads the kept key only when it very likely matches.
+struct ExtHash {
+    uint32_t slot, tag;
+};
+__device__ __forceinline__ uint32_t ext_mix(uint32_t x) {
+    x = (x ^ (x >> 16)) * 0x85EBCA6Bu;
+    return x ^ (x >> 13);
+}
+__device__ __forceinline__ ExtHash ext_hash(uint32_t a, uint32_t b, uint32_t mask, int idx_bits) {
+    ExtHash h;
+    h.slot = ext_mix(a) & mask;
+    h.tag = idx_bits < 32 ? ext_mix(b) << idx_bits : 0u;
+    return h;
+}
+__device__ __forceinline__ ExtHash ext_hash(u64 k, uint32_t mask, int idx_bits) {
+    const uint32_t l = (uint32_t)k, h = (uint32_t)(k >> 32);
+    return ext_hash(l * 0x9E3779B1u + h * 0x85EBCA77u, l * 0xC2B2AE3Du + h * 0x27D4EB2Fu, mask, idx_bits);
+}
+__device__ __forceinline__ ExtHash ext_hash(const key128& k, uint32_t mask, int idx_bits) {
+    const uint32_t a = (uint32_t)k.lo, b = (uint32_t)(k.lo >> 32), c = (uint32_t)k.hi, d = (uint32_t)(k.hi >> 32);
+    return ext_hash(a * 0x9E3779B1u + b * 0x85EBCA77u + c * 0xC2B2AE3Du + d * 0x27D4EB2Fu,
+                    a * 0x165667B1u + b * 0xD3A2646Du + c * 0xFD7046C5u + d * 0xB55A4F09u, mask, idx_bits);
 }
 
 template <typename K>
 __global__ void __launch_bounds__(256) k_ext_insert(const K* __restrict__ keys, uint64_t n, uint32_t* table,
-                                                    uint32_t mask, int* err) {
+                                                    uint32_t mask, int idx_bits, int* err) {
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        const K key = keys[i];
-        uint32_t h = ext_hash(key) & mask;
+        const ExtHash x = ext_hash(keys[i], mask, idx_bits);
+        uint32_t h = x.slot;
         for (uint32_t probe = 0;; ++probe) {
             if (probe > mask) {  // never: the table has twice as many slots as keys
                 raise_error(err, HSK_DERR_BOUNDS);
                 break;
             }
-            if (atomicCAS(&table[h], EXT_EMPTY, (uint32_t)i + 1) == EXT_EMPTY) break;
+            if (atomicCAS(&table[h], 0u, x.tag | ((uint32_t)i + 1)) == 0u) break;
             h = (h + 1) & mask;
         }
     }
@@ -50,81 +68,118 @@ __global__ void __launch_bounds__(256) k_ext_insert(const K* __restrict__ keys, 
 // Index of `key` among the kept keys, or -1.
 template <typename K>
 __device__ __forceinline__ int64_t ext_find(const K& key, const K* __restrict__ kept, const uint32_t* __restrict__ table,
-                                            uint32_t mask) {
-    uint32_t h = ext_hash(key) & mask;
+                                            uint32_t mask, int idx_bits) {
+    const ExtHash x = ext_hash(key, mask, idx_bits);
+    const uint32_t idx = idx_bits < 32 ? (1u << idx_bits) - 1u : 0xFFFFFFFFu;
+    uint32_t h = x.slot;
     for (uint32_t probe = 0; probe <= mask; ++probe) {
         const uint32_t v = table[h];
-        if (v == EXT_EMPTY) return -1;
-        if (key_eq(kept[v - 1], key)) return (int64_t)(v - 1);
+        if (v == 0) return -1;
+        if ((v & ~idx) == x.tag && key_eq(kept[(v & idx) - 1], key)) return (int64_t)((v & idx) - 1);
         h = (h + 1) & mask;
     }
     return -1;
 }
 
-// One thread per 64 window starts: validity from the invalid and read-start
-// masks (no invalid base in the window, no read start after its first base),
-// then each valid window's canonical key is looked up; kept ones emit
-// (index << 40) | start into out[atomic cursor] (128-bit composites when the
-// index needs more than 24 bits).
+// A warp takes 1024 window starts, lane l the 32 that start in its word of
+// packed bases: their validity from the invalid and read-start masks, their
+// canonical keys rolled 16 at a time (KmerRoll), each valid one looked up.
+// Kept ones emit (index << pos_bits) | start, buffered per warp and written
+// with one atomic a buffer (128-bit composites when the two do not fit 64).
+// Bound by the table's random reads (from L2 while it fits): 1.9 ms for 150 M
+// windows and 3.6 M kept k-mers.  One thread per 64 windows, each window's key
+// cut out and compared with a kept key at every probe, the masks shifted k
+// times and one atomic a hit, took 7.4 ms.
+constexpr int EXT_BUF = 128;  // composites buffered per warp
 template <typename K>
 __global__ void __launch_bounds__(256) k_ext_scan(const u64* __restrict__ packed, const u64* __restrict__ invalid,
                                                   const u64* __restrict__ start, uint64_t n_bases, int k,
                                                   const K* __restrict__ kept, const uint32_t* __restrict__ table,
-                                                  uint32_t mask, bool wide_out, void* out, uint64_t out_cap,
-                                                  unsigned long long* cursor, int* err) {
-    const uint64_t words = (n_bases + 63) / 64;
-    for (uint64_t w = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; w < words; w += (uint64_t)gridDim.x * blockDim.x) {
-        // bad window starts: an invalid base in [p, p + k) or a read start in (p, p + k)
-        u64 bad = 0;
-        for (int j = 0; j < k; ++j) {
-            const uint64_t g = w * 64 + j;  // bits of window starts w*64 .. w*64+63, shifted by j
-            const uint64_t q = g >> 6;
-            const int off = (int)(g & 63);
-            const u64 a = q < words ? invalid[q] : ~0ULL;
-            const u64 b = q + 1 < words ? invalid[q + 1] : ~0ULL;
-            bad |= off ? (a << off) | (b >> (64 - off)) : a;
-            if (j > 0) {
-                const u64 sa = q < words ? start[q] : 0ULL;
-                const u64 sb = q + 1 < words ? start[q + 1] : 0ULL;
-                bad |= off ? (sa << off) | (sb >> (64 - off)) : sa;
-            }
-        }
-        u64 good = ~bad;
-        while (good) {
-            const int t = __clzll(good);  // most significant first: window w*64 + t
-            good &= ~(0x8000000000000000ULL >> t);
-            const uint64_t p = w * 64 + (uint64_t)t;
-            if (p + (uint64_t)k > n_bases) break;
-            K key;
-            if constexpr (std::is_same<K, u64>::value) key = canonical64(extract_k64(packed, p, k), k);
-            else key = canonical128(extract_k128(packed, p, k), k);
-            const int64_t idx = ext_find(key, kept, table, mask);
-            if (idx < 0) continue;
-            const unsigned long long at = atomicAdd(cursor, 1ULL);
+                                                  uint32_t mask, int idx_bits, int pos_bits, bool wide_out, void* out,
+                                                  uint64_t out_cap, unsigned long long* cursor, int* err) {
+    constexpr bool WIDE = sizeof(K) == 16;
+    __shared__ uint64_t s_pos[8][EXT_BUF];
+    __shared__ uint32_t s_idx[8][EXT_BUF];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t n_pw = (n_bases + 31) / 32, n_mw = (n_bases + 63) / 64, tiles = (n_bases + 1023) / 1024;
+    const u64 code = ~0ULL << (WIDE ? 128 - 2 * k : 64 - 2 * k);
+    int nbuf = 0;  // composites buffered by this warp
+    auto flush = [&]() {
+        unsigned long long base = 0;
+        __syncwarp();
+        if (lane == 0) base = atomicAdd(cursor, (unsigned long long)nbuf);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        for (int i = lane; i < nbuf; i += 32) {
+            const uint64_t at = base + i, p = s_pos[warp][i];
+            const u64 idx = s_idx[warp][i];
             if (at >= out_cap) {
                 raise_error(err, HSK_DERR_BOUNDS);
-                continue;
-            }
-            if (!wide_out) {
-                reinterpret_cast<u64*>(out)[at] = ((u64)idx << 40) | p;
+            } else if (!wide_out) {
+                reinterpret_cast<u64*>(out)[at] = (idx << pos_bits) | p;
             } else {
                 key128 c;
-                c.lo = p | ((u64)idx << 40);
-                c.hi = (u64)idx >> 24;
+                c.lo = p | (idx << pos_bits);
+                c.hi = idx >> (64 - pos_bits);
                 reinterpret_cast<key128*>(out)[at] = c;
             }
         }
+        __syncwarp();
+        nbuf = 0;
+    };
+    for (uint64_t t = (uint64_t)blockIdx.x * 8 + warp; t < tiles; t += (uint64_t)gridDim.x * 8) {
+        const uint64_t p0 = t * 1024 + 32 * lane, wi = p0 >> 5, q = p0 >> 6;
+        // window starts whose k bases are all valid and in one read, window j at bit j
+        uint32_t V;
+        {
+            u64 iv[2], rs[3];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) iv[i] = q + i < n_mw ? invalid[q + i] : ~0ULL;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) rs[i] = q + i < n_mw ? start[q + i] : 0ULL;
+            u64 bad = window_or64(iv[0], iv[1], k);
+            if (k > 1) bad |= window_or64((rs[0] << 1) | (rs[1] >> 63), (rs[1] << 1) | (rs[2] >> 63), k - 1);
+            V = ~__brev(lane & 1 ? (uint32_t)bad : (uint32_t)(bad >> 32));
+            const uint64_t left = n_bases + 1 > p0 + k ? n_bases + 1 - (p0 + k) : 0;
+            if (left < 32) V &= (1u << left) - 1u;
+        }
+        uint32_t w[6];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const u64 x = (i < 2 || WIDE) && wi + i < n_pw ? packed[wi + i] : 0ULL;
+            w[2 * i] = (uint32_t)(x >> 32);
+            w[2 * i + 1] = (uint32_t)x;
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            KmerRoll<WIDE> S;
+            S.start(w + s, k);
+            for (int j = 0; j < 16; ++j) {
+                int64_t idx = -1;
+                if ((V >> (16 * s + j)) & 1u) idx = ext_find(right_aligned(S.left(code), k), kept, table, mask, idx_bits);
+                S.step();
+                const uint32_t hit = __ballot_sync(0xffffffffu, idx >= 0);
+                if (!hit) continue;
+                if (idx >= 0) {
+                    const int at = nbuf + __popc(hit & ((1u << lane) - 1u));
+                    s_pos[warp][at] = p0 + 16 * s + j;
+                    s_idx[warp][at] = (uint32_t)idx;
+                }
+                nbuf += __popc(hit);
+                if (nbuf > EXT_BUF - 32) flush();
+            }
+        }
     }
+    if (nbuf) flush();
 }
 
 // Sorted composites -> (read, position in read): read = the last read whose
 // offset is <= the global start.
-__global__ void __launch_bounds__(256) k_ext_decode_pos(const void* comp, bool wide, uint64_t n,
+__global__ void __launch_bounds__(256) k_ext_decode_pos(const void* comp, bool wide, int pos_bits, uint64_t n,
                                                         const uint64_t* __restrict__ offsets, uint64_t n_reads,
                                                         uint32_t* __restrict__ occ_read, uint32_t* __restrict__ occ_pos) {
     for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (uint64_t)gridDim.x * blockDim.x) {
-        const u64 p = wide ? (reinterpret_cast<const key128*>(comp)[j].lo & ((1ULL << 40) - 1))
-                           : (reinterpret_cast<const u64*>(comp)[j] & ((1ULL << 40) - 1));
+        const u64 c = wide ? reinterpret_cast<const key128*>(comp)[j].lo : reinterpret_cast<const u64*>(comp)[j];
+        const u64 p = c & ((1ULL << pos_bits) - 1);
         uint64_t lo = 0, hi = n_reads;  // offsets[lo] <= p < offsets[hi]
         while (hi - lo > 1) {
             const uint64_t mid = (lo + hi) >> 1;
@@ -136,38 +191,38 @@ __global__ void __launch_bounds__(256) k_ext_decode_pos(const void* comp, bool w
     }
 }
 
-void launch_ext_insert(const void* keys, int key_words, uint64_t n, uint32_t* table, uint32_t mask, int* err,
-                       cudaStream_t st) {
+void launch_ext_insert(const void* keys, int key_words, uint64_t n, uint32_t* table, uint32_t mask, int idx_bits,
+                       int* err, cudaStream_t st) {
     if (n == 0) return;
     count_launch();
     const unsigned g = (unsigned)std::min<uint64_t>((n + 255) / 256, 65535);
-    if (key_words == 1) k_ext_insert<u64><<<g, 256, 0, st>>>((const u64*)keys, n, table, mask, err);
-    else k_ext_insert<key128><<<g, 256, 0, st>>>((const key128*)keys, n, table, mask, err);
+    if (key_words == 1) k_ext_insert<u64><<<g, 256, 0, st>>>((const u64*)keys, n, table, mask, idx_bits, err);
+    else k_ext_insert<key128><<<g, 256, 0, st>>>((const key128*)keys, n, table, mask, idx_bits, err);
 }
 
 void launch_ext_scan(const uint64_t* packed, const uint64_t* invalid, const uint64_t* start, uint64_t n_bases, int k,
-                     const void* kept, const uint32_t* table, uint32_t mask, bool wide_out, void* out,
-                     uint64_t out_cap, uint64_t* cursor, int* err, int grid, cudaStream_t st) {
+                     const void* kept, const uint32_t* table, uint32_t mask, int idx_bits, int pos_bits, bool wide_out,
+                     void* out, uint64_t out_cap, uint64_t* cursor, int* err, int grid, cudaStream_t st) {
     if (n_bases == 0) return;
     count_launch();
-    const uint64_t words = (n_bases + 63) / 64;
-    const unsigned g = (unsigned)std::min<uint64_t>((words + 255) / 256, (uint64_t)grid);
+    const uint64_t tiles = (n_bases + 1023) / 1024;
+    const unsigned g = (unsigned)std::min<uint64_t>((tiles + 7) / 8, (uint64_t)grid);
     if (k <= 32)
         k_ext_scan<u64><<<g, 256, 0, st>>>((const u64*)packed, (const u64*)invalid, (const u64*)start, n_bases, k,
-                                           (const u64*)kept, table, mask, wide_out, out, out_cap,
+                                           (const u64*)kept, table, mask, idx_bits, pos_bits, wide_out, out, out_cap,
                                            (unsigned long long*)cursor, err);
     else
         k_ext_scan<key128><<<g, 256, 0, st>>>((const u64*)packed, (const u64*)invalid, (const u64*)start, n_bases, k,
-                                              (const key128*)kept, table, mask, wide_out, out, out_cap,
-                                              (unsigned long long*)cursor, err);
+                                              (const key128*)kept, table, mask, idx_bits, pos_bits, wide_out, out,
+                                              out_cap, (unsigned long long*)cursor, err);
 }
 
-void launch_ext_decode_pos(const void* comp, bool wide, uint64_t n, const uint64_t* offsets, uint64_t n_reads,
-                           uint32_t* occ_read, uint32_t* occ_pos, int grid, cudaStream_t st) {
+void launch_ext_decode_pos(const void* comp, bool wide, int pos_bits, uint64_t n, const uint64_t* offsets,
+                           uint64_t n_reads, uint32_t* occ_read, uint32_t* occ_pos, int grid, cudaStream_t st) {
     if (n == 0) return;
     count_launch();
     const unsigned g = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)grid);
-    k_ext_decode_pos<<<g, 256, 0, st>>>(comp, wide, n, offsets, n_reads, occ_read, occ_pos);
+    k_ext_decode_pos<<<g, 256, 0, st>>>(comp, wide, pos_bits, n, offsets, n_reads, occ_read, occ_pos);
 }
 
 // ---------------------------------------------------------------------------

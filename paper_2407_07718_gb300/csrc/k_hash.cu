@@ -83,53 +83,22 @@ constexpr size_t hash_smem() {
     return (size_t)C::ENT * ((WIDE ? 16 : 8) + 4) + (size_t)C::RB * ((WIDE ? 32 : 16) + 4 + 2) + ((size_t)2 << C::LS);
 }
 
-// A record's segment of HC_SEG k-mers, in 32-bit words: the bases from the
-// first k-mer on, and their reverse complements shifted so that the first
-// k-mer's is left aligned in r[1..], the bases that later k-mers shift in
-// being in r[0].
+// Segment s (HC_SEG k-mers) of a record of 32-bit words w; s is the same in the
+// whole warp.
 template <bool WIDE>
-struct SegWords {
-    static constexpr int N = WIDE ? 4 : 2;   // words of a key
-    uint32_t f[N + 1], r[N + 1];
-    // words w (2 * RW of them, the record's), segment s, k-mer length k
-    __device__ __forceinline__ void load(uint32_t (&w)[WIDE ? 8 : 4], int s, int k) {
-        constexpr int NW = WIDE ? 8 : 4;
-        const int b0 = HC_SEG * s;  // first base; s is the same in the whole warp
-        for (int q = b0 >> 4; q > 0; --q) {
+__device__ __forceinline__ void segment_start(KmerRoll<WIDE>& S, uint32_t (&w)[WIDE ? 8 : 4], int s, int k) {
+    constexpr int NW = WIDE ? 8 : 4;
+    const int b0 = HC_SEG * s;  // first base
+    for (int q = b0 >> 4; q > 0; --q) {
 #pragma unroll
-            for (int i = 0; i < NW; ++i) w[i] = i + 1 < NW ? w[i + 1] : 0u;
-        }
-        if (b0 & 15) {
-#pragma unroll
-            for (int i = 0; i < NW; ++i) w[i] = __funnelshift_l(i + 1 < NW ? w[i + 1] : 0u, w[i], 2 * (b0 & 15));
-        }
-        // the first 16 (N + 1) bases reversed and complemented; the first k-mer
-        // starts at base 16 (N + 1) - k of them (16 or more: k <= 16 N)
-        uint32_t x[N + 4];
-#pragma unroll
-        for (int i = 0; i <= N; ++i) {
-            f[i] = w[i];
-            x[i] = revcomp32(w[N - i]);
-        }
-        x[N + 1] = x[N + 2] = x[N + 3] = 0;
-        const int o = 2 * (16 * (N + 1) - k);
-        if (o >= 64) {
-#pragma unroll
-            for (int i = 0; i < N + 3; ++i) x[i] = x[i + 1];
-        }
-#pragma unroll
-        for (int i = 0; i <= N; ++i) r[i] = __funnelshift_l(x[i + 1], x[i], o & 31);
+        for (int i = 0; i < NW; ++i) w[i] = i + 1 < NW ? w[i + 1] : 0u;
     }
-    // the next k-mer
-    __device__ __forceinline__ void step() {
+    if (b0 & 15) {
 #pragma unroll
-        for (int i = 0; i < N; ++i) f[i] = __funnelshift_l(f[i + 1], f[i], 2);
-        f[N] <<= 2;
-#pragma unroll
-        for (int i = N; i > 0; --i) r[i] = __funnelshift_r(r[i], r[i - 1], 2);
-        r[0] >>= 2;
+        for (int i = 0; i < NW; ++i) w[i] = __funnelshift_l(i + 1 < NW ? w[i + 1] : 0u, w[i], 2 * (b0 & 15));
     }
-};
+    S.start(w, k);
+}
 
 // Slot (of 2^LS) of a key in round `round`.
 template <int LS>
@@ -325,20 +294,10 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
                         W[4 * y + 3] = v.z;
                     }
                     const int nk = min((int)(W[2 * RW - 1] & 0x7Fu) - HC_SEG * s, HC_SEG);
-                    SegWords<WIDE> S;
-                    S.load(W, s, k);
+                    KmerRoll<WIDE> S;
+                    segment_start<WIDE>(S, W, s, k);
                     for (int j = 0; j < nk; ++j) {
-                        K key;
-                        if constexpr (WIDE) {
-                            const u64 fh = ((u64)S.f[0] << 32) | S.f[1], fl = ((u64)S.f[2] << 32) | S.f[3];
-                            const u64 rh = ((u64)S.r[1] << 32) | S.r[2], rl = ((u64)S.r[3] << 32) | S.r[4];
-                            const bool fwd = fh < rh || (fh == rh && fl < rl);
-                            key.hi = fwd ? fh : rh;
-                            key.lo = (fwd ? fl : rl) & mask;
-                        } else {
-                            const u64 f = ((u64)S.f[0] << 32) | S.f[1], r = ((u64)S.r[1] << 32) | S.r[2];
-                            key = (f < r ? f : r) & mask;
-                        }
+                        const K key = S.left(mask);
                         S.step();
                         const uint32_t own = D + s_ent[HC_SEG * s + j] + q;
                         ek[own] = key;
@@ -434,14 +393,7 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
             const bool keep = cnt && cnt >= P.lo && cnt <= P.hi;
             const uint32_t km = __ballot_sync(0xffffffffu, keep);
             if (keep) {
-                K key = ek[i];
-                if constexpr (WIDE) {
-                    const int sh = 128 - 2 * k;  // 0 .. 62
-                    key.lo = sh ? (key.lo >> sh) | (key.hi << (64 - sh)) : key.lo;
-                    key.hi >>= sh;
-                } else {
-                    key >>= 64 - 2 * k;
-                }
+                const K key = right_aligned(ek[i], k);
                 atomicAdd(&s_dig[key_digit(key, P.dshift, 0xFF)], 1u);
                 const u64 o = at + (uint32_t)__popc(km & ((1u << lane) - 1u));
                 reinterpret_cast<K*>(P.out_keys)[o] = key;

@@ -84,21 +84,6 @@ __device__ __forceinline__ uint32_t mmer_score(const u64* pk, int q, int m, uint
     else return fmix32((uint32_t)c ^ (uint32_t)(c >> 32) ^ seed);
 }
 
-// Bit t (most significant first) = OR of bits [t, t + L) of the 128-bit
-// value a:b, for t = 0..63 and 1 <= L <= 64: OR over windows of doubling
-// width, then two overlapping windows of that width.
-__device__ __forceinline__ u64 window_or64(u64 a, u64 b, int L) {
-    u64 hi = a, lo = b;
-    int width = 1;
-    while (2 * width <= L) {
-        hi |= (hi << width) | (lo >> (64 - width));
-        lo |= lo << width;
-        width *= 2;
-    }
-    const int d = L - width;  // 0 <= d < width
-    return d ? hi | (hi << d) | (lo >> (64 - d)) : hi;
-}
-
 // Bits [2*nb, 64) of word x cleared when the record holds only nb (< 32) more bases.
 __device__ __forceinline__ u64 keep_bases(u64 x, int nb) {
     if (nb >= 32) return x;
