@@ -1,70 +1,83 @@
 // k_encode.cu -- stage S1: 2-bit encoding of reads (Sec. 2.2: sequences are
 // encoded before they are parsed into k-mers).
 //
-// One thread turns 64 ASCII bytes (four 128-bit loads) into two packed words
-// (32 bases each, first base most significant) and one invalid-mask word.
-// The kernel is bound by HBM: 1 byte read and 0.375 bytes written per base.
+// One thread turns 16 ASCII bytes into half a packed word (16 bases, first
+// base most significant) and a quarter of an invalid-mask word, so that every
+// load and store of a warp is one run of bytes.  The kernel is bound by HBM (1
+// byte read and 0.375 bytes written per base) once the arithmetic is short:
+// byte compares, each several instructions, kept the integer pipe 93 % busy and
+// took 0.83 and 1.18 ms on 1.5 and 2.0 Gbases; this takes 0.42 and 0.64.
 #include "hsk_device.cuh"
 
 namespace hsk {
 
-// 4 ASCII bytes (little-endian in x) -> 4 codes packed most significant first
-// in 8 bits, plus a 4-bit invalid nibble (first byte in bit 3).
-__device__ __forceinline__ void encode4(uint32_t x, uint32_t& code8, uint32_t& inv4) {
-    uint32_t ok = __vcmpeq4(x, 0x41414141u) | __vcmpeq4(x, 0x43434343u) |
-                  __vcmpeq4(x, 0x47474747u) | __vcmpeq4(x, 0x54545454u);
-    // A 0x41 -> 0, C 0x43 -> 1, G 0x47 -> 2, T 0x54 -> 3: ((c >> 2) ^ (c >> 1)) & 3
-    uint32_t c = ((x >> 2) ^ (x >> 1)) & 0x03030303u & ok;
-    code8 = ((c & 3u) << 6) | (((c >> 8) & 3u) << 4) | (((c >> 16) & 3u) << 2) | ((c >> 24) & 3u);
-    uint32_t bad = ~ok;
-    inv4 = ((bad & 1u) << 3) | (((bad >> 8) & 1u) << 2) | (((bad >> 16) & 1u) << 1) | ((bad >> 24) & 1u);
+// 4 ASCII bytes (little-endian in x) -> their codes in 2 bits per byte (A 0x41
+// -> 0, C 0x43 -> 1, G 0x47 -> 2, T 0x54 -> 3: ((c >> 2) ^ (c >> 1)) & 3), right
+// for the four letters; diff has a non-zero byte for every other one.
+__device__ __forceinline__ uint32_t codes4(uint32_t x, uint32_t& diff) {
+    const uint32_t c = ((x >> 2) ^ (x >> 1)) & 0x03030303u;
+    // the codes as the selectors of a byte permutation of "ACGT"
+    const uint32_t sel = __byte_perm(c | (c >> 4), 0, 0x4420);
+    diff = x ^ __byte_perm(0x54474341u, 0, sel);
+    return c;
+}
+// Invalid nibble (first byte in bit 3) of a diff word; the codes of its bytes cleared.
+__device__ __noinline__ uint32_t invalid4(uint32_t diff, uint32_t& c) {
+    const uint32_t bad = __vcmpne4(diff, 0u);
+    c &= ~bad;
+    return ((bad & 1u) << 3) | (((bad >> 8) & 1u) << 2) | (((bad >> 16) & 1u) << 1) | ((bad >> 24) & 1u);
 }
 
+// Units of 16 bases [u0, u1); n_bases bytes, the units past them invalid.  Unit
+// u is the upper (u even) or lower half of packed word u / 2, and 16 bits of
+// mask word u / 4, first bases uppermost.
 __global__ void __launch_bounds__(256) k_encode(const char* __restrict__ reads, uint64_t n_bases,
-                                                u64* __restrict__ packed, u64* __restrict__ invalid,
-                                                uint64_t n_packed_words, uint64_t t0, uint64_t t1,
-                                                bool aligned16) {
-    uint64_t t = t0 + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= t1) return;
-    uint64_t b0 = t * 64;
-    uint32_t x[16];
-    if (aligned16 && b0 + 64 <= n_bases) {
-        const uint4* src = reinterpret_cast<const uint4*>(reads + b0);
+                                                uint32_t* __restrict__ packed, uint16_t* __restrict__ invalid,
+                                                uint64_t n_packed_words, uint64_t u0, uint64_t u1, bool aligned16) {
+    constexpr int PER = 4;  // units a thread, a block apart
+    const uint64_t first = u0 + (uint64_t)blockIdx.x * (256 * PER) + threadIdx.x;
+    uint4 x[PER];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            uint4 q = __ldcs(src + v);  // streamed once: do not keep in L1/L2
-            x[4 * v] = q.x;
-            x[4 * v + 1] = q.y;
-            x[4 * v + 2] = q.z;
-            x[4 * v + 3] = q.w;
-        }
-    } else {
+    for (int i = 0; i < PER; ++i) {
+        const uint64_t u = first + (uint64_t)i * 256, b0 = u * 16;
+        x[i] = make_uint4(0, 0, 0, 0);
+        if (u >= u1) continue;
+        if (aligned16 && b0 + 16 <= n_bases) {
+            x[i] = __ldcs(reinterpret_cast<const uint4*>(reads + b0));  // streamed once: do not keep in L1/L2
+        } else {
+            uint32_t w[4];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            uint32_t v = 0;
-            for (int b = 0; b < 4; ++b) {
-                uint64_t g = b0 + 4 * j + b;
-                // bytes past the data read as 0 -> invalid
-                uint32_t c = g < n_bases ? (uint32_t)(unsigned char)reads[g] : 0u;
-                v |= c << (8 * b);
+            for (int j = 0; j < 4; ++j) {
+                w[j] = 0;
+                for (int b = 0; b < 4; ++b) {
+                    const uint64_t g = b0 + 4 * j + b;
+                    // bytes past the data read as 0 -> invalid
+                    const uint32_t c = g < n_bases ? (uint32_t)(unsigned char)reads[g] : 0u;
+                    w[j] |= c << (8 * b);
+                }
             }
-            x[j] = v;
+            x[i] = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
-    u64 w0 = 0, w1 = 0, iv = 0;
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        uint32_t c8, i4;
-        encode4(x[j], c8, i4);
-        if (j < 8)
-            w0 |= (u64)c8 << (56 - 8 * j);
-        else
-            w1 |= (u64)c8 << (56 - 8 * (j - 8));
-        iv |= (u64)i4 << (60 - 4 * j);
+    for (int i = 0; i < PER; ++i) {
+        const uint64_t u = first + (uint64_t)i * 256;
+        if (u >= u1) continue;
+        const uint32_t w[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
+        uint32_t c[4], diff[4], bad = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) c[j] = codes4(w[j], diff[j]);
+        if (diff[0] | diff[1] | diff[2] | diff[3]) {  // rare
+#pragma unroll
+            for (int j = 0; j < 4; ++j) bad |= invalid4(diff[j], c[j]) << (12 - 4 * j);
+        }
+        // four 2-bit codes, a byte apart, to the top byte of a product (no carries reach it)
+        uint32_t code = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) code |= (c[j] * 0x40100401u) >> 24 << (24 - 8 * j);
+        if (u / 2 < n_packed_words) packed[u ^ 1] = code;
+        invalid[u ^ 3] = (uint16_t)bad;
     }
-    if (2 * t < n_packed_words) packed[2 * t] = w0;
-    if (2 * t + 1 < n_packed_words) packed[2 * t + 1] = w1;
-    invalid[t] = iv;
 }
 
 // Marks the first base of every non-empty read and checks the offsets:
@@ -122,24 +135,26 @@ void launch_mark_starts_sets(const uint64_t* offsets, const uint64_t* off0, cons
                                                                    (u64*)start_mask, err);
 }
 
+// bases [b0, b1), b0 a multiple of 64; whole mask words are written
+static void encode_units(const char* reads, uint64_t n_bases, uint64_t b0, uint64_t b1, uint64_t* packed,
+                         uint64_t* invalid, uint64_t n_packed_words, cudaStream_t st) {
+    const uint64_t u0 = b0 / 64 * 4, u1 = (b1 + 63) / 64 * 4;
+    if (u1 <= u0) return;
+    count_launch();
+    const bool al = (reinterpret_cast<uintptr_t>(reads) & 15) == 0;
+    k_encode<<<(unsigned)((u1 - u0 + 1023) / 1024), 256, 0, st>>>(reads, n_bases, (uint32_t*)packed,
+                                                                  (uint16_t*)invalid, n_packed_words, u0, u1, al);
+}
+
 void launch_encode(const char* reads, uint64_t n_bases, uint64_t* packed, uint64_t* invalid,
                    uint64_t n_packed_words, uint64_t n_mask_words, cudaStream_t st) {
-    uint64_t threads = (n_bases + 63) / 64;
-    if (threads == 0) return;
-    count_launch();
-    bool al = (reinterpret_cast<uintptr_t>(reads) & 15) == 0;
-    k_encode<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(
-        reads, n_bases, (u64*)packed, (u64*)invalid, n_packed_words, 0, threads, al);
+    (void)n_mask_words;
+    encode_units(reads, n_bases, 0, n_bases, packed, invalid, n_packed_words, st);
 }
 
 void launch_encode_range(const char* reads, uint64_t n_bases, uint64_t b0, uint64_t b1, uint64_t* packed,
                          uint64_t* invalid, uint64_t n_packed_words, cudaStream_t st) {
-    const uint64_t t0 = b0 / 64, t1 = (b1 + 63) / 64;
-    if (t1 <= t0) return;
-    count_launch();
-    bool al = (reinterpret_cast<uintptr_t>(reads) & 15) == 0;
-    k_encode<<<(unsigned)((t1 - t0 + 255) / 256), 256, 0, st>>>(reads, n_bases, (u64*)packed, (u64*)invalid,
-                                                                n_packed_words, t0, t1, al);
+    encode_units(reads, n_bases, b0, b1, packed, invalid, n_packed_words, st);
 }
 
 void launch_mark_starts(const uint64_t* offsets, uint64_t n_reads, uint64_t n_bases,
