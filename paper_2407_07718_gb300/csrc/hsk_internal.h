@@ -28,7 +28,7 @@ void launch_encode_range(const char* reads, uint64_t n_bases, uint64_t b0, uint6
                          uint64_t* invalid, uint64_t n_packed_words, cudaStream_t st);
 constexpr uint64_t SM_TILE_BASES = 1024;   // windows per S2 warp tile
 constexpr uint64_t SM_TILE_REACH = 1280;   // bases past a tile's start that its walk reads
-constexpr int SM_CTA_WARPS = 8;            // warps per CTA of the walk
+constexpr int SM_CTA_WARPS = 32;           // warps per CTA of the walk at most
 void launch_mark_starts(const uint64_t* offsets, uint64_t n_reads, uint64_t n_bases,
                         uint64_t* start_mask, int* err, cudaStream_t st);
 
@@ -53,6 +53,7 @@ struct SmParams {
     int nmax;                 // k-mers per supermer record at most
     int rec_words;            // 2 (k <= 32) or 4 (k <= 64)
     uint32_t grid;
+    int warps;                // warps per CTA
     uint64_t tile_begin, tile_end;     // warp tiles [begin, end) of 1024 windows (end 0 = all)
     // Fine partitions (part_rec != nullptr): the sub_bits (at most 8) hash bits
     // above the bucket's split every bucket into 2^sub_bits of them; windows of
@@ -83,8 +84,9 @@ struct SmParams {
     int* err;
 };
 
-size_t supermer_smem_bytes(int mode, uint32_t n_buckets);
-int supermer_max_ctas_per_sm(int mode, int m, bool lexical, uint32_t n_buckets);
+// warps per CTA and CTAs for a walk over n_tiles warp tiles
+void supermer_shape(int mode, int m, bool lexical, uint32_t n_buckets, uint64_t n_tiles, int num_sms, int* warps,
+                    uint32_t* grid);
 void launch_supermer(int mode, const SmParams& p, cudaStream_t st);
 // records from descriptors, in bucket order, or with part_cursor in order of
 // fine partitions (their first records; advanced) and in one orientation for

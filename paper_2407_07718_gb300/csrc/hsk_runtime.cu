@@ -438,10 +438,8 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
     }
     const bool fine = sub_bits >= 0;
     const uint64_t F = fine ? (uint64_t)B << sub_bits : 0;
-    const int occ = supermer_max_ctas_per_sm(SM_DESC, m, P.lexical, B);
-    const uint64_t warp_tiles = (E.n_bases + 1023) / 1024;
-    uint64_t g = std::min<uint64_t>((uint64_t)c->num_sms * occ, (warp_tiles + SM_CTA_WARPS - 1) / SM_CTA_WARPS);
-    P.grid = (uint32_t)std::max<uint64_t>(g, 1);
+    supermer_shape(SM_DESC, m, P.lexical, B, (E.n_bases + SM_TILE_BASES - 1) / SM_TILE_BASES, c->num_sms, &P.warps,
+                   &P.grid);
     TRY(hsk_ensure(c, c->bucket_kmers, (uint64_t)B * 8, false));
     TRY(hsk_ensure(c, c->bucket_rec, ((uint64_t)B + 1) * 8, false));
     // records per bucket, then the bucket cursors of the scatter (spread out);
@@ -500,7 +498,7 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
                 if (t_end > t_done) {
                     P.tile_begin = t_done;
                     P.tile_end = t_end;
-                    P.grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(grid, (t_end - t_done + SM_CTA_WARPS - 1) / SM_CTA_WARPS));
+                    P.grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(grid, (t_end - t_done + P.warps - 1) / P.warps));
                     launch_supermer(SM_DESC, P, st);
                     t_done = t_end;
                 }
@@ -1542,8 +1540,8 @@ extern "C" int hsk_stage_windows(hsk_ctx* c, const char* d_reads, const uint64_t
         TRY(hsk_encode_into(c, d_reads, n_bases, d_offsets, n_reads, c->pk, c->iv, c->rs, E, st, false));
         SmParams P;
         fill_sm_params(c, E, k, m, 1, P);
-        uint64_t warp_tiles = (n_bases + 1023) / 1024;
-        P.grid = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)c->num_sms * 4, (warp_tiles + SM_CTA_WARPS - 1) / SM_CTA_WARPS));
+        supermer_shape(SM_DUMP, m, P.lexical, 1, (n_bases + SM_TILE_BASES - 1) / SM_TILE_BASES, c->num_sms, &P.warps,
+                       &P.grid);
         P.dump_valid = d_valid;
         P.dump_key = d_key;
         P.dump_minhash = d_minhash;

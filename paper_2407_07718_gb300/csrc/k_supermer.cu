@@ -21,22 +21,24 @@
 // supermer starts where a bit is set, and ends at the next set bit of the
 // cuts, in this lane or a later one.  Every supermer becomes an 8-byte
 // descriptor (start base, k-mer count, bucket), appended to a global list with
-// one atomic per tile (or one for even and one for odd buckets); per-bucket record and k-mer counts are kept in shared
-// memory.  A second, light kernel scatters records into their buckets from
-// the descriptors.  DUMP mode writes per-window keys and scores for the stage
-// test.
+// one atomic per tile (or two, when S3 takes the buckets in two halves);
+// per-bucket record and k-mer counts are kept in shared memory.  A second, light
+// kernel scatters records into their buckets from the descriptors.  DUMP mode
+// writes per-window keys and scores for the stage test.
 //
-// The kernel is bound by instruction issue.  With 32 windows a lane it takes
-// 3.9 ms on 1.5 G windows of long reads (k = 31, w = 15) and 5.3 ms on 1.27 G
-// of short reads (k = 55, w = 35); one window a lane and step, with the window
-// minima and the cuts found by shuffles and ballots across lanes, took 8.7
-// warp instructions per window and 14.4 and 17.0 ms.
+// The kernel is bound by the integer pipe (ncu: 75 % busy, 67 thread
+// instructions per window).  With 32 windows a lane it takes 3.8 ms on 1.5 G
+// windows of long reads (k = 31, w = 15) and 4.6 ms on 1.27 G of short reads (k
+// = 55, w = 35), with 32 warps a CTA; 8 warps and three CTAs per SM took 4.4 and
+// 5.4 ms (fewer registers allow 32 warps per SM instead of 24, and one table
+// serves them all).  One window a lane and step, with the window minima and the
+// cuts found by shuffles and ballots across lanes, took 8.7 warp instructions
+// per window and 14.4 and 17.0 ms.  Right shifts done by the multiply pipe (12 %
+// busy) made no difference.
 #include "hsk_device.cuh"
 
 namespace hsk {
 
-constexpr int SM_WARPS = SM_CTA_WARPS;
-constexpr int SM_CTAS = 3;                // CTAs per SM (registers, shared memory)
 constexpr int SM_TW = 32 * 32;            // windows per warp tile, 32 per lane
 constexpr int SM_PW = SM_TW / 32 + 6;     // packed words staged per warp (even)
 constexpr int SM_MW = SM_TW / 64 + 4;     // mask words staged per warp (even)
@@ -52,8 +54,8 @@ static_assert(SM_PW * 32 <= (int)SM_TILE_REACH && SM_MW * 64 <= (int)SM_TILE_REA
 // size of the largest table (SM_MAX_BUCKETS buckets), never to its own, so
 // one thread cannot lower it under another's launch.
 constexpr uint32_t SM_MAX_BUCKETS = 8192;
-size_t supermer_smem_bytes(int mode, uint32_t n_buckets) {
-    size_t s = (size_t)SM_WARPS * ((SM_PW + 2 * SM_MW + SM_VW) * sizeof(u64) + SM_ROWS * sizeof(uint32_t));
+size_t supermer_smem_bytes(int mode, uint32_t n_buckets, int warps) {
+    size_t s = (size_t)warps * ((SM_PW + 2 * SM_MW + SM_VW) * sizeof(u64) + SM_ROWS * sizeof(uint32_t));
     if (mode == SM_DESC) s += (size_t)n_buckets * 2 * sizeof(uint32_t);
     return s;
 }
@@ -159,52 +161,59 @@ __device__ __forceinline__ uint32_t row_at(const uint32_t* rows, int lane, int j
 // reverse complements are funnels of the reversed and complemented words,
 // shifted once so that those shifts are constant too.  Codes stay left
 // aligned with the following bases below them: two codes that differ compare
-// by their own bits, and equal ones are the same m-mer.
+// by their own bits, and equal ones are the same m-mer.  For m > 16 the first
+// 16 bases decide: an m-mer and its reverse complement that agree there (base i
+// and base m - 1 - i are complements for every i < 16, and m <= 32) are equal,
+// and the code's low word comes from the words shifted by the other m - 16 bases.
 template <bool SHORT, bool LEX>
 __device__ __forceinline__ void mmer_scores32(u64 W0, u64 W1, int m, uint32_t seed, uint32_t (&a)[32]) {
     u64 R0 = reverse_pairs(~W1), R1 = reverse_pairs(~W0);
-    const uint32_t s = 2 * (33 - m);  // 2 .. 64
-    if (s == 64) {
-        R0 = R1;
-        R1 = 0;
-    } else {
-        R0 = (R0 << s) | (R1 >> (64 - s));
-        R1 <<= s;
-    }
+    auto shift = [](u64& h, u64& l, uint32_t s) {  // s in 0 .. 64
+        if (s == 64) {
+            h = l;
+            l = 0;
+        } else if (s) {
+            h = (h << s) | (l >> (64 - s));
+            l <<= s;
+        }
+    };
+    shift(R0, R1, 2 * (33 - m));
     const uint32_t F[5] = {(uint32_t)(W0 >> 32), (uint32_t)W0, (uint32_t)(W1 >> 32), (uint32_t)W1, 0u};
     const uint32_t C[5] = {(uint32_t)(R0 >> 32), (uint32_t)R0, (uint32_t)(R1 >> 32), (uint32_t)R1, 0u};
-    const uint32_t sh = SHORT ? 32 - 2 * m : 64 - 2 * m;  // < 32
+    if constexpr (SHORT || LEX) {
+        const int sh = SHORT ? 32 - 2 * m : 0;
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        const int fi = j / 16, fs = 2 * (j % 16), ci = (31 - j) / 16, cs = 2 * ((31 - j) % 16);
-        const uint32_t fh = __funnelshift_l(F[fi + 1], F[fi], fs), ch = __funnelshift_l(C[ci + 1], C[ci], cs);
-        if constexpr (SHORT) {
-            const uint32_t c = min(fh, ch) >> sh;
+        for (int j = 0; j < 32; ++j) {
+            const int fi = j / 16, fs = 2 * (j % 16), ci = (31 - j) / 16, cs = 2 * ((31 - j) % 16);
+            const uint32_t c = min(__funnelshift_l(F[fi + 1], F[fi], fs), __funnelshift_l(C[ci + 1], C[ci], cs)) >> sh;
             a[j] = LEX ? c : fmix32(c ^ seed);
-        } else {
-            if constexpr (LEX) {
-                a[j] = min(fh, ch);
-            } else {
-                const uint32_t fl = __funnelshift_l(F[fi + 2], F[fi + 1], fs);
-                const uint32_t cl = __funnelshift_l(C[ci + 2], C[ci + 1], cs);
-                const u64 f = ((u64)fh << 32) | fl, r = ((u64)ch << 32) | cl;
-                const u64 c = f < r ? f : r;
-                const uint32_t h = (uint32_t)(c >> 32), l = (uint32_t)c;
-                a[j] = fmix32(__funnelshift_r(l, h, sh) ^ (h >> sh) ^ seed);
-            }
+        }
+    } else {
+        shift(W0, W1, 2 * (m - 16));
+        shift(R0, R1, 2 * (m - 16));
+        const uint32_t G[5] = {(uint32_t)(W0 >> 32), (uint32_t)W0, (uint32_t)(W1 >> 32), (uint32_t)W1, 0u};
+        const uint32_t E[5] = {(uint32_t)(R0 >> 32), (uint32_t)R0, (uint32_t)(R1 >> 32), (uint32_t)R1, 0u};
+        const int sh = 64 - 2 * m;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+            const int fi = j / 16, fs = 2 * (j % 16), ci = (31 - j) / 16, cs = 2 * ((31 - j) % 16);
+            const uint32_t fh = __funnelshift_l(F[fi + 1], F[fi], fs), ch = __funnelshift_l(C[ci + 1], C[ci], cs);
+            const uint32_t fl = __funnelshift_l(G[fi + 1], G[fi], fs), cl = __funnelshift_l(E[ci + 1], E[ci], cs);
+            a[j] = fmix32((fh < ch ? fl : cl) ^ (min(fh, ch) >> sh) ^ seed);
         }
     }
 }
 
 template <int MODE, bool SHORT, bool LEX, bool TWO_ENDED>
-__global__ void __launch_bounds__(SM_WARPS * 32, SM_CTAS) k_supermer(const __grid_constant__ SmParams P) {
+__global__ void __launch_bounds__(SM_CTA_WARPS * 32, 1) k_supermer(const __grid_constant__ SmParams P) {
     extern __shared__ __align__(16) unsigned char smem[];
     u64* s_pk = reinterpret_cast<u64*>(smem);
-    u64* s_iv = s_pk + SM_WARPS * SM_PW;
-    u64* s_rs = s_iv + SM_WARPS * SM_MW;
-    u64* s_val = s_rs + SM_WARPS * SM_MW;
-    uint32_t* s_rows = reinterpret_cast<uint32_t*>(s_val + SM_WARPS * SM_VW);
-    uint32_t* s_cnt = s_rows + SM_WARPS * SM_ROWS;  // DESC
+    const int warps = blockDim.x >> 5;
+    u64* s_iv = s_pk + warps * SM_PW;
+    u64* s_rs = s_iv + warps * SM_MW;
+    u64* s_val = s_rs + warps * SM_MW;
+    uint32_t* s_rows = reinterpret_cast<uint32_t*>(s_val + warps * SM_VW);
+    uint32_t* s_cnt = s_rows + warps * SM_ROWS;  // DESC
     uint32_t* s_km = s_cnt + P.n_buckets;           // DESC
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -223,7 +232,7 @@ __global__ void __launch_bounds__(SM_WARPS * 32, SM_CTAS) k_supermer(const __gri
     uint32_t* rows = s_rows + warp * SM_ROWS;
     const u64 n_tiles = P.tile_end ? P.tile_end : (P.n_bases + SM_TW - 1) / SM_TW;
 
-    for (u64 t = P.tile_begin + (u64)blockIdx.x * SM_WARPS + warp; t < n_tiles; t += (u64)gridDim.x * SM_WARPS) {
+    for (u64 t = P.tile_begin + (u64)blockIdx.x * warps + warp; t < n_tiles; t += (u64)gridDim.x * warps) {
         const u64 p0 = t * SM_TW;
         // buckets of the tile's set (packed sets: the set holding tile t)
         uint32_t bbase = 0, bmask = B - 1u;
@@ -414,22 +423,33 @@ static SmKernel walk_kernel(int mode, int m, bool lexical, bool two_ended) {
     SmKernel fn = mode != SM_DESC ? walk_kernel<SM_DUMP, false>(m, lexical)
                   : two_ended     ? walk_kernel<SM_DESC, true>(m, lexical)
                                   : walk_kernel<SM_DESC, false>(m, lexical);
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)supermer_smem_bytes(mode, SM_MAX_BUCKETS));
+    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)supermer_smem_bytes(mode, SM_MAX_BUCKETS, SM_CTA_WARPS));
     return fn;
 }
 
 void launch_supermer(int mode, const SmParams& p, cudaStream_t st) {
     if (p.n_bases == 0) return;
     count_launch();
-    walk_kernel(mode, p.m, p.lexical, p.two_ended)<<<p.grid, SM_WARPS * 32, supermer_smem_bytes(mode, p.n_buckets), st>>>(p);
+    walk_kernel(mode, p.m, p.lexical, p.two_ended)<<<p.grid, p.warps * 32, supermer_smem_bytes(mode, p.n_buckets, p.warps), st>>>(p);
 }
 
-int supermer_max_ctas_per_sm(int mode, int m, bool lexical, uint32_t n_buckets) {
+// As many warps a CTA as leave every SM one (at most SM_CTA_WARPS, at least 4):
+// the CTA's table of bucket counters, and adding it up at the end, is shared by
+// its warps.  One CTA of 16, 20, 24 and 32 warps per SM took 4.2, 3.9, 3.8 and 3.8
+// ms on the long reads, 5.1, 4.9, 4.8 and 4.7 ms on the short ones; on 300 K
+// windows all of them take the same.
+void supermer_shape(int mode, int m, bool lexical, uint32_t n_buckets, uint64_t n_tiles, int num_sms, int* warps,
+                    uint32_t* grid) {
+    const uint64_t per_sm = (n_tiles + num_sms - 1) / num_sms;
+    *warps = (int)(per_sm < 4 ? 4 : per_sm > SM_CTA_WARPS ? SM_CTA_WARPS : per_sm);
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel(mode, m, lexical, false), SM_WARPS * 32,
-                                                      supermer_smem_bytes(mode, n_buckets)) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel(mode, m, lexical, false), *warps * 32,
+                                                      supermer_smem_bytes(mode, n_buckets, *warps)) != cudaSuccess)
         n = 1;
-    return n > 0 ? n : 1;
+    if (n < 1) n = 1;
+    const uint64_t want = (n_tiles + *warps - 1) / *warps, most = (uint64_t)num_sms * n;
+    *grid = (uint32_t)(want < 1 ? 1 : want < most ? want : most);
 }
 
 // A record's nb bases (left aligned, the rest 0) or their reverse complement,
