@@ -20,6 +20,16 @@ namespace hsk {
 // Kernels launched by this library (all launch_* wrappers add to it).
 void count_launch(unsigned n = 1);
 
+// Small regions zeroed by one launch, where a memset each would cost a launch
+// each (words of 4 bytes).
+constexpr int ZERO_MAX = 8;
+struct ZeroList {
+    void* p[ZERO_MAX];
+    uint64_t words[ZERO_MAX];
+    int n = 0;
+};
+void launch_zero(const ZeroList& L, cudaStream_t st);
+
 // ---- S1 encode ----------------------------------------------------------
 void launch_encode(const char* reads, uint64_t n_bases, uint64_t* packed, uint64_t* invalid,
                    uint64_t n_packed_words, uint64_t n_mask_words, cudaStream_t st);
@@ -204,16 +214,16 @@ constexpr int HASH_MAX_SUB_BITS = 8;             // fine partitions of a bucket:
 constexpr uint64_t HASH_MAX_BASES = 1ull << 36;  // bases a descriptor with a sub-partition can address
 uint32_t hash_count_cap(int key_words);      // distinct k-mers the first tier's table holds
 // Counts partitions (all of them, or the n_part listed in `only`): kept pairs
-// to places out_base[0] .. out_base[1] of (out_keys, out_counts) in no
-// particular order, out_n[0] of them; partitions that overfill the tier's
+// to places 0 .. out_cap of (out_keys, out_counts) in no particular order,
+// out_n[0] of them; partitions that overfill the tier's
 // batch listed in ov_list, ov_stats = {listed, their records}; dig_hist[256]
 // += kept pairs per top digit.  bucket_set (packed passes): the set of every
-// bucket of 2^sub_bits partitions, with out_base, out_n, dig_hist and the
-// statistics per set.
+// bucket of 2^sub_bits partitions, with places out_base[s] .. out_base[s + 1],
+// out_n, dig_hist and the statistics per set.
 void launch_hash_count(const uint64_t* records, const uint64_t* part_off, const uint32_t* only, uint32_t n_part,
                        int tier, int k, int nmax, uint32_t lo, uint32_t hi, void* out_keys, uint32_t* out_counts,
-                       const uint32_t* bucket_set, int sub_bits, const uint64_t* out_base, uint64_t* out_n,
-                       uint32_t* ov_list, uint64_t* ov_stats, uint64_t* hist, uint32_t hist_len, uint32_t* max_count,
+                       const uint32_t* bucket_set, int sub_bits, const uint64_t* out_base, uint64_t out_cap,
+                       uint64_t* out_n, uint32_t* ov_list, uint64_t* ov_stats, uint64_t* hist, uint32_t hist_len, uint32_t* max_count,
                        uint64_t* n_distinct, uint64_t* dig_hist, uint32_t* claim, int* err, int num_sms,
                        cudaStream_t st);
 // sets' pairs from src_off[s] on -> dst_off[s] .. dst_off[s + 1] (n in all)

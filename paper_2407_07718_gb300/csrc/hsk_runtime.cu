@@ -93,6 +93,32 @@ int hsk_ensure(hsk_ctx* c, DevBuf& b, size_t bytes, bool zero_new) {
     return HSK_OK;
 }
 
+// Host room of at least `words` words behind the error words
+// (hsk_read_device_error).  Asked for more than it ever held it moves, so no copy
+// into it is under way then; it stays where it is for ROOM_MIN words or fewer.
+constexpr size_t ROOM_ERR = 8, ROOM_MIN = 32768;
+uint64_t* hsk_host_room(hsk_ctx* c, size_t words) {
+    c->h_room.resize(std::max(words + ROOM_ERR, ROOM_MIN));
+    return c->h_room.data() + ROOM_ERR;
+}
+
+// Zero-fills regions (of whole 4-byte words): the small ones in one launch, larger ones by memset.
+int hsk_zero(hsk_ctx* c, cudaStream_t st, std::initializer_list<std::pair<void*, size_t>> regions) {
+    ZeroList L;
+    for (const auto& r : regions) {
+        if (r.second == 0) continue;
+        if (r.second > (1u << 20) || L.n == ZERO_MAX) {
+            CK(cudaMemsetAsync(r.first, 0, r.second, st));
+        } else {
+            L.p[L.n] = r.first;
+            L.words[L.n++] = r.second / 4;
+        }
+    }
+    launch_zero(L, st);
+    CK(cudaGetLastError());
+    return HSK_OK;
+}
+
 static void free_buf(hsk_ctx* c, DevBuf& b) {
     if (b.p) {
         cudaFree(b.p);
@@ -186,6 +212,7 @@ extern "C" int hsk_create(hsk_ctx** out, const hsk_config* cfg_in) {
             c->cfg.tune_cache = nullptr;  // the caller's string is not kept
             hsk_tune_load(c);
         }
+        c->h_room.pinned = true;
         c->host_res.set_pinned(true);  // hsk_count's results: reused from call to call
         c->allocated = HSK_SMALL_BYTES;
         char* s = (char*)c->small;
@@ -222,7 +249,6 @@ extern "C" void hsk_destroy(hsk_ctx* c) {
     }
     for (int i = 0; i < HSK_MAX_PIPE; ++i)
         if (c->pipe_ev[i]) cudaEventDestroy(c->pipe_ev[i]);
-    if (c->h_pin) cudaFreeHost(c->h_pin);
     delete c;
 }
 
@@ -342,8 +368,8 @@ static int check_args(hsk_ctx* c, const void* reads, const void* offsets, uint64
 // Reads the device error word (and the largest count, stored 8 bytes after it)
 // once the stream's work is done.
 int hsk_read_device_error(hsk_ctx* c, cudaStream_t st, uint32_t* max_count) {
-    uint32_t w[3] = {0, 0, 0};
-    CK(cudaMemcpyAsync(w, c->d_err, sizeof(w), cudaMemcpyDeviceToHost, st));
+    uint32_t* w = reinterpret_cast<uint32_t*>(hsk_host_room(c, 0) - ROOM_ERR);
+    CK(cudaMemcpyAsync(w, c->d_err, 12, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     const int derr = (int)w[0];
     if (max_count) *max_count = w[2];
@@ -374,9 +400,7 @@ int hsk_encode_into(hsk_ctx* c, const char* d_reads, uint64_t n_bases, const uin
     TRY(hsk_ensure(c, pk, (E.n_pw + 8) * 8, false));
     TRY(hsk_ensure(c, iv, (E.n_mw + 8) * 8, false));
     TRY(hsk_ensure(c, rs, (E.n_mw + 8) * 8, false));
-    CK(cudaMemsetAsync((uint64_t*)pk.p + E.n_pw, 0, 8 * 8, st));
-    CK(cudaMemsetAsync((uint64_t*)iv.p + E.n_mw, 0, 8 * 8, st));
-    CK(cudaMemsetAsync(rs.p, 0, (E.n_mw + 8) * 8, st));
+    TRY(hsk_zero(c, st, {{(uint64_t*)pk.p + E.n_pw, 64}, {(uint64_t*)iv.p + E.n_mw, 64}, {rs.p, (E.n_mw + 8) * 8}}));
     launch_mark_starts(d_offsets, n_reads, n_bases, (uint64_t*)rs.p, c->d_err, st);
     // with defer_bases the bases are encoded chunk by chunk as they arrive (hsk_supermers)
     if (!defer_bases) launch_encode(d_reads, n_bases, (uint64_t*)pk.p, (uint64_t*)iv.p, E.n_pw, E.n_mw, st);
@@ -467,10 +491,7 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
     S.h_bucket_rec.resize((size_t)B + 1);
     for (int attempt = 0; attempt < 2; ++attempt) {
         TRY(hsk_ensure(c, c->cta_off, cap * 8, false));
-        CK(cudaMemsetAsync(c->bucket_kmers.p, 0, (size_t)B * 8, st));
-        if (fine) CK(cudaMemsetAsync(d_rec_cnt, 0, F * 4, st));
-        else CK(cudaMemsetAsync(d_rec_cnt, 0, cnt_bytes, st));
-        CK(cudaMemsetAsync(c->d_ndesc, 0, 16, st));
+        TRY(hsk_zero(c, st, {{c->bucket_kmers.p, (size_t)B * 8}, {d_rec_cnt, fine ? F * 4 : cnt_bytes}, {c->d_ndesc, 16}}));
         P.desc = (uint64_t*)c->cta_off.p;
         P.desc_cap = cap;
         P.desc_count = (unsigned long long*)c->d_ndesc;
@@ -521,10 +542,14 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
             launch_scan_u32(d_rec_cnt, B, (uint64_t*)c->bucket_rec.p, (uint64_t*)c->lb_status.p, ctr, ep, c->d_err, st);
         CK(cudaGetLastError());
         // bucket statistics to the host (needed to size records and plan chunks)
-        CK(cudaMemcpyAsync(n_end, c->d_ndesc, 16, cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(S.h_bucket_kmers.data(), c->bucket_kmers.p, (size_t)B * 8, cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(S.h_bucket_rec.data(), c->bucket_rec.p, ((size_t)B + 1) * 8, cudaMemcpyDeviceToHost, st));
+        uint64_t* room = hsk_host_room(c, 2 + 2 * (size_t)B + 1);
+        CK(cudaMemcpyAsync(room, c->d_ndesc, 16, cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(room + 2, c->bucket_kmers.p, (size_t)B * 8, cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(room + 2 + B, c->bucket_rec.p, ((size_t)B + 1) * 8, cudaMemcpyDeviceToHost, st));
         TRY(hsk_read_device_error(c, st));
+        memcpy(n_end, room, 16);
+        memcpy(S.h_bucket_kmers.data(), room + 2, (size_t)B * 8);
+        memcpy(S.h_bucket_rec.data(), room + 2 + B, ((size_t)B + 1) * 8);
         n_desc = n_end[0] + n_end[1];
         if (n_desc <= cap) break;
         cap = n_desc;  // the walk counted every supermer: one more run fits them all
@@ -720,38 +745,36 @@ int hsk_order_pairs(hsk_ctx* c, void* keys, uint32_t* counts, uint64_t n, int ke
 int hsk_top_digit_pass(hsk_ctx* c, const void* keys, const uint32_t* counts, uint32_t S, const uint64_t* seg,
                        const uint64_t* hist, int kw, int key_bits, cudaStream_t st) {
     const uint64_t TILE = split_tile_keys(kw);
-    std::vector<uint64_t>& hb = c->s6_h;
-    hb.resize((size_t)S * 256 + 1);
-    std::vector<uint64_t> up(S + 1 + (S + 2) / 2);  // segments, then their first tiles
-    uint32_t* ts = reinterpret_cast<uint32_t*>(up.data() + S + 1);
+    // range starts | the same (the pass's cursors) | segments | their first tiles
+    const size_t R = (size_t)S * 256 + 1;
+    std::vector<uint64_t> up(2 * R + S + 1 + (S + 2) / 2);
+    uint64_t* h_seg = up.data() + 2 * R;
+    uint32_t* ts = reinterpret_cast<uint32_t*>(h_seg + S + 1);
     uint64_t tiles = 0;
     for (uint32_t i = 0; i < S; ++i) {
-        up[i] = seg[i];
+        h_seg[i] = seg[i];
         ts[i] = (uint32_t)tiles;
         tiles += (seg[i + 1] - seg[i] + TILE - 1) / TILE;
         uint64_t at = seg[i];
         for (int d = 0; d < 256; ++d) {
-            hb[(size_t)i * 256 + d] = at;
+            up[(size_t)i * 256 + d] = at;
             at += hist[(size_t)i * 256 + d];
         }
     }
-    up[S] = seg[S];
+    h_seg[S] = up[R - 1] = seg[S];
     ts[S] = (uint32_t)tiles;
-    hb[(size_t)S * 256] = seg[S];
+    memcpy(up.data() + R, up.data(), R * 8);
+    c->s6_h.assign(up.begin(), up.begin() + R);
     if (tiles >= 0xFFFFFFFFull) {
         hsk_set_error(c, "%llu sort tiles", (unsigned long long)tiles);
         return HSK_EOVERFLOW;
     }
-    TRY(hsk_ensure(c, c->s6_bounds, hb.size() * 8, false));
-    TRY(hsk_ensure(c, c->digit_off, hb.size() * 8, false));  // the pass's cursors
-    TRY(hsk_ensure(c, c->seg, up.size() * 8, false));
-    CK(cudaMemcpyAsync(c->s6_bounds.p, hb.data(), hb.size() * 8, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(c->seg.p, up.data(), up.size() * 8, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(c->digit_off.p, hb.data(), hb.size() * 8, cudaMemcpyHostToDevice, st));
-    const uint64_t* d_seg = (const uint64_t*)c->seg.p;
-    launch_split_pairs(keys, counts, c->out_keys.p, (uint32_t*)c->out_counts.p, d_seg, S,
-                       (const uint32_t*)(d_seg + S + 1), (uint32_t)tiles, kw, key_bits - 8,
-                       (uint64_t*)c->digit_off.p, c->d_err, st);
+    TRY(hsk_ensure(c, c->s6_bounds, up.size() * 8, false));
+    uint64_t* d_up = (uint64_t*)c->s6_bounds.p;
+    CK(cudaMemcpyAsync(d_up, up.data(), up.size() * 8, cudaMemcpyHostToDevice, st));
+    launch_split_pairs(keys, counts, c->out_keys.p, (uint32_t*)c->out_counts.p, d_up + 2 * R, S,
+                       (const uint32_t*)(d_up + 2 * R + S + 1), (uint32_t)tiles, kw, key_bits - 8, d_up + R, c->d_err,
+                       st);
     CK(cudaGetLastError());
     return HSK_OK;
 }
@@ -1126,19 +1149,21 @@ int hsk_hash_tiers(hsk_ctx* c, const uint64_t* recs, const uint64_t* part_off, u
     R.S = S;
     R.h.resize(words);
     CK(cudaMemsetAsync(ctl, 0, words * 8, st));
-    CK(cudaMemcpyAsync(d_base, out_base, ((size_t)S + 1) * 8, cudaMemcpyHostToDevice, st));
+    if (bucket_set) CK(cudaMemcpyAsync(d_base, out_base, ((size_t)S + 1) * 8, cudaMemcpyHostToDevice, st));
+    uint64_t* room = hsk_host_room(c, words);
     for (int tier = 0; tier < 2; ++tier) {
         const uint32_t n = tier ? (uint32_t)R.h[0] : n_part;
         if (n == 0) break;
         uint32_t* ctr;
         TRY(hsk_next_counter(c, st, &ctr));
         launch_hash_count(recs, part_off, tier ? list1 : nullptr, n, tier, k, SM.nmax, lo, hi, c->keys.p,
-                          (uint32_t*)c->alt.p, bucket_set, SM.sub_bits, d_base, ctl + 4, tier ? R.list : list1,
+                          (uint32_t*)c->alt.p, bucket_set, SM.sub_bits, d_base, out_base[1], ctl + 4, tier ? R.list : list1,
                           ctl + 2 * tier, (uint64_t*)c->hist.p, H, d_max, ctl + 4 + S, ctl + 4 + 2 * (size_t)S, ctr,
                           c->d_err, c->num_sms, st);
         CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(R.h.data(), ctl, words * 8, cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(room, ctl, words * 8, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
+        memcpy(R.h.data(), room, words * 8);
     }
     R.n_left = (uint32_t)R.h[2];
     return HSK_OK;
@@ -1228,9 +1253,8 @@ int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, ui
     const uint32_t H = c->cfg.hist_len;
     TRY(hsk_ensure(c, c->hist, (size_t)H * 8, false));
     CK(cudaEventRecord(c->ev0, st));
-    CK(cudaMemsetAsync(c->hist.p, 0, (size_t)H * 8, st));
-    CK(cudaMemsetAsync(c->small, 0, 64, st));  // err, max, n_heads, n_out
-    CK(cudaMemsetAsync(c->counters, 0, HSK_N_COUNTERS * sizeof(uint32_t), st));
+    // histogram; err, max, n_heads, n_out; tile counters
+    TRY(hsk_zero(c, st, {{c->hist.p, (size_t)H * 8}, {c->small, 64}, {c->counters, HSK_N_COUNTERS * sizeof(uint32_t)}}));
     c->ctr_used = 0;
     c->marks.clear();
     prof_mark(c, st, -1);

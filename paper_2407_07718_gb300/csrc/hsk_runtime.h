@@ -5,6 +5,7 @@
 #include <condition_variable>
 #include <cstdint>
 #include <deque>
+#include <initializer_list>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -321,8 +322,9 @@ struct hsk_ctx {
     std::vector<std::pair<std::string, Tune>> tuned;  // (class key, parameters)
     bool tuning = false;                 // hsk_autotune is running its trials
 
-    void* h_pin = nullptr;
-    size_t h_pin_cap = 0;
+    // host room for the small copies from the device inside a call (page-locked:
+    // such a copy into pageable memory waits for itself); see hsk_host_room
+    HostArr<uint64_t> h_room;
 
     HostPool result_pool;                // host blocks of batched and served results (outlives them)
     HostResult host_res;                 // result of the last hsk_count
@@ -410,6 +412,8 @@ int hsk_guarded(hsk_ctx* c, F&& body) {
     }
 }
 int hsk_ensure(hsk_ctx* c, DevBuf& b, size_t bytes, bool zero_new);
+uint64_t* hsk_host_room(hsk_ctx* c, size_t words);
+int hsk_zero(hsk_ctx* c, cudaStream_t st, std::initializer_list<std::pair<void*, size_t>> regions);
 int hsk_ensure_status(hsk_ctx* c, uint64_t words, cudaStream_t st);
 int hsk_next_epoch(hsk_ctx* c, cudaStream_t st, uint32_t* epoch);
 int hsk_next_counter(hsk_ctx* c, cudaStream_t st, uint32_t** ctr);

@@ -123,6 +123,22 @@ __global__ void k_mark_starts_sets(const uint64_t* __restrict__ offsets, const u
     }
 }
 
+// Zero-fills up to ZERO_MAX regions in one launch (block row y: region y).
+__global__ void __launch_bounds__(256) k_zero(const __grid_constant__ ZeroList L) {
+    uint32_t* p = (uint32_t*)L.p[blockIdx.y];
+    const uint64_t n = L.words[blockIdx.y];
+    for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256) p[i] = 0;
+}
+
+void launch_zero(const ZeroList& L, cudaStream_t st) {
+    if (L.n == 0) return;
+    uint64_t most = 0;
+    for (int i = 0; i < L.n; ++i) most = L.words[i] > most ? L.words[i] : most;
+    count_launch();
+    const uint64_t bx = (most + 1023) / 1024;
+    k_zero<<<dim3((unsigned)(bx < 1 ? 1 : bx > 256 ? 256 : bx), (unsigned)L.n), 256, 0, st>>>(L);
+}
+
 void launch_mark_starts_sets(const uint64_t* offsets, const uint64_t* off0, const uint64_t* n_reads,
                              const uint64_t* base, uint32_t n_sets, uint64_t max_reads, char* reads,
                              uint64_t* start_mask, int* err, cudaStream_t st) {

@@ -124,12 +124,13 @@ struct HashArgs {
     uint32_t* out_counts;
     // Sets (packed passes): bucket b belongs to set bucket_set[b] (nullptr: one
     // set); partition p to bucket p >> sub_bits.  Set s's kept pairs go to
-    // places out_base[s] .. out_base[s + 1], out_n[s] of them, and its
-    // statistics to hist + s * hist_len, max_count[s], n_distinct[s] and
-    // dig_hist + s * 256.
+    // places out_base[s] .. out_base[s + 1] (one set: 0 .. out_cap), out_n[s] of
+    // them, and its statistics to hist + s * hist_len, max_count[s],
+    // n_distinct[s] and dig_hist + s * 256.
     const uint32_t* bucket_set;
     int sub_bits;
     const u64* out_base;
+    u64 out_cap;
     unsigned long long* out_n;  // kept pairs
     uint32_t* ov_list;
     unsigned long long* ov_stats;  // {partitions listed, their records}
@@ -177,7 +178,11 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
     u64 my_distinct = 0;
     uint32_t my_max = 0, my_ones = 0;
     uint32_t set = 0;  // the set whose statistics are held here
-    u64 out0 = P.out_base[0], out1 = P.out_base[1];
+    u64 out0 = 0, out1 = P.out_cap;
+    if (P.bucket_set) {
+        out0 = P.out_base[0];
+        out1 = P.out_base[1];
+    }
     u64* hist = P.hist;
 
     // Records [r0, r0 + nr) into shared memory, equal ones merged (most of
@@ -553,8 +558,8 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
 
 void launch_hash_count(const uint64_t* records, const uint64_t* part_off, const uint32_t* only, uint32_t n_part,
                        int tier, int k, int nmax, uint32_t lo, uint32_t hi, void* out_keys, uint32_t* out_counts,
-                       const uint32_t* bucket_set, int sub_bits, const uint64_t* out_base, uint64_t* out_n,
-                       uint32_t* ov_list, uint64_t* ov_stats, uint64_t* hist, uint32_t hist_len, uint32_t* max_count,
+                       const uint32_t* bucket_set, int sub_bits, const uint64_t* out_base, uint64_t out_cap,
+                       uint64_t* out_n, uint32_t* ov_list, uint64_t* ov_stats, uint64_t* hist, uint32_t hist_len, uint32_t* max_count,
                        uint64_t* n_distinct, uint64_t* dig_hist, uint32_t* claim, int* err, int num_sms,
                        cudaStream_t st) {
     if (n_part == 0) return;
@@ -574,6 +579,7 @@ void launch_hash_count(const uint64_t* records, const uint64_t* part_off, const 
     P.bucket_set = bucket_set;
     P.sub_bits = sub_bits;
     P.out_base = (const u64*)out_base;
+    P.out_cap = out_cap;
     P.out_n = (unsigned long long*)out_n;
     P.ov_list = ov_list;
     P.ov_stats = (unsigned long long*)ov_stats;
