@@ -24,7 +24,7 @@
 // What it replaces and measured (one GB300): writing every key to its (group,
 // top digit) sub-segment and sorting the sub-segments on chip (k_local.cu)
 // took 39 ms on 1.5 G windows of 30x long reads (k = 31) and 45 ms on 1.27 G
-// of 20x short reads (k = 55); this takes 4.9 and 13.0 ms.
+// of 20x short reads (k = 55); this takes 4.7 and 11.9 ms.
 #include "hsk_device.cuh"
 
 namespace hsk {
@@ -46,13 +46,16 @@ namespace hsk {
 // its phases (about half the issue slots used); an open-addressing table with
 // compare-and-swap took three times the instructions, as the lanes of a warp
 // wait for its longest probe sequence: 10.2 and 26.8 ms on the two workloads
-// above (four tags read at once 10.2 and 27.7), against 4.9 and 13.0.
+// above (four tags read at once 10.2 and 27.7), against 4.9 and 13.0.  Visiting
+// only the kept entries when the pairs are written (one in nine of the short
+// reads') took that to 4.7 and 11.9.
 //
 // Sizes, by trial.  64-bit keys, on the long reads and on 8x short reads of a
 // 20 Mbp genome: 384 threads x 3 CTAs and 3072 entries 5.1 and 0.74 ms, 512 x
 // 2 and 4096 5.8 and 0.92, 256 x 4 and 2304 5.5 and 0.77.  128-bit keys, on
 // the short reads: 512 x 2 and 3840 entries 12.9 ms, 3584 13.3, 1024 x 1 and
-// 7680 14.1.
+// 7680 14.1.  With the kept entries listed (emit): 3840 12.1 ms, 4032 (what two
+// CTAs can hold) 11.9; 64-bit keys 3072 4.72, 3200 4.76.
 template <bool WIDE, int TIER>
 struct HashCfg;
 template <>
@@ -65,7 +68,7 @@ struct HashCfg<false, 1> {
 };
 template <>
 struct HashCfg<true, 0> {
-    static constexpr int NT = 512, CTAS = 2, ENT = 3840, LS = 13, RB = 384;
+    static constexpr int NT = 512, CTAS = 2, ENT = 4032, LS = 13, RB = 384;
 };
 template <>
 struct HashCfg<true, 1> {
@@ -165,7 +168,7 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
     __shared__ uint32_t s_bin[128], s_base[128], s_ent[128];
     __shared__ uint32_t s_hist[HC_HS], s_dig[256], s_wk[NW];
     __shared__ u64 s_off[HC_CHUNK + 1], s_obase;
-    __shared__ uint32_t s_claim, s_U, s_nl[2];
+    __shared__ uint32_t s_claim, s_U, s_nl[2], s_kept;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t hs = P.hist_len < (uint32_t)HC_HS ? P.hist_len : (uint32_t)HC_HS;
     const int k = P.k;
@@ -175,8 +178,8 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
     for (int i = tid; i < 256; i += NT) s_dig[i] = 0;
     if (tid < 128) s_bin[tid] = 0;
     if (tid < 2) s_nl[tid] = 0;
-    u64 my_distinct = 0;
-    uint32_t my_max = 0, my_ones = 0;
+    uint32_t my_max = 0, my_ones = 0, my_more = 0;  // largest count; k-mers seen once, more often
+    if (tid == 0) s_kept = 0;
     uint32_t set = 0;  // the set whose statistics are held here
     u64 out0 = 0, out1 = P.out_cap;
     if (P.bucket_set) {
@@ -355,56 +358,51 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
         if (tid < 2) s_nl[tid] = 0;  // read next after later barriers
     };
 
-    // Statistics, filter and kept pairs of the U merged entries (count 0: merged into another).
+    // Statistics, filter and kept pairs of the U merged entries (count 0:
+    // merged into another).  The kept ones are listed, so that only they are
+    // visited again.
     auto emit = [&](uint32_t U) {
-        uint32_t kept = 0;
-        for (uint32_t i = tid; i < U; i += NT) {
-            const uint32_t cnt = ec[i];
-            if (!cnt) continue;
-            ++my_distinct;
-            if (cnt == 1) {
-                ++my_ones;
-            } else {
-                const uint32_t b = cnt < P.hist_len - 1 ? cnt : P.hist_len - 1;
-                if (b < hs) atomicAdd(&s_hist[b], 1u);
-                else atomicAdd(reinterpret_cast<unsigned long long*>(hist + b), 1ULL);
-            }
-            my_max = cnt > my_max ? cnt : my_max;
-            kept += (cnt >= P.lo && cnt <= P.hi) ? 1u : 0u;
-        }
-        kept = __reduce_add_sync(0xffffffffu, kept);
-        if (lane == 0) s_wk[warp] = kept;
-        __syncthreads();
-        if (warp == 0) {
-            const uint32_t v = lane < NW ? s_wk[lane] : 0u;
-            const uint32_t inc = warp_incl_sum<uint32_t>(v);
-            if (lane < NW) s_wk[lane] = inc - v;
-            const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
-            if (lane == 0) {
-                u64 at = out0 + (total ? atomicAdd(P.out_n + set, (unsigned long long)total) : 0ULL);
-                if (at + total > out1) {
-                    raise_error(P.err, HSK_DERR_BOUNDS);
-                    at = ~0ULL;
-                }
-                s_obase = total ? at : ~0ULL;
-            }
-        }
-        __syncthreads();
-        if (s_obase == ~0ULL) return;  // nothing kept
-        u64 at = s_obase + s_wk[warp];
         for (uint32_t i0 = 0; i0 < U; i0 += NT) {
             const uint32_t i = i0 + tid;
             const uint32_t cnt = i < U ? ec[i] : 0u;
+            if (cnt > 1) {
+                const uint32_t b = cnt < P.hist_len - 1 ? cnt : P.hist_len - 1;
+                if (b < hs) atomicAdd(&s_hist[b], 1u);
+                else atomicAdd(reinterpret_cast<unsigned long long*>(hist + b), 1ULL);
+                ++my_more;
+            }
+            my_ones += cnt == 1 ? 1u : 0u;
+            my_max = cnt > my_max ? cnt : my_max;
             const bool keep = cnt && cnt >= P.lo && cnt <= P.hi;
             const uint32_t km = __ballot_sync(0xffffffffu, keep);
-            if (keep) {
-                const K key = right_aligned(ek[i], k);
-                atomicAdd(&s_dig[key_digit(key, P.dshift, 0xFF)], 1u);
-                const u64 o = at + (uint32_t)__popc(km & ((1u << lane) - 1u));
-                reinterpret_cast<K*>(P.out_keys)[o] = key;
-                P.out_counts[o] = cnt;
+            if (km) {
+                uint32_t at = 0;
+                if (lane == 0) at = atomicAdd(&s_kept, (uint32_t)__popc(km));
+                at = __shfl_sync(0xffffffffu, at, 0);
+                if (keep) s_list[at + (uint32_t)__popc(km & ((1u << lane) - 1u))] = (uint16_t)i;
             }
-            at += (uint32_t)__popc(km);
+        }
+        __syncthreads();
+        const uint32_t kept = s_kept;
+        if (kept == 0) return;
+        if (tid == 0) {
+            u64 at = out0 + atomicAdd(P.out_n + set, (unsigned long long)kept);
+            if (at + kept > out1) {
+                raise_error(P.err, HSK_DERR_BOUNDS);
+                at = ~0ULL;
+            }
+            s_obase = at;
+        }
+        __syncthreads();
+        const u64 at = s_obase;
+        if (tid == 0) s_kept = 0;
+        if (at == ~0ULL) return;
+        for (uint32_t q = tid; q < kept; q += NT) {
+            const uint32_t i = s_list[q];
+            const K key = right_aligned(ek[i], k);
+            atomicAdd(&s_dig[key_digit(key, P.dshift, 0xFF)], 1u);
+            reinterpret_cast<K*>(P.out_keys)[at + q] = key;
+            P.out_counts[at + q] = ec[i];
         }
     };
 
@@ -420,12 +418,11 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
             if (s_dig[i]) atomicAdd(P.dig_hist + (u64)set * 256 + i, (unsigned long long)s_dig[i]);
             s_dig[i] = 0;
         }
-        const u64 d = warp_incl_sum<u64>(my_distinct);
+        const u64 d = warp_incl_sum<u64>((u64)my_ones + my_more);
         const uint32_t mx = __reduce_max_sync(0xffffffffu, my_max);
         if (lane == 31 && d) atomicAdd(P.n_distinct + set, (unsigned long long)d);
         if (lane == 0 && mx) atomicMax(P.max_count + set, mx);
-        my_distinct = 0;
-        my_max = my_ones = 0;
+        my_max = my_ones = my_more = 0;
         __syncthreads();
     };
     // Moves the entries in use to the front; returns their number.
