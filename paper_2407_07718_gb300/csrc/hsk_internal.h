@@ -108,7 +108,7 @@ void launch_supermer(int mode, const SmParams& p, cudaStream_t st);
 constexpr uint32_t SCATTER_CURSOR_STRIDE = 32;
 void launch_scatter_desc(const uint64_t* desc, uint64_t n_desc, const uint64_t* packed, int k,
                          const uint64_t* bucket_off, uint32_t* cursor, uint64_t* part_cursor, int sub_bits,
-                         uint64_t* records, uint64_t n_records, int* err, int grid, cudaStream_t st);
+                         uint64_t* records, uint64_t n_records, int* err, cudaStream_t st);
 
 // exclusive scan of n uint32 counts into uint64 offsets; offsets[n] = total.
 // Scratch: scan_status_words(n) uint64 words.  copy: the offsets once more;

@@ -570,7 +570,7 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
     for (int half = 0; half < 2; ++half)
         launch_scatter_desc((const uint64_t*)c->cta_off.p + (half ? cap - n_end[1] : 0), n_end[half], E.packed, k,
                             (const uint64_t*)c->bucket_rec.p, d_cursor, d_part_cursor, fine ? sub_bits : 0,
-                            (uint64_t*)c->records.p, S.n_records, c->d_err, c->num_sms * 8, st);
+                            (uint64_t*)c->records.p, S.n_records, c->d_err, st);
     CK(cudaGetLastError());
     S.records = (const uint64_t*)c->records.p;
     return HSK_OK;

@@ -492,79 +492,89 @@ __device__ __forceinline__ void one_strand(u64 (&r)[RW], int nb) {
 // ---------------------------------------------------------------------------
 // A slot in the supermer's bucket from the bucket's cursor, the record's
 // bases gathered from the packed reads (the descriptors of a warp come from
-// one tile, so these reads hit L1/L2).  The kernel waits on memory: each
-// thread takes SD descriptors at a time and issues their loads and cursor
-// atomics together (SD = 4: long-read S3 5.35 -> 4.40 ms; 8 was slower).
+// one tile, so these reads hit L1/L2).
 //
 // FINE: straight into the fine partitions, whose cursors start at their first
 // record.  The records of a partition arrive one by one, but the partitions'
 // open sectors (1 M x 32 bytes) stay in L2, so they leave it whole.  What
-// bounds it is L2 requests: one atomic and one write per record.  Scattering
-// into the buckets (4.4 and 3.8 ms; 5.9 and 4.4 with the sub-partition beside
-// each record) and from there into the partitions (2.1 and 1.3 ms) took 8.0
-// and 5.7 ms on the long- and short-read workloads; this takes 5.0 to 5.8 and
-// 3.9 (and 0.1 of the walk, which counts records per partition).
+// bounds it is L2 requests: one atomic and one write per record, at random.
+// Scattering into the buckets (4.4 and 3.8 ms; 5.9 and 4.4 with the
+// sub-partition beside each record) and from there into the partitions (2.1 and
+// 1.3 ms) took 8.0 and 5.7 ms on the long- and short-read workloads; this takes
+// 4.0 and 3.3 (and 0.1 of the walk, which counts records per partition).
+//
+// SMs differ in how far the cursors and lines they need are, so every CTA takes
+// its few descriptors and is done, and the next one goes where there is room:
+// with 8 looping CTAs per SM some SMs were idle for the last fifth (4.5 and 3.9
+// ms).  Few records in flight keep the open sectors few: descriptors a thread
+// takes at a time, in CTAs of 512: 16-byte records 1 4.0 ms, 2 4.0, 3 4.1, 8 4.7;
+// 32-byte records 3 3.6 ms, 4 3.4, 5 3.25, 6 3.25 (whose registers let fewer
+// threads run); a tile's words are loaded before the slots are waited for.
+constexpr int SD_NT = 512, SD_NARROW = 1, SD_WIDE = 5;  // threads a CTA, descriptors a thread
 template <bool WIDE, bool FINE>
-__global__ void __launch_bounds__(256) k_scatter_desc(const u64* __restrict__ desc, u64 n_desc,
+__global__ void __launch_bounds__(SD_NT) k_scatter_desc(const u64* __restrict__ desc, u64 n_desc,
                                                       const u64* __restrict__ packed, int k,
                                                       const u64* __restrict__ bucket_off, uint32_t* cursor,
                                                       unsigned long long* part_cursor, int sub_bits,
                                                       u64* __restrict__ records, u64 n_records, int* err) {
-    constexpr int SD = 4;
+    constexpr int SD = WIDE ? SD_WIDE : SD_NARROW;
     constexpr int RW = WIDE ? 4 : 2;
-    const u64 stride = (u64)gridDim.x * blockDim.x * SD;
-    for (u64 i0 = (u64)blockIdx.x * blockDim.x * SD + threadIdx.x; i0 < n_desc; i0 += stride) {
-        u64 dd[SD], slot[SD];
+    const u64 i0 = (u64)blockIdx.x * blockDim.x * SD + threadIdx.x;
+    u64 dd[SD], slot[SD], w[SD][RW + 1];
 #pragma unroll
-        for (int j = 0; j < SD; ++j) {
-            const u64 i = i0 + (u64)j * blockDim.x;
-            dd[j] = i < n_desc ? desc[i] : ~0ULL;
-        }
+    for (int j = 0; j < SD; ++j) {
+        const u64 i = i0 + (u64)j * blockDim.x;
+        dd[j] = i < n_desc ? __ldcs(desc + i) : ~0ULL;
+    }
 #pragma unroll
-        for (int j = 0; j < SD; ++j) {
-            slot[j] = ~0ULL;
-            if (dd[j] != ~0ULL) {
-                if constexpr (FINE) {
-                    const uint32_t b = (uint32_t)(dd[j] >> 43) & 0x1FFFu, sub = (uint32_t)(dd[j] >> 56);
-                    slot[j] = atomicAdd(part_cursor + ((b << sub_bits) | sub), 1ULL);
-                } else {
-                    const uint32_t b = (uint32_t)(dd[j] >> 48);
-                    slot[j] = bucket_off[b] + atomicAdd(cursor + (size_t)b * SCATTER_CURSOR_STRIDE, 1u);
-                }
+    for (int j = 0; j < SD; ++j) {
+        slot[j] = ~0ULL;
+        if (dd[j] != ~0ULL) {
+            if constexpr (FINE) {
+                const uint32_t b = (uint32_t)(dd[j] >> 43) & 0x1FFFu, sub = (uint32_t)(dd[j] >> 56);
+                slot[j] = atomicAdd(part_cursor + ((b << sub_bits) | sub), 1ULL);
+            } else {
+                const uint32_t b = (uint32_t)(dd[j] >> 48);
+                slot[j] = bucket_off[b] + atomicAdd(cursor + (size_t)b * SCATTER_CURSOR_STRIDE, 1u);
             }
         }
+    }
 #pragma unroll
-        for (int j = 0; j < SD; ++j) {
-            if (dd[j] == ~0ULL) continue;
-            const u64 d = dd[j];
-            const u64 pos = d & (FINE ? (1ULL << 36) - 1 : (1ULL << 40) - 1);
-            const uint32_t n = FINE ? (uint32_t)(d >> 36) & 0x7F : (uint32_t)(d >> 40) & 0xFF;
-            if (slot[j] >= n_records || (!FINE && slot[j] >= bucket_off[(uint32_t)(d >> 48) + 1])) {
-                raise_error(err, HSK_DERR_BOUNDS);
-                continue;
-            }
-            const int nb = (int)n + k - 1;  // bases in the record
-            u64 r[RW];
+    for (int j = 0; j < SD; ++j) {  // up to RW words past the bases: the stream is padded
+        const u64 pos = dd[j] == ~0ULL ? 0 : dd[j] & (FINE ? (1ULL << 36) - 1 : (1ULL << 40) - 1);
 #pragma unroll
-            for (int q = 0; q < RW; ++q) r[q] = keep_bases(extract_k64(packed, pos + 32 * q, 32), nb - 32 * q);
-            if (FINE) one_strand<RW>(r, nb);
-            r[RW - 1] |= (u64)n;
-            ulonglong2* dst = reinterpret_cast<ulonglong2*>(records) + (RW / 2) * slot[j];
+        for (int q = 0; q <= RW; ++q) w[j][q] = packed[(pos >> 5) + q];
+    }
 #pragma unroll
-            for (int q = 0; q < RW / 2; ++q) dst[q] = make_ulonglong2(r[2 * q], r[2 * q + 1]);
+    for (int j = 0; j < SD; ++j) {
+        const u64 d = dd[j];
+        if (d == ~0ULL) continue;
+        const uint32_t n = FINE ? (uint32_t)(d >> 36) & 0x7F : (uint32_t)(d >> 40) & 0xFF;
+        const int nb = (int)n + k - 1;  // bases in the record
+        const uint32_t off = 2 * ((uint32_t)d & 31u);
+        u64 r[RW];
+#pragma unroll
+        for (int q = 0; q < RW; ++q) r[q] = keep_bases(funnel64(w[j][q], w[j][q + 1], off), nb - 32 * q);
+        if (FINE) one_strand<RW>(r, nb);
+        r[RW - 1] |= (u64)n;
+        if (slot[j] >= n_records || (!FINE && slot[j] >= bucket_off[(uint32_t)(d >> 48) + 1])) {
+            raise_error(err, HSK_DERR_BOUNDS);
+            continue;
         }
+        ulonglong2* dst = reinterpret_cast<ulonglong2*>(records) + (RW / 2) * slot[j];
+#pragma unroll
+        for (int q = 0; q < RW / 2; ++q) dst[q] = make_ulonglong2(r[2 * q], r[2 * q + 1]);
     }
 }
 
 void launch_scatter_desc(const uint64_t* desc, uint64_t n_desc, const uint64_t* packed, int k,
                          const uint64_t* bucket_off, uint32_t* cursor, uint64_t* part_cursor, int sub_bits,
-                         uint64_t* records, uint64_t n_records, int* err, int grid, cudaStream_t st) {
+                         uint64_t* records, uint64_t n_records, int* err, cudaStream_t st) {
     if (n_desc == 0) return;
     count_launch();
-    uint64_t need = (n_desc + 4 * 256 - 1) / (4 * 256);  // four descriptors a thread
-    unsigned g = (unsigned)(need < (uint64_t)grid ? need : (uint64_t)grid);
+    const uint64_t per = SD_NT * (k <= 32 ? SD_NARROW : SD_WIDE), g = (n_desc + per - 1) / per;
     auto go = [&](auto kern) {
-        kern<<<g, 256, 0, st>>>((const u64*)desc, n_desc, (const u64*)packed, k, (const u64*)bucket_off, cursor,
+        kern<<<(unsigned)g, SD_NT, 0, st>>>((const u64*)desc, n_desc, (const u64*)packed, k, (const u64*)bucket_off, cursor,
                                 (unsigned long long*)part_cursor, sub_bits, (u64*)records, n_records, err);
     };
     if (part_cursor) {
