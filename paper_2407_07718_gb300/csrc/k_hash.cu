@@ -24,7 +24,7 @@
 // What it replaces and measured (one GB300): writing every key to its (group,
 // top digit) sub-segment and sorting the sub-segments on chip (k_local.cu)
 // took 39 ms on 1.5 G windows of 30x long reads (k = 31) and 45 ms on 1.27 G
-// of 20x short reads (k = 55); this takes 4.7 and 11.9 ms.
+// of 20x short reads (k = 55); this takes 4.6 and 11.5 ms.
 #include "hsk_device.cuh"
 
 namespace hsk {
@@ -48,7 +48,7 @@ namespace hsk {
 // wait for its longest probe sequence: 10.2 and 26.8 ms on the two workloads
 // above (four tags read at once 10.2 and 27.7), against 4.9 and 13.0.  Visiting
 // only the kept entries when the pairs are written (one in nine of the short
-// reads') took that to 4.7 and 11.9.
+// reads') took that to 4.7 and 11.9, the last rounds by one warp to 4.6 and 11.5.
 //
 // Sizes, by trial.  64-bit keys, on the long reads and on 8x short reads of a
 // 20 Mbp genome: 384 threads x 3 CTAs and 3072 entries 5.1 and 0.74 ms, 512 x
@@ -339,6 +339,44 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
         for (uint32_t round = 1;; ++round) {  // at least one key a slot is settled every round
             const uint32_t nl = s_nl[(round - 1) & 1];
             if (nl == 0) break;
+            // the last few: one warp, without the CTA's barriers (long reads 4.73 ->
+            // 4.60 ms, short reads 11.9 -> 11.5; 32 4.63, 128 4.59, 256 4.73)
+            if (nl <= 64) {
+                if (warp == 0) {
+                    uint32_t e[2];
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const uint32_t q = 32 * j + lane;
+                        e[j] = q < nl ? s_list[q] : 0xFFFFFFFFu;
+                    }
+                    for (uint32_t r = round;; ++r) {
+#pragma unroll
+                        for (int j = 0; j < 2; ++j)
+                            if (e[j] != 0xFFFFFFFFu) *(volatile uint16_t*)&s_slot[key_slot<LS>(ek[e[j]], r)] = (uint16_t)e[j];
+                        __syncwarp();
+                        bool left = false;
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            if (e[j] == 0xFFFFFFFFu) continue;
+                            const K key = ek[e[j]];
+                            const uint32_t win = *(volatile uint16_t*)&s_slot[key_slot<LS>(key, r)];
+                            if (win == e[j]) {
+                                e[j] = 0xFFFFFFFFu;
+                            } else if (key_eq(ek[win], key)) {
+                                atomicAdd(&ec[win], ec[e[j]]);
+                                ec[e[j]] = 0;
+                                e[j] = 0xFFFFFFFFu;
+                            } else {
+                                left = true;
+                            }
+                        }
+                        if (!__any_sync(0xffffffffu, left)) break;
+                        __syncwarp();
+                    }
+                }
+                __syncthreads();
+                break;
+            }
             // this thread's entries, in registers: the list is written again
             constexpr int LPT = (ENT + NT - 1) / NT;
             uint32_t e[LPT];

@@ -93,6 +93,19 @@ def test_one_record_many_times(hsk, k):
         assert_same_result(ctx.count(reads, offs, k, 17, 1, 1 << 30), want, "repeats")
 
 
+@pytest.mark.parametrize("k,m", [(31, 17), (55, 21)])
+@pytest.mark.parametrize("copies", [2, 4, 6, 8, 60])
+def test_few_entries_left_after_the_first_round(hsk, k, m, copies):
+    """Every read `copies` times: a batch of records holds ever fewer distinct
+    k-mers, so that about 300 down to none of them share a slot at first (the
+    last 64 are settled by one warp)."""
+    rng = np.random.default_rng(100 * k + copies)
+    reads = ["".join("ACGT"[x] for x in rng.integers(0, 4, 2000)) for _ in range(max(1, 120 // copies))]
+    r, o = _join(reads * copies)
+    with hsk.Context() as ctx:
+        assert_same_result(ctx.count(r, o, k, m, 1, 1 << 30), oracle.count(r, o, k, 1, 1 << 30), f"{copies} copies")
+
+
 def test_chunks_and_small_histogram(hsk):
     rs = datagen.batched_set(datagen.derive_seed(9, 9), 400_000, 12.0)
     want = oracle.count(rs.reads, rs.offsets, 31, 1, 5, hist_len=7)
