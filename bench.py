@@ -759,22 +759,22 @@ def main():
                     "peak_source": f"{peaks['source']} (MEASURED_PEAKS hbm_gbs copy bandwidth)",
                     "bytes_per_launch": bytes_per_launch, "launch_ms": launch_ms}
     else:
-        # on-chip path: the sub-segment sort (k_local_sort, all tiers) reads
-        # every key once and writes the kept pairs; it is bound by instruction
-        # issue and shared-memory latency, so its roofline is the issue rate
+        # on-chip path: the hash count (k_hash_count, both tiers) reads every
+        # supermer record once and writes the kept pairs; it is bound by
+        # instructions and the shared-memory pipe, so its roofline is the issue rate
         launch_ms = stage_ms[4] / args.steps
-        sha = source_sha(os.path.join(ROOT, "paper_2407_07718_gb300", "csrc", "k_local.cu"))
+        sha = source_sha(os.path.join(ROOT, "paper_2407_07718_gb300", "csrc", "k_hash.cu"))
         cnt = NCU_PER_KEY.get((args.workload, sha))
         n_sms = torch.cuda.get_device_properties(dev).multi_processor_count
         peak_issue = n_sms * SCHEDULERS_PER_SM * clk_mhz / 1e3  # G warp-instructions / s
         inst = cnt["inst"] * n_windows if cnt else None
         achieved = inst / (launch_ms / 1e3) / 1e9 if inst and launch_ms > 0 else None
-        hbm_bytes = n_windows * kb + int(res.n_pairs) * (kb + 4)
+        hbm_bytes = int(res.n_supermers) * 2 * kb + int(res.n_pairs) * (kb + 4)  # a record is two keys long
         hbm_achieved = hbm_bytes / (launch_ms / 1e3) / 1e9 if launch_ms > 0 else 0.0
         wav = cnt.get("smem_wavefronts") * n_windows if cnt else None
         smem_peak = n_sms * clk_mhz / 1e3  # G wavefronts / s: one per SM per cycle
         smem_achieved = wav / (launch_ms / 1e3) / 1e9 if wav and launch_ms > 0 else None
-        roofline = {"bound": "alu", "kernel": "k_local_sort (sub-segment sort + count in shared memory, all tiers)",
+        roofline = {"bound": "alu", "kernel": "k_hash_count (k-mers of supermer records counted by hashing in shared memory, both tiers)",
                     "achieved": achieved, "peak": peak_issue, "unit": "G warp-instructions/s",
                     "frac": achieved / peak_issue if achieved else None,
                     "traffic": cnt["dram"] * n_windows if cnt else None,
@@ -797,14 +797,14 @@ def main():
                + n_windows * kb * (1 + 2 * P)              # keys written, P passes
                + n_windows * kb + int(res.n_pairs) * (kb + 4))  # S5: keys read, kept pairs written
     else:
-        s45 = (2 * n_sm * rec_b                            # S4: records read to count, then to scatter
-               + n_windows * kb * 2                        # keys written by the scatter, read on chip
-               + int(res.n_pairs) * (kb + 4) * 3)          # kept pairs written, compacted (read + write)
+        s45 = (n_sm * rec_b                                # S4 + S5: records read
+               + int(res.n_pairs) * (kb + 4) * 3)          # kept pairs written, split by top digit (read + write)
     e2e_bytes = (rs.n_bases * (1 + 0.25 + 0.25)            # S1: ASCII in, packed + masks out
                  + 2 * rs.n_bases * 0.5                    # S2 + S3: packed + masks read twice
                  + n_sm * rec_b                            # S3 records written
                  + s45
-                 + int(res.n_pairs) * (kb + 4) * 2 * P)    # S6: output pairs sorted
+                 # S6: output pairs sorted (on-chip path: a second-digit split, then ranges on chip)
+                 + int(res.n_pairs) * (kb + 4) * 2 * (P if passes > 0 else 2))
     step_s = ms_max / args.steps / 1e3
     roofline["end_to_end"] = {"bytes_per_step": e2e_bytes, "achieved": e2e_bytes / step_s / 1e9,
                               "frac": e2e_bytes / step_s / 1e9 / peaks["hbm_gbs"]}

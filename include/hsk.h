@@ -17,9 +17,11 @@
  *
  * How (all on the GPU, no CPU fallback): 2-bit encoding (Sec. 2.2); canonical
  * k-mers with hash-scored minimizers and supermers (Sec. 3.2); supermers
- * scattered into minimizer-hashed buckets, the paper's tasks (Sec. 3.4);
- * an LSD radix sort of packed keys (Sec. 3.1); a run-length scan with the
- * filter and histogram (Sec. 3.1).
+ * scattered into minimizer-hashed partitions, the paper's tasks (Sec. 3.4),
+ * cut fine enough that the k-mers of one are counted in an SM's shared memory
+ * by hashing, with the filter and histogram; the kept pairs sorted by key.
+ * Where partitions cannot be cut so fine: a radix sort of the k-mers and a
+ * run-length scan (Sec. 3.1).
  *
  * Keys: k <= 32 -> one uint64 word per k-mer (the 2k-bit code, right
  * aligned); 33 <= k <= 64 -> two uint64 words per k-mer, little-endian
@@ -62,10 +64,10 @@ typedef struct {
     int autotune;          /* 1 = hsk_count_batch applies the parameters that
                               hsk_autotune recorded for its class of job mix (if
                               any); 0 = built-in or last applied parameters */
-    int local_sort;        /* 1 (default) = sort and count sub-segments that fit in
-                              shared memory on chip, the rest with global radix
-                              passes; 0 = global radix passes only.  The result is
-                              the same either way. */
+    int local_sort;        /* 1 (default) = count partitions that fit in shared
+                              memory on chip, the rest with global radix passes;
+                              0 = global radix passes only.  The result is the
+                              same either way. */
     const char* tune_cache; /* file of tuned parameters: read at hsk_create,
                                appended to by hsk_autotune; NULL = none */
     int minimizer_order;    /* 0 (default) = m-mers ordered by a hash of the
@@ -200,7 +202,8 @@ int hsk_host_unpin(void* p);
 
 /* Parameters of the batched and served forms chosen by hsk_autotune. */
 typedef struct {
-    uint32_t group_div;          /* keys of a bucket group = 256 x on-chip sub-segment capacity / group_div */
+    uint32_t group_div;          /* keys of a bucket group = 256 x on-chip sub-segment capacity / group_div
+                                    (jobs and packs that are counted by sorting) */
     uint32_t plain_bucket_shift; /* large jobs run alone use (4096, or 8192 for k > 32) >> shift buckets */
     uint64_t pack_bases;         /* bases of one packed pass at most */
     uint64_t pack_small;         /* jobs of more bases run alone */

@@ -8,19 +8,21 @@
 //     an invalid byte, so no window reaches across it);
 //   * each set owns a range of minimizer buckets, so no bucket, bucket group
 //     or sub-segment ever holds k-mers of two sets;
-//   * S1 encode, S2 walk, S3 scatter, the S4 partition and the S4/S5 on-chip
-//     sort run once over the pack; the on-chip sort keeps each set's
-//     histogram, distinct count and largest count apart;
-//   * S6 sorts every set's kept pairs as one segment of a segmented LSD sort;
+//   * S1 encode, S2 walk, S3 scatter and the S4/S5 hash count (packs under 4 M
+//     bases: the S4 partition and the on-chip sort) run once over the pack; the
+//     counting kernels keep each set's histogram, distinct count and largest
+//     count apart;
+//   * S6 splits every set's kept pairs by their top digit and sorts the ranges;
 //   * the results are copied back set by set.
 // A set is counted exactly as hsk_count counts it alone: windows never cross
 // a read, buckets only partition the k-mers, and the output order is the
 // global key order of the set.
 //
-// A set whose keys do not all fit the on-chip sort (a sub-segment that no
-// on-chip tier nor the heavy-hitter lists take: repeat-rich input) is counted again alone through
-// the plain path, which handles that case; the pack's partial result for it
-// is dropped.
+// A set whose keys do not all fit on chip (a partition that no tier of the hash
+// count takes; a sub-segment that no tier of the on-chip sort nor the
+// heavy-hitter lists take: repeat-rich input) is counted again alone through the
+// plain path, which handles that case; the pack's partial result for it is
+// dropped.
 #include <algorithm>
 #include <cstring>
 #include <vector>

@@ -5,15 +5,20 @@
 // word and the look-back bookkeeping (epoch-tagged status words, tile
 // counters).  hsk_count_device runs the whole pipeline on one stream:
 //
-//   S1 encode -> S2 supermer walk (descriptors, per-bucket counts) -> scan
-//   -> S3 scatter records into buckets -> plan chunks of buckets under the
-//   budget -> per chunk: group buckets, S4 count + scatter keys into
-//   (group, top digit) sub-segments, S4/S5 sort and count each sub-segment
-//   on chip (k_local.cu; the ones that do not fit go through the 8-bit LSD
-//   passes of k_sort.cu and the run scan of k_rle.cu) -> S6 order the kept
-//   pairs.  With local_sort = 0 every chunk takes the LSD passes and the run
-//   scan.  hsk_count copies large inputs in chunks on the copy stream while
-//   S1/S2 run on the chunks already there.
+//   S1 encode -> S2 supermer walk (descriptors, counts per bucket and fine
+//   partition) -> scan -> S3 scatter records into the fine partitions -> plan
+//   chunks of buckets under the budget -> per chunk: S4/S5 count the k-mers of
+//   the partitions on chip, straight from the records (k_hash.cu) -> S6 split
+//   the kept pairs by their top digit and sort the ranges.
+//
+// Where the partitions would not fit an SM (hsk_hash_path_fits), and for the
+// few that do not: S3 scatters into buckets (or the partitions' records are
+// gathered), buckets are grouped, S4 counts + scatters keys into (group, top
+// digit) sub-segments, S4/S5 sorts and counts each sub-segment on chip
+// (k_local.cu; the ones that do not fit go through the 8-bit LSD passes of
+// k_sort.cu and the run scan of k_rle.cu).  With local_sort = 0 every chunk
+// takes the LSD passes and the run scan.  hsk_count copies large inputs in
+// chunks on the copy stream while S1/S2 run on the chunks already there.
 //
 // Buckets are the paper's tasks (Sec. 3.4): a k-mer value never lands in two
 // of them, so chunks and groups of buckets are sorted and counted

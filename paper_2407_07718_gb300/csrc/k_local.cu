@@ -1,7 +1,9 @@
 // k_local.cu -- stage S4 + S5 on chip: each minimizer-bucket group is cut by
 // the top digit of its keys into 256 sub-segments, and every sub-segment that
 // fits shared memory is sorted, run-length counted, histogrammed and filtered
-// by one CTA without going back to HBM.
+// by one CTA without going back to HBM.  This is the path for what the hash
+// count (k_hash.cu) cannot take: small jobs and short k-mers, jobs with too few
+// minimizers, and single partitions over its capacity.
 //
 // The paper's tasks (Sec. 3.4) are independent groups of k-mers that each
 // worker sorts on its own and then counts with one linear scan (Sec. 3.1).

@@ -9,7 +9,8 @@
 //
 // This is the global path: it sorts the sub-segments that do not fit the
 // on-chip sort (k_local.cu), the whole job when local_sort is off, the keys
-// of hsk_stage_sort / hsk_sort_keys_noalloc, and the output pairs (S6).
+// of hsk_stage_sort / hsk_sort_keys_noalloc, and the output pairs of chunked
+// jobs.  The other output pairs (S6) take k_split_pairs and k_range_sort.
 //
 // Segments.  The keys of a job are split into C segments, each a group of
 // minimizer buckets -- the paper's tasks (Sec. 3.4), which never share a
