@@ -46,16 +46,16 @@ UNIT = "k-mers/s"
 # Per-key counters of the dominant kernel from one ncu capture, keyed by the
 # workload and the SHA-256 (first 16 hex digits) of the kernel's source code
 # (comments stripped) at capture time; used only while that code is unchanged.
-#   inst  : warp instructions issued per key (all on-chip tiers)
-#   dram  : DRAM bytes read + written per key (all tiers)
-#   smem_wavefronts : shared-memory wavefronts per key (all tiers); an SM's
+#   inst  : warp instructions issued per k-mer (both tiers)
+#   dram  : DRAM bytes read + written per k-mer (both tiers)
+#   smem_wavefronts : shared-memory wavefronts per k-mer (both tiers); an SM's
 #           shared-memory pipe processes at most one wavefront per cycle
 # The commands that produced them are in profiles/.
 NCU_PER_KEY = {
-    # long-read workload, k=31: k_local_sort tiers 0, 1 and 2 (the heavy-hitter kernel does not
-    # run at this scale), smsp__inst_executed.sum, DRAM bytes and shared-memory wavefronts
-    # (l1tex__data_pipe_lsu_wavefronts_mem_shared.sum) from the 0.1-scale case (149.6 M keys)
-    ("long_read", "068cb6efb5eb6836"): {"inst": 10.1611, "dram": 8.3749, "smem_wavefronts": 2.2143},
+    # long-read workload, k=31: k_hash_count tiers 0 and 1, smsp__inst_executed.sum, DRAM bytes and
+    # shared-memory wavefronts (l1tex__data_pipe_lsu_wavefronts_mem_shared.sum) of one count of the
+    # full workload, one counter a run
+    ("long_read", "36754e016be9d5cb"): {"inst": 2.2121, "dram": 2.1101, "smem_wavefronts": 0.4340},
 }
 # Warp schedulers per SM (Blackwell): each issues at most one warp instruction
 # per cycle; the issue peak is SMs (queried from the device) x this x the SM
