@@ -589,7 +589,11 @@ int hsk_grow_output(hsk_ctx* c, const Output& O, uint64_t need, int key_words, c
     if (c->out_keys.cap >= need * kb && c->out_counts.cap >= need * 4) return HSK_OK;
     DevBuf nk, ncn;
     TRY(hsk_ensure(c, nk, need * kb + need * kb / 4, false));
-    TRY(hsk_ensure(c, ncn, need * 4 + need, false));
+    const int rc = hsk_ensure(c, ncn, need * 4 + need, false);
+    if (rc != HSK_OK) {
+        free_buf(c, nk);
+        return rc;
+    }
     if (O.n_pairs) {
         CK(cudaMemcpyAsync(nk.p, c->out_keys.p, O.n_pairs * kb, cudaMemcpyDeviceToDevice, st));
         CK(cudaMemcpyAsync(ncn.p, c->out_counts.p, O.n_pairs * 4, cudaMemcpyDeviceToDevice, st));

@@ -1,0 +1,30 @@
+"""Device memory: a call that fails for want of memory keeps none of it."""
+import pytest
+
+import datagen
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_reads", [400, 20_000])  # counted by sorting, by hashing
+def test_a_failed_allocation_leaks_nothing(hsk, n_reads):
+    """Whichever allocation of a call fails, the context holds as much after a
+    later good call as one that never failed."""
+    reads, offs = datagen.random_reads(7, n_reads, 150, 150)
+    with hsk.Context() as ctx:
+        ctx.count(reads, offs, 31, 17, 1, 1000)
+        want = ctx.allocated()
+    failed = 0
+    for i in range(60):
+        with hsk.Context() as ctx:
+            ctx.fail_alloc_after(i)
+            try:
+                ctx.count(reads, offs, 31, 17, 1, 1000)
+                break
+            except hsk.HskError as e:
+                assert e.code == hsk.HSK_ENOMEM
+            failed += 1
+            ctx.fail_alloc_after(-1)
+            ctx.count(reads, offs, 31, 17, 1, 1000)
+            assert ctx.allocated() == want, f"allocation {i}"
+    assert failed > 15
