@@ -76,6 +76,7 @@ int hsk_ensure(hsk_ctx* c, DevBuf& b, size_t bytes, bool zero_new) {
         b.cap = 0;
     }
     if (c->fail_alloc_after >= 0 && c->fail_alloc_after-- == 0) {
+        c->alloc_injected = true;
         hsk_set_error(c, "injected allocation failure");
         return HSK_ENOMEM;
     }
@@ -131,6 +132,12 @@ static void free_buf(hsk_ctx* c, DevBuf& b) {
     }
     b.p = nullptr;
     b.cap = 0;
+}
+
+// Gives back every buffer but the ones named.
+void hsk_free_except(hsk_ctx* c, std::initializer_list<DevBuf*> keep) {
+    for (DevBuf* b : c->all_bufs())
+        if (std::find(keep.begin(), keep.end(), b) == keep.end()) free_buf(c, *b);
 }
 
 // A fresh epoch for a look-back launch (status words of other launches never
@@ -1248,9 +1255,10 @@ static int hash_chunk(hsk_ctx* c, const Supermers& S, uint32_t b0, uint32_t b1, 
     return HSK_OK;
 }
 
-int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, uint64_t n_reads,
-                  uint64_t n_bases, int k, int m, uint32_t lo, uint32_t hi, cudaStream_t st,
-                  DevResult& R, InputPipe* pipe) {
+// One count; hash: the hash path may be taken (cleared when it was not).
+static int run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, uint64_t n_reads, uint64_t n_bases,
+                     int k, int m, uint32_t lo, uint32_t hi, cudaStream_t st, DevResult& R, InputPipe* pipe,
+                     bool& may_hash) {
     memset(&R, 0, sizeof(R));
     c->zst = st;
     if (n_bases >= (1ull << 40)) {
@@ -1277,7 +1285,8 @@ int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, ui
     Supermers S;
     uint32_t B = hsk_pick_buckets(c, n_bases, k);
     int sub_bits = -1;
-    if (n_bases < HASH_MAX_BASES && hsk_hash_path_fits(c, n_bases, B, k, m)) {
+    may_hash = may_hash && n_bases < HASH_MAX_BASES && hsk_hash_path_fits(c, n_bases, B, k, m);
+    if (may_hash) {
         // fine partitions of half a batch's k-mers at most
         for (sub_bits = 0; sub_bits < HASH_MAX_SUB_BITS;) {
             if (n_bases <= ((uint64_t)B << sub_bits) * (hash_count_cap(kw) / 2)) break;
@@ -1391,6 +1400,24 @@ int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, ui
     R.hist_len = H;
     R.device_ms = ms;
     return HSK_OK;
+}
+
+int hsk_run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets, uint64_t n_reads,
+                  uint64_t n_bases, int k, int m, uint32_t lo, uint32_t hi, cudaStream_t st,
+                  DevResult& R, InputPipe* pipe) {
+    bool hash = true;
+    c->alloc_injected = false;
+    int rc = run_count(c, d_reads, d_offsets, n_reads, n_bases, k, m, lo, hi, st, R, pipe, hash);
+    // The hash path holds tables of the fine partitions, and gathers the records
+    // of those it cannot count beside the originals: a budget may be enough for
+    // the sorting path alone.
+    if (rc == HSK_ENOMEM && hash && !c->alloc_injected) {
+        CK(cudaStreamSynchronize(st));
+        hsk_free_except(c, {&c->in_reads, &c->in_offsets});
+        hash = false;
+        rc = run_count(c, d_reads, d_offsets, n_reads, n_bases, k, m, lo, hi, st, R, pipe, hash);
+    }
+    return rc;
 }
 
 static void to_public(const DevResult& R, hsk_result* out) {

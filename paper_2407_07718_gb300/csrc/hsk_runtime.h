@@ -279,6 +279,7 @@ struct hsk_ctx {
     std::string err_msg;
     size_t budget = 0, allocated = 0;
     int fail_alloc_after = -1;
+    bool alloc_injected = false;  // an allocation of the call failed by fail_alloc_after
 
     // small device scalars: error word, max count, run count, kept count, tile counters
     void* small = nullptr;
@@ -412,6 +413,7 @@ int hsk_guarded(hsk_ctx* c, F&& body) {
     }
 }
 int hsk_ensure(hsk_ctx* c, DevBuf& b, size_t bytes, bool zero_new);
+void hsk_free_except(hsk_ctx* c, std::initializer_list<DevBuf*> keep);
 uint64_t* hsk_host_room(hsk_ctx* c, size_t words);
 int hsk_zero(hsk_ctx* c, cudaStream_t st, std::initializer_list<std::pair<void*, size_t>> regions);
 int hsk_ensure_status(hsk_ctx* c, uint64_t words, cudaStream_t st);

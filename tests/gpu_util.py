@@ -40,3 +40,33 @@ def assert_same_result(got, want, label=""):
     assert np.array_equal(got.kmers, want.kmers), label
     assert np.array_equal(got.counts, want.counts), label
     assert np.array_equal(got.hist, want.hist), label
+
+
+ACGT = np.frombuffer(b"ACGT", np.uint8)
+
+
+def reads_of(template, n_reads, length, err, seed):
+    """n_reads reads of `length` bases from either strand of a template, with
+    substitutions at rate err; (ASCII bases, offsets)."""
+    rng = np.random.default_rng(seed)
+    start = rng.integers(0, len(template) - length + 1, n_reads)
+    x = template[start[:, None] + np.arange(length)]
+    flip = rng.random(n_reads) < 0.5
+    x[flip] = 3 - x[flip, ::-1]
+    hit = rng.random(x.shape, dtype=np.float32) < err
+    x = np.where(hit, (x + rng.integers(1, 4, x.shape, dtype=np.uint8)) & 3, x)
+    return ACGT[x].reshape(-1), np.arange(n_reads + 1, dtype=np.uint64) * np.uint64(length)
+
+
+def join(*sets):
+    at = np.cumsum([0] + [int(o[-1]) for _, o in sets])
+    offs = [o[:-1] + np.uint64(a) for (_, o), a in zip(sets, at)] + [np.array([at[-1]], np.uint64)]
+    return np.concatenate([r for r, _ in sets]), np.concatenate(offs)
+
+
+def bases(n, seed):
+    return np.random.default_rng(seed).integers(0, 4, n, dtype=np.uint8)
+
+
+def amplicon(n_bases, seed, err=0.01):
+    return reads_of(bases(400, seed), n_bases // 400, 400, err, seed + 1)

@@ -2,6 +2,8 @@
 import pytest
 
 import datagen
+import oracle
+from gpu_util import amplicon, assert_same_result
 
 pytestmark = pytest.mark.gpu
 
@@ -28,3 +30,15 @@ def test_a_failed_allocation_leaks_nothing(hsk, n_reads):
             ctx.count(reads, offs, 31, 17, 1, 1000)
             assert ctx.allocated() == want, f"allocation {i}"
     assert failed > 15
+
+
+@pytest.mark.parametrize("budget_mb", [176, 180])
+def test_a_budget_for_the_sorting_path_is_enough(hsk, budget_mb):
+    """Partitions that the hash count cannot take are gathered beside the
+    originals; where the budget has no room for that, the sorting path alone
+    counts the job."""
+    reads, offs = amplicon(12_000_000, 1)
+    want = oracle.count(reads, offs, 55, 1, 1000)
+    with hsk.Context(hbm_budget=budget_mb << 20) as ctx:
+        assert_same_result(ctx.count(reads, offs, 55, 21, 1, 1000), want, f"{budget_mb} MB")
+        assert ctx.allocated() <= budget_mb << 20
