@@ -35,11 +35,7 @@ extern "C" int hsk_count_ext(hsk_ctx* c, const char* reads, const uint64_t* offs
         c->ext_off.pinned = c->ext_read.pinned = c->ext_pos.pinned = true;
         c->ext_off.resize(np + 1);
         uint64_t n_occ = 0;
-        if (np == 0) {
-            c->ext_off.data()[0] = 0;
-            c->ext_read.resize(0);
-            c->ext_pos.resize(0);
-        } else {
+        auto occurrences = [&]() -> int {
             // the kept keys (sorted, on the device since the count) into a table of indices
             uint32_t slots = 1024;
             while (slots < 2 * np) slots <<= 1;
@@ -92,7 +88,20 @@ extern "C" int hsk_count_ext(hsk_ctx* c, const char* reads, const uint64_t* offs
             CK(cudaMemcpyAsync(c->ext_off.data(), occ_off, (np + 1) * 8, cudaMemcpyDeviceToHost, st));
             CK(cudaMemcpyAsync(c->ext_read.data(), occ_read, n_occ * 4, cudaMemcpyDeviceToHost, st));
             CK(cudaMemcpyAsync(c->ext_pos.data(), occ_pos, n_occ * 4, cudaMemcpyDeviceToHost, st));
-            TRY(hsk_read_device_error(c, st));
+            return hsk_read_device_error(c, st);
+        };
+        if (np == 0) {
+            c->ext_off.data()[0] = 0;
+            c->ext_read.resize(0);
+            c->ext_pos.resize(0);
+        } else {
+            int rc = occurrences();
+            if (rc == HSK_ENOMEM && !c->alloc_injected) {  // without what only the count needed
+                CK(cudaStreamSynchronize(st));
+                hsk_free_except(c, {&c->in_offsets, &c->pk, &c->iv, &c->rs, &c->hist, &c->out_keys, &c->out_counts});
+                rc = occurrences();
+            }
+            TRY(rc);
         }
         memset(out, 0, sizeof(*out));
         out->counts = plain;

@@ -1,4 +1,5 @@
 """Device memory: a call that fails for want of memory keeps none of it."""
+import numpy as np
 import pytest
 
 import datagen
@@ -42,3 +43,14 @@ def test_a_budget_for_the_sorting_path_is_enough(hsk, budget_mb):
     with hsk.Context(hbm_budget=budget_mb << 20) as ctx:
         assert_same_result(ctx.count(reads, offs, 55, 21, 1, 1000), want, f"{budget_mb} MB")
         assert ctx.allocated() <= budget_mb << 20
+
+
+def test_occurrences_within_a_budget_for_the_sorting_path(hsk):
+    """The arrays that only the count needs make room for the occurrence lists."""
+    reads, offs = amplicon(12_000_000, 1)
+    want = oracle.count_ext(reads, offs, 55, 2, 1000)
+    with hsk.Context(hbm_budget=218 << 20) as ctx:
+        res, off, rd, ps = ctx.count_ext(reads, offs, 55, 21, 2, 1000)
+    assert np.array_equal(res.kmers, want.kmers) and np.array_equal(res.counts, want.counts)
+    assert np.array_equal(off, want.occ_offsets)
+    assert np.array_equal(rd, want.occ_read) and np.array_equal(ps, want.occ_pos)
