@@ -27,8 +27,8 @@
 // writes per-window keys and scores for the stage test.
 //
 // The kernel is bound by the integer pipe (ncu: 75 % busy, 67 thread
-// instructions per window).  With 32 windows a lane it takes 3.8 ms on 1.5 G
-// windows of long reads (k = 31, w = 15) and 4.6 ms on 1.27 G of short reads (k
+// instructions per window).  With 32 windows a lane it takes 3.9 ms on 1.5 G
+// windows of long reads (k = 31, w = 15) and 4.7 ms on 1.27 G of short reads (k
 // = 55, w = 35), with 32 warps a CTA; 8 warps and three CTAs per SM took 4.4 and
 // 5.4 ms (fewer registers allow 32 warps per SM instead of 24, and one table
 // serves them all).  One window a lane and step, with the window minima and the
@@ -364,27 +364,52 @@ __global__ void __launch_bounds__(SM_CTA_WARPS * 32, 1) k_supermer(const __grid_
                 };
                 reserve(incl - mine, total);
                 uint32_t extra = 0;  // pieces past the first of runs of more than nmax k-mers, counted like `mine`
-                auto put = [&](int pos, int n, uint32_t id) {
+                // TWO_ENDED: the id's lowest bit is the bucket's highest, so the two
+                // kinds are the two halves of the records
+                auto bucket_of = [&](uint32_t id) {
+                    const uint32_t in = id & bmask;
+                    return bbase + (TWO_ENDED ? (in >> 1) | ((in & 1u) << (bb - 1)) : in);
+                };
+                auto part_of = [&](uint32_t id, uint32_t b) { return (b << P.sub_bits) | (id >> bb); };
+                auto put = [&](int pos, int n, uint32_t id, uint32_t b) {
                     const bool down = TWO_ENDED && (id & 1u);
                     const u64 at = down ? P.desc_cap - 1 - at1++ : at0++;  // past the capacity: not written
-                    // TWO_ENDED: that bit is the bucket's highest, so the two kinds
-                    // are the two halves of the records
-                    const uint32_t in = id & bmask;
-                    const uint32_t b = bbase + (TWO_ENDED ? (in >> 1) | ((in & 1u) << (bb - 1)) : in);
-                    if (P.part_rec) atomicAdd(P.part_rec + ((b << P.sub_bits) | (id >> bb)), 1u);
-                    else atomicAdd(&s_cnt[b], 1u);
-                    atomicAdd(&s_km[b], (uint32_t)n);
                     if (at < P.desc_cap)
                         P.desc[at] = make_desc(p0 + pos, (uint32_t)n, b | (id >> bb) << 13, P.part_rec != nullptr);
                 };
+                // Records per fine partition: one atomic for all pieces of a run, and the
+                // records of the first window's partition added up over the tile.  Reads
+                // crowded around one minimizer have nearly all of theirs there, and an
+                // atomic per record queues at its address, 1.3 a nanosecond: 150 Mbp of
+                // one-base reads took 3.3 ms (now 0.45), with 1 % errors 3.8 (now 0.58).
+                // Other reads pay 3 % of the walk for it.
+                const uint32_t id0 = min(rows[0], row_at(rows, 0, off)) & idmask;
+                const uint32_t hot = part_of(id0, bucket_of(id0));
+                uint32_t hot_n = 0;
                 for (uint32_t S = start; S; S &= S - 1) {
                     const int j = __ffs(S) - 1;
                     const uint32_t rest = ev & ~((2u << j) - 1u);
                     const int len = (rest ? 32 * lane + __ffs(rest) - 1 : open_end) - (32 * lane + j);
                     const uint32_t id = min(row_at(rows, lane, j), row_at(rows, lane, j + off)) & idmask;
-                    if (len > nmax) extra += (uint32_t)((len - 1) / nmax) << (TWO_ENDED && (id & 1u) ? 16 : 0);
-                    put(32 * lane + j, min(len, nmax), id);
+                    const uint32_t b = bucket_of(id);
+                    uint32_t n_rec = 1;
+                    if (len > nmax) {
+                        const uint32_t more = (uint32_t)((len - 1) / nmax);
+                        extra += more << (TWO_ENDED && (id & 1u) ? 16 : 0);
+                        n_rec += more;
+                    }
+                    if (P.part_rec) {
+                        const uint32_t part = part_of(id, b);
+                        if (part == hot) hot_n += n_rec;
+                        else atomicAdd(P.part_rec + part, n_rec);
+                    } else {
+                        atomicAdd(&s_cnt[b], n_rec);
+                    }
+                    atomicAdd(&s_km[b], (uint32_t)len);
+                    put(32 * lane + j, min(len, nmax), id, b);
                 }
+                hot_n = __reduce_add_sync(0xffffffffu, hot_n);
+                if (lane == 0 && hot_n) atomicAdd(P.part_rec + hot, hot_n);
                 if (__any_sync(0xffffffffu, extra)) {
                     const uint32_t xi = warp_incl_sum<uint32_t>(extra);
                     at0 = at1 = 0;
@@ -394,7 +419,8 @@ __global__ void __launch_bounds__(SM_CTA_WARPS * 32, 1) k_supermer(const __grid_
                         const uint32_t rest = ev & ~((2u << j) - 1u);
                         const int end = rest ? 32 * lane + __ffs(rest) - 1 : open_end;
                         const uint32_t id = min(row_at(rows, lane, j), row_at(rows, lane, j + off)) & idmask;
-                        for (int q = 32 * lane + j + nmax; q < end; q += nmax) put(q, min(end - q, nmax), id);
+                        const uint32_t b = bucket_of(id);
+                        for (int q = 32 * lane + j + nmax; q < end; q += nmax) put(q, min(end - q, nmax), id, b);
                     }
                 }
             }
