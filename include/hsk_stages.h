@@ -149,6 +149,19 @@ uint64_t hsk_debug_allocated(hsk_ctx* ctx);
 /* Keys of the context's last counting call that did not fit the on-chip
  * sort and went through the global radix passes instead (0 when none). */
 uint64_t hsk_debug_last_overflow(hsk_ctx* ctx);
+/* How the context's last counting call (not a batched or served one) counted
+ * by hashing: [0] fine partitions (0: the whole job was sorted), [1] those too
+ * full for the first table and left to the second, [2] those of so many records,
+ * or too full for the second, that they were cut into slices, [3] (k-mer, count)
+ * pairs the slices left, [4] partitions that went on to the sorting path. */
+#define HSK_N_HASH_STATS 5
+int hsk_debug_hash_stats(hsk_ctx* ctx, uint64_t out[HSK_N_HASH_STATS]);
+/* Sets one of the context's built-in limits, so that small inputs reach what
+ * lies beyond (results do not change; before the first batched or served call
+ * the serving slots take the limits too):
+ *   HSK_LIMIT_PAIRS  (2^24) pairs of slices; with more, the sorting path. */
+enum { HSK_LIMIT_PAIRS = 0, HSK_N_LIMITS = 1 };
+int hsk_debug_limit(hsk_ctx* ctx, int which, uint64_t value);
 /* Failure detection without a GPU fault: runs the decoupled look-back wait
  * that the scans and radix passes use, on a predecessor status word that
  * nothing ever publishes, giving up after spin_limit polls (1 .. 2^24).

@@ -113,6 +113,8 @@ def load():
             "hsk_debug_fail_alloc_after": ([P, i32], i32),
             "hsk_debug_allocated": ([P], u64),
             "hsk_debug_last_overflow": ([P], u64),
+            "hsk_debug_limit": ([P, i32, u64], i32),
+            "hsk_debug_hash_stats": ([P, C.POINTER(u64)], i32),
             "hsk_debug_wait_timeout": ([P, u32], C.c_int),
             "hsk_debug_host_pool_check": ([], C.c_int),
             "hsk_profile_enable": ([P, i32], i32),
@@ -481,6 +483,18 @@ class Context:
         msg = self.lib.hsk_debug_pack_failure(self.h, C.byref(f)).decode()
         return {"passes": a.value, "sets": b.value, "alone": c.value, "failed_passes": f.value,
                 "last_failure": msg}
+
+    LIMITS = ("pairs",)
+
+    def debug_limit(self, name: str, value: int):
+        """Set a built-in limit for a test (hsk_debug_limit)."""
+        self._check(self.lib.hsk_debug_limit(self.h, self.LIMITS.index(name), value))
+
+    def hash_stats(self) -> dict:
+        """How the last counting call counted by hashing (hsk_debug_hash_stats)."""
+        a = (C.c_uint64 * 5)()
+        self._check(self.lib.hsk_debug_hash_stats(self.h, a))
+        return dict(zip(("partitions", "overfull", "heavy", "pairs", "sorted"), (int(x) for x in a)))
 
     def last_overflow(self) -> int:
         """Keys of the last call that went through the global radix passes

@@ -213,19 +213,47 @@ void launch_ov_gather(const uint64_t* sub_off, const uint32_t* ov_list, uint32_t
 constexpr int HASH_MAX_SUB_BITS = 8;             // fine partitions of a bucket: 2^8 at most
 constexpr uint64_t HASH_MAX_BASES = 1ull << 36;  // bases a descriptor with a sub-partition can address
 uint32_t hash_count_cap(int key_words);      // distinct k-mers the first tier's table holds
-// Counts partitions (all of them, or the n_part listed in `only`): kept pairs
-// to places 0 .. out_cap of (out_keys, out_counts) in no particular order,
-// out_n[0] of them; partitions that overfill the tier's
-// batch listed in ov_list, ov_stats = {listed, their records}; dig_hist[256]
-// += kept pairs per top digit.  bucket_set (packed passes): the set of every
-// bucket of 2^sub_bits partitions, with places out_base[s] .. out_base[s + 1],
-// out_n, dig_hist and the statistics per set.
-void launch_hash_count(const uint64_t* records, const uint64_t* part_off, const uint32_t* only, uint32_t n_part,
-                       int tier, int k, int nmax, uint32_t lo, uint32_t hi, void* out_keys, uint32_t* out_counts,
-                       const uint32_t* bucket_set, int sub_bits, const uint64_t* out_base, uint64_t out_cap,
-                       uint64_t* out_n, uint32_t* ov_list, uint64_t* ov_stats, uint64_t* hist, uint32_t hist_len, uint32_t* max_count,
-                       uint64_t* n_distinct, uint64_t* dig_hist, uint32_t* claim, int* err, int num_sms,
-                       cudaStream_t st);
+uint32_t hash_slice_records(int key_words);  // records of a slice at least (a batch of tier 1)
+// What a count of partitions reads and where its results go: kept pairs to
+// places 0 .. out_cap of (out_keys, out_counts) in no particular order, out_n[0]
+// of them; dig_hist[256] += kept pairs per top digit.  bucket_set (packed
+// passes): the set of every bucket of 2^sub_bits partitions, with places
+// out_base[s] .. out_base[s + 1], out_n, dig_hist and the statistics per set.
+struct HashJob {
+    const uint64_t *records, *part_off;
+    int k, nmax;
+    uint32_t lo, hi;
+    void* out_keys;
+    uint32_t* out_counts;
+    const uint32_t* bucket_set;
+    int sub_bits;
+    const uint64_t* out_base;
+    uint64_t out_cap;
+    uint64_t* out_n;
+    uint64_t* hist;
+    uint32_t hist_len;
+    uint32_t* max_count;
+    uint64_t *n_distinct, *dig_hist;
+    int* err;
+};
+// Counts partitions 0 .. n_part - 1, or the n_part listed in `only`; partitions
+// that overfill tier 0's batch, or tier 1's table, are listed in ov_list,
+// ov_stats = {listed, their records}.  Those of tier 0 with more than heavy_min
+// records and those of tier 1 are listed as {first record, records, partition}
+// in heavy instead while it has room (heavy_cap), heavy_n = {listed, or more than
+// heavy_cap, their records}.
+void launch_hash_count(const HashJob& J, const uint32_t* only, uint32_t n_part, int tier, uint32_t* ov_list,
+                       uint64_t* ov_stats, uint64_t* heavy, uint32_t heavy_cap, uint64_t heavy_min, uint64_t* heavy_n,
+                       uint32_t* claim, int num_sms, cudaStream_t st);
+// Those partitions: the k-mers of every slice {first record, records,
+// partition} as pairs (a k-mer may have several) with their sets (pair_set ==
+// nullptr: one set), pair_n of them; more than pair_cap: incomplete.
+void launch_hash_slices(const HashJob& J, const uint64_t* slices, uint32_t n_slices, void* pair_keys,
+                        uint32_t* pair_counts, uint32_t* pair_set, uint64_t pair_cap, uint64_t* pair_n,
+                        uint32_t* claim, int num_sms, cudaStream_t st);
+// n of those pairs to the job's results; table: mask + 1 >= 2 n zeroed slots
+void launch_pairs(const HashJob& J, void* pair_keys, uint32_t* pair_counts, uint32_t* pair_set, uint32_t n,
+                  uint32_t* table, uint32_t mask, int num_sms, cudaStream_t st);
 // sets' pairs from src_off[s] on -> dst_off[s] .. dst_off[s + 1] (n in all)
 void launch_close_sets(const void* src_keys, const uint32_t* src_counts, const uint64_t* src_off,
                        const uint64_t* dst_off, uint32_t n_sets, uint64_t n, int key_words, void* dst_keys,

@@ -293,6 +293,16 @@ extern "C" int hsk_debug_fail_alloc_after(hsk_ctx* c, int n) {
 
 extern "C" uint64_t hsk_debug_allocated(hsk_ctx* c) { return c ? c->allocated : 0; }
 extern "C" uint64_t hsk_debug_last_overflow(hsk_ctx* c) { return c ? c->last_ov_keys : 0; }
+extern "C" int hsk_debug_limit(hsk_ctx* c, int which, uint64_t value) {
+    if (!c || which < 0 || which >= HSK_N_LIMITS) return HSK_EINVAL;
+    c->limits[which] = value;
+    return HSK_OK;
+}
+extern "C" int hsk_debug_hash_stats(hsk_ctx* c, uint64_t* out) {
+    if (!c || !out) return HSK_EINVAL;
+    memcpy(out, c->hash_stats, sizeof(c->hash_stats));
+    return HSK_OK;
+}
 
 
 // ---------------------------------------------------------------------------
@@ -1147,41 +1157,149 @@ bool hsk_hash_path_fits(hsk_ctx* c, uint64_t n_windows, uint32_t B, int k, int m
     return n_windows >= HASH_MIN_KMERS && per_part <= cap && per_min <= cap;
 }
 
+// Room of a buffer without running out of the budget.
+static bool fits_budget(hsk_ctx* c, const DevBuf& b, size_t bytes) {
+    return b.cap >= bytes || c->allocated - b.cap + bytes + (2u << 20) <= c->budget;
+}
+
+// Partitions of a hash count ({first record, records, partition} in list) cut
+// into slices for all SMs, whose pairs are merged in a table.  *done = false: not
+// counted, as the slices leave too many pairs or the budget has no room for them.
+// The limit (2^24 pairs): so many k-mers that mostly differ fill the SMs on the
+// sorting path too.
+static int count_heavy(hsk_ctx* c, const HashJob& J, const std::vector<uint64_t>& list, uint64_t* d_pair_n,
+                       cudaStream_t st, bool* done) {
+    *done = false;
+    const int kw = J.k <= 32 ? 1 : 2;
+    uint64_t n_rec = 0;
+    for (size_t i = 0; i < list.size(); i += 3) n_rec += list[i + 1];
+    // four slices an SM, of a batch at least
+    const uint64_t len = std::max<uint64_t>(hash_slice_records(kw), (n_rec + 4 * c->num_sms - 1) / (4 * c->num_sms));
+    std::vector<uint64_t> sl;
+    for (size_t i = 0; i < list.size(); i += 3)
+        for (uint64_t r = 0; r < list[i + 1]; r += len) {
+            const uint64_t s[3] = {list[i] + r, std::min(len, list[i + 1] - r), list[i + 2]};
+            sl.insert(sl.end(), s, s + 3);
+        }
+    const uint64_t cap = std::min<uint64_t>(c->limits[HSK_LIMIT_PAIRS], n_rec * J.nmax);
+    const size_t kb = (size_t)kw * 8, bytes = cap * (kb + 4 + (J.bucket_set ? 4 : 0)) + sl.size() * 8;
+    if (!fits_budget(c, c->heavy, bytes)) return HSK_OK;
+    TRY(hsk_ensure(c, c->heavy, bytes, false));
+    uint64_t* d_sl = (uint64_t*)((char*)c->heavy.p + cap * kb);
+    uint32_t* d_cnt = (uint32_t*)(d_sl + sl.size());
+    uint32_t* d_set = J.bucket_set ? d_cnt + cap : nullptr;
+    CK(cudaMemcpyAsync(d_sl, sl.data(), sl.size() * 8, cudaMemcpyHostToDevice, st));
+    uint32_t* ctr;
+    TRY(hsk_next_counter(c, st, &ctr));
+    launch_hash_slices(J, d_sl, (uint32_t)(sl.size() / 3), c->heavy.p, d_cnt, d_set, cap, d_pair_n, ctr, c->num_sms, st);
+    CK(cudaGetLastError());
+    uint64_t* room = hsk_host_room(c, 1);
+    CK(cudaMemcpyAsync(room, d_pair_n, 8, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    const uint64_t n = room[0];
+    if (n > cap) return HSK_OK;
+    uint64_t slots = 1024;
+    while (slots < 2 * n) slots *= 2;
+    if (!fits_budget(c, c->loc_tab, slots * 4)) return HSK_OK;
+    TRY(hsk_ensure(c, c->loc_tab, slots * 4, false));
+    CK(cudaMemsetAsync(c->loc_tab.p, 0, slots * 4, st));
+    launch_pairs(J, c->heavy.p, d_cnt, d_set, (uint32_t)n, (uint32_t*)c->loc_tab.p, (uint32_t)(slots - 1), c->num_sms, st);
+    CK(cudaGetLastError());
+    *done = true;
+    return HSK_OK;
+}
+
 // The hash count of n_part partitions of S sets (bucket_set: the set of every
 // bucket; nullptr with one set): kept pairs of set s to places out_base[s] ..
 // out_base[s + 1] of (c->keys, c->alt); histograms to c->hist, largest counts
 // to d_max[s].  R receives the rest.
+// A partition is heavy, and not left to one CTA of tier 1, when it holds more
+// than a part of an SM's share of the records: a quarter of 64-bit keys, a
+// sixteenth of 128-bit keys, of which tier 1's table holds fewer and so rejects
+// more partitions after it walked them.  30 kb sequenced 20,000 times (600 Mbp, all
+// partitions overfull) takes 1.13 and 9.0 ms with a quarter, 1.22 and 6.2 with a
+// sixteenth (k = 31 and 55); 50 amplicons (150 Mbp) 0.37 and 2.29, 0.42 and 1.56.
+constexpr uint32_t HEAVY_MAX = 16384;  // partitions listed for slices
 int hsk_hash_tiers(hsk_ctx* c, const uint64_t* recs, const uint64_t* part_off, uint32_t n_part, const Supermers& SM,
                    int k, uint32_t lo, uint32_t hi, uint32_t H, uint32_t S, const uint64_t* out_base,
                    const uint32_t* bucket_set, uint32_t* d_max, HashRun& R, cudaStream_t st) {
-    // {listed, their records} of the two tiers | kept pairs, distinct k-mers
-    // and kept pairs per top digit of every set || out_base || two lists
-    const size_t words = 4 + 258 * (size_t)S;
-    TRY(hsk_ensure(c, c->hash_ctl, (words + S + 1) * 8 + (size_t)n_part * 8, false));
+    // control words (HASH_CTL) | kept pairs, distinct k-mers and kept pairs per
+    // top digit of every set || out_base || heavy partitions || two lists
+    const int kw = k <= 32 ? 1 : 2;
+    const size_t words = HASH_CTL + 258 * (size_t)S;
+    TRY(hsk_ensure(c, c->hash_ctl, (words + S + 1 + 3 * HEAVY_MAX) * 8 + (size_t)n_part * 8, false));
     uint64_t* ctl = (uint64_t*)c->hash_ctl.p;
     uint64_t* d_base = ctl + words;
-    uint32_t* list1 = (uint32_t*)(d_base + S + 1);
+    uint64_t* d_heavy = d_base + S + 1;
+    uint32_t* list1 = (uint32_t*)(d_heavy + 3 * HEAVY_MAX);
     R.list = list1 + n_part;
     R.S = S;
     R.h.resize(words);
+    HashJob J;
+    J.records = recs;
+    J.part_off = part_off;
+    J.k = k;
+    J.nmax = SM.nmax;
+    J.lo = lo;
+    J.hi = hi;
+    J.out_keys = c->keys.p;
+    J.out_counts = (uint32_t*)c->alt.p;
+    J.bucket_set = bucket_set;
+    J.sub_bits = SM.sub_bits;
+    J.out_base = d_base;
+    J.out_cap = out_base[1];
+    J.out_n = ctl + HASH_CTL;
+    J.hist = (uint64_t*)c->hist.p;
+    J.hist_len = H;
+    J.max_count = d_max;
+    J.n_distinct = ctl + HASH_CTL + S;
+    J.dig_hist = ctl + HASH_CTL + 2 * (size_t)S;
+    J.err = c->d_err;
     CK(cudaMemsetAsync(ctl, 0, words * 8, st));
     if (bucket_set) CK(cudaMemcpyAsync(d_base, out_base, ((size_t)S + 1) * 8, cudaMemcpyHostToDevice, st));
-    uint64_t* room = hsk_host_room(c, words);
-    for (int tier = 0; tier < 2; ++tier) {
-        const uint32_t n = tier ? (uint32_t)R.h[0] : n_part;
-        if (n == 0) break;
-        uint32_t* ctr;
-        TRY(hsk_next_counter(c, st, &ctr));
-        launch_hash_count(recs, part_off, tier ? list1 : nullptr, n, tier, k, SM.nmax, lo, hi, c->keys.p,
-                          (uint32_t*)c->alt.p, bucket_set, SM.sub_bits, d_base, out_base[1], ctl + 4, tier ? R.list : list1,
-                          ctl + 2 * tier, (uint64_t*)c->hist.p, H, d_max, ctl + 4 + S, ctl + 4 + 2 * (size_t)S, ctr,
-                          c->d_err, c->num_sms, st);
-        CK(cudaGetLastError());
+    auto read_ctl = [&]() -> int {
+        uint64_t* room = hsk_host_room(c, words);
         CK(cudaMemcpyAsync(room, ctl, words * 8, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
         memcpy(R.h.data(), room, words * 8);
+        return HSK_OK;
+    };
+    uint32_t* ctr;
+    TRY(hsk_next_counter(c, st, &ctr));
+    const uint64_t n_rec = (uint64_t)((double)SM.n_records * n_part / ((uint64_t)SM.B << SM.sub_bits));
+    const uint64_t heavy_min = std::max<uint64_t>(4 * hash_slice_records(kw), n_rec / ((kw == 1 ? 4 : 16) * (uint64_t)c->num_sms));
+    launch_hash_count(J, nullptr, n_part, 0, list1, ctl, d_heavy, HEAVY_MAX, heavy_min, ctl + 4, ctr, c->num_sms, st);
+    CK(cudaGetLastError());
+    TRY(read_ctl());
+    c->hash_stats[0] += n_part;
+    const uint32_t n1 = (uint32_t)R.h[0];
+    if (n1) {
+        TRY(hsk_next_counter(c, st, &ctr));
+        launch_hash_count(J, list1, n1, 1, R.list, ctl + 2, d_heavy, HEAVY_MAX, 0, ctl + 4, ctr, c->num_sms, st);
+        CK(cudaGetLastError());
+        TRY(read_ctl());
+    }
+    const uint32_t n_heavy = (uint32_t)std::min<uint64_t>(R.h[4], HEAVY_MAX);
+    std::vector<uint32_t> left;  // of those, not counted
+    if (n_heavy) {
+        std::vector<uint64_t> list(3 * (size_t)n_heavy);
+        CK(cudaMemcpyAsync(list.data(), d_heavy, list.size() * 8, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        bool done = false;
+        TRY(count_heavy(c, J, list, ctl + 6, st, &done));
+        if (!done)
+            for (size_t i = 2; i < list.size(); i += 3) left.push_back((uint32_t)list[i]);
+        TRY(read_ctl());
     }
     R.n_left = (uint32_t)R.h[2];
+    if (!left.empty()) {
+        CK(cudaMemcpyAsync(R.list + R.n_left, left.data(), left.size() * 4, cudaMemcpyHostToDevice, st));
+        R.n_left += (uint32_t)left.size();
+    }
+    c->hash_stats[1] += n1;
+    c->hash_stats[2] += n_heavy;
+    c->hash_stats[3] += R.h[6];
+    c->hash_stats[4] += R.n_left;
     return HSK_OK;
 }
 
@@ -1273,6 +1391,7 @@ static int run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets,
     // histogram; err, max, n_heads, n_out; tile counters
     TRY(hsk_zero(c, st, {{c->hist.p, (size_t)H * 8}, {c->small, 64}, {c->counters, HSK_N_COUNTERS * sizeof(uint32_t)}}));
     c->ctr_used = 0;
+    memset(c->hash_stats, 0, sizeof(c->hash_stats));
     c->marks.clear();
     prof_mark(c, st, -1);
     Output O;

@@ -19,6 +19,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/hsk.h"
+#include "../../include/hsk_stages.h"
 
 #define HSK_N_COUNTERS 16384
 #define HSK_SMALL_BYTES (256 + HSK_N_COUNTERS * 4)
@@ -50,16 +51,19 @@ struct Supermers {
     int sub_bits = -1;                     // records in order of 2^sub_bits fine partitions per bucket; -1: none
 };
 
+// Control words of a hash count before those of the sets: {listed, their
+// records} of tiers 0 and 1, the same of heavy partitions, pairs of their slices.
+constexpr size_t HASH_CTL = 8;
 // What a hash count leaves on the host (and its list of uncounted partitions
 // on the device).
 struct HashRun {
     uint32_t S = 1;              // sets
     std::vector<uint64_t> h;     // control words
-    uint32_t n_left = 0;         // partitions that no tier holds
+    uint32_t n_left = 0;         // partitions that were not counted
     uint32_t* list = nullptr;
-    const uint64_t* out_n() const { return h.data() + 4; }             // kept pairs per set
-    const uint64_t* distinct() const { return h.data() + 4 + S; }
-    const uint64_t* digits() const { return h.data() + 4 + 2 * (size_t)S; }  // S x 256 kept pairs per top digit
+    const uint64_t* out_n() const { return h.data() + HASH_CTL; }             // kept pairs per set
+    const uint64_t* distinct() const { return h.data() + HASH_CTL + S; }
+    const uint64_t* digits() const { return h.data() + HASH_CTL + 2 * (size_t)S; }  // S x 256 kept pairs per top digit
 };
 
 // Jobs of fewer k-mers than this take the sorting path.
@@ -307,6 +311,7 @@ struct hsk_ctx {
     DevBuf ext_tab, ext_occ;                                       // extension information: key table, occurrence arrays
     DevBuf s6_bounds;                                              // S6: where each top digit's kept pairs start
     DevBuf part_off, hash_ctl, ov_records;                         // hash path: partitions, control words and lists
+    DevBuf heavy;                                                  // hash path: pairs and slices of heavy partitions
     bool s6_digit_major = false;                                   // the output holds only digit-major pairs
     std::vector<uint64_t> s6_h;                                    // S6: host copy of s6_bounds, when known
 
@@ -346,6 +351,8 @@ struct hsk_ctx {
     std::vector<std::pair<int, int>> marks;  // (event index, stage id; -1 = start)
     double prof_ms[8] = {0};
     uint64_t prof_passes = 0;
+    uint64_t limits[HSK_N_LIMITS] = {1ull << 24};           // hsk_debug_limit
+    uint64_t hash_stats[HSK_N_HASH_STATS] = {0};  // of the last counting call (hsk_debug_hash_stats)
     uint64_t last_ov_keys = 0;  // keys of the last job that did not fit the on-chip sort
 
     std::vector<DevBuf*> all_bufs() {
@@ -353,7 +360,7 @@ struct hsk_ctx {
                 &bucket_rec, &records, &keys, &alt, &pass_hist, &digit_off, &lb_status, &seg, &heads, &rle_tiles,
                 &out_keys, &out_counts, &hist, &pair_alt_keys, &pair_alt_counts, &loc_tab, &batch_a,
                 &batch_b, &batch_c, &batch_d, &pack_tab, &pack_stat, &ext_tab, &ext_occ, &s6_bounds,
-                &part_off, &hash_ctl, &ov_records};
+                &part_off, &hash_ctl, &ov_records, &heavy};
     }
 };
 

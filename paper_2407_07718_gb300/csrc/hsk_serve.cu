@@ -284,6 +284,7 @@ static int serve_start(hsk_ctx* c) {
             return rc;
         }
         child->tune = c->tune;
+        memcpy(child->limits, c->limits, sizeof(c->limits));
         S->slots.push_back(child);
         S->slot_est.push_back(0);
         S->slot_busy.push_back(0);

@@ -16,10 +16,15 @@
 //                    the record's multiplicity, equal ones merged, and the
 //                    counts go to the statistics, the filter and the output.
 //                    Tier 1 is the same kernel with one CTA per SM and a
-//                    larger batch, for partitions that overfill tier 0's;
-//                    what overfills that is listed for the sorting path
-//                    (k_local.cu).
-//   k_list_gather -- records of listed partitions -> one array for that path.
+//                    larger batch, for partitions that overfill tier 0's.
+//   k_pair_merge, k_pair_emit
+//                 -- partitions of very many records (reads crowded around one
+//                    minimizer), and those that overfill tier 1's table, are cut
+//                    into slices that any CTA counts (tier 2 of k_hash_count);
+//                    the slices' (k-mer, count) pairs are merged in one table in
+//                    global memory.
+//   k_list_gather -- records of the partitions whose slices leave too many pairs
+//                    -> one array for the sorting path (k_local.cu).
 //
 // What it replaces and measured (one GB300): writing every key to its (group,
 // top digit) sub-segment and sorting the sub-segments on chip (k_local.cu)
@@ -74,11 +79,15 @@ template <>
 struct HashCfg<true, 1> {
     static constexpr int NT = 512, CTAS = 1, ENT = 6144, LS = 14, RB = 1536;
 };
+template <bool WIDE>
+struct HashCfg<WIDE, 2> : HashCfg<WIDE, 1> {};
 constexpr int HC_HS = 128;      // count-histogram bins kept in shared memory
 constexpr int HC_SEG = 16;      // k-mers of a record one lane takes at a time (at most 16)
 constexpr int HC_CHUNK = 32;    // most partitions claimed at a time
 
 uint32_t hash_count_cap(int key_words) { return key_words == 1 ? HashCfg<false, 0>::ENT : HashCfg<true, 0>::ENT; }
+
+uint32_t hash_slice_records(int key_words) { return key_words == 1 ? HashCfg<false, 1>::RB : HashCfg<true, 1>::RB; }
 
 template <bool WIDE, int TIER>
 constexpr size_t hash_smem() {
@@ -144,6 +153,22 @@ struct HashArgs {
     unsigned long long* dig_hist;  // kept pairs per top digit
     uint32_t* claim;
     int* err;
+    // Partitions for the slices {first record, records, partition}, while there is
+    // room; heavy_n = {listed (or more), records of those in the list}: of tier 0
+    // those of more than heavy_min records, of tier 1 all that it cannot take
+    u64* heavy;
+    u64 heavy_min;
+    uint32_t heavy_cap;
+    unsigned long long* heavy_n;
+    // Tier 2: n_part slices {first record, records, partition}; their pairs (keys
+    // left aligned) with their sets (nullptr: one set), pair_n of them or more
+    // than pair_cap
+    const u64* slice;
+    void* pair_keys;
+    uint32_t* pair_counts;
+    uint32_t* pair_set;
+    u64 pair_cap;
+    unsigned long long* pair_n;
 };
 
 template <bool WIDE, int TIER>
@@ -529,6 +554,61 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
         const uint32_t t = nr * (uint32_t)(ENT / 16 * 15) / (U ? U : 1u);  // nr <= 4096, ENT <= 8192: no overflow
         return t > (uint32_t)RB ? (uint32_t)RB : t;
     };
+    if constexpr (TIER == 2) {
+        // the D entries as pairs
+        auto put_pairs = [&](uint32_t D) {
+            D = close_up(D);
+            if (tid == 0) s_obase = atomicAdd(P.pair_n, (unsigned long long)D);
+            __syncthreads();
+            const u64 at = s_obase;
+            if (at + D <= P.pair_cap)
+                for (uint32_t i = tid; i < D; i += NT) {
+                    reinterpret_cast<K*>(P.pair_keys)[at + i] = ek[i];
+                    P.pair_counts[at + i] = ec[i];
+                    if (P.pair_set) P.pair_set[at + i] = set;
+                }
+            __syncthreads();
+        };
+        for (;;) {
+            __syncthreads();
+            if (tid == 0) s_claim = atomicAdd(P.claim, 1u);
+            __syncthreads();
+            if (s_claim >= P.n_part) break;
+            const u64* sl = P.slice + 3 * (u64)s_claim;
+            u64 r = sl[0];
+            const u64 end = r + sl[1];
+            if (P.bucket_set) set = P.bucket_set[sl[2] >> P.sub_bits];
+            uint32_t D = 0, take = RB;
+            while (r < end) {
+                if (tid == 0) s_kept = *(volatile unsigned long long*)P.pair_n > P.pair_cap;
+                __syncthreads();
+                if (s_kept) break;  // too many pairs already: all are dropped
+                const uint32_t n = end - r < (u64)take ? (uint32_t)(end - r) : take;
+                const uint32_t U = stage(r, n);
+                if (D + U > (uint32_t)ENT) D = close_up(D);
+                if (D + U > (uint32_t)ENT && D > (uint32_t)ENT / 2) {
+                    put_pairs(D);
+                    D = 0;
+                }
+                if (D + U > (uint32_t)ENT) {  // more than 16 records: those have fewer k-mers than half the entries
+                    take = next_part(n, U, (uint32_t)ENT - D);
+                    continue;
+                }
+                expand(D);
+                for (uint32_t i = tid; i < D; i += NT) *(volatile uint16_t*)&s_slot[key_slot<LS>(ek[i], 0)] = (uint16_t)i;
+                __syncthreads();
+                merge(D + U);
+                __syncthreads();
+                D += U;
+                r += n;
+                // about three eighths of the entries a part
+                const uint32_t t = n * (uint32_t)(ENT / 8 * 3) / (U ? U : 1u);
+                take = t < 16 ? 16 : t > (uint32_t)RB ? (uint32_t)RB : t;
+            }
+            put_pairs(D);
+        }
+        return;
+    }
     uint32_t target = RB;
     for (;;) {
         __syncthreads();
@@ -571,8 +651,17 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
                 // partition p alone is more than a batch
                 if (TIER == 0 || !count_in_parts(r0, nr, U)) {
                     if (tid == 0) {
-                        P.ov_list[atomicAdd(reinterpret_cast<unsigned int*>(P.ov_stats), 1u)] = (uint32_t)(first + p);
-                        atomicAdd(P.ov_stats + 1, (unsigned long long)nr);
+                        u64 at = P.heavy_cap;
+                        if (TIER == 1 || nr > P.heavy_min) at = atomicAdd(P.heavy_n, 1ULL);
+                        if (at < (u64)P.heavy_cap) {
+                            P.heavy[3 * at] = r0;
+                            P.heavy[3 * at + 1] = nr;
+                            P.heavy[3 * at + 2] = first + p;
+                            atomicAdd(P.heavy_n + 1, (unsigned long long)nr);
+                        } else {
+                            P.ov_list[atomicAdd(reinterpret_cast<unsigned int*>(P.ov_stats), 1u)] = (uint32_t)(first + p);
+                            atomicAdd(P.ov_stats + 1, (unsigned long long)nr);
+                        }
                     }
                     __syncthreads();
                 }
@@ -591,65 +680,231 @@ __global__ void __launch_bounds__(HashCfg<WIDE, TIER>::NT, HashCfg<WIDE, TIER>::
     flush_stats();
 }
 
-void launch_hash_count(const uint64_t* records, const uint64_t* part_off, const uint32_t* only, uint32_t n_part,
-                       int tier, int k, int nmax, uint32_t lo, uint32_t hi, void* out_keys, uint32_t* out_counts,
-                       const uint32_t* bucket_set, int sub_bits, const uint64_t* out_base, uint64_t out_cap,
-                       uint64_t* out_n, uint32_t* ov_list, uint64_t* ov_stats, uint64_t* hist, uint32_t hist_len, uint32_t* max_count,
-                       uint64_t* n_distinct, uint64_t* dig_hist, uint32_t* claim, int* err, int num_sms,
-                       cudaStream_t st) {
+template <bool WIDE, int TIER>
+static void go_hash_count(HashArgs& P, int num_sms, cudaStream_t st) {
+    using C = HashCfg<WIDE, TIER>;
+    const size_t dyn = hash_smem<WIDE, TIER>();
+    cudaFuncSetAttribute(k_hash_count<WIDE, TIER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    const uint64_t slots = (uint64_t)num_sms * C::CTAS;
+    // enough claims that the CTAs end together, few enough that a claim spans several batches
+    uint64_t ch = P.only || TIER == 2 ? 1 : P.n_part / (slots * 8);
+    if (ch < 1) ch = 1;
+    if (ch > HC_CHUNK) ch = HC_CHUNK;
+    if (P.bucket_set) {  // a power of two, at most a bucket's partitions
+        uint64_t c2 = 1;
+        while (c2 * 2 <= ch && c2 * 2 <= (1ull << P.sub_bits)) c2 *= 2;
+        ch = c2;
+    }
+    P.chunk = (uint32_t)ch;
+    const uint64_t want = (P.n_part + P.chunk - 1) / P.chunk;
+    k_hash_count<WIDE, TIER><<<(unsigned)(want < slots ? want : slots), C::NT, dyn, st>>>(P);
+}
+
+static HashArgs hash_args(const HashJob& J) {
+    HashArgs P{};
+    P.rec = (const u64*)J.records;
+    P.part_off = (const u64*)J.part_off;
+    P.k = J.k;
+    P.dshift = 2 * J.k > 8 ? 2 * J.k - 8 : 0;
+    P.rec_n = J.nmax;
+    P.lo = J.lo;
+    P.hi = J.hi;
+    P.out_keys = J.out_keys;
+    P.out_counts = J.out_counts;
+    P.bucket_set = J.bucket_set;
+    P.sub_bits = J.sub_bits;
+    P.out_base = (const u64*)J.out_base;
+    P.out_cap = J.out_cap;
+    P.out_n = (unsigned long long*)J.out_n;
+    P.hist = (u64*)J.hist;
+    P.hist_len = J.hist_len;
+    P.max_count = J.max_count;
+    P.n_distinct = (unsigned long long*)J.n_distinct;
+    P.dig_hist = (unsigned long long*)J.dig_hist;
+    P.err = J.err;
+    return P;
+}
+
+void launch_hash_count(const HashJob& J, const uint32_t* only, uint32_t n_part, int tier, uint32_t* ov_list,
+                       uint64_t* ov_stats, uint64_t* heavy, uint32_t heavy_cap, uint64_t heavy_min, uint64_t* heavy_n,
+                       uint32_t* claim, int num_sms, cudaStream_t st) {
     if (n_part == 0) return;
     count_launch();
-    HashArgs P;
-    P.rec = (const u64*)records;
-    P.part_off = (const u64*)part_off;
+    HashArgs P = hash_args(J);
     P.only = only;
     P.n_part = n_part;
-    P.k = k;
-    P.dshift = 2 * k > 8 ? 2 * k - 8 : 0;
-    P.rec_n = nmax;
-    P.lo = lo;
-    P.hi = hi;
-    P.out_keys = out_keys;
-    P.out_counts = out_counts;
-    P.bucket_set = bucket_set;
-    P.sub_bits = sub_bits;
-    P.out_base = (const u64*)out_base;
-    P.out_cap = out_cap;
-    P.out_n = (unsigned long long*)out_n;
     P.ov_list = ov_list;
     P.ov_stats = (unsigned long long*)ov_stats;
-    P.hist = (u64*)hist;
-    P.hist_len = hist_len;
-    P.max_count = max_count;
-    P.n_distinct = (unsigned long long*)n_distinct;
-    P.dig_hist = (unsigned long long*)dig_hist;
+    P.heavy = (u64*)heavy;
+    P.heavy_min = heavy_min;
+    P.heavy_cap = heavy_cap;
+    P.heavy_n = (unsigned long long*)heavy_n;
     P.claim = claim;
-    P.err = err;
-    auto go = [&](auto kern, int nt, int ctas, size_t dyn) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-        const uint64_t slots = (uint64_t)num_sms * ctas;
-        // enough claims that the CTAs end together, few enough that a claim spans several batches
-        uint64_t ch = only ? 1 : n_part / (slots * 8);
-        if (ch < 1) ch = 1;
-        if (ch > HC_CHUNK) ch = HC_CHUNK;
-        if (bucket_set) {  // a power of two, at most a bucket's partitions
-            uint64_t c2 = 1;
-            while (c2 * 2 <= ch && c2 * 2 <= (1ull << sub_bits)) c2 *= 2;
-            ch = c2;
+    if (J.k <= 32) tier ? go_hash_count<false, 1>(P, num_sms, st) : go_hash_count<false, 0>(P, num_sms, st);
+    else tier ? go_hash_count<true, 1>(P, num_sms, st) : go_hash_count<true, 0>(P, num_sms, st);
+}
+
+void launch_hash_slices(const HashJob& J, const uint64_t* slices, uint32_t n_slices, void* pair_keys,
+                        uint32_t* pair_counts, uint32_t* pair_set, uint64_t pair_cap, uint64_t* pair_n,
+                        uint32_t* claim, int num_sms, cudaStream_t st) {
+    if (n_slices == 0) return;
+    count_launch();
+    HashArgs P = hash_args(J);
+    P.slice = (const u64*)slices;
+    P.n_part = n_slices;
+    P.pair_keys = pair_keys;
+    P.pair_counts = pair_counts;
+    P.pair_set = pair_set;
+    P.pair_cap = pair_cap;
+    P.pair_n = (unsigned long long*)pair_n;
+    P.claim = claim;
+    if (J.k <= 32) go_hash_count<false, 2>(P, num_sms, st);
+    else go_hash_count<true, 2>(P, num_sms, st);
+}
+
+// ---------------------------------------------------------------------------
+// pairs of the slices -> counts of k-mers
+// ---------------------------------------------------------------------------
+// Merges equal k-mers (of one set) of n pairs: every pair looks for its k-mer in
+// an open-addressing table of pair numbers (+ 1), zeroed, with twice as many slots
+// as pairs; the one that enters it keeps the sum, the others end with count 0.
+// Bound by the table's random accesses.  With the slices it counts 150 Mbp of
+// 150-base reads of one base with 1 % errors in 0.4 and 2.4 ms (k = 31 and 55),
+// where one CTA took 30 and 81; one 400-base amplicon (150 Mbp) in 0.6 and 3.1,
+// where most of it went on to the sorting path (4.1 and 23 ms in all).
+template <typename K>
+__global__ void __launch_bounds__(256) k_pair_merge(const K* __restrict__ keys, uint32_t* counts,
+                                                    const uint32_t* __restrict__ sets, uint32_t n, uint32_t* table,
+                                                    uint32_t mask, int* err) {
+    for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
+        const K key = keys[i];
+        const uint32_t cnt = counts[i], set = sets ? sets[i] : 0u;
+        uint32_t h = key_slot<32>(key, 0) ^ set * 0x9E3779B1u;
+        h = (h ^ (h >> 16)) & mask;
+        for (uint32_t probe = 0;; ++probe) {
+            if (probe > mask) {  // never: the table has twice as many slots as pairs
+                raise_error(err, HSK_DERR_BOUNDS);
+                break;
+            }
+            const uint32_t v = atomicCAS(&table[h], 0u, i + 1);
+            if (v == 0) break;
+            if (key_eq(keys[v - 1], key) && (!sets || sets[v - 1] == set)) {
+                atomicAdd(&counts[v - 1], cnt);
+                counts[i] = 0;
+                break;
+            }
+            h = (h + 1) & mask;
         }
-        P.chunk = (uint32_t)ch;
-        const uint64_t want = (n_part + P.chunk - 1) / P.chunk;
-        kern<<<(unsigned)(want < slots ? want : slots), nt, dyn, st>>>(P);
-    };
-#define HC_GO(W, T) go(k_hash_count<W, T>, HashCfg<W, T>::NT, HashCfg<W, T>::CTAS, hash_smem<W, T>())
-    if (k <= 32) {
-        if (tier) HC_GO(false, 1);
-        else HC_GO(false, 0);
-    } else {
-        if (tier) HC_GO(true, 1);
-        else HC_GO(true, 0);
     }
-#undef HC_GO
+}
+
+// Statistics, filter and kept pairs of n merged pairs (as k_hash_count's emit).
+// A CTA takes a run of pairs; pairs of one set lie together in slices, so tiles
+// of several sets, which go to memory pair by pair, are few.
+template <typename K>
+__global__ void __launch_bounds__(256) k_pair_emit(const __grid_constant__ HashArgs P, uint32_t n) {
+    __shared__ uint32_t s_hist[HC_HS], s_dig[256], s_n;
+    __shared__ u64 s_at;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const K* keys = reinterpret_cast<const K*>(P.pair_keys);
+    const uint32_t hs = P.hist_len < (uint32_t)HC_HS ? P.hist_len : (uint32_t)HC_HS;
+    const uint32_t i0 = (uint32_t)((u64)n * blockIdx.x / gridDim.x), i1 = (uint32_t)((u64)n * (blockIdx.x + 1) / gridDim.x);
+    if (i0 >= i1) return;
+    uint32_t set = P.pair_set ? P.pair_set[i0] : 0u, my_max = 0, my_n = 0;
+    for (int i = tid; i < HC_HS; i += 256) s_hist[i] = 0;
+    s_dig[tid] = 0;
+    if (tid == 0) s_n = 0;
+    auto bin_of = [&](uint32_t c) { return c < P.hist_len - 1 ? c : P.hist_len - 1; };
+    auto flush = [&]() {
+        __syncthreads();
+        for (uint32_t i = tid; i < hs; i += 256) {
+            if (s_hist[i]) atomicAdd((unsigned long long*)(P.hist + (u64)set * P.hist_len + i), (unsigned long long)s_hist[i]);
+            s_hist[i] = 0;
+        }
+        if (s_dig[tid]) atomicAdd(P.dig_hist + (u64)set * 256 + tid, (unsigned long long)s_dig[tid]);
+        s_dig[tid] = 0;
+        const uint32_t d = __reduce_add_sync(0xffffffffu, my_n), mx = __reduce_max_sync(0xffffffffu, my_max);
+        if (lane == 0 && d) atomicAdd(P.n_distinct + set, (unsigned long long)d);
+        if (lane == 0 && mx) atomicMax(P.max_count + set, mx);
+        my_n = my_max = 0;
+        __syncthreads();
+    };
+    __syncthreads();
+    for (uint32_t b = i0; b < i1; b += 256) {
+        const uint32_t i = b + tid;
+        const uint32_t cnt = i < i1 ? P.pair_counts[i] : 0u;
+        const bool keep = cnt && cnt >= P.lo && cnt <= P.hi;
+        const uint32_t mine = cnt && P.pair_set ? P.pair_set[i] : set;
+        if (!__syncthreads_and(mine == set)) {
+            flush();
+            if (cnt) {
+                atomicAdd((unsigned long long*)(P.hist + (u64)mine * P.hist_len + bin_of(cnt)), 1ULL);
+                atomicAdd(P.n_distinct + mine, 1ULL);
+                atomicMax(P.max_count + mine, cnt);
+            }
+            if (keep) {
+                const K key = right_aligned(keys[i], P.k);
+                const u64 at = P.out_base[mine] + atomicAdd(P.out_n + mine, 1ULL);
+                atomicAdd(P.dig_hist + (u64)mine * 256 + key_digit(key, P.dshift, 0xFF), 1ULL);
+                if (at < P.out_base[mine + 1]) {
+                    reinterpret_cast<K*>(P.out_keys)[at] = key;
+                    P.out_counts[at] = cnt;
+                } else {
+                    raise_error(P.err, HSK_DERR_BOUNDS);
+                }
+            }
+            set = P.pair_set[i1 - b > 256 ? b + 255 : i1 - 1];
+            continue;
+        }
+        if (cnt) {
+            const uint32_t c = bin_of(cnt);
+            if (c < hs) atomicAdd(&s_hist[c], 1u);
+            else atomicAdd((unsigned long long*)(P.hist + (u64)set * P.hist_len + c), 1ULL);
+            ++my_n;
+            my_max = cnt > my_max ? cnt : my_max;
+        }
+        const uint32_t km = __ballot_sync(0xffffffffu, keep);
+        uint32_t q = 0;
+        if (lane == 0 && km) q = atomicAdd(&s_n, (uint32_t)__popc(km));
+        q = __shfl_sync(0xffffffffu, q, 0) + (uint32_t)__popc(km & ((1u << lane) - 1u));
+        __syncthreads();
+        if (tid == 0) {
+            const u64 base = P.bucket_set ? P.out_base[set] : 0, top = P.bucket_set ? P.out_base[set + 1] : P.out_cap;
+            u64 at = s_n ? base + atomicAdd(P.out_n + set, (unsigned long long)s_n) : 0;
+            if (at + s_n > top) {
+                raise_error(P.err, HSK_DERR_BOUNDS);
+                at = ~0ULL;
+            }
+            s_at = at;
+            s_n = 0;
+        }
+        __syncthreads();
+        if (keep && s_at != ~0ULL) {
+            const K key = right_aligned(keys[i], P.k);
+            atomicAdd(&s_dig[key_digit(key, P.dshift, 0xFF)], 1u);
+            reinterpret_cast<K*>(P.out_keys)[s_at + q] = key;
+            P.out_counts[s_at + q] = cnt;
+        }
+    }
+    flush();
+}
+
+void launch_pairs(const HashJob& J, void* pair_keys, uint32_t* pair_counts, uint32_t* pair_set, uint32_t n,
+                  uint32_t* table, uint32_t mask, int num_sms, cudaStream_t st) {
+    if (n == 0) return;
+    count_launch(2);
+    HashArgs P = hash_args(J);
+    P.pair_keys = pair_keys;
+    P.pair_counts = pair_counts;
+    P.pair_set = pair_set;
+    const uint32_t want = (n + 255) / 256, most = (uint32_t)num_sms * 8, g = want < most ? want : most;
+    if (J.k <= 32) {
+        k_pair_merge<u64><<<g, 256, 0, st>>>((const u64*)pair_keys, pair_counts, pair_set, n, table, mask, J.err);
+        k_pair_emit<u64><<<g, 256, 0, st>>>(P, n);
+    } else {
+        k_pair_merge<key128><<<g, 256, 0, st>>>((const key128*)pair_keys, pair_counts, pair_set, n, table, mask, J.err);
+        k_pair_emit<key128><<<g, 256, 0, st>>>(P, n);
+    }
 }
 
 // ---------------------------------------------------------------------------

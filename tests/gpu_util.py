@@ -70,3 +70,17 @@ def bases(n, seed):
 
 def amplicon(n_bases, seed, err=0.01):
     return reads_of(bases(400, seed), n_bases // 400, 400, err, seed + 1)
+
+
+def low_score_mmer(rng, m, seed=0x9E3779B97F4A7C15):
+    """The base codes of an m-mer whose score (the minimizers' hash) is the least
+    of 200,000 random ones."""
+    c = rng.integers(0, 4, size=(200_000, m), dtype=np.uint8)
+    w = (np.uint64(1) << (2 * np.arange(m - 1, -1, -1)).astype(np.uint64))
+    v = np.minimum((c.astype(np.uint64) * w).sum(1, dtype=np.uint64),
+                   ((3 - c[:, ::-1]).astype(np.uint64) * w).sum(1, dtype=np.uint64))
+    h = (v & np.uint64(0xFFFFFFFF)).astype(np.uint32) ^ (v >> np.uint64(32)).astype(np.uint32) ^ np.uint32(seed & 0xFFFFFFFF)
+    for shift, mul in ((16, 0x85EBCA6B), (13, 0xC2B2AE35), (16, 1)):
+        h ^= h >> np.uint32(shift)
+        h = (h.astype(np.uint64) * np.uint64(mul) & np.uint64(0xFFFFFFFF)).astype(np.uint32)
+    return c[int(np.argmin(h))]

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 import oracle
-from gpu_util import assert_same_result, bases, join, reads_of
+from gpu_util import ACGT, assert_same_result, bases, join, low_score_mmer, reads_of
 
 pytestmark = pytest.mark.gpu
 
@@ -46,3 +46,82 @@ def test_walk_is_as_fast_on_one_minimizer(hsk):
     with hsk.Context() as ctx:
         a, b = (_stage_ms(ctx, 1, r, offs, 31, 17) for r in (crowd, spread))
     assert a < 3 * b, (a, b)
+
+
+def crowd(n, m, side, seed):
+    """n reads, each with its own `side` bases on both sides of one m-mer that no
+    other scores below, so that all their k-mers of m + side bases share it."""
+    low = low_score_mmer(np.random.default_rng(seed), m)
+    x = np.empty((n, m + 2 * side), np.uint8)
+    x[:, :side], x[:, side + m:] = (bases(n * side, seed + i).reshape(n, side) for i in (1, 2))
+    x[:, side: side + m] = low
+    return ACGT[x].reshape(-1), np.arange(n + 1, dtype=np.uint64) * np.uint64(x.shape[1])
+
+
+@pytest.mark.parametrize("k,m", [(31, 17), (55, 21), (32, 16), (33, 17)])
+@pytest.mark.parametrize("lo,hi", [(1, 1 << 30), (2, 50)])
+def test_partitions_cut_into_slices(hsk, k, m, lo, hi):
+    """Partitions of more records than one CTA should walk: of few distinct
+    k-mers, of more than its table holds, of distinct ones only; and one of few
+    records that overfills the second table.  With a low limit on the slices' pairs
+    the same partitions go on to the sorting path."""
+    spread = reads_of(bases(50_000, 1), 10_000, 150, 0.002, 2)
+    few = reads_of(poly("A", 1000), 30_000, 150, 0.0, 3)
+    many = reads_of(bases(120, 4), 60_000, 120, 0.01, 5)
+    for label, sets in (("few", (spread, few)), ("many", (many, spread, few)),
+                        ("distinct", (few, crowd(40_000, m, k - m, 6), spread)),
+                        ("alone", (crowd(40_000, m, k - m, 6), spread)),
+                        ("rejected", (crowd(1500, m, k - m, 7), spread))):
+        reads, offs = join(*sets)
+        want = oracle.count(reads, offs, k, lo, hi)
+        with hsk.Context() as ctx:
+            for _ in range(2):
+                assert_same_result(ctx.count(reads, offs, k, m, lo, hi), want, f"k={k} {label}")
+            s = ctx.hash_stats()
+            assert s["heavy"] > 0 and s["sorted"] == 0 and (s["overfull"] > 0 or label != "rejected"), (label, s)
+            assert label != "many" or s["pairs"] > 20_000, s  # slices that outgrew the table
+            ctx.debug_limit("pairs", 4000)
+            assert_same_result(ctx.count(reads, offs, k, m, lo, hi), want, f"k={k} {label}, sorted")
+            t = ctx.hash_stats()
+            assert t["sorted"] == (s["heavy"] if s["pairs"] > 4000 else 0), (label, s, t)
+
+
+@pytest.mark.parametrize("around", [-1, 0, 1])
+@pytest.mark.parametrize("k,m,most", [(31, 17, 16384), (55, 21, 6144)])
+def test_either_side_of_a_heavy_partition(hsk, k, m, most, around):
+    """Exactly so many records, all in one partition: reads of a full record (two
+    when they cross a 1024-window tile), then reads of one k-mer."""
+    per = (60 if k <= 32 else 124) - k + 1
+    length, at, n_rec, lens = per + k - 1, 0, 0, []
+    while n_rec < most + around:
+        full = n_rec + 2 <= most + around
+        lens.append(length if full else k)
+        n_rec += (at + per - 1) // 1024 - at // 1024 + 1 if full else 1
+        at += lens[-1]
+    offs = np.cumsum([0] + lens).astype(np.uint64)
+    reads = np.full(at, ord("A"), np.uint8)
+    want = oracle.count(reads, offs, k, 1, 1 << 30)
+    with hsk.Context() as ctx:
+        assert_same_result(ctx.count(reads, offs, k, m, 1, 1 << 30), want, f"{most + around}")
+        s = ctx.hash_stats()
+    assert s["heavy"] == (1 if around > 0 else 0) and s["heavy"] + s["overfull"] == 1, s
+
+
+@pytest.mark.parametrize("k,m", [(31, 17), (55, 21)])
+def test_heavy_partitions_of_packed_sets(hsk, k, m):
+    """The same k-mers are heavy in several sets of a pack, and counted for each."""
+    spread = reads_of(bases(300_000, 1), 20_000, 150, 0.002, 2)
+    jobs = [spread] + [join(reads_of(poly("A", 1000), 30_000 + 1000 * i, 150, 0.002 * i, 3 + i),
+                            reads_of(bases(30_000, 9), 3000, 150, 0.0, 20 + i)) for i in range(4)] + [spread]
+    wants = [oracle.count(r, o, k, 2, 1 << 20) for r, o in jobs]
+    for limit in (None, 100):
+        with hsk.Context() as ctx:
+            ctx.tune_set(slots=1)
+            if limit:
+                ctx.debug_limit("pairs", limit)
+            for _ in range(2):
+                for i, (g, w) in enumerate(zip(ctx.count_batch([(r, o, k, m, 2, 1 << 20) for r, o in jobs]), wants)):
+                    assert_same_result(g, w, f"k={k} set {i}")
+            st = ctx.pack_stats()
+        assert st["sets"] == 2 * len(jobs) and st["failed_passes"] == 0, st
+        assert st["alone"] == (8 if limit else 0), st
