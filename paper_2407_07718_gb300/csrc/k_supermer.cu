@@ -27,8 +27,8 @@
 // writes per-window keys and scores for the stage test.
 //
 // The kernel is bound by the integer pipe (ncu: 75 % busy, 67 thread
-// instructions per window).  With 32 windows a lane it takes 3.9 ms on 1.5 G
-// windows of long reads (k = 31, w = 15) and 4.7 ms on 1.27 G of short reads (k
+// instructions per window).  With 32 windows a lane it takes 3.7 ms on 1.5 G
+// windows of long reads (k = 31, w = 15) and 4.6 ms on 1.27 G of short reads (k
 // = 55, w = 35), with 32 warps a CTA; 8 warps and three CTAs per SM took 4.4 and
 // 5.4 ms (fewer registers allow 32 warps per SM instead of 24, and one table
 // serves them all).  One window a lane and step, with the window minima and the
@@ -204,7 +204,7 @@ __device__ __forceinline__ void mmer_scores32(u64 W0, u64 W1, int m, uint32_t se
     }
 }
 
-template <int MODE, bool SHORT, bool LEX, bool TWO_ENDED>
+template <int MODE, bool SHORT, bool LEX, bool FINE, bool TWO_ENDED>
 __global__ void __launch_bounds__(SM_CTA_WARPS * 32, 1) k_supermer(const __grid_constant__ SmParams P) {
     extern __shared__ __align__(16) unsigned char smem[];
     u64* s_pk = reinterpret_cast<u64*>(smem);
@@ -213,15 +213,15 @@ __global__ void __launch_bounds__(SM_CTA_WARPS * 32, 1) k_supermer(const __grid_
     u64* s_rs = s_iv + warps * SM_MW;
     u64* s_val = s_rs + warps * SM_MW;
     uint32_t* s_rows = reinterpret_cast<uint32_t*>(s_val + warps * SM_VW);
-    uint32_t* s_cnt = s_rows + warps * SM_ROWS;  // DESC
-    uint32_t* s_km = s_cnt + P.n_buckets;           // DESC
+    uint32_t* s_km = s_rows + warps * SM_ROWS;  // DESC: k-mers per bucket
+    uint32_t* s_cnt = s_km + P.n_buckets;       // DESC without fine partitions: records per bucket
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t B = P.n_buckets;
     const int k = P.k, m = P.m, w = P.w, nmax = P.nmax;
 
     if (MODE == SM_DESC) {
-        for (uint32_t b = threadIdx.x; b < B; b += blockDim.x) s_cnt[b] = s_km[b] = 0;
+        for (uint32_t b = threadIdx.x; b < (FINE ? B : 2 * B); b += blockDim.x) s_km[b] = 0;
         __syncthreads();
     }
 
@@ -375,17 +375,18 @@ __global__ void __launch_bounds__(SM_CTA_WARPS * 32, 1) k_supermer(const __grid_
                     const bool down = TWO_ENDED && (id & 1u);
                     const u64 at = down ? P.desc_cap - 1 - at1++ : at0++;  // past the capacity: not written
                     if (at < P.desc_cap)
-                        P.desc[at] = make_desc(p0 + pos, (uint32_t)n, b | (id >> bb) << 13, P.part_rec != nullptr);
+                        P.desc[at] = make_desc(p0 + pos, (uint32_t)n, b | (id >> bb) << 13, FINE);
                 };
                 // Records per fine partition: one atomic for all pieces of a run, and the
                 // records of the first window's partition added up over the tile.  Reads
                 // crowded around one minimizer have nearly all of theirs there, and an
                 // atomic per record queues at its address, 1.3 a nanosecond: 150 Mbp of
                 // one-base reads took 3.3 ms (now 0.45), with 1 % errors 3.8 (now 0.58).
-                // Other reads pay 3 % of the walk for it.
-                const uint32_t id0 = min(rows[0], row_at(rows, 0, off)) & idmask;
-                const uint32_t hot = part_of(id0, bucket_of(id0));
-                uint32_t hot_n = 0;
+                // Other reads pay 3 % of the walk for it, and get as much back from kernels
+                // of their own for fine partitions.
+                [[maybe_unused]] const uint32_t id0 = min(rows[0], row_at(rows, 0, off)) & idmask;
+                [[maybe_unused]] const uint32_t hot = part_of(id0, bucket_of(id0));
+                [[maybe_unused]] uint32_t hot_n = 0;
                 for (uint32_t S = start; S; S &= S - 1) {
                     const int j = __ffs(S) - 1;
                     const uint32_t rest = ev & ~((2u << j) - 1u);
@@ -398,7 +399,7 @@ __global__ void __launch_bounds__(SM_CTA_WARPS * 32, 1) k_supermer(const __grid_
                         extra += more << (TWO_ENDED && (id & 1u) ? 16 : 0);
                         n_rec += more;
                     }
-                    if (P.part_rec) {
+                    if (FINE) {
                         const uint32_t part = part_of(id, b);
                         if (part == hot) hot_n += n_rec;
                         else atomicAdd(P.part_rec + part, n_rec);
@@ -408,8 +409,10 @@ __global__ void __launch_bounds__(SM_CTA_WARPS * 32, 1) k_supermer(const __grid_
                     atomicAdd(&s_km[b], (uint32_t)len);
                     put(32 * lane + j, min(len, nmax), id, b);
                 }
-                hot_n = __reduce_add_sync(0xffffffffu, hot_n);
-                if (lane == 0 && hot_n) atomicAdd(P.part_rec + hot, hot_n);
+                if (FINE) {
+                    hot_n = __reduce_add_sync(0xffffffffu, hot_n);
+                    if (lane == 0 && hot_n) atomicAdd(P.part_rec + hot, hot_n);
+                }
                 if (__any_sync(0xffffffffu, extra)) {
                     const uint32_t xi = warp_incl_sum<uint32_t>(extra);
                     at0 = at1 = 0;
@@ -431,7 +434,7 @@ __global__ void __launch_bounds__(SM_CTA_WARPS * 32, 1) k_supermer(const __grid_
     if (MODE == SM_DESC) {
         __syncthreads();
         for (uint32_t b = threadIdx.x; b < B; b += blockDim.x) {
-            if (s_cnt[b]) atomicAdd(P.bucket_rec + b, s_cnt[b]);
+            if (!FINE && s_cnt[b]) atomicAdd(P.bucket_rec + b, s_cnt[b]);
             if (s_km[b]) atomicAdd(reinterpret_cast<unsigned long long*>(P.bucket_kmers + b),
                                    (unsigned long long)s_km[b]);
         }
@@ -439,16 +442,19 @@ __global__ void __launch_bounds__(SM_CTA_WARPS * 32, 1) k_supermer(const __grid_
 }
 
 using SmKernel = void (*)(SmParams);
-template <int MODE, bool TWO_ENDED>
+template <int MODE, bool FINE, bool TWO_ENDED>
 static SmKernel walk_kernel(int m, bool lexical) {
     if (m <= 16)
-        return lexical ? (SmKernel)k_supermer<MODE, true, true, TWO_ENDED> : (SmKernel)k_supermer<MODE, true, false, TWO_ENDED>;
-    return lexical ? (SmKernel)k_supermer<MODE, false, true, TWO_ENDED> : (SmKernel)k_supermer<MODE, false, false, TWO_ENDED>;
+        return lexical ? (SmKernel)k_supermer<MODE, true, true, FINE, TWO_ENDED>
+                       : (SmKernel)k_supermer<MODE, true, false, FINE, TWO_ENDED>;
+    return lexical ? (SmKernel)k_supermer<MODE, false, true, FINE, TWO_ENDED>
+                   : (SmKernel)k_supermer<MODE, false, false, FINE, TWO_ENDED>;
 }
-static SmKernel walk_kernel(int mode, int m, bool lexical, bool two_ended) {
-    SmKernel fn = mode != SM_DESC ? walk_kernel<SM_DUMP, false>(m, lexical)
-                  : two_ended     ? walk_kernel<SM_DESC, true>(m, lexical)
-                                  : walk_kernel<SM_DESC, false>(m, lexical);
+static SmKernel walk_kernel(int mode, int m, bool lexical, bool fine, bool two_ended) {
+    SmKernel fn = mode != SM_DESC ? walk_kernel<SM_DUMP, false, false>(m, lexical)
+                  : two_ended     ? walk_kernel<SM_DESC, true, true>(m, lexical)
+                  : fine          ? walk_kernel<SM_DESC, true, false>(m, lexical)
+                                  : walk_kernel<SM_DESC, false, false>(m, lexical);
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)supermer_smem_bytes(mode, SM_MAX_BUCKETS, SM_CTA_WARPS));
     return fn;
@@ -457,7 +463,7 @@ static SmKernel walk_kernel(int mode, int m, bool lexical, bool two_ended) {
 void launch_supermer(int mode, const SmParams& p, cudaStream_t st) {
     if (p.n_bases == 0) return;
     count_launch();
-    walk_kernel(mode, p.m, p.lexical, p.two_ended)<<<p.grid, p.warps * 32, supermer_smem_bytes(mode, p.n_buckets, p.warps), st>>>(p);
+    walk_kernel(mode, p.m, p.lexical, p.part_rec != nullptr, p.two_ended)<<<p.grid, p.warps * 32, supermer_smem_bytes(mode, p.n_buckets, p.warps), st>>>(p);
 }
 
 // As many warps a CTA as leave every SM one (at most SM_CTA_WARPS, at least 4):
@@ -470,7 +476,7 @@ void supermer_shape(int mode, int m, bool lexical, uint32_t n_buckets, uint64_t 
     const uint64_t per_sm = (n_tiles + num_sms - 1) / num_sms;
     *warps = (int)(per_sm < 4 ? 4 : per_sm > SM_CTA_WARPS ? SM_CTA_WARPS : per_sm);
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel(mode, m, lexical, false), *warps * 32,
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel(mode, m, lexical, true, false), *warps * 32,
                                                       supermer_smem_bytes(mode, n_buckets, *warps)) != cudaSuccess)
         n = 1;
     if (n < 1) n = 1;
