@@ -898,6 +898,50 @@ template <>
 struct RangeCfg<key128, 1> {
     static constexpr int CAP = 8192, CTAS = 1;
 };
+// A bin of more keys than this (they share 20 to 28 bits: variants of a few
+// sequences) would cost more to rank, each against the whole bin, than a sort of
+// the range by exchanges.  1.7 M pairs of 128-bit keys from one 400-base amplicon
+// took 5.4 ms all ranked, and 0.66 with 256 (512 0.66, 1024 0.63; other inputs
+// lose 0.1 with those); 64-bit keys are compared faster (150 Mbp of reads of one
+// base with errors, k = 21: 256 0.44, 512 0.37, 1024 0.31, all ranked 0.32; an
+// amplicon, k = 31: 0.35 with 1024, 0.43 with 2048).
+template <typename K>
+constexpr uint32_t range_crowd() { return sizeof(K) == 8 ? 1024 : 256; }
+
+// Sorts n pairs in shared memory by key: bitonic merges whose first step mirrors
+// the upper half, so that every exchange puts the smaller key first and n need not
+// be a power of two.  Starts with a barrier, ends with one.
+template <typename K>
+__device__ __noinline__ void sort_crowded(K* sk, uint32_t* sv, uint32_t n) {
+    const uint32_t half = n > 1 ? 1u << (31 - __clz(n - 1)) : 0u;  // half the power of two that holds n
+    auto exchange = [&](uint32_t i, uint32_t j) {
+        if (j >= n) return;
+        const K x = sk[i], y = sk[j];
+        if (key_lt(y, x)) {
+            sk[i] = y;
+            sk[j] = x;
+            const uint32_t v = sv[i];
+            sv[i] = sv[j];
+            sv[j] = v;
+        }
+    };
+    __syncthreads();
+    for (uint32_t w = 1; w <= half; w *= 2) {  // sorted runs of w -> of 2 w
+        for (uint32_t t = threadIdx.x; t < half; t += RS_NT) {
+            const uint32_t base = t / w * 2 * w, o = t & (w - 1);
+            exchange(base + o, base + 2 * w - 1 - o);
+        }
+        __syncthreads();
+        for (uint32_t d = w / 2; d > 0; d /= 2) {
+            for (uint32_t t = threadIdx.x; t < half; t += RS_NT) {
+                const uint32_t i = t / d * 2 * d + (t & (d - 1));
+                exchange(i, i + d);
+            }
+            __syncthreads();
+        }
+    }
+}
+
 uint32_t range_sort_cap(int key_words) { return key_words == 1 ? RangeCfg<u64, 0>::CAP : RangeCfg<key128, 0>::CAP; }
 
 template <typename K, int TIER>
@@ -915,7 +959,7 @@ __global__ void __launch_bounds__(RS_NT, RangeCfg<K, TIER>::CTAS)
     uint32_t* s_bin = sv + CAP;  // [RS_BINS] counts, then starts
     __shared__ uint32_t s_scr[RS_NT / 32];
     __shared__ u64 s_b[RS_GROUP + 1];
-    __shared__ uint32_t s_next;
+    __shared__ uint32_t s_next, s_crowd;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (;;) {
         __syncthreads();
@@ -940,6 +984,7 @@ __global__ void __launch_bounds__(RS_NT, RangeCfg<K, TIER>::CTAS)
             const uint32_t n = (uint32_t)len;
 #pragma unroll
             for (int t = 0; t < BPT; ++t) s_bin[t * RS_NT + tid] = 0;
+            if (tid == 0) s_crowd = 0;
             __syncthreads();
             K key[PT];
             uint32_t at[PT];
@@ -954,17 +999,36 @@ __global__ void __launch_bounds__(RS_NT, RangeCfg<K, TIER>::CTAS)
                 if (q < n) at[t] = atomicAdd(&s_bin[key_digit(key[t], shift, mask)], 1u);
             }
             __syncthreads();
-            uint32_t c[BPT], sum = 0;
+            uint32_t c[BPT], sum = 0, most = 0;
 #pragma unroll
             for (int t = 0; t < BPT; ++t) {
                 c[t] = s_bin[tid * BPT + t];
                 sum += c[t];
+                most = max(most, c[t]);
             }
+            if (most > range_crowd<K>()) s_crowd = 1;
             const uint32_t inc = warp_incl_sum<uint32_t>(sum);
             if (lane == 31) s_scr[warp] = inc;
             __syncthreads();
             uint32_t run = inc - sum;
             for (int w = 0; w < warp; ++w) run += s_scr[w];
+            if (s_crowd) {
+#pragma unroll
+                for (int t = 0; t < PT; ++t) {
+                    const uint32_t q = (uint32_t)t * RS_NT + tid;
+                    if (q < n) {
+                        sk[q] = key[t];
+                        sv[q] = vin[b + q];
+                    }
+                }
+                sort_crowded(sk, sv, n);
+                for (uint32_t q = tid; q < n; q += RS_NT) {
+                    kout[b + q] = sk[q];
+                    vout[b + q] = sv[q];
+                }
+                __syncthreads();
+                continue;
+            }
 #pragma unroll
             for (int t = 0; t < BPT; ++t) {
                 s_bin[tid * BPT + t] = run;

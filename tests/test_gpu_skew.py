@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 import oracle
-from gpu_util import ACGT, assert_same_result, bases, join, low_score_mmer, reads_of
+from gpu_util import ACGT, amplicon, assert_same_result, bases, join, low_score_mmer, reads_of
 
 pytestmark = pytest.mark.gpu
 
@@ -125,3 +125,38 @@ def test_heavy_partitions_of_packed_sets(hsk, k, m):
             st = ctx.pack_stats()
         assert st["sets"] == 2 * len(jobs) and st["failed_passes"] == 0, st
         assert st["alone"] == (8 if limit else 0), st
+
+
+@pytest.mark.parametrize("k,m,sizes", [(31, 17, (1023, 1024, 1025, 4000, 6143, 6144, 6145, 8192, 8193)),
+                                       (55, 21, (255, 256, 257, 2048, 4095, 4096, 4097, 8192, 8193))])
+@pytest.mark.parametrize("prefix", [9, 11, 13, 16])
+def test_output_keys_that_share_their_top_bits(hsk, k, m, sizes, prefix):
+    """So many k-mers with one prefix (of 18 to 32 bits) next to others: bins on
+    either side of what is ranked, ranges on either side of what fits an SM."""
+    sets = [reads_of(bases(30_000, 1), 4000, 150, 0.0, 2)]
+    for i, n in enumerate(sizes):
+        x = bases(n * k, 10 + i).reshape(n, k)
+        x[:, :prefix] = [0, 0, 1 + i % 3] + [i // 3] * 2 + [3] * (prefix - 5)  # below the reverse complement's start
+        sets.append((ACGT[x].reshape(-1), np.arange(n + 1, dtype=np.uint64) * np.uint64(k)))
+    for some in ([sets[0]] + sets[1:4], sets):
+        reads, offs = join(*some)
+        want = oracle.count(reads, offs, k, 1, 1000)
+        with hsk.Context() as ctx:
+            assert_same_result(ctx.count(reads, offs, k, m, 1, 1000), want, f"k={k} prefix {prefix}")
+
+
+def test_output_order_of_crowded_keys_is_not_quadratic(hsk):
+    """S6 on the variants of an amplicon's k-mers against as many k-mers of random
+    reads (fifteen times as long when every key is ranked in its bin)."""
+    crowd = amplicon(12_000_000, 1)
+    spread = reads_of(bases(1_000_000, 2), 60_000, 150, 0.0, 3)
+    with hsk.Context() as ctx:
+        ctx.profile()
+        ms = []
+        for reads, offs in (crowd, spread):
+            best = 1e9
+            for _ in range(5):
+                n = ctx.count(reads, offs, 55, 21, 1, 1000, copy=False).extra["n_pairs"]
+                best = min(best, ctx.profile_read()[0][6])
+            ms.append(best / n)
+    assert ms[0] < 8 * ms[1], ms
