@@ -153,8 +153,9 @@ uint64_t hsk_debug_last_overflow(hsk_ctx* ctx);
  * by hashing: [0] fine partitions (0: the whole job was sorted), [1] those too
  * full for the first table and left to the second, [2] those of so many records,
  * or too full for the second, that they were cut into slices, [3] (k-mer, count)
- * pairs the slices left, [4] partitions that went on to the sorting path. */
-#define HSK_N_HASH_STATS 5
+ * pairs the slices left, [4] partitions that went on to the sorting path; and
+ * [5] packed passes of the batched and served forms so far that did. */
+#define HSK_N_HASH_STATS 6
 int hsk_debug_hash_stats(hsk_ctx* ctx, uint64_t out[HSK_N_HASH_STATS]);
 /* Sets one of the context's built-in limits, so that small inputs reach what
  * lies beyond (results do not change; before the first batched or served call

@@ -492,9 +492,9 @@ class Context:
 
     def hash_stats(self) -> dict:
         """How the last counting call counted by hashing (hsk_debug_hash_stats)."""
-        a = (C.c_uint64 * 5)()
+        a = (C.c_uint64 * 6)()
         self._check(self.lib.hsk_debug_hash_stats(self.h, a))
-        return dict(zip(("partitions", "overfull", "heavy", "pairs", "sorted"), (int(x) for x in a)))
+        return dict(zip(("partitions", "overfull", "heavy", "pairs", "sorted", "packs"), (int(x) for x in a)))
 
     def last_overflow(self) -> int:
         """Keys of the last call that went through the global radix passes

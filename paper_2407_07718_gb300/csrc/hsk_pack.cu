@@ -34,13 +34,15 @@
 
 using namespace hsk;
 
-// Buckets of one set in a pack: about one bucket group per bucket (a group
-// holds a third of 256 sub-segments' on-chip capacity), a power of two.
+// Buckets of one set in a pack, a power of two: about one bucket group per bucket
+// (a group holds a third of 256 sub-segments' on-chip capacity), but never more
+// bases in one than the fine partitions of the hash count divide well (393,216,
+// with 128-bit keys 516,096), whatever group_div was tuned to.
 uint32_t hsk_pack_set_buckets(uint64_t n_bases, int key_words, uint64_t group_keys) {
-    const uint64_t groups = (n_bases + group_keys - 1) / group_keys;
+    const uint64_t most = std::min<uint64_t>(group_keys, (uint64_t)(hash_count_cap(key_words) / 2) << HASH_MAX_SUB_BITS);
+    const uint64_t groups = (n_bases + most - 1) / most;
     uint32_t b = 1;
     while (b < groups && b < HSK_PACK_MAX_SET_BUCKETS) b <<= 1;
-    (void)key_words;
     return b;
 }
 
@@ -146,6 +148,7 @@ static int pack_pass(hsk_ctx* c, std::vector<PackSet*>& sets, const std::vector<
     CK(cudaMemsetAsync(c->small, 0, 64, st));
     CK(cudaMemsetAsync(c->counters, 0, HSK_N_COUNTERS * sizeof(uint32_t), st));
     c->ctr_used = 0;
+    c->pass_hashed = false;
 
     // ---- inputs and set tables to the device
     TRY(hsk_ensure(c, c->in_reads, NB + 64, false));
@@ -278,6 +281,7 @@ static int pack_pass(hsk_ctx* c, std::vector<PackSet*>& sets, const std::vector<
         HashRun R;
         TRY(hsk_hash_tiers(c, SMR.records, (const uint64_t*)c->part_off.p, B_total << sub_bits, SMR, k, lo, hi, H, S,
                            at.data(), (const uint32_t*)c->batch_d.p, d_max, R, st));
+        c->pass_hashed = true;
         if (R.n_left) {  // sets with a partition that no tier holds: counted again alone
             std::vector<uint32_t> left(R.n_left);
             CK(cudaMemcpyAsync(left.data(), R.list, (size_t)R.n_left * 4, cudaMemcpyDeviceToHost, st));

@@ -301,6 +301,7 @@ extern "C" int hsk_debug_limit(hsk_ctx* c, int which, uint64_t value) {
 extern "C" int hsk_debug_hash_stats(hsk_ctx* c, uint64_t* out) {
     if (!c || !out) return HSK_EINVAL;
     memcpy(out, c->hash_stats, sizeof(c->hash_stats));
+    out[HSK_N_HASH_STATS - 1] = c->pack_hashed.load();
     return HSK_OK;
 }
 

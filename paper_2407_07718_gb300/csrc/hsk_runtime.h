@@ -342,6 +342,8 @@ struct hsk_ctx {
     // packed passes run for this context's batched and served jobs, the sets
     // they held, and the sets among them counted again alone
     std::atomic<uint64_t> pack_passes{0}, pack_sets{0}, pack_redo{0};
+    std::atomic<uint64_t> pack_hashed{0};  // of those passes, the ones that counted by hashing
+    bool pass_hashed = false;              // whether this (a slot's) context's last pass did
     std::atomic<uint64_t> pack_fail{0};  // passes that failed as a whole (their sets were counted alone)
     std::string pack_fail_msg;           // the last such failure's reason (under tune_mu)
 
@@ -352,7 +354,7 @@ struct hsk_ctx {
     double prof_ms[8] = {0};
     uint64_t prof_passes = 0;
     uint64_t limits[HSK_N_LIMITS] = {1ull << 24};           // hsk_debug_limit
-    uint64_t hash_stats[HSK_N_HASH_STATS] = {0};  // of the last counting call (hsk_debug_hash_stats)
+    uint64_t hash_stats[HSK_N_HASH_STATS - 1] = {0};  // of the last counting call (hsk_debug_hash_stats)
     uint64_t last_ov_keys = 0;  // keys of the last job that did not fit the on-chip sort
 
     std::vector<DevBuf*> all_bufs() {

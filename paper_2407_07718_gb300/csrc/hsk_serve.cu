@@ -240,6 +240,7 @@ static void worker_main(hsk_ctx* parent, ServeState* S, int slot) {
                 if (ps[i].alone) parent->pack_redo.fetch_add(1);
             }
             parent->pack_passes.fetch_add(1);
+            if (c->pass_hashed) parent->pack_hashed.fetch_add(1);
             parent->pack_sets.fetch_add(group.size());
         }
         lk.lock();
