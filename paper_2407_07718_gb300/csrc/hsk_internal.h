@@ -211,7 +211,8 @@ void launch_ov_gather(const uint64_t* sub_off, const uint32_t* ov_list, uint32_t
 
 // ---- S4 + S5 by hashing (k_hash.cu) -------------------------------------------
 constexpr int HASH_MAX_SUB_BITS = 8;             // fine partitions of a bucket: 2^8 at most
-constexpr uint64_t HASH_MAX_BASES = 1ull << 36;  // bases a descriptor with a sub-partition can address
+constexpr uint64_t HASH_MAX_BASES = 1ull << 36;  // bases a descriptor with a sub-partition can address (the size of the
+                                                 // partitions ends the hash path long before: hash_buckets)
 uint32_t hash_count_cap(int key_words);      // distinct k-mers the first tier's table holds
 uint32_t hash_slice_records(int key_words);  // records of a slice at least (a batch of tier 1)
 // What a count of partitions reads and where its results go: kept pairs to

@@ -438,13 +438,25 @@ uint32_t hsk_pick_buckets(hsk_ctx* c, uint64_t n_bases, int k) {
     if (c->cfg.n_buckets) return c->cfg.n_buckets;
     // small jobs: fewer buckets keep the per-CTA tables cheap
     if (n_bases < (1ull << 22)) return 256;
-    // 4096 buckets for both key widths.  128-bit keys fit half as many per
-    // sub-segment, but twice the groups (8192 buckets) measured about 1 ms
-    // slower on the short-read workload once the middle on-chip tier took
-    // the sub-segments over the first tier's capacity
+    // 4096 buckets for both key widths, by the sorting path: 128-bit keys fit half
+    // as many per sub-segment, but twice the groups (8192 buckets) measured about 1
+    // ms slower on the short-read workload once the middle on-chip tier took the
+    // sub-segments over the first tier's capacity.  The hash count takes more where
+    // it needs them (hash_buckets).
     (void)k;
     const uint32_t B = 4096;
     return c->tune.plain_bucket_shift ? std::max<uint32_t>(256, B >> c->tune.plain_bucket_shift) : B;
+}
+
+// Buckets for the hash count of n_windows (at most) when it fits, else 0: B, or
+// more of them where partitions of B buckets would be too large (over 3.2 G
+// windows of 64-bit keys with 4096 buckets, or a smaller B by plain_bucket_shift).
+// 8192 buckets take 6.4 G, and 8.5 G of 128-bit keys.
+static uint32_t hash_buckets(hsk_ctx* c, uint64_t n_windows, uint32_t B, int k, int m) {
+    const uint32_t most = c->cfg.n_buckets ? B : HSK_MAX_BUCKETS;
+    for (; B <= most; B *= 2)
+        if (hsk_hash_path_fits(c, n_windows, B, k, m)) return B;
+    return 0;
 }
 
 static void fill_sm_params(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, SmParams& P) {
@@ -1405,8 +1417,10 @@ static int run_count(hsk_ctx* c, const char* d_reads, const uint64_t* d_offsets,
     Supermers S;
     uint32_t B = hsk_pick_buckets(c, n_bases, k);
     int sub_bits = -1;
-    may_hash = may_hash && n_bases < HASH_MAX_BASES && hsk_hash_path_fits(c, n_bases, B, k, m);
+    const uint32_t hash_B = may_hash && n_bases < HASH_MAX_BASES ? hash_buckets(c, n_bases, B, k, m) : 0;
+    may_hash = hash_B != 0;
     if (may_hash) {
+        B = hash_B;
         // fine partitions of half a batch's k-mers at most
         for (sub_bits = 0; sub_bits < HASH_MAX_SUB_BITS;) {
             if (n_bases <= ((uint64_t)B << sub_bits) * (hash_count_cap(kw) / 2)) break;
