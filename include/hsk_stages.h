@@ -160,8 +160,19 @@ int hsk_debug_hash_stats(hsk_ctx* ctx, uint64_t out[HSK_N_HASH_STATS]);
 /* Sets one of the context's built-in limits, so that small inputs reach what
  * lies beyond (results do not change; before the first batched or served call
  * the serving slots take the limits too):
- *   HSK_LIMIT_PAIRS  (2^24) pairs of slices; with more, the sorting path. */
-enum { HSK_LIMIT_PAIRS = 0, HSK_N_LIMITS = 1 };
+ *   HSK_LIMIT_PAIRS           (2^24) pairs of slices; with more, the sorting path
+ *   HSK_LIMIT_ONE_SCATTER     (2^19) fine partitions scattered into at once; with
+ *                             more, in two halves
+ *   HSK_LIMIT_DESCRIPTORS     (none) supermers the walk has room for at first
+ *   HSK_LIMIT_COMPOSITE_BITS  (64) bits of an occurrence's k-mer and position that
+ *                             are sorted as one word; with more, as two */
+enum {
+    HSK_LIMIT_PAIRS = 0,
+    HSK_LIMIT_ONE_SCATTER = 1,
+    HSK_LIMIT_DESCRIPTORS = 2,
+    HSK_LIMIT_COMPOSITE_BITS = 3,
+    HSK_N_LIMITS = 4
+};
 int hsk_debug_limit(hsk_ctx* ctx, int which, uint64_t value);
 /* Failure detection without a GPU fault: runs the decoupled look-back wait
  * that the scans and radix passes use, on a predecessor status word that

@@ -484,7 +484,7 @@ class Context:
         return {"passes": a.value, "sets": b.value, "alone": c.value, "failed_passes": f.value,
                 "last_failure": msg}
 
-    LIMITS = ("pairs",)
+    LIMITS = ("pairs", "one_scatter", "descriptors", "composite_bits")
 
     def debug_limit(self, name: str, value: int):
         """Set a built-in limit for a test (hsk_debug_limit)."""

@@ -43,7 +43,7 @@ extern "C" int hsk_count_ext(hsk_ctx* c, const char* reads, const uint64_t* offs
             int ib = 1, pb = 1;
             while ((1ull << ib) <= np) ++ib;
             while ((1ull << pb) < n_bases) ++pb;
-            const bool wide = ib + pb > 64;
+            const bool wide = ib + pb > (int)c->limits[HSK_LIMIT_COMPOSITE_BITS];
             const int comp_bits = ib + pb;
             const size_t cb = wide ? 16 : 8;
             // occurrence offsets = exclusive scan of the kept counts

@@ -294,7 +294,8 @@ extern "C" int hsk_debug_fail_alloc_after(hsk_ctx* c, int n) {
 extern "C" uint64_t hsk_debug_allocated(hsk_ctx* c) { return c ? c->allocated : 0; }
 extern "C" uint64_t hsk_debug_last_overflow(hsk_ctx* c) { return c ? c->last_ov_keys : 0; }
 extern "C" int hsk_debug_limit(hsk_ctx* c, int which, uint64_t value) {
-    if (!c || which < 0 || which >= HSK_N_LIMITS) return HSK_EINVAL;
+    static const uint64_t most[HSK_N_LIMITS] = {1ull << 24, ~0ull, ~0ull, 64};
+    if (!c || which < 0 || which >= HSK_N_LIMITS || value > most[which]) return HSK_EINVAL;
     c->limits[which] = value;
     return HSK_OK;
 }
@@ -520,7 +521,8 @@ int hsk_supermers(hsk_ctx* c, const Encoded& E, int k, int m, uint32_t B, Superm
     // the partitions, then the second (long-read workload, 2^20 partitions: 6.0
     // ms in one go, 4.7 in two, for 0.3 ms more in the walk).  32-byte records
     // fill whole sectors and gain nothing (3.9 and 3.7 ms).
-    P.two_ended = F > (1u << 19) && k <= 32 && !sets;
+    P.two_ended = F > c->limits[HSK_LIMIT_ONE_SCATTER] && k <= 32 && !sets && B > 1;
+    cap = std::min(cap, c->limits[HSK_LIMIT_DESCRIPTORS]);
     S.B = B;
     S.h_bucket_kmers.resize(B);
     S.h_bucket_rec.resize((size_t)B + 1);
