@@ -160,7 +160,7 @@ int hsk_debug_hash_stats(hsk_ctx* ctx, uint64_t out[HSK_N_HASH_STATS]);
 /* Sets one of the context's built-in limits, so that small inputs reach what
  * lies beyond (results do not change; before the first batched or served call
  * the serving slots take the limits too):
- *   HSK_LIMIT_PAIRS           (2^24) pairs of slices; with more, the sorting path
+ *   HSK_LIMIT_PAIRS           (2^30) pairs of slices; with more, the sorting path
  *   HSK_LIMIT_ONE_SCATTER     (2^19) fine partitions scattered into at once; with
  *                             more, in two halves
  *   HSK_LIMIT_DESCRIPTORS     (none) supermers the walk has room for at first

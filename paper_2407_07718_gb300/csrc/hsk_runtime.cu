@@ -294,7 +294,7 @@ extern "C" int hsk_debug_fail_alloc_after(hsk_ctx* c, int n) {
 extern "C" uint64_t hsk_debug_allocated(hsk_ctx* c) { return c ? c->allocated : 0; }
 extern "C" uint64_t hsk_debug_last_overflow(hsk_ctx* c) { return c ? c->last_ov_keys : 0; }
 extern "C" int hsk_debug_limit(hsk_ctx* c, int which, uint64_t value) {
-    static const uint64_t most[HSK_N_LIMITS] = {1ull << 24, ~0ull, ~0ull, 64};
+    static const uint64_t most[HSK_N_LIMITS] = {1ull << 30, ~0ull, ~0ull, 64};
     if (!c || which < 0 || which >= HSK_N_LIMITS || value > most[which]) return HSK_EINVAL;
     c->limits[which] = value;
     return HSK_OK;
@@ -1177,13 +1177,15 @@ static bool fits_budget(hsk_ctx* c, const DevBuf& b, size_t bytes) {
     return b.cap >= bytes || c->allocated - b.cap + bytes + (2u << 20) <= c->budget;
 }
 
-// Partitions of a hash count ({first record, records, partition} in list) cut
-// into slices for all SMs, whose pairs are merged in a table.  *done = false: not
-// counted, as the slices leave too many pairs or the budget has no room for them.
-// The limit (2^24 pairs): so many k-mers that mostly differ fill the SMs on the
-// sorting path too.
-static int count_heavy(hsk_ctx* c, const HashJob& J, const std::vector<uint64_t>& list, uint64_t* d_pair_n,
-                       cudaStream_t st, bool* done) {
+// Partitions of a hash count ({first record, records, partition} in list; of
+// n_kmers k-mers at most) cut into slices for all SMs, whose pairs are merged in a
+// table.  *done = false: not counted, as the slices leave more pairs than the limit
+// or the budget has no room for them; the sorting path takes them then.  The limit
+// (2^30) is what 32-bit pair numbers and twice as many slots allow: mostly distinct
+// k-mers are counted faster so too (22 M of 64-bit keys around one minimizer 3.7
+// ms, sorted 9.4; 66 M 11.3 and 20.7).
+static int count_heavy(hsk_ctx* c, const HashJob& J, const std::vector<uint64_t>& list, uint64_t n_kmers,
+                       uint64_t* d_pair_n, cudaStream_t st, bool* done) {
     *done = false;
     const int kw = J.k <= 32 ? 1 : 2;
     uint64_t n_rec = 0;
@@ -1196,7 +1198,7 @@ static int count_heavy(hsk_ctx* c, const HashJob& J, const std::vector<uint64_t>
             const uint64_t s[3] = {list[i] + r, std::min(len, list[i + 1] - r), list[i + 2]};
             sl.insert(sl.end(), s, s + 3);
         }
-    const uint64_t cap = std::min<uint64_t>(c->limits[HSK_LIMIT_PAIRS], n_rec * J.nmax);
+    const uint64_t cap = std::min({c->limits[HSK_LIMIT_PAIRS], n_kmers, n_rec * J.nmax});
     const size_t kb = (size_t)kw * 8, bytes = cap * (kb + 4 + (J.bucket_set ? 4 : 0)) + sl.size() * 8;
     if (!fits_budget(c, c->heavy, bytes)) return HSK_OK;
     TRY(hsk_ensure(c, c->heavy, bytes, false));
@@ -1300,8 +1302,16 @@ int hsk_hash_tiers(hsk_ctx* c, const uint64_t* recs, const uint64_t* part_off, u
         std::vector<uint64_t> list(3 * (size_t)n_heavy);
         CK(cudaMemcpyAsync(list.data(), d_heavy, list.size() * 8, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
+        // at most the k-mers of the buckets they lie in
+        const uint64_t b0 = (uint64_t)(part_off - (const uint64_t*)c->part_off.p) >> SM.sub_bits;
+        std::vector<uint64_t> in(n_heavy);
+        for (size_t i = 0; i < in.size(); ++i) in[i] = b0 + (list[3 * i + 2] >> SM.sub_bits);
+        std::sort(in.begin(), in.end());
+        in.erase(std::unique(in.begin(), in.end()), in.end());
+        uint64_t n_kmers = 0;
+        for (uint64_t b : in) n_kmers += SM.h_bucket_kmers[b];
         bool done = false;
-        TRY(count_heavy(c, J, list, ctl + 6, st, &done));
+        TRY(count_heavy(c, J, list, n_kmers, ctl + 6, st, &done));
         if (!done)
             for (size_t i = 2; i < list.size(); i += 3) left.push_back((uint32_t)list[i]);
         TRY(read_ctl());

@@ -353,7 +353,7 @@ struct hsk_ctx {
     std::vector<std::pair<int, int>> marks;  // (event index, stage id; -1 = start)
     double prof_ms[8] = {0};
     uint64_t prof_passes = 0;
-    uint64_t limits[HSK_N_LIMITS] = {1ull << 24, 1ull << 19, ~0ull, 64};  // hsk_debug_limit
+    uint64_t limits[HSK_N_LIMITS] = {1ull << 30, 1ull << 19, ~0ull, 64};  // hsk_debug_limit
     uint64_t hash_stats[HSK_N_HASH_STATS - 1] = {0};  // of the last counting call (hsk_debug_hash_stats)
     uint64_t last_ov_keys = 0;  // keys of the last job that did not fit the on-chip sort
 
