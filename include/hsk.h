@@ -204,7 +204,8 @@ int hsk_host_unpin(void* p);
 typedef struct {
     uint32_t group_div;          /* keys of a bucket group = 256 x on-chip sub-segment capacity / group_div
                                     (jobs and packs that are counted by sorting) */
-    uint32_t plain_bucket_shift; /* large jobs run alone use (4096, or 8192 for k > 32) >> shift buckets */
+    uint32_t plain_bucket_shift; /* large jobs run alone use 4096 >> shift buckets (more where the
+                                    count by hashing needs them) */
     uint64_t pack_bases;         /* bases of one packed pass at most */
     uint64_t pack_small;         /* jobs of more bases run alone */
     int slots;                   /* serving slots (streams with their own arenas) */

@@ -203,8 +203,12 @@ int hsk_debug_host_pool_check(void);
  * CUDA events on its own stream at the boundaries of its stages and adds the
  * device time between them to per-stage totals:
  *   0 S1 encode, 1 S2 k-mers/minimizers + supermer count + bucket scan,
- *   2 S3 supermer scatter, 3 S4 record expansion + digit histograms,
- *   4 S4 radix passes, 5 S5 run-length count/filter/histogram, 6 S6 order.
+ *   2 S3 supermer scatter,
+ *   3 S4 keys written (sorting path only): expansion or partition of the records,
+ *   4 S4 + S5 count: the hash count, or the on-chip sort, or the radix passes,
+ *   5 S5 kept pairs: split by their top digit, or compacted; after radix passes
+ *     the run-length count, filter and histogram,
+ *   6 S6 order.
  * hsk_profile_read copies HSK_N_STAGES totals (ms) and the number of radix-pass
  * launches they include, then clears them when reset != 0.
  * hsk_launch_count: kernels launched by this library in this process so far. */

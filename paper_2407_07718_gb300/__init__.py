@@ -448,8 +448,8 @@ class Context:
         self._check(self.lib.hsk_stage_order(self.h, _tptr(keys_t), _tptr(counts_t), n, key_words, key_bits,
                                              _stream_ptr(stream)))
 
-    STAGES = ("S1 encode", "S2 k-mers+minimizers+count", "S3 scatter", "S4 expand+hist", "S4 radix passes",
-              "S5 rle+filter+hist", "S6 order")
+    STAGES = ("S1 encode", "S2 k-mers+minimizers+count", "S3 scatter", "S4 keys written (sorting path)",
+              "S4+S5 count", "S5 kept pairs", "S6 order")
 
     def profile(self, on: bool = True):
         self._check(self.lib.hsk_profile_enable(self.h, int(on)))

@@ -11,8 +11,8 @@
 //   the partitions on chip, straight from the records (k_hash.cu) -> S6 split
 //   the kept pairs by their top digit and sort the ranges.
 //
-// Where the partitions would not fit an SM (hsk_hash_path_fits), and for the
-// few that do not: S3 scatters into buckets (or the partitions' records are
+// Where the partitions would not fit an SM (hsk_hash_path_fits), and for single
+// ones that memory has no room for: S3 scatters into buckets (or the partitions' records are
 // gathered), buckets are grouped, S4 counts + scatters keys into (group, top
 // digit) sub-segments, S4/S5 sorts and counts each sub-segment on chip
 // (k_local.cu; the ones that do not fit go through the 8-bit LSD passes of
@@ -939,7 +939,9 @@ std::vector<uint32_t> hsk_group_buckets(const Supermers& S, uint32_t b0, uint32_
     return cut;
 }
 
-// Plan chunks of consecutive buckets whose keys fit the sort budget.
+// Plan chunks of consecutive buckets whose keys fit the budget of the sorting path,
+// whose run heads also limit a chunk to 0xF0000000 keys.  (The hash count holds
+// less per k-mer and has no such limit, but shares the plan.)
 int hsk_plan_chunks(hsk_ctx* c, const Supermers& S, int key_words,
                     std::vector<std::pair<uint32_t, uint32_t>>& chunks) {
     chunks.clear();

@@ -61,6 +61,12 @@ namespace hsk {
 // the short reads: 512 x 2 and 3840 entries 12.9 ms, 3584 13.3, 1024 x 1 and
 // 7680 14.1.  With the kept entries listed (emit): 3840 12.1 ms, 4032 (what two
 // CTAs can hold) 11.9; 64-bit keys 3072 4.72, 3200 4.76.
+//
+// Tier 1 (and 2), the whole count stage where partitions are overfull.  64-bit keys,
+// on 5 Mbp of long reads with repeats and on 30 kb sequenced 20,000 times: 1024
+// threads and 8192 entries 0.64 and 1.13 ms, 512 threads 0.65 and 1.18, 512 x 2 CTAs
+// and 4864 entries 0.59 and 1.34.  128-bit keys: 512 threads 2.30 and 6.13, 768 2.28
+// and 6.09, 1024 2.36 and 6.49.
 template <bool WIDE, int TIER>
 struct HashCfg;
 template <>

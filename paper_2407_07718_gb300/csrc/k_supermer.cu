@@ -30,8 +30,8 @@
 // instructions per window).  With 32 windows a lane it takes 3.7 ms on 1.5 G
 // windows of long reads (k = 31, w = 15) and 4.6 ms on 1.27 G of short reads (k
 // = 55, w = 35), with 32 warps a CTA; 8 warps and three CTAs per SM took 4.4 and
-// 5.4 ms (fewer registers allow 32 warps per SM instead of 24, and one table
-// serves them all).  One window a lane and step, with the window minima and the
+// 5.4 ms (64 registers allow 32 warps per SM instead of 24, for some 140 bytes a
+// thread spilled, and one table serves them all).  One window a lane and step, with the window minima and the
 // cuts found by shuffles and ballots across lanes, took 8.7 warp instructions
 // per window and 14.4 and 17.0 ms.  Right shifts done by the multiply pipe (12 %
 // busy) made no difference.
