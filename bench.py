@@ -55,7 +55,7 @@ NCU_PER_KEY = {
     # long-read workload, k=31: k_hash_count tiers 0 and 1, smsp__inst_executed.sum, DRAM bytes and
     # shared-memory wavefronts (l1tex__data_pipe_lsu_wavefronts_mem_shared.sum) of one count of the
     # full workload, one counter a run
-    ("long_read", "36754e016be9d5cb"): {"inst": 2.2121, "dram": 2.1101, "smem_wavefronts": 0.4340},
+    ("long_read", "86065891c0285906"): {"inst": 2.2111, "dram": 2.1097, "smem_wavefronts": 0.4343},
 }
 # Warp schedulers per SM (Blackwell): each issues at most one warp instruction
 # per cycle; the issue peak is SMs (queried from the device) x this x the SM

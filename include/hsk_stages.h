@@ -184,8 +184,9 @@ int hsk_debug_wait_timeout(hsk_ctx* ctx, uint32_t spin_limit);
 /* Packing of the batched and served forms: *passes = packed passes run so
  * far on this context (each counts several small jobs of one k, m and
  * filter together), *sets = jobs they held, *alone = jobs among those that a
- * pass could not finish (a sub-segment too large for the on-chip sort) and
- * that were then counted alone.  NULL outputs are skipped. */
+ * pass could not finish (a sub-segment too large for the on-chip sort, or
+ * overfull partitions with too many pairs for memory) and that were then
+ * counted alone.  NULL outputs are skipped. */
 int hsk_debug_pack_stats(hsk_ctx* ctx, uint64_t* passes, uint64_t* sets, uint64_t* alone);
 /* Packed passes that failed as a whole (their jobs were then counted alone,
  * so results are unaffected): *failed_passes (may be NULL) receives their
