@@ -999,14 +999,17 @@ __global__ void __launch_bounds__(RS_NT, RangeCfg<K, TIER>::CTAS)
                 if (q < n) at[t] = atomicAdd(&s_bin[key_digit(key[t], shift, mask)], 1u);
             }
             __syncthreads();
-            uint32_t c[BPT], sum = 0, most = 0;
+            uint32_t c[BPT], sum = 0;
 #pragma unroll
             for (int t = 0; t < BPT; ++t) {
                 c[t] = s_bin[tid * BPT + t];
                 sum += c[t];
-                most = max(most, c[t]);
             }
-            if (most > range_crowd<K>()) s_crowd = 1;
+            if (sum > range_crowd<K>()) {  // rare (looking at every bin: S6 of 54 M 64-bit pairs 1.15 -> 1.17 ms)
+#pragma unroll
+                for (int t = 0; t < BPT; ++t)
+                    if (c[t] > range_crowd<K>()) s_crowd = 1;
+            }
             const uint32_t inc = warp_incl_sum<uint32_t>(sum);
             if (lane == 31) s_scr[warp] = inc;
             __syncthreads();
